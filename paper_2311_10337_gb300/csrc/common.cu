@@ -21,6 +21,30 @@ dgec_status read_counters(Ctx *c, const int64_t *d, int n, int64_t *host) {
     CU_TRY(c, cudaMemcpyAsync(c->h_pinned, d, sizeof(int64_t) * n, cudaMemcpyDeviceToHost, c->stream));
     CU_TRY(c, cudaStreamSynchronize(c->stream));
     memcpy(host, c->h_pinned, sizeof(int64_t) * n);
+    return coop_check(c);
+}
+
+dgec_status coop_begin(Ctx *c, unsigned *bar) {
+    c->bar = bar;
+    *(volatile unsigned *)c->bar_err = 0u;
+    CU_TRY(c, cudaMemsetAsync(bar, 0, sizeof(unsigned) * kBarWords, c->stream));
+    return DGEC_OK;
+}
+
+dgec_status coop_check(Ctx *c) {
+    if (*(volatile unsigned *)c->bar_err) return set_err(c, DGEC_ERR_TIMEOUT, "a grid barrier gave up");
+    return DGEC_OK;
+}
+
+dgec_status coop_grid(Ctx *c, CoopKernel which, const void *fn, int threads, size_t smem, int *grid) {
+    if (!c->coop_ctas[which]) {
+        int per_sm = 0;
+        CU_TRY(c, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        CU_TRY(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem));
+        if (per_sm < 1) return set_err(c, DGEC_ERR_INTERNAL, "a cooperative kernel does not fit an SM");
+        c->coop_ctas[which] = per_sm * c->num_sms;
+    }
+    *grid = c->coop_ctas[which];
     return DGEC_OK;
 }
 

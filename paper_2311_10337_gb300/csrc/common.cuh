@@ -43,6 +43,9 @@ struct StageTimer {
     int n = 0;
 };
 
+// Cooperative kernels whose resident-CTA count a context remembers.
+enum CoopKernel { kCoopSortK, kCoopSortKV, kCoopCount };
+
 struct Ctx {
     int device = 0;
     int knn_block = 128;           // launch configuration (dgec_set_launch_config)
@@ -55,7 +58,19 @@ struct Ctx {
     cudaStream_t stream = nullptr;
     KernelTimer *kt = nullptr;
     StageTimer stages;
+    int coop_ctas[kCoopCount] = {};  // CTAs of each cooperative kernel the device holds at once; 0 = not asked yet
+    unsigned *bar = nullptr;         // barrier words of the current call (in its workspace)
+    unsigned *bar_err = nullptr;     // host-mapped: 1 once a grid barrier gave up
 };
+
+// The current call's barrier words, zeroed on its stream.
+constexpr int kBarWords = 64;
+dgec_status coop_begin(Ctx *c, unsigned *bar);
+// DGEC_ERR_TIMEOUT if a grid barrier gave up (after a stream synchronisation).
+dgec_status coop_check(Ctx *c);
+// How many CTAs of the kernel fit on the device at once (also raises its
+// dynamic shared memory limit).
+dgec_status coop_grid(Ctx *c, CoopKernel which, const void *fn, int threads, size_t smem, int *grid);
 
 void stage_start(Ctx *c);
 void stage_mark(Ctx *c, const char *name);
@@ -157,6 +172,16 @@ inline int bits_for(uint64_t maxval) {  // bits to hold values 0..maxval
     int b = 0;
     while (b < 64 && (maxval >> b) != 0) b++;
     return b;
+}
+
+// Launch a cooperative kernel of one by-value argument struct.
+template <class A>
+dgec_status coop_launch(Ctx *c, const char *name, const void *fn, int grid, int threads, size_t smem, A a) {
+    void *args[] = {&a};
+    cudaError_t e;
+    TK(c, name, e = cudaLaunchCooperativeKernel(fn, dim3((unsigned)grid), dim3((unsigned)threads), args, smem, c->stream));
+    if (e != cudaSuccess) return set_err(c, DGEC_ERR_CUDA, "%s launch: %s", name, cudaGetErrorString(e));
+    return DGEC_OK;
 }
 
 // Read n int64 counters from device memory (synchronises the stream).

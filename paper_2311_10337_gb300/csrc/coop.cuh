@@ -1,0 +1,64 @@
+// Cooperative building blocks: a grid barrier for kernels whose CTAs are all
+// resident (launched through coop_launch), and the stable LSD radix sort as
+// one such kernel.
+#pragma once
+
+#include "common.cuh"
+
+namespace dgec {
+
+// The barrier words of a call (kBarWords of them): [0] arrivals, [1] exits.
+// Zeroed once per call; the last CTA out of a kernel leaves them zero again.
+
+// Polls before a barrier gives up (about a microsecond each). CTAs of a
+// cooperative launch are co-resident, so this only bounds the wait should
+// that ever not hold.
+constexpr unsigned kBarPolls = 1u << 24;
+
+// Barrier over every CTA of a cooperative launch. Arrivals count up without
+// a reset between barriers (compared by signed difference). A barrier that
+// gives up writes 1 to *err (host-mapped memory) and returns false in every
+// thread of its CTA; the kernel must then return at once (the other CTAs
+// give up likewise).
+struct GridBar {
+    unsigned *word;
+    unsigned *err;
+    unsigned nblk, target;
+    __device__ __forceinline__ GridBar(unsigned *w, unsigned *e) : word(w), err(e), nblk(gridDim.x), target(0) {}
+    __device__ __forceinline__ bool sync() {
+        if (nblk == 1) {
+            __syncthreads();
+            return true;
+        }
+        __syncthreads();
+        bool bad = false;
+        target += nblk;
+        if (threadIdx.x == 0) {
+            __threadfence();
+            atomicAdd(word, 1u);
+            unsigned polls = 0;
+            for (;;) {
+                unsigned v;
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(word) : "memory");
+                if ((int)(v - target) >= 0) break;
+                if (++polls > kBarPolls) {
+                    bad = true;
+                    *(volatile unsigned *)err = 1u;
+                    break;
+                }
+            }
+            __threadfence();
+        }
+        return !__syncthreads_or(bad);
+    }
+    // every CTA calls this after its last barrier
+    __device__ __forceinline__ void finish() {
+        if (nblk == 1 || threadIdx.x != 0) return;
+        if (atomicAdd(word + 1, 1u) == nblk - 1) {
+            word[0] = 0u;
+            word[1] = 0u;
+        }
+    }
+};
+
+}  // namespace dgec

@@ -13,6 +13,7 @@ namespace {
 // Workspace = per-graph tables and outputs (kept) followed by one scratch
 // region that every stage reuses in turn (sized for the largest stage).
 struct Layout {
+    unsigned *bar;
     int64_t *eoff, *voff, *knn_off;
     int32_t *gk, *gM, *egraph;
     Csr csr;
@@ -70,6 +71,7 @@ Problem make_problem(const HostBatch &hb) {
 Layout plan(void *base, const Problem &p) {
     Layout L;
     Arena a(base, SIZE_MAX);
+    L.bar = a.take<unsigned>(kBarWords);
     L.eoff = a.take<int64_t>(p.G + 1);
     L.voff = a.take<int64_t>(p.G + 1);
     L.knn_off = a.take<int64_t>(p.G + 1);
@@ -193,6 +195,7 @@ dgec_status run_pipeline(Ctx *c, const HostBatch &hb, const int32_t *d_src, cons
     size_t need = plan(nullptr, p).total;
     if (ws_bytes < need) return set_err(c, DGEC_ERR_OOM, "workspace %zu bytes < %zu needed", ws_bytes, need);
     Layout L = plan(d_ws, p);
+    DG_TRY(coop_begin(c, L.bar));
     DG_TRY(upload_tables(c, hb, L.eoff, L.voff, L.knn_off, L.gk, L.gM));
     p.eoff = L.eoff;
     p.voff = L.voff;
@@ -227,6 +230,7 @@ dgec_status run_pipeline(Ctx *c, const HostBatch &hb, const int32_t *d_src, cons
                                 L.msf.goff, L.lmu, L.lmv, L.lla, L.llb));
     CU_TRY(c, cudaStreamSynchronize(c->stream));
     CU_TRY(c, cudaGetLastError());
+    DG_TRY(coop_check(c));
     kt_collect(c);
     stage_collect(c);
     *out_layout = L;
@@ -276,6 +280,7 @@ void fill_result(const Layout &L, dgec_result *out) {
 // ------------------------------------------------- discrete dendrogram run
 
 struct LvLayout {
+    unsigned *bar;
     int64_t *eoff, *voff, *knn_off;
     int32_t *gk, *gM, *egraph;
     Csr csr;
@@ -290,6 +295,7 @@ struct LvLayout {
 LvLayout plan_lv(void *base, const Problem &p, int q, bool dense, bool condense) {
     LvLayout L;
     Arena a(base, SIZE_MAX);
+    L.bar = a.take<unsigned>(kBarWords);
     L.eoff = a.take<int64_t>(2);
     L.voff = a.take<int64_t>(2);
     L.knn_off = a.take<int64_t>(2);
@@ -360,6 +366,7 @@ dgec_status dgec_create(dgec_ctx **out, int device) {
     cudaError_t e = cudaSetDevice(device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device);
     if (e == cudaSuccess) e = cudaMallocHost((void **)&c->h_pinned, 4096);
+    if (e == cudaSuccess) c->bar_err = (unsigned *)(c->h_pinned + 511);  // last word pair of the 4 KB, read and written by kernels too
     c->kt = new (std::nothrow) KernelTimer();
     if (e != cudaSuccess || !c->kt) {
         if (c->h_pinned) cudaFreeHost(c->h_pinned);
@@ -625,6 +632,7 @@ dgec_status dgec_run_levels(dgec_ctx *x, const int32_t *d_src, const int32_t *d_
     p.dst = d_dst;
     p.t = d_t;
     HostBatch hb = d.hb();
+    DG_TRY(coop_begin(c, L.bar));
     DG_TRY(upload_tables(c, hb, L.eoff, L.voff, L.knn_off, L.gk, L.gM));
     p.eoff = L.eoff;
     p.voff = L.voff;
@@ -644,6 +652,7 @@ dgec_status dgec_run_levels(dgec_ctx *x, const int32_t *d_src, const int32_t *d_
     }
     CU_TRY(c, cudaStreamSynchronize(c->stream));
     CU_TRY(c, cudaGetLastError());
+    DG_TRY(coop_check(c));
     kt_collect(c);
     stage_collect(c);
     out->sk_u = L.skel.u;

@@ -398,6 +398,7 @@ namespace {
 using namespace dgec;
 
 struct HLayout {
+    unsigned *bar;
     int64_t *eoff, *voff, *knn_off;
     int32_t *gk, *gM, *egraph;
     Csr csr;
@@ -427,6 +428,7 @@ Problem hyper_problem(const HyperProblem &h, int32_t M) {
 HLayout plan_hlayout(void *base, const HyperProblem &h, const Problem &p) {
     HLayout L;
     Arena a(base, SIZE_MAX);
+    L.bar = a.take<unsigned>(kBarWords);
     L.eoff = a.take<int64_t>(2);
     L.voff = a.take<int64_t>(2);
     L.knn_off = a.take<int64_t>(2);
@@ -514,6 +516,7 @@ dgec_status dgec_run_hyper(dgec_ctx *x, const int64_t *d_t, int64_t n_hyperedges
     size_t need = plan_hlayout(nullptr, h, p).total;
     if (ws_bytes < need) return set_err(c, DGEC_ERR_OOM, "workspace %zu bytes < %zu needed", ws_bytes, need);
     HLayout L = plan_hlayout(d_ws, h, p);
+    DG_TRY(coop_begin(c, L.bar));
     // the one-graph tables the shared stages read
     {
         int64_t tab[6] = {0, h.E, 0, h.V, 0, 0};
@@ -540,6 +543,7 @@ dgec_status dgec_run_hyper(dgec_ctx *x, const int64_t *d_t, int64_t n_hyperedges
     DG_STAGE("D2 condense and labels", stage_condense(c, p, L.msf, L.den, L.cond, L.scratch));
     CU_TRY(c, cudaStreamSynchronize(c->stream));
     CU_TRY(c, cudaGetLastError());
+    DG_TRY(coop_check(c));
     kt_collect(c);
     stage_collect(c);
     out->src_voff = L.S.voff;
