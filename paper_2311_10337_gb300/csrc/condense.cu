@@ -21,10 +21,11 @@
 // Everything is computed by data-parallel passes: pointer jumping for the
 // equal-weight runs and for "which cluster does this merge belong to",
 // short upward walks (< M steps) for where a point leaves, 128-bit atomics
-// for stabilities, and a rake-and-compress tree contraction over the
-// cluster tree for the EOM maximisation, whose per-node update
+// for stabilities, and upward walks plus a rake-and-compress contraction of
+// what they leave for the EOM maximisation, whose per-node update
 // S = max(stab, sum of children) composes along unary chains as
 // x -> max(a, c + x).
+#include "coop.cuh"
 #include "stages.cuh"
 
 namespace dgec {
@@ -329,33 +330,35 @@ __global__ void k_c_compact(int64_t E, int64_t m, const int *isc, const long lon
 
 struct Eom {
     int64_t ncl;
-    int64_t R0;  // node ids >= R0 are virtual roots (never selected)
+    int64_t root0;  // clusters [root0, ncl) are the virtual roots (never selected, nothing reads their sums)
+    int64_t R0;     // node ids >= R0 are virtual roots
     const int32_t *clist, *cidx, *cparent;  // cparent by node id
     int32_t *par;                            // compact parent, -1 root
-    int *pending, *done, *state;             // state: 1 done this phase
+    int *pending, *done, *fin;
     u128 *stab, *S, *Fa, *Fc, *Fa2, *Fc2;
-    unsigned long long *acc_hi, *acc_lo;
-    int32_t *ucand, *nxt, *nxt2;
-    const int32_t *alist;  // open clusters this phase
-    int64_t nact;
-    unsigned long long *flag;  // [0] changed
+    const unsigned long long *csz;        // total size of the child clusters (0: none)
+    unsigned long long *acc_hi, *acc_lo;  // sum of the children's S
+    int32_t *ucand, *nxt, *nxt2, *al, *al2;
+    unsigned long long *slot;  // (next ancestor << 32) | highest selected on the way there
+    int32_t *H;                // highest selected ancestor-or-self, -1
+    unsigned long long *cnt;   // [0], [1] open clusters, [2..4] flags, [5] error; zeroed before the kernel
+    unsigned *bar, *err;
 };
 
 __global__ void k_e_init(Eom e, const unsigned long long *st_hi, const unsigned long long *st_lo,
-                         const unsigned long long *cbirth, const unsigned long long *cdeath,
-                         const unsigned long long *csz) {
+                         const unsigned long long *cbirth, const unsigned long long *cdeath) {
     for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < e.ncl;
          c += (int64_t)gridDim.x * blockDim.x) {
         int node = e.clist[c];
         int pn = e.cparent[node];
         e.par[c] = pn < 0 ? -1 : e.cidx[pn];
-        const unsigned long long kids = csz[c];
+        const unsigned long long kids = e.csz[c];
         const u128 from_kids = kids ? (u128)(cdeath[node] - cbirth[node]) * kids : (u128)0;
         e.stab[c] = (((u128)st_hi[node] << 64) | st_lo[node]) + from_kids;
         e.done[c] = 0;
         e.acc_hi[c] = 0;
         e.acc_lo[c] = 0;
-        if (pn >= 0) atomicAdd(&e.pending[e.cidx[pn]], 1);
+        if (pn >= 0 && pn < e.R0) atomicAdd(&e.pending[e.par[c]], 1);
     }
 }
 
@@ -363,209 +366,209 @@ __device__ __forceinline__ u128 acc_of(const Eom &e, int64_t c) {
     return ((u128)e.acc_hi[c] << 64) | e.acc_lo[c];
 }
 
-// unary clusters learn their one pending child; F = (stab, acc)
-__global__ void k_e_unary(Eom e) {
-    for (int64_t ix = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; ix < e.nact;
-         ix += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t c = e.alist[ix];
-        e.state[c] = 0;
-        if (e.done[c]) continue;
-        int p = e.par[c];
-        if (p >= 0 && e.pending[p] == 1) e.ucand[p] = (int32_t)c;
+__device__ __forceinline__ void acc_add(const Eom &e, int p, u128 s) {
+    atomic_add_u128(&e.acc_hi[p], &e.acc_lo[p], (unsigned long long)(s >> 64), (unsigned long long)s);
+}
+
+// From a cluster c whose children have all reported, up while this thread is
+// the last child to report: S = max(stab, sum of the children's S) is added
+// to the parent's sum, and the last report makes the parent ready. At most
+// kEomWalk clusters; the one reached then stays open (ready, not done).
+constexpr int kEomWalk = 24;
+__device__ __forceinline__ void e_walk(const Eom &e, int c) {
+    for (int step = 0; step < kEomWalk; step++) {
+        const u128 acc = ((u128) * (volatile unsigned long long *)&e.acc_hi[c] << 64) |
+                         *(volatile unsigned long long *)&e.acc_lo[c];
+        const u128 st = e.stab[c];
+        const int p = e.par[c];
+        e.done[c] = 1;
+        if (p < 0 || p >= e.root0) return;
+        acc_add(e, p, st > acc ? st : acc);
+        __threadfence();
+        if (atomicSub(&e.pending[p], 1) != 1) return;
+        __threadfence();
+        c = p;
     }
 }
 
-__global__ void k_e_fninit(Eom e) {
-    for (int64_t ix = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; ix < e.nact;
-         ix += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t c = e.alist[ix];
-        if (!e.done[c] && e.pending[c] == 1) {
-            e.nxt[c] = e.ucand[c];
-            e.Fa[c] = e.stab[c];
-            e.Fc[c] = acc_of(e, c);
-        } else {
-            e.nxt[c] = -1;
+// Excess of mass over the cluster tree in one cooperative kernel: every
+// cluster's sum of its children's S = max(stab, that sum), then for every
+// cluster its highest selected ancestor-or-self (selected: stab >= the sum,
+// ties to the parent; a virtual root never).
+//   1. Every leaf cluster walks up (e_walk): all subtrees of height up to
+//      kEomWalk, which is nearly every cluster, are done in this one pass.
+//   2. What stays open are the long spines. Contraction over the open list
+//      only: runs of clusters with one open child compose x -> max(a, c + x)
+//      by doubling; runs that end in a ready cluster resolve and report to
+//      the parent above, whose last report walks on. Repeated until nothing
+//      is open; a phase at least halves the spines' branchings.
+//   3. Walks toward the root that leave a (next, highest selected) shortcut
+//      in their slot, in descending order, so the clusters near the root
+//      finish first and later walks are short; a walk cut at kTopWalk steps
+//      is taken up again in another round.
+// What bounds it: the random 8 and 16-byte accesses of the walks' reports at
+// large trees, the barriers (about 2 us each) of the contraction at small ones.
+// Against a contraction of the whole tree phase by phase (up to 160 launches
+// and a host read every other one; a serial sweep up to 4,096 clusters): 0.06 ms
+// for 0.55 at 20,000 edges, 0.63 for 2.7 at 10M, 4.7 for about 15 at 100M hub
+// edges.
+__global__ void __launch_bounds__(256, 4) k_e_tree(Eom e) {
+    GridBar bar(e.bar, e.err);
+    const int64_t gsize = (int64_t)gridDim.x * blockDim.x, g0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
+    for (int64_t c = g0; c < e.root0; c += gsize)
+        if (e.csz[c] == 0) e_walk(e, (int)c);  // no child cluster
+    if (!bar.sync()) return;
+    int32_t *al = e.al, *al2 = e.al2;
+    int64_t nact = e.root0;
+    for (int phase = 0;; phase++) {
+        if (phase > 4096) {
+            if (lead) e.cnt[5] = 1;
+            break;
         }
-    }
-}
-
-// one synchronous doubling step: F(c) <- F(c) o F(nxt c) while nxt is unary
-__global__ void k_e_double(Eom e, const int32_t *nin, int32_t *nout, const u128 *ain, const u128 *cin,
-                           u128 *aout, u128 *cout) {
-    bool moved = false;
-    for (int64_t ix = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; ix < e.nact;
-         ix += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t c = e.alist[ix];
-        int x = nin[c];
-        u128 a = ain[c], cc = cin[c];
-        if (x >= 0 && nin[x] >= 0) {
-            // x is unary: compose (apply x's function first)
-            u128 a2 = ain[x], c2 = cin[x];
-            u128 t = cc + a2;
-            a = a > t ? a : t;
-            cc = cc + c2;
-            x = nin[x];
-            moved = true;
+        // the open clusters; each tells a parent that waits for it alone
+        for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < nact; base += gsize) {  // CTA-uniform
+            const int64_t ix = base + threadIdx.x;
+            bool open = false;
+            int c = 0;
+            if (ix < nact) {
+                c = phase == 0 ? (int)ix : al[ix];
+                open = !e.done[c];
+                if (open) {
+                    const int p = e.par[c];
+                    if (p >= 0 && p < e.root0 && e.pending[p] == 1) e.ucand[p] = c;
+                }
+            }
+            const long long at = cta_reserve(open, e.cnt + (phase & 1));
+            if (open) al2[at] = c;
         }
-        nout[c] = x;
-        aout[c] = a;
-        cout[c] = cc;
-    }
-    if (__any_sync(0xffffffffu, moved) && lane_id() == 0) e.flag[0] = 1;
-}
-
-// rake ready clusters (all children done)
-__global__ void k_e_rake(Eom e) {
-    for (int64_t ix = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; ix < e.nact;
-         ix += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t c = e.alist[ix];
-        if (e.done[c] || e.pending[c] != 0) continue;
-        u128 acc = acc_of(e, c);
-        e.S[c] = e.stab[c] > acc ? e.stab[c] : acc;
-        e.state[c] = 1;
-    }
-}
-
-// unary clusters whose chain bottom was just raked resolve through F
-__global__ void k_e_resolve(Eom e, const int32_t *nfin, const u128 *afin, const u128 *cfin) {
-    for (int64_t ix = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; ix < e.nact;
-         ix += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t c = e.alist[ix];
-        if (e.done[c] || e.pending[c] != 1) continue;
-        int x = nfin[c];
-        if (x < 0 || e.state[x] != 1 || e.pending[x] != 0) continue;
-        u128 t = cfin[c] + e.S[x];
-        e.S[c] = afin[c] > t ? afin[c] : t;
-        e.state[c] = 2;
-    }
-}
-
-// clusters finished this phase report to a parent that is still open
-__global__ void k_e_report(Eom e) {
-    for (int64_t ix = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; ix < e.nact;
-         ix += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t c = e.alist[ix];
-        if (!e.state[c]) continue;
-        int p = e.par[c];
-        if (p >= 0 && !e.state[p] && !e.done[p]) {
-            u128 s = e.S[c];
-            atomic_add_u128(&e.acc_hi[p], &e.acc_lo[p], (unsigned long long)(s >> 64),
-                            (unsigned long long)s);
-            atomicSub(&e.pending[p], 1);
+        if (!bar.sync()) return;
+        nact = (int64_t) * (volatile unsigned long long *)(e.cnt + (phase & 1));
+        if (nact == 0) break;
+        {
+            int32_t *t = al;
+            al = al2;
+            al2 = t;
         }
-    }
-}
-
-__global__ void k_e_commit(Eom e, int32_t *alist2, unsigned long long *n_open) {
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < e.nact;
-         base += (int64_t)gridDim.x * blockDim.x) {  // CTA-uniform
-        int64_t ix = base + threadIdx.x;
-        bool open = false;
-        int64_t c = 0;
-        if (ix < e.nact) {
-            c = e.alist[ix];
-            if (e.state[c]) e.done[c] = 1;
-            open = !e.done[c];
+        for (int64_t ix = g0; ix < nact; ix += gsize) {
+            const int c = al[ix];
+            const int pd = e.pending[c];
+            const u128 acc = acc_of(e, c), st = e.stab[c];
+            if (pd == 0) e.S[c] = st > acc ? st : acc;
+            e.nxt[c] = pd == 1 ? e.ucand[c] : -1;
+            e.Fa[c] = st;
+            e.Fc[c] = acc;
         }
-        long long at = cta_reserve(open, n_open);
-        if (open) alist2[at] = (int32_t)c;
-    }
-}
-
-// Small cluster trees (at most kEomSmall clusters) in one CTA. Clusters are
-// numbered in ascending node id, and a parent cluster starts at a merge
-// above its children's, so every child comes before its parent: one
-// bottom-up sweep gives S = max(stab, sum of children's S) and the
-// children's sums, one top-down sweep the highest selected ancestor-or-self.
-// The sweeps are sequential (one thread, shared memory); loading and storing
-// are spread over the CTA. Same results as the contraction below.
-constexpr int kEomSmall = 4096;
-constexpr int kEomThreads = 1024;
-constexpr size_t kEomSmem = (size_t)kEomSmall * (16 + 16 + 4 + 4);
-__global__ void __launch_bounds__(kEomThreads) k_e_small(Eom e, int32_t *H) {
-    extern __shared__ __align__(16) unsigned long long esm[];
-    u128 *sst = reinterpret_cast<u128 *>(esm);       // stab
-    u128 *sacc = sst + kEomSmall;                    // children's S
-    int32_t *spar = reinterpret_cast<int32_t *>(sacc + kEomSmall);
-    int32_t *sh = spar + kEomSmall;
-    const int n = (int)e.ncl;
-    for (int c = threadIdx.x; c < n; c += kEomThreads) {
-        sst[c] = e.stab[c];
-        sacc[c] = 0;
-        spar[c] = e.par[c];
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int c = 0; c < n; c++) {  // children first
-            const u128 a = sacc[c], st = sst[c];
-            const int p = spar[c];
-            if (p >= 0) sacc[p] += st > a ? st : a;
+        if (lead) e.cnt[(phase & 1) ^ 1] = 0;
+        if (!bar.sync()) return;
+        int32_t *ni = e.nxt, *no = e.nxt2;
+        u128 *ai = e.Fa, *ao = e.Fa2, *ci = e.Fc, *co = e.Fc2;
+        for (int it = 0;; it++) {  // at most 32: chains are shorter than 2^31
+            bool moved = false;
+            for (int64_t ix = g0; ix < nact; ix += gsize) {
+                const int c = al[ix];
+                int x = ni[c];
+                u128 a = ai[c], cc = ci[c];
+                if (x >= 0) {
+                    const int nx = ni[x];
+                    if (nx >= 0) {  // x is unary: compose (x's function applies first)
+                        const u128 t = cc + ai[x];
+                        a = a > t ? a : t;
+                        cc = cc + ci[x];
+                        x = nx;
+                        moved = true;
+                    }
+                }
+                no[c] = x;
+                ao[c] = a;
+                co[c] = cc;
+            }
+            if (__syncthreads_or(moved) && threadIdx.x == 0) *(volatile unsigned long long *)(e.cnt + 2 + it % 3) = 1;
+            if (lead) e.cnt[2 + (it + 1) % 3] = 0;
+            if (!bar.sync()) return;
+            {
+                int32_t *t = ni;
+                ni = no;
+                no = t;
+                u128 *u = ai;
+                ai = ao;
+                ao = u;
+                u = ci;
+                ci = co;
+                co = u;
+            }
+            if (*(volatile unsigned long long *)(e.cnt + 2 + it % 3) == 0) break;
         }
-        for (int c = n - 1; c >= 0; c--) {  // parents first
-            const bool sel = e.clist[c] < e.R0 && sst[c] >= sacc[c];
-            const int p = spar[c];
-            const int hp = p >= 0 ? sh[p] : -1;
-            sh[c] = hp >= 0 ? hp : (sel ? c : -1);
+        for (int64_t ix = g0; ix < nact; ix += gsize) {
+            const int c = al[ix];
+            const int pd = e.pending[c];
+            int f = pd == 0;
+            if (pd == 1) {
+                const int x = ni[c];
+                if (e.pending[x] == 0) {
+                    const u128 t = ci[c] + e.S[x];
+                    e.S[c] = ai[c] > t ? ai[c] : t;
+                    f = 1;
+                }
+            }
+            e.fin[c] = f;
         }
-    }
-    __syncthreads();
-    for (int c = threadIdx.x; c < n; c += kEomThreads) {
-        e.acc_hi[c] = (unsigned long long)(sacc[c] >> 64);
-        e.acc_lo[c] = (unsigned long long)sacc[c];
-        H[c] = sh[c];
-    }
-}
-
-__global__ void k_e_iota(int64_t n, int32_t *a) {
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n;
-         x += (int64_t)gridDim.x * blockDim.x)
-        a[x] = (int32_t)x;
-}
-
-// selection: stab(K) >= sum of children's S (ties to the parent)
-__global__ void k_e_childsum(Eom e) {
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < e.ncl;
-         c += (int64_t)gridDim.x * blockDim.x) {
-        e.acc_hi[c] = 0;
-        e.acc_lo[c] = 0;
-    }
-}
-__global__ void k_e_childsum2(Eom e) {
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < e.ncl;
-         c += (int64_t)gridDim.x * blockDim.x) {
-        int p = e.par[c];
-        if (p < 0) continue;
-        u128 s = e.S[c];
-        atomic_add_u128(&e.acc_hi[p], &e.acc_lo[p], (unsigned long long)(s >> 64), (unsigned long long)s);
-    }
-}
-__global__ void k_e_select(Eom e, int32_t *H, int32_t *J) {
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < e.ncl;
-         c += (int64_t)gridDim.x * blockDim.x) {
-        bool sel = (e.clist[c] < e.R0) && e.stab[c] >= acc_of(e, c);
-        H[c] = sel ? (int32_t)c : -1;
-        J[c] = e.par[c];
-    }
-}
-
-// highest selected ancestor-or-self, by synchronous doubling
-__global__ void k_e_hdouble(int64_t ncl, const int32_t *Hin, const int32_t *Jin, int32_t *Hout,
-                            int32_t *Jout, unsigned long long *flag) {
-    bool live = false;
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < ncl;
-         c += (int64_t)gridDim.x * blockDim.x) {
-        int j = Jin[c];
-        if (j >= 0) {
-            int h = Hin[j];
-            Hout[c] = h >= 0 ? h : Hin[c];
-            Jout[c] = Jin[j];
-            live |= Jin[j] >= 0;
-        } else {
-            Hout[c] = Hin[c];
-            Jout[c] = -1;
+        if (lead) e.cnt[2] = e.cnt[3] = e.cnt[4] = 0;
+        if (!bar.sync()) return;
+        for (int64_t ix = g0; ix < nact; ix += gsize) {
+            const int c = al[ix];
+            if (!e.fin[c]) continue;
+            e.done[c] = 1;
+            const int p = e.par[c];
+            if (p < 0 || p >= e.root0) continue;
+            acc_add(e, p, e.S[c]);
+            if (e.fin[p]) continue;  // resolved in this phase too
+            __threadfence();
+            if (atomicSub(&e.pending[p], 1) == 1) {
+                __threadfence();
+                e_walk(e, p);
+            }
         }
+        if (!bar.sync()) return;
     }
-    if (__any_sync(0xffffffffu, live) && lane_id() == 0) flag[0] = 1;
+    // highest selected ancestor-or-self
+    for (int64_t c = g0; c < e.ncl; c += gsize) {
+        const bool sel = c < e.root0 && e.stab[c] >= acc_of(e, c);
+        e.slot[c] = ((unsigned long long)(unsigned)e.par[c] << 32) | (unsigned)(sel ? (int)c : -1);
+        e.fin[c] = 0;
+    }
+    if (lead) e.cnt[2] = 0;
+    if (!bar.sync()) return;
+    for (int round = 0;; round++) {
+        if (round > 4096) {
+            if (lead) e.cnt[5] = 2;
+            break;
+        }
+        bool cut = false;
+        for (int64_t t = g0; t < e.ncl; t += gsize) {
+            const int64_t c = e.ncl - 1 - t;
+            if (e.fin[c]) continue;
+            unsigned long long v = e.slot[c];
+            int it = 0;
+            while ((int)(v >> 32) >= 0 && it < kTopWalk) {
+                const unsigned long long u = *(volatile unsigned long long *)(e.slot + (v >> 32));
+                v = (u & 0xffffffff00000000ull) | ((int)(unsigned)u >= 0 ? (unsigned)u : (unsigned)v);
+                *(volatile unsigned long long *)(e.slot + c) = v;
+                it++;
+            }
+            if ((int)(v >> 32) >= 0) {
+                cut = true;
+            } else {
+                e.H[c] = (int)(unsigned)v;
+                e.fin[c] = 1;
+            }
+        }
+        if (__syncthreads_or(cut) && threadIdx.x == 0) *(volatile unsigned long long *)(e.cnt + 2 + round % 3) = 1;
+        if (lead) e.cnt[2 + (round + 1) % 3] = 0;
+        if (!bar.sync()) return;
+        if (*(volatile unsigned long long *)(e.cnt + 2 + round % 3) == 0) break;
+    }
+    bar.finish();
 }
 
 __global__ void k_e_labels(int64_t E, const int32_t *fall_cluster, const int32_t *cidx,
@@ -661,9 +664,9 @@ void plan_condensed(Arena &ws, const Problem &p, Condensed &o) {
 }
 
 struct CScratch {
-    int32_t *up, *cpar, *link, *cparent, *clist, *cidx, *par, *ucand, *nxt, *nxt2, *H, *J, *H2, *J2,
+    int32_t *up, *cpar, *link, *cparent, *clist, *cidx, *par, *ucand, *nxt, *nxt2, *H,
         *rank, *al1, *al2;
-    int *isrep, *isc, *pending, *done, *state, *minmem, *flag;
+    int *isrep, *isc, *pending, *done, *fin, *minmem, *flag;
     unsigned long long *cbirth, *cdeath, *st_hi, *st_lo, *acc_hi, *acc_lo, *csz, *cnt, *k1, *k2, *v1, *v2, *jflag;
     long long *cpos, *scan_tmp;
     int64_t *gstart;
@@ -690,7 +693,7 @@ static CScratch carve_condense(Arena &a, const Problem &p) {
     s.par = a.take<int32_t>(E + p.G + 1);
     s.pending = a.take<int>(E + p.G + 1);
     s.done = a.take<int>(E + p.G + 1);
-    s.state = a.take<int>(E + p.G + 1);
+    s.fin = a.take<int>(E + p.G + 1);
     s.ucand = a.take<int32_t>(E + p.G + 1);
     s.nxt = a.take<int32_t>(E + p.G + 1);
     s.nxt2 = a.take<int32_t>(E + p.G + 1);
@@ -704,16 +707,13 @@ static CScratch carve_condense(Arena &a, const Problem &p) {
     s.acc_lo = a.take<unsigned long long>(E + p.G + 1);
     s.csz = a.take<unsigned long long>(E + p.G + 1);
     s.H = a.take<int32_t>(E + p.G + 1);
-    s.J = a.take<int32_t>(E + p.G + 1);
-    s.H2 = a.take<int32_t>(E + p.G + 1);
-    s.J2 = a.take<int32_t>(E + p.G + 1);
     s.minmem = a.take<int>(E + p.G + 1);
     s.flag = a.take<int>(E + p.G + 2);
     s.rank = a.take<int32_t>(E + p.G + 1);
     s.gstart = a.take<int64_t>(p.G + 1);
     s.al1 = a.take<int32_t>(E + p.G + 1);
     s.al2 = a.take<int32_t>(E + p.G + 1);
-    s.cnt = a.take<unsigned long long>(4);
+    s.cnt = a.take<unsigned long long>(8);
     s.jflag = a.take<unsigned long long>(1);
     s.k1 = a.take<unsigned long long>(E + p.G + 1);
     s.k2 = a.take<unsigned long long>(E + p.G + 1);
@@ -780,6 +780,7 @@ dgec_status stage_condense(Ctx *c, const Problem &p, const Msf &m, const Dendro 
     // ---- excess of mass over the cluster tree
     Eom e;
     e.ncl = ncl;
+    e.root0 = ncl - p.G;  // every virtual root is a cluster, and their node ids are the last
     e.R0 = E + n;
     e.clist = s.clist;
     e.cidx = s.cidx;
@@ -787,98 +788,44 @@ dgec_status stage_condense(Ctx *c, const Problem &p, const Msf &m, const Dendro 
     e.par = s.par;
     e.pending = s.pending;
     e.done = s.done;
-    e.state = s.state;
+    e.fin = s.fin;
     e.stab = s.stab;
     e.S = s.S;
     e.Fa = s.Fa;
     e.Fc = s.Fc;
     e.Fa2 = s.Fa2;
     e.Fc2 = s.Fc2;
+    e.csz = s.csz;
     e.acc_hi = s.acc_hi;
     e.acc_lo = s.acc_lo;
     e.ucand = s.ucand;
     e.nxt = s.nxt;
     e.nxt2 = s.nxt2;
+    e.al = s.al1;
+    e.al2 = s.al2;
+    e.slot = s.k1;
+    e.H = s.H;
+    e.cnt = s.cnt;
+    e.bar = c->bar;
+    e.err = c->bar_err;
     const int gc = grid_for(ncl + 1, kBlock, kStreamCap);
-    e.flag = s.cnt + 2;
     CU_TRY(c, cudaMemsetAsync(s.pending, 0, sizeof(int) * (ncl + 1), st));
-    TK(c, "k_e_init", k_e_init<<<gc, kBlock, 0, st>>>(e, s.st_hi, s.st_lo, s.cbirth, s.cdeath, s.csz));
-    int32_t *Hi = s.H;  // highest selected ancestor-or-self of every cluster
-    if (ncl <= kEomSmall) {
-        CU_TRY(c, cudaFuncSetAttribute(k_e_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEomSmem));
-        TK(c, "k_e_small", k_e_small<<<1, kEomThreads, kEomSmem, st>>>(e, Hi));
-    } else {
-    TK(c, "k_e_iota", k_e_iota<<<gc, kBlock, 0, st>>>(ncl, s.al1));
-    int32_t *al = s.al1, *al2 = s.al2;
-    int64_t nact = ncl;
-    const int kMaxDouble = 40;  // chains are shorter than 2^31
-    for (int phase = 0;; phase++) {
-        if (phase > 4096) return set_err(c, DGEC_ERR_TIMEOUT, "EOM contraction exceeded 4096 phases");
-        e.alist = al;
-        e.nact = nact;
-        const int ga = grid_for(nact, kBlock, kStreamCap);
-        TK(c, "k_e_unary", k_e_unary<<<ga, kBlock, 0, st>>>(e));
-        TK(c, "k_e_fninit", k_e_fninit<<<ga, kBlock, 0, st>>>(e));
-        int32_t *ni = s.nxt, *no = s.nxt2;
-        u128 *ai = s.Fa, *ao = s.Fa2, *ci = s.Fc, *co = s.Fc2;
-        // synchronous doubling until no pointer moves (checked every 2 steps)
-        for (int it = 0; it < kMaxDouble; it++) {
-            if ((it & 1) == 0) CU_TRY(c, cudaMemsetAsync(e.flag, 0, sizeof(unsigned long long), st));
-            TK(c, "k_e_double", k_e_double<<<ga, kBlock, 0, st>>>(e, ni, no, ai, ci, ao, co));
-            int32_t *t = ni;
-            ni = no;
-            no = t;
-            u128 *ta = ai;
-            ai = ao;
-            ao = ta;
-            ta = ci;
-            ci = co;
-            co = ta;
-            if (it & 1) {
-                int64_t moved;
-                DG_TRY(read_counters(c, (const int64_t *)e.flag, 1, &moved));
-                if (!moved) break;
-            }
-        }
-        TK(c, "k_e_rake", k_e_rake<<<ga, kBlock, 0, st>>>(e));
-        TK(c, "k_e_resolve", k_e_resolve<<<ga, kBlock, 0, st>>>(e, ni, ai, ci));
-        TK(c, "k_e_report", k_e_report<<<ga, kBlock, 0, st>>>(e));
-        CU_TRY(c, cudaMemsetAsync(s.cnt, 0, sizeof(unsigned long long), st));
-        TK(c, "k_e_commit", k_e_commit<<<ga, kBlock, 0, st>>>(e, al2, s.cnt));
-        int64_t open;
-        DG_TRY(read_counters(c, (const int64_t *)s.cnt, 1, &open));
-        if (open == 0) break;
-        int32_t *t = al;
-        al = al2;
-        al2 = t;
-        nact = open;
-    }
-    TK(c, "k_e_childsum", k_e_childsum<<<gc, kBlock, 0, st>>>(e));
-    TK(c, "k_e_childsum2", k_e_childsum2<<<gc, kBlock, 0, st>>>(e));
-    TK(c, "k_e_select", k_e_select<<<gc, kBlock, 0, st>>>(e, s.H, s.J));
-    int32_t *Ji = s.J, *Ho = s.H2, *Jo = s.J2;
-    for (int it = 0; it < kMaxDouble; it++) {
-        if ((it & 1) == 0) CU_TRY(c, cudaMemsetAsync(e.flag, 0, sizeof(unsigned long long), st));
-        TK(c, "k_e_hdouble", k_e_hdouble<<<gc, kBlock, 0, st>>>(ncl, Hi, Ji, Ho, Jo, e.flag));
-        int32_t *t = Hi;
-        Hi = Ho;
-        Ho = t;
-        t = Ji;
-        Ji = Jo;
-        Jo = t;
-        if (it & 1) {
-            int64_t live;
-            DG_TRY(read_counters(c, (const int64_t *)e.flag, 1, &live));
-            if (!live) break;
-        }
-    }
+    CU_TRY(c, cudaMemsetAsync(s.cnt, 0, 8 * sizeof(unsigned long long), st));
+    TK(c, "k_e_init", k_e_init<<<gc, kBlock, 0, st>>>(e, s.st_hi, s.st_lo, s.cbirth, s.cdeath));
+    {
+        int grid = 1;
+        DG_TRY(coop_grid(c, kCoopEom, (const void *)k_e_tree, kBlock, 0, &grid));
+        const int64_t want = cdiv(ncl, 2 * kBlock);
+        DG_TRY(coop_launch(c, "k_e_tree", (const void *)k_e_tree, want < grid ? (int)want : grid, kBlock, 0, e));
     }
     TK(c, "k_fill_i32", k_fill_i32<<<gc, kBlock, 0, st>>>(s.minmem, ncl + 1, INT_MAX));
-    TK(c, "k_e_labels", k_e_labels<<<gE, kBlock, 0, st>>>(E, o.fall_cluster, s.cidx, Hi, o.labels, s.minmem));
-    TK(c, "k_e_final_keys", k_e_final_keys<<<gc, kBlock, 0, st>>>(ncl, Hi, s.minmem, s.flag));
+    TK(c, "k_e_labels", k_e_labels<<<gE, kBlock, 0, st>>>(E, o.fall_cluster, s.cidx, s.H, o.labels, s.minmem));
+    TK(c, "k_e_final_keys", k_e_final_keys<<<gc, kBlock, 0, st>>>(ncl, s.H, s.minmem, s.flag));
     DG_TRY(exclusive_scan_i32(c, s.flag, s.cpos, ncl + 1, s.scan_tmp));
     int64_t nf;
+    CU_TRY(c, cudaMemcpyAsync(c->h_pinned + 8, s.cnt + 5, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     DG_TRY(read_counters(c, (const int64_t *)(s.cpos + ncl), 1, &nf));
+    if (c->h_pinned[8]) return set_err(c, DGEC_ERR_TIMEOUT, "the EOM pass exceeded its round bound");
     o.n_clusters = (int32_t)nf;
     if (nf > 0) {
         TK(c, "k_e_final_emit", k_e_final_emit<<<gc, kBlock, 0, st>>>(ncl, s.flag, s.cpos, s.minmem, s.k1, s.v1));
@@ -892,7 +839,7 @@ dgec_status stage_condense(Ctx *c, const Problem &p, const Msf &m, const Dendro 
         TK(c, "k_e_rank", k_e_rank<<<gf, kBlock, 0, st>>>(nf, kk, vv, p.egraph, s.gstart, s.rank));
         TK(c, "k_e_relabel", k_e_relabel<<<gE, kBlock, 0, st>>>(E, s.rank, o.labels));
     }
-    TK(c, "k_e_out", k_e_out<<<gc, kBlock, 0, st>>>(e, gv, d.size, s.cbirth, s.cdeath, Hi, o.cl_id, o.cl_parent,
+    TK(c, "k_e_out", k_e_out<<<gc, kBlock, 0, st>>>(e, gv, d.size, s.cbirth, s.cdeath, s.H, o.cl_id, o.cl_parent,
                                    o.cl_birth, o.cl_death, o.cl_size, o.cl_stab_hi, o.cl_stab_lo,
                                    o.cl_selected));
     return DGEC_OK;
