@@ -481,8 +481,9 @@ dgec_status radix_sort(Ctx *c, RadixBuffers buf, int64_t n, int begin_bit, int e
     unsigned *w = (unsigned *)scratch;
     // digits of at most kSBits bits (see kSNarrow)
     const int most = buf.va && n > kSNarrow ? kSBits - 1 : kSBits;
-    SortArgs a{buf.ka, buf.kb, buf.va, buf.vb, n, begin_bit, end_bit, most, w, w + (size_t)kSRanges * kSBins,
-               w + (size_t)2 * kSRanges * kSBins, w + (size_t)(2 * kSRanges + 1) * kSBins, c->bar, c->bar_err};
+    const size_t R = (size_t)sort_max_ranges(n) * kSBins;
+    SortArgs a{buf.ka, buf.kb, buf.va, buf.vb, n, begin_bit, end_bit, most, w, w + R, w + 2 * R, w + 2 * R + kSBins,
+               c->bar, c->bar_err};
     const int passes = (end_bit - begin_bit + most - 1) / most;
     *in_b = n <= kSTile || (passes & 1);
     return buf.va ? launch_sort<true>(c, a) : launch_sort<false>(c, a);
