@@ -3,11 +3,14 @@
 //
 // The order (w, min id, max id) is strict (a pair appears once in L*), so
 // the forest is unique. Each round: every live edge between two components
-// bids its w into both components with atomicMin, then the edges that match
-// a component's best w bid their packed (u << 32 | v); each component hooks
-// along its winning edge, a mutual pair keeps the smaller label as root,
-// labels are pointer-jumped to their roots, and edges inside one component
-// are dropped while the survivors are compacted for the next round.
+// bids its key into both, each component hooks along its winning edge, a
+// mutual pair keeps the smaller label as root, labels are pointer-jumped to
+// their roots, and edges inside one component are dropped while the survivors
+// are compacted for the next round. The pipeline's form is k_m_forest; the
+// kernels before it serve dgec_msf_static.
+#include <utility>
+
+#include "coop.cuh"
 #include "stages.cuh"
 
 namespace dgec {
@@ -169,6 +172,9 @@ __global__ void k_iota(int64_t E, int32_t *comp) {
 // ----- the pipeline's forest stage: nodes are internal ids r; each edge
 // carries its original ends (u < v) for the (w, u, v) tie-break key.
 
+// ---- large rounds: one kernel a step (more threads resident than the
+// cooperative kernel below allows, which the random accesses need here)
+
 // Edges carry the labels (cu, cv) of the components at their ends; the
 // labels move one hop per round (par of the old root), so no per-node
 // label array is swept. Live edges: (cu, cv) labels, (u, v) original ends
@@ -189,7 +195,7 @@ __global__ void k_m_bid(const int32_t *cu, const int32_t *cv, const int64_t *w, 
 
 // Items per thread between two slot reservations of the compacting
 // kernels below (one atomic on the shared counter per 2,048 items).
-constexpr int kRes = 8;
+constexpr int kRes8 = 8;
 
 // Move labels one hop to the merged roots, drop edges inside one
 // component, compact the rest and bid w.
@@ -197,12 +203,12 @@ __global__ void k_m_filter_bid(const int32_t *cu, const int32_t *cv, const int32
                                const int64_t *w, int64_t n, const int32_t *par, int32_t *cu2,
                                int32_t *cv2, int32_t *u2, int32_t *v2, int64_t *w2,
                                unsigned long long *cnt, unsigned long long *bw) {
-    const int64_t tile = (int64_t)blockDim.x * kRes;
+    const int64_t tile = (int64_t)blockDim.x * kRes8;
     for (int64_t base = (int64_t)blockIdx.x * tile; base < n; base += (int64_t)gridDim.x * tile) {  // CTA-uniform
-        int a[kRes], b[kRes];
+        int a[kRes8], b[kRes8];
         unsigned keep = 0;
 #pragma unroll
-        for (int q = 0; q < kRes; q++) {
+        for (int q = 0; q < kRes8; q++) {
             const int64_t x = base + (int64_t)q * blockDim.x + threadIdx.x;
             a[q] = b[q] = 0;
             if (x < n) {
@@ -213,7 +219,7 @@ __global__ void k_m_filter_bid(const int32_t *cu, const int32_t *cv, const int32
         }
         long long at = cta_reserve_count(__popc(keep), cnt);
 #pragma unroll
-        for (int q = 0; q < kRes; q++) {
+        for (int q = 0; q < kRes8; q++) {
             if (!((keep >> q) & 1u)) continue;
             const int64_t x = base + (int64_t)q * blockDim.x + threadIdx.x;
             const unsigned long long uw = (unsigned long long)w[x];
@@ -273,17 +279,17 @@ __global__ void k_m_hook(const int32_t *__restrict__ roots, int64_t nr, const un
                          const int32_t *__restrict__ v, const int64_t *__restrict__ w,
                          const int32_t *__restrict__ rank_of, int32_t *__restrict__ par, FEdge *__restrict__ fe,
                          unsigned long long *n_out) {
-    const int64_t tile = (int64_t)blockDim.x * kRes;
+    const int64_t tile = (int64_t)blockDim.x * kRes8;
     for (int64_t base = (int64_t)blockIdx.x * tile; base < nr; base += (int64_t)gridDim.x * tile) {  // CTA-uniform
-        int xs[kRes], ps[kRes], wx[kRes];
+        int xs[kRes8], ps[kRes8], wx[kRes8];
         unsigned live = 0, mutual = 0;
 #pragma unroll
-        for (int q = 0; q < kRes; q++) {
+        for (int q = 0; q < kRes8; q++) {
             const int64_t ix = base + (int64_t)q * blockDim.x + threadIdx.x;
             xs[q] = ix < nr ? roots[ix] : -1;
         }
 #pragma unroll
-        for (int q = 0; q < kRes; q++) {
+        for (int q = 0; q < kRes8; q++) {
             ps[q] = wx[q] = 0;
             if (xs[q] < 0) continue;
             if (bw[xs[q]] != kMax64) {
@@ -293,14 +299,14 @@ __global__ void k_m_hook(const int32_t *__restrict__ roots, int64_t nr, const un
             }
         }
 #pragma unroll
-        for (int q = 0; q < kRes; q++) {
+        for (int q = 0; q < kRes8; q++) {
             if (!((live >> q) & 1u)) continue;
             const int x = xs[q], p = ps[q];
             if (bp[p] == x && buv[p] == buv[x]) mutual |= 1u << q;
         }
         unsigned emit = 0;
 #pragma unroll
-        for (int q = 0; q < kRes; q++) {
+        for (int q = 0; q < kRes8; q++) {
             if (xs[q] < 0) continue;
             const int x = xs[q];
             if (!((live >> q) & 1u)) {
@@ -313,7 +319,7 @@ __global__ void k_m_hook(const int32_t *__restrict__ roots, int64_t nr, const un
         }
         long long at = cta_reserve_count(__popc(emit), n_out);
 #pragma unroll
-        for (int q = 0; q < kRes; q++) {
+        for (int q = 0; q < kRes8; q++) {
             if (!((emit >> q) & 1u)) continue;
             const int a = u[wx[q]], b = v[wx[q]];
             FEdge f;
@@ -347,27 +353,27 @@ __global__ void k_m_jump(const int32_t *roots, int64_t nr, int32_t *par) {
 __global__ void k_m_next_roots(const int32_t *__restrict__ roots, int64_t nr, const int32_t *__restrict__ par,
                                unsigned long long *__restrict__ bw, unsigned long long *__restrict__ buv,
                                int32_t *__restrict__ roots2, unsigned long long *cnt) {
-    const int64_t tile = (int64_t)blockDim.x * kRes;
+    const int64_t tile = (int64_t)blockDim.x * kRes8;
     for (int64_t base = (int64_t)blockIdx.x * tile; base < nr; base += (int64_t)gridDim.x * tile) {  // CTA-uniform
-        int xs[kRes];
+        int xs[kRes8];
         unsigned keep = 0;
 #pragma unroll
-        for (int q = 0; q < kRes; q++) {
+        for (int q = 0; q < kRes8; q++) {
             const int64_t ix = base + (int64_t)q * blockDim.x + threadIdx.x;
             xs[q] = ix < nr ? roots[ix] : -1;
         }
 #pragma unroll
-        for (int q = 0; q < kRes; q++)
+        for (int q = 0; q < kRes8; q++)
             if (xs[q] >= 0 && par[xs[q]] == xs[q] && bw[xs[q]] != kMax64) keep |= 1u << q;
 #pragma unroll
-        for (int q = 0; q < kRes; q++) {
+        for (int q = 0; q < kRes8; q++) {
             if (xs[q] < 0) continue;
             bw[xs[q]] = kMax64;
             buv[xs[q]] = kMax64;
         }
         long long at = cta_reserve_count(__popc(keep), cnt);
 #pragma unroll
-        for (int q = 0; q < kRes; q++)
+        for (int q = 0; q < kRes8; q++)
             if ((keep >> q) & 1u) roots2[at++] = xs[q];
     }
 }
@@ -381,6 +387,233 @@ __global__ void k_m_init(int64_t E, int32_t *par, int32_t *roots, unsigned long 
         bw[x] = kMax64;
         buv[x] = kMax64;
     }
+}
+
+// ---- the other rounds, in one cooperative kernel
+
+typedef unsigned __int128 u128;
+
+// A live edge after the first round: the labels of the components at its
+// ends, and its packed key.
+struct MsfArgs {
+    int64_t nr0, n0;
+    const int32_t *roots0;           // the roots to begin with (null: 0 .. nr0-1)
+    const int32_t *ru, *rv, *u, *v;  // the edges to begin with: labels of the ends, original ends
+    const int64_t *w;
+    const int32_t *rank_of;
+    int32_t *par, *roots, *roots2, *bp;
+    ulonglong2 *slot;       // best key bid at each root (all ones: none)
+    int2 *la, *lb;          // live edges: labels
+    ulonglong2 *ka, *kb;    // live edges: keys without the label
+    FEdge *fe;
+    unsigned long long *cnt;  // [0], [1] live edges, [2], [3] roots, [4] forest edges, [5] error; zeroed before
+    int ib, lbits;            // bits of an original id, of the label in a key (0: none)
+    unsigned *bar, *err;
+};
+
+__device__ __forceinline__ u128 as_u128(ulonglong2 x) { return ((u128)x.y << 64) | x.x; }
+__device__ __forceinline__ ulonglong2 as_pair(u128 x) {
+    return make_ulonglong2((unsigned long long)x, (unsigned long long)(x >> 64));
+}
+__device__ __forceinline__ u128 cas_u128(ulonglong2 *p, u128 cmp, u128 val) {
+    unsigned long long lo, hi;
+    asm volatile(
+        "{\n\t.reg .b128 c, v, o;\n\t"
+        "mov.b128 c, {%2, %3};\n\t"
+        "mov.b128 v, {%4, %5};\n\t"
+        "atom.relaxed.gpu.global.cas.b128 o, [%6], c, v;\n\t"
+        "mov.b128 {%0, %1}, o;\n\t}"
+        : "=l"(lo), "=l"(hi)
+        : "l"((unsigned long long)cmp), "l"((unsigned long long)(cmp >> 64)), "l"((unsigned long long)val),
+          "l"((unsigned long long)(val >> 64)), "l"(p)
+        : "memory");
+    return ((u128)hi << 64) | lo;
+}
+// Minimum into a slot. The read before skips bids that cannot win (most, at a
+// large component). It trusts the high word alone, which only falls: the two
+// words of the read need not belong together, so where the high words tie, a
+// swap of the value for itself reads it whole.
+__device__ __forceinline__ void bid_u128(ulonglong2 *slot, u128 key) {
+    const ulonglong2 seen = *slot;
+    if ((unsigned long long)(key >> 64) > seen.y) return;
+    u128 cur = as_u128(seen);
+    if (key >= cur) cur = cas_u128(slot, cur, cur);
+    while (key < cur) {
+        const u128 old = cas_u128(slot, cur, key);
+        if (old == cur) return;
+        cur = old;
+    }
+}
+
+// Borůvka, all rounds in one cooperative kernel. A root's slot takes the
+// smallest bid by 128-bit compare-and-swap: the bid packs (w, u, v) and, in
+// its low bits, the label at the edge's other end, so one pass over the live
+// edges bids, and the roots then hook from the slots alone. (When the bits do
+// not fit -- w bits + 3 id bits > 127 -- the label is left out and a pass over
+// the live edges tells each root its winner's other end.) Per round:
+//   hook:   each root follows its best edge; a mutual pair keeps the smaller
+//           label as root; every forest edge is appended once;
+//   jump:   the old roots walk to their new root; those that stayed roots are
+//           the next round's, their slots cleared;
+//   filter: labels move one hop, edges inside one component are dropped, the
+//           rest is compacted and bids again.
+constexpr int kRes = 4;          // items a thread has in flight between slot reservations
+__global__ void __launch_bounds__(kBlock, 4) k_m_forest(MsfArgs a) {
+    GridBar bar(a.bar, a.err);
+    const int64_t gsize = (int64_t)gridDim.x * blockDim.x, g0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t tile = (int64_t)blockDim.x * kRes;
+    const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
+    const int ib = a.ib, lb = a.lbits;
+    const u128 none = ~(u128)0;
+    const unsigned lmask = (1u << lb) - 1u, imask = (unsigned)((1ull << ib) - 1ull);
+    for (int64_t ix = g0; ix < a.nr0; ix += gsize) {
+        const int x = a.roots0 ? a.roots0[ix] : (int)ix;
+        a.par[x] = x;
+        a.slot[x] = as_pair(none);
+    }
+    if (!bar.sync()) return;
+    auto pack = [&](int64_t x) {
+        return ((((u128)(unsigned long long)a.w[x] << ib | (unsigned)a.u[x]) << ib) | (unsigned)a.v[x]) << lb;
+    };
+    for (int64_t x = g0; x < a.n0; x += gsize) {
+        const int cu = a.ru[x], cv = a.rv[x];
+        const u128 key = pack(x);
+        bid_u128(a.slot + cu, key | (lb ? (unsigned)cv : 0u));
+        bid_u128(a.slot + cv, key | (lb ? (unsigned)cu : 0u));
+    }
+    if (!bar.sync()) return;
+    int64_t n = a.n0, nr = a.nr0;
+    const int32_t *roots = a.roots0;
+    int32_t *rout = a.roots, *rnext = a.roots2;
+    int2 *lin = a.la, *lout = a.lb;
+    ulonglong2 *kin = a.ka, *kout = a.kb;
+    for (int round = 0;; round++) {
+        if (round >= 64) {
+            if (lead) a.cnt[5] = 1;
+            break;
+        }
+        if (!lb) {  // the winner of each slot records the label at its other end
+            for (int64_t x = g0; x < n; x += gsize) {
+                const int2 l = round ? lin[x] : make_int2(a.ru[x], a.rv[x]);
+                const u128 key = round ? as_u128(kin[x]) : pack(x);
+                if (as_u128(a.slot[l.x]) == key) a.bp[l.x] = l.y;
+                if (as_u128(a.slot[l.y]) == key) a.bp[l.y] = l.x;
+            }
+            if (!bar.sync()) return;
+        }
+        for (int64_t base = (int64_t)blockIdx.x * tile; base < nr; base += gsize * kRes) {  // CTA-uniform
+            int xs[kRes], ps[kRes];
+            u128 key[kRes];
+            unsigned emit = 0;
+#pragma unroll
+            for (int q = 0; q < kRes; q++) {
+                const int64_t ix = base + (int64_t)q * blockDim.x + threadIdx.x;
+                xs[q] = ix < nr ? (roots ? roots[ix] : (int)ix) : -1;
+            }
+#pragma unroll
+            for (int q = 0; q < kRes; q++) {
+                key[q] = xs[q] >= 0 ? as_u128(a.slot[xs[q]]) : none;
+                ps[q] = -1;
+                if (key[q] != none) ps[q] = lb ? (int)((unsigned)key[q] & lmask) : a.bp[xs[q]];
+            }
+#pragma unroll
+            for (int q = 0; q < kRes; q++) {
+                if (ps[q] < 0) continue;  // no edge left: par[x] stays x
+                const bool mutual = (as_u128(a.slot[ps[q]]) >> lb) == (key[q] >> lb);
+                if (!mutual || xs[q] < ps[q]) emit |= 1u << q;
+                if (!mutual || xs[q] > ps[q]) a.par[xs[q]] = ps[q];
+            }
+            long long at = cta_reserve_count(__popc(emit), a.cnt + 4);
+#pragma unroll
+            for (int q = 0; q < kRes; q++) {
+                if (!((emit >> q) & 1u)) continue;
+                const u128 k = key[q] >> lb;
+                FEdge f;
+                f.v = (int32_t)((unsigned)k & imask);
+                f.u = (int32_t)((unsigned)(k >> ib) & imask);
+                f.w = (int64_t)(unsigned long long)(k >> (2 * ib));
+                f.ru = a.rank_of[f.u];
+                f.rv = a.rank_of[f.v];
+                a.fe[at++] = f;
+            }
+        }
+        if (lead) a.cnt[round & 1] = 0;  // the live count written in this round's filter
+        if (!bar.sync()) return;
+        for (int64_t base = (int64_t)blockIdx.x * tile; base < nr; base += gsize * kRes) {  // CTA-uniform
+            int xs[kRes];
+            unsigned keep = 0;
+#pragma unroll
+            for (int q = 0; q < kRes; q++) {
+                const int64_t ix = base + (int64_t)q * blockDim.x + threadIdx.x;
+                xs[q] = ix < nr ? (roots ? roots[ix] : (int)ix) : -1;
+                if (xs[q] < 0) continue;
+                int r = a.par[xs[q]];
+                if (r == xs[q]) {
+                    if (as_u128(a.slot[r]) != none) keep |= 1u << q;
+                    continue;
+                }
+                for (int it = 0; it < kMaxWalk; it++) {  // bounded: pointers form a forest
+                    const int rr = a.par[r];
+                    if (rr == r) break;
+                    r = rr;
+                    a.par[xs[q]] = r;
+                }
+            }
+            long long at = cta_reserve_count(__popc(keep), a.cnt + 2 + (round & 1));
+#pragma unroll
+            for (int q = 0; q < kRes; q++) {
+                if (!((keep >> q) & 1u)) continue;
+                a.slot[xs[q]] = as_pair(none);
+                rout[at++] = xs[q];
+            }
+        }
+        if (!bar.sync()) return;
+        nr = (int64_t) * (volatile unsigned long long *)(a.cnt + 2 + (round & 1));
+        for (int64_t base = (int64_t)blockIdx.x * tile; base < n; base += gsize * kRes) {  // CTA-uniform
+            int ca[kRes], cb[kRes];
+            unsigned keep = 0;
+#pragma unroll
+            for (int q = 0; q < kRes; q++) {
+                const int64_t x = base + (int64_t)q * blockDim.x + threadIdx.x;
+                ca[q] = cb[q] = 0;
+                if (x < n) {
+                    const int2 l = round ? lin[x] : make_int2(a.ru[x], a.rv[x]);
+                    ca[q] = a.par[l.x];
+                    cb[q] = a.par[l.y];
+                    if (ca[q] != cb[q]) keep |= 1u << q;
+                }
+            }
+            long long at = cta_reserve_count(__popc(keep), a.cnt + (round & 1));
+#pragma unroll
+            for (int q = 0; q < kRes; q++) {
+                if (!((keep >> q) & 1u)) continue;
+                const int64_t x = base + (int64_t)q * blockDim.x + threadIdx.x;
+                const u128 key = round ? as_u128(kin[x]) : pack(x);
+                lout[at] = make_int2(ca[q], cb[q]);
+                kout[at] = as_pair(key);
+                at++;
+                bid_u128(a.slot + ca[q], key | (lb ? (unsigned)cb[q] : 0u));
+                bid_u128(a.slot + cb[q], key | (lb ? (unsigned)ca[q] : 0u));
+            }
+        }
+        if (lead) a.cnt[2 + ((round & 1) ^ 1)] = 0;
+        if (!bar.sync()) return;
+        n = (int64_t) * (volatile unsigned long long *)(a.cnt + (round & 1));
+        if (n == 0) break;
+        {
+            int32_t *t = rout;
+            roots = rout;
+            rout = rnext;
+            rnext = t;
+            int2 *tl = lin;
+            lin = lout;
+            lout = tl;
+            ulonglong2 *tk = kin;
+            kin = kout;
+            kout = tk;
+        }
+    }
+    bar.finish();
 }
 
 __global__ void k_pack_uv_idx(const FEdge *fe, int64_t n, int idbits, unsigned long long *k,
@@ -470,12 +703,41 @@ void plan_msf(Arena &ws, const Problem &p, Msf &o) {
     o.w = ws.take<int64_t>(p.E);
 }
 
+// Live edges above which the host launches every step of a round by itself:
+// the 64-bit bids in three passes at full occupancy beat the one 128-bit pass
+// there (100M hub edges, 190M links: 25.4 against 28.6 ms for all rounds; 50M
+// edges 17.4 against 18.8), while below, the launches and the host's read of
+// every round cost more than they save (316,229 edges: 0.93 -> 0.61 ms for the
+// stage, 20,000: 0.60 -> 0.48, 3M: 2.4 -> 2.1; the line measured flat from 2^20 to
+// 2^24).
+constexpr int64_t kMLarge = int64_t(1) << 22;
+// One side of the live edges: 24 bytes each, as five columns in the large
+// rounds, as labels and keys in the cooperative kernel.
+struct LiveSide {
+    int32_t *cu, *cv, *u, *v;
+    int64_t *w;
+    ulonglong2 *key;
+    int2 *lab;
+};
+static LiveSide carve_side(Arena &a, int64_t S) {
+    const int64_t n = (S + 3) & ~int64_t(3);
+    char *p = a.take<char>(24 * n);
+    LiveSide s;
+    s.cu = (int32_t *)p;
+    s.cv = s.cu + n;
+    s.u = s.cv + n;
+    s.v = s.u + n;
+    s.w = (int64_t *)(s.v + n);
+    s.key = (ulonglong2 *)p;
+    s.lab = (int2 *)(s.key + n);
+    return s;
+}
 struct MsfScratch {
     int32_t *par, *roots, *roots2, *bp, *win;
-    int32_t *cua, *cva, *ua, *va, *cub, *cvb, *ub, *vb;
-    int64_t *wa, *wb;
+    LiveSide side[2];
+    ulonglong2 *slot;
     FEdge *fe;
-    unsigned long long *bw, *buv, *cnt;
+    unsigned long long *cnt;
     unsigned long long *k1, *k2, *v1, *v2;
     void *radix;
 };
@@ -487,20 +749,11 @@ static MsfScratch carve_msf(Arena &a, const Problem &p) {
     s.roots2 = a.take<int32_t>(E);
     s.bp = a.take<int32_t>(E);
     s.win = a.take<int32_t>(E);
-    s.cua = a.take<int32_t>(S);
-    s.cva = a.take<int32_t>(S);
-    s.ua = a.take<int32_t>(S);
-    s.va = a.take<int32_t>(S);
-    s.wa = a.take<int64_t>(S);
-    s.cub = a.take<int32_t>(S);
-    s.cvb = a.take<int32_t>(S);
-    s.ub = a.take<int32_t>(S);
-    s.vb = a.take<int32_t>(S);
-    s.wb = a.take<int64_t>(S);
+    s.side[0] = carve_side(a, S);
+    s.side[1] = carve_side(a, S);
+    s.slot = a.take<ulonglong2>(E);
     s.fe = a.take<FEdge>(E);
-    s.bw = a.take<unsigned long long>(E);
-    s.buv = a.take<unsigned long long>(E);
-    s.cnt = a.take<unsigned long long>(4);
+    s.cnt = a.take<unsigned long long>(8);
     s.k1 = a.take<unsigned long long>(E);
     s.k2 = a.take<unsigned long long>(E);
     s.v1 = a.take<unsigned long long>(E);
@@ -522,56 +775,62 @@ dgec_status stage_msf(Ctx *c, const Problem &p, const Csr &g, const Skel &sk, Ms
     if (E == 0 || sk.n == 0) return DGEC_OK;
     Arena a(scratch, SIZE_MAX);
     MsfScratch s = carve_msf(a, p);
-    const int gE = grid_for(E, kBlock, kStreamCap);
-    TK(c, "k_m_init", k_m_init<<<gE, kBlock, 0, st>>>(E, s.par, s.roots, s.bw, s.buv));
-    CU_TRY(c, cudaMemsetAsync(s.cnt, 0, 4 * sizeof(unsigned long long), st));
+    CU_TRY(c, cudaMemsetAsync(s.cnt, 0, 8 * sizeof(unsigned long long), st));
     // live edges: (cu, cv) component labels, (u, v) original ends, w; the
     // first round reads the skeleton itself (labels = internal ids)
-    const int32_t *ccu = sk.ru, *ccv = sk.rv, *cu = sk.u, *cv = sk.v;
+    const int32_t *ccu = sk.ru, *ccv = sk.rv, *cu = sk.u, *cv = sk.v, *roots0 = nullptr;
     const int64_t *cw = sk.w;
     int64_t n = sk.n, nr = E;
+    int which = 0;  // the side the next filter writes
     int32_t *roots = s.roots, *roots2 = s.roots2;
-    int which = 0;
-    for (int round = 0;; round++) {
-        if (round >= 64) return set_err(c, DGEC_ERR_TIMEOUT, "Boruvka did not finish in 64 rounds");
-        if (round == 0) {
-            TK(c, "k_m_bid", k_m_bid<<<grid_for(n, kBlock, kStreamCap), kBlock, 0, st>>>(ccu, ccv, cw, n, s.bw));
-        } else {
-            int32_t *ncu = which ? s.cub : s.cua, *ncv = which ? s.cvb : s.cva;
-            int32_t *nu = which ? s.ub : s.ua, *nv = which ? s.vb : s.va;
-            int64_t *nw = which ? s.wb : s.wa;
-            CU_TRY(c, cudaMemsetAsync(s.cnt, 0, sizeof(unsigned long long), st));
-            TK(c, "k_m_filter_bid", k_m_filter_bid<<<grid_for(n, kBlock * kRes, kStreamCap), kBlock, 0, st>>>(
-                                      ccu, ccv, cu, cv, cw, n, s.par, ncu, ncv, nu, nv, nw, s.cnt, s.bw));
-            int64_t h[3];
-            DG_TRY(read_counters(c, (const int64_t *)s.cnt, 3, h));
+    if (n > kMLarge) {
+        unsigned long long *bw = (unsigned long long *)s.slot, *buv = bw + E;
+        TK(c, "k_m_init", k_m_init<<<grid_for(E, kBlock, kStreamCap), kBlock, 0, st>>>(E, s.par, roots, bw, buv));
+        for (int round = 0; n > kMLarge; round++) {
+            if (round >= 64) return set_err(c, DGEC_ERR_TIMEOUT, "Boruvka did not finish in 64 rounds");
+            const int gn = grid_for(n, kBlock, kStreamCap), gr = grid_for(nr, kBlock, kStreamCap),
+                      grk = grid_for(nr, kBlock * kRes8, kStreamCap);
+            if (round == 0) TK(c, "k_m_bid", k_m_bid<<<gn, kBlock, 0, st>>>(ccu, ccv, cw, n, bw));
+            TK(c, "k_m_bid_uv", k_m_bid_uv<<<gn, kBlock, 0, st>>>(ccu, ccv, cu, cv, cw, n, bw, buv));
+            TK(c, "k_m_claim", k_m_claim<<<gn, kBlock, 0, st>>>(ccu, ccv, cu, cv, n, buv, s.bp, s.win));
+            TK(c, "k_m_hook", k_m_hook<<<grk, kBlock, 0, st>>>(roots, nr, bw, buv, s.bp, s.win, cu, cv, cw, g.rank_of,
+                                                            s.par, s.fe, s.cnt + 4));
+            TK(c, "k_m_jump", k_m_jump<<<gr, kBlock, 0, st>>>(roots, nr, s.par));
+            CU_TRY(c, cudaMemsetAsync(s.cnt, 0, 4 * sizeof(unsigned long long), st));
+            TK(c, "k_m_next_roots", k_m_next_roots<<<grk, kBlock, 0, st>>>(roots, nr, s.par, bw, buv, roots2, s.cnt + 1));
+            std::swap(roots, roots2);
+            const LiveSide &o = s.side[which];
+            TK(c, "k_m_filter_bid", k_m_filter_bid<<<grid_for(n, kBlock * kRes8, kStreamCap), kBlock, 0, st>>>(
+                                      ccu, ccv, cu, cv, cw, n, s.par, o.cu, o.cv, o.u, o.v, o.w, s.cnt, bw));
+            int64_t h[2];
+            DG_TRY(read_counters(c, (const int64_t *)s.cnt, 2, h));
             n = h[0];
-            nr = h[2];
-            if (n == 0) break;
-            ccu = ncu;
-            ccv = ncv;
-            cu = nu;
-            cv = nv;
-            cw = nw;
+            nr = h[1];
+            ccu = o.cu;
+            ccv = o.cv;
+            cu = o.u;
+            cv = o.v;
+            cw = o.w;
             which ^= 1;
         }
-        const int gn = grid_for(n, kBlock, kStreamCap), gr = grid_for(nr, kBlock, kStreamCap),
-                  grk = grid_for(nr, kBlock * kRes, kStreamCap);
-        TK(c, "k_m_bid_uv", k_m_bid_uv<<<gn, kBlock, 0, st>>>(ccu, ccv, cu, cv, cw, n, s.bw, s.buv));
-        TK(c, "k_m_claim", k_m_claim<<<gn, kBlock, 0, st>>>(ccu, ccv, cu, cv, n, s.buv, s.bp, s.win));
-        TK(c, "k_m_hook", k_m_hook<<<grk, kBlock, 0, st>>>(roots, nr, s.bw, s.buv, s.bp, s.win, cu, cv, cw,
-                                                        g.rank_of, s.par, s.fe,
-                                                        s.cnt + 1));
-        TK(c, "k_m_jump", k_m_jump<<<gr, kBlock, 0, st>>>(roots, nr, s.par));
-        CU_TRY(c, cudaMemsetAsync(s.cnt + 2, 0, sizeof(unsigned long long), st));
-        TK(c, "k_m_next_roots", k_m_next_roots<<<grk, kBlock, 0, st>>>(roots, nr, s.par, s.bw, s.buv, roots2,
-                                                                    s.cnt + 2));
-        int32_t *tr = roots;
-        roots = roots2;
-        roots2 = tr;
+        roots0 = roots;
+        CU_TRY(c, cudaMemsetAsync(s.cnt, 0, 4 * sizeof(unsigned long long), st));
     }
-    int64_t m;
-    DG_TRY(read_counters(c, (const int64_t *)(s.cnt + 1), 1, &m));
+    if (n > 0) {
+        // the kernel's first filter writes lb/kb: not the side its edges come from
+        const LiveSide &in = s.side[which ^ 1], &out = s.side[which];
+        MsfArgs f{nr, n, roots0, ccu, ccv, cu, cv, cw, g.rank_of, s.par, roots0 ? roots2 : roots, roots0 ? roots : roots2,
+                  s.bp, s.slot, in.lab, out.lab, in.key, out.key, s.fe, s.cnt, p.idbits,
+                  p.tbits + 3 * p.idbits <= 127 ? p.idbits : 0, c->bar, c->bar_err};
+        int grid = 1;
+        DG_TRY(coop_grid(c, kCoopMsf, (const void *)k_m_forest, kBlock, 0, &grid));
+        const int64_t want = cdiv(n > nr ? n : nr, kBlock * kRes);
+        DG_TRY(coop_launch(c, "k_m_forest", (const void *)k_m_forest, want < grid ? (int)want : grid, kBlock, 0, f));
+    }
+    int64_t h[2];
+    DG_TRY(read_counters(c, (const int64_t *)(s.cnt + 4), 2, h));
+    if (h[1]) return set_err(c, DGEC_ERR_TIMEOUT, "Boruvka did not finish in 64 rounds");
+    const int64_t m = h[0];
     o.n = m;
     if (m == 0) return DGEC_OK;
     // order by (w, u, v): stable radix by the packed original ends, then by w,
