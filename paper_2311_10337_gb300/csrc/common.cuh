@@ -44,7 +44,7 @@ struct StageTimer {
 };
 
 // Cooperative kernels whose resident-CTA count a context remembers.
-enum CoopKernel { kCoopSortK, kCoopSortKV, kCoopEom, kCoopMsf, kCoopCount };
+enum CoopKernel { kCoopSortK, kCoopSortKV, kCoopEom, kCoopMsf, kCoopDendro, kCoopCount };
 
 struct Ctx {
     int device = 0;

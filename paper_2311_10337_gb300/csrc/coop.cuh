@@ -23,7 +23,7 @@ constexpr unsigned kBarPolls = 1u << 24;
 struct GridBar {
     unsigned *word;
     unsigned *err;
-    unsigned nblk, target;
+    unsigned nblk, target;  // nblk = 1 once one CTA goes on alone
     __device__ __forceinline__ GridBar(unsigned *w, unsigned *e) : word(w), err(e), nblk(gridDim.x), target(0) {}
     __device__ __forceinline__ bool sync() {
         if (nblk == 1) {
@@ -53,8 +53,8 @@ struct GridBar {
     }
     // every CTA calls this after its last barrier
     __device__ __forceinline__ void finish() {
-        if (nblk == 1 || threadIdx.x != 0) return;
-        if (atomicAdd(word + 1, 1u) == nblk - 1) {
+        if (gridDim.x == 1 || threadIdx.x != 0) return;
+        if (atomicAdd(word + 1, 1u) == gridDim.x - 1) {
             word[0] = 0u;
             word[1] = 0u;
         }

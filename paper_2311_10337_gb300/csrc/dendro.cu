@@ -19,6 +19,9 @@
 // pointer tree with no interfering edge is placed whole (a star is one
 // round), so the round count follows the depth of interference, not the
 // dendrogram height.
+#include <algorithm>
+
+#include "sort_dev.cuh"
 #include "stages.cuh"
 
 namespace dgec {
@@ -50,171 +53,18 @@ __global__ void k_d_init(int64_t E, int64_t n, const int32_t *mu, const int32_t 
                          const int32_t *orig_of, int32_t *svpar, SvRec *sv,
                          unsigned long long *minr, unsigned long long *tau, int32_t *parent, int32_t *act, int32_t *ecu,
                          int32_t *ecv) {
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < E + n;
+    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < E;
          x += (int64_t)gridDim.x * blockDim.x) {
         parent[x] = -1;
-        if (x < E) {
-            svpar[x] = (int32_t)x;
-            sv[x] = SvRec{1, orig_of[x], 0};
-            minr[x] = ~0ull;
-            tau[x] = ~0ull;
+        svpar[x] = (int32_t)x;
+        sv[x] = SvRec{1, orig_of[x], 0};
+        minr[x] = ~0ull;
+        tau[x] = ~0ull;
+        if (n == 1 && x == 0) {  // (more rows come ordered, from k_d_order_act)
+            act[0] = 0;
+            ecu[0] = mu[0];
+            ecv[0] = mv[0];
         }
-        if (x < n) {
-            act[x] = (int32_t)x;
-            ecu[x] = mu[x];
-            ecv[x] = mv[x];
-        }
-    }
-}
-
-// Every live forest edge bids its rank into the super-vertices at its ends.
-// The labels (ecu, ecv) travel with the edge and are moved one hop after
-// each round's merges, so no label chain is ever walked. A read before the
-// atomic skips bids that cannot win (slots only decrease).
-__global__ void k_d_bid(const int32_t *act, int64_t na, const int32_t *ecu, const int32_t *ecv,
-                        unsigned long long *minr, unsigned stamp) {
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < na;
-         j += (int64_t)gridDim.x * blockDim.x) {
-        int s = act[j];
-        int cu = ecu[j], cv = ecv[j];
-        const unsigned long long key = rkey(stamp, s);
-        if (key < minr[cu]) atomicMin(&minr[cu], key);
-        if (key < minr[cv]) atomicMin(&minr[cv], key);
-    }
-}
-
-__global__ void k_d_ptr(const int32_t *act, int64_t na, const int32_t *ecu, const int32_t *ecv,
-                        const unsigned long long *minr, unsigned stamp, int32_t *gp) {
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < na;
-         j += (int64_t)gridDim.x * blockDim.x) {
-        int s = act[j], cu = ecu[j], cv = ecv[j];
-        bool pu = rval(minr[cu], stamp) == s, pv = rval(minr[cv], stamp) == s;
-        if (pu && pv) {
-            int r = cu < cv ? cu : cv;
-            gp[cu] = r;
-            gp[cv] = r;
-        } else {
-            if (pu) gp[cu] = cv;
-            if (pv) gp[cv] = cu;
-        }
-    }
-}
-
-__global__ void k_d_gjump(const int32_t *act, int64_t na, const int32_t *ecu, const int32_t *ecv,
-                          const unsigned long long *minr, unsigned stamp, int32_t *gp) {
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < na;
-         j += (int64_t)gridDim.x * blockDim.x) {
-        int s = act[j];
-#pragma unroll
-        for (int side = 0; side < 2; side++) {
-            int c = side ? ecv[j] : ecu[j];
-            if (rval(minr[c], stamp) != s) continue;
-            int r = gp[c];
-            for (int it = 0; it < kMaxWalk; it++) {  // bounded: pointer trees
-                int rr = gp[r];
-                if (rr == r) break;
-                r = rr;
-                gp[c] = r;
-            }
-        }
-    }
-}
-
-__global__ void k_d_tau(const int32_t *act, int64_t na, const int32_t *ecu, const int32_t *ecv,
-                        const unsigned long long *minr, unsigned stamp, const int32_t *gp,
-                        unsigned long long *tau) {
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < na;
-         j += (int64_t)gridDim.x * blockDim.x) {
-        int s = act[j], cu = ecu[j], cv = ecv[j];
-        if (rval(minr[cu], stamp) != s && rval(minr[cv], stamp) != s) {
-            const int gu = gp[cu], gv = gp[cv];
-            const unsigned long long key = rkey(stamp, s);
-            if (key < tau[gu]) atomicMin(&tau[gu], key);
-            if (key < tau[gv]) atomicMin(&tau[gv], key);
-        }
-    }
-}
-
-__global__ void k_d_accept(const int32_t *act, int64_t na, const int32_t *ecu, const int32_t *ecv,
-                           const unsigned long long *minr, unsigned stamp, const int32_t *gp,
-                           const unsigned long long *tau, int *flag) {
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j <= na;
-         j += (int64_t)gridDim.x * blockDim.x) {
-        if (j == na) {
-            flag[j] = 0;
-            continue;
-        }
-        int s = act[j], cu = ecu[j], cv = ecv[j];
-        bool ptr = rval(minr[cu], stamp) == s || rval(minr[cv], stamp) == s;
-        flag[j] = ptr && s < rval(tau[gp[cu]], stamp);
-    }
-}
-
-// accepted edges keyed (group, rank) so a sort puts each group's chain in
-// rank order; the value carries the edge's two super-vertices, the one
-// whose pointer the edge is first (either for the group's mutual edge)
-__global__ void k_d_emit(const int32_t *act, int64_t na, const int32_t *ecu, const int32_t *ecv,
-                         const unsigned long long *minr, unsigned stamp, const int32_t *gp, const int *flag,
-                         const long long *pos,
-                         int sbits, unsigned long long *key, unsigned long long *val) {
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < na;
-         j += (int64_t)gridDim.x * blockDim.x) {
-        if (!flag[j]) continue;
-        const int64_t at = pos[j];
-        const int s = act[j], cu = ecu[j], cv = ecv[j];
-        const bool own_u = rval(minr[cu], stamp) == s;
-        const unsigned Y = (unsigned)(own_u ? cu : cv), O = (unsigned)(own_u ? cv : cu);
-        key[at] = ((unsigned long long)gp[cu] << sbits) | (unsigned long long)s;
-        val[at] = ((unsigned long long)Y << 32) | O;
-    }
-}
-
-__global__ void k_d_chain(const unsigned long long *__restrict__ key, const unsigned long long *__restrict__ val,
-                          int64_t nacc, int64_t E, int sbits, const SvRec *__restrict__ sv, int2 *__restrict__ lab,
-                          int32_t *__restrict__ parent, long long *__restrict__ contrib, int *__restrict__ head) {
-    const unsigned long long smask = (1ull << sbits) - 1ull;
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < nacc;
-         x += (int64_t)gridDim.x * blockDim.x) {
-        const unsigned long long k = key[x], vv = val[x];
-        const unsigned long long G = k >> sbits;
-        const int s = (int)(k & smask);
-        const int Y = (int)(vv >> 32), O = (int)(vv & 0xffffffffu);  // Y: the pointer's owner
-        const bool h = (x == 0) || (key[x - 1] >> sbits) != G;
-        int c1, c2;
-        long long add;
-        const SvRec ry = sv[Y];
-        if (h) {
-            const SvRec ro = sv[O];
-            c1 = ry.root;
-            c2 = ro.root;
-            add = ry.size + ro.size;
-        } else {
-            c1 = (int)(E + (int64_t)(key[x - 1] & smask));
-            c2 = ry.root;
-            add = ry.size;
-        }
-        lab[s] = c1 < c2 ? make_int2(c1, c2) : make_int2(c2, c1);  // one sector per row
-        parent[c1] = (int32_t)(E + s);
-        parent[c2] = (int32_t)(E + s);
-        contrib[x] = add;
-        head[x] = h;
-    }
-}
-
-__global__ void k_d_sizes(const unsigned long long *__restrict__ key, const unsigned long long *__restrict__ val,
-                          int64_t nacc, int64_t E, int sbits, const long long *__restrict__ csum,
-                          int64_t *__restrict__ lsize, int32_t *__restrict__ svpar, SvRec *__restrict__ sv) {
-    const unsigned long long smask = (1ull << sbits) - 1ull;
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < nacc;
-         x += (int64_t)gridDim.x * blockDim.x) {
-        const unsigned long long k = key[x], vv = val[x];
-        const unsigned long long G = k >> sbits;
-        const int s = (int)(k & smask);
-        lsize[s] = csum[x];
-        svpar[(int)(vv >> 32)] = (int32_t)G;
-        svpar[(int)(vv & 0xffffffffu)] = (int32_t)G;
-        bool tail = (x == nacc - 1) || (key[x + 1] >> sbits) != G;
-        if (tail) sv[G] = SvRec{csum[x], (int32_t)(E + s), 0};
     }
 }
 
@@ -240,31 +90,696 @@ __global__ void k_d_order_act(const unsigned long long *k, int64_t n, int sbits,
     }
 }
 
-__global__ void k_d_keep(const int32_t *__restrict__ act, int64_t na, const int *__restrict__ flag,
-                         const long long *__restrict__ pos, int32_t *__restrict__ act2,
-                         const int32_t *__restrict__ ecu, const int32_t *__restrict__ ecv,
-                         int32_t *__restrict__ ecu2, int32_t *__restrict__ ecv2,
-                         const int32_t *__restrict__ svpar) {
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < na;
-         j += (int64_t)gridDim.x * blockDim.x) {
+// A dendrogram row as the rounds write it: one whole sector. `parent` is the
+// merge above (a node id, -1 at a root).
+struct __align__(32) DRow {
+    int32_t a, b, parent, pad;
+    int64_t size, pad2;
+};
+
+__global__ void k_d_split(const DRow *__restrict__ row, int64_t n, int32_t *__restrict__ la,
+                          int32_t *__restrict__ lb, int64_t *__restrict__ size, int32_t *__restrict__ mparent) {
+    for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n;
+         s += (int64_t)gridDim.x * blockDim.x) {
+        const int4 r = *reinterpret_cast<const int4 *>(row + s);
+        la[s] = r.x;
+        lb[s] = r.y;
+        mparent[s] = r.z;
+        size[s] = row[s].size;
+    }
+}
+
+struct DArgs {
+    int64_t E, n;
+    int lb, sbits;  // bits of a label, of a rank
+    int32_t *act, *act2, *ecu, *ecu2, *ecv, *ecv2;  // live edges: rank, labels of the super-vertices at the ends
+    unsigned char *st;                              // per live edge: bit 0/1 it is the pointer of ecu/ecv, bit 2 accepted
+    unsigned long long *minr, *tau;
+    int32_t *gp, *svpar;
+    SvRec *sv;
+    // accepted edges of small groups, group by group
+    int *gcnt;       // [E] by group: its accepted edges (zero between rounds)
+    int2 *gseg;      // [E] by group: (first place, edges); first -1: a large group
+    int32_t *slot;   // [E] by live edge: place within its group
+    int2 *segA;      // (rank, leaves the edge adds)
+    int4 *segB;      // (pointer's owner, group, owner's root, the mutual pair's other root or -1)
+    int2 *segC;      // its group's (first place, edges)
+    unsigned long long *tot;  // [0], [1] places of small groups taken (by round parity), [2], [3] edges of large groups
+    // accepted edges of large groups, sorted by (group, rank)
+    int2 *kids;          // the nodes the edge merges
+    long long *contrib;  // (leaves it adds << 1) | first of its chain
+    DRow *row;
+    int32_t *parent;     // [E] of the leaves
+    SortArgs sort;       // n and bits are set every round
+    unsigned *ccnt;      // [CTAs] accepted edges of each CTA's chunk
+    SegVal *cagg;        // [CTAs] chain sum over each CTA's chunk
+    int *state;          // [0] rounds run, [1] error, [2] live edges (accepted ones after a large round's emit)
+    int max_rounds;
+    unsigned *bar, *err;
+};
+
+// The last rounds (k_d_tail) take over at this many live edges; above
+// kDLarge the host launches every step by itself: the steps are bound by
+// random accesses there and want more threads than the cooperative kernel's
+// 1,024 an SM (every round in that kernel: 53.6 ms for the stage at 100M hub
+// edges, 34 with the large rounds apart); below, its barriers (about 2 us)
+// replace launches and a host read (3M edges: 2.18 ms with the line at 2^19, 2.22
+// at 2^20, 2.78 at 2^22).
+constexpr int kTailMax = 8192;
+constexpr int64_t kDLarge = int64_t(1) << 19;
+// Groups of at most this many accepted edges skip the sort: each edge scans
+// its group (316,229 edges: 1.08 ms for the stage at 16, 0.92 at 32, 0.87 at 64
+// and 128; 10M edges 5.7 at 64, 5.4 at 128).
+constexpr int kDSmall = 128;
+constexpr int kDItems = 4;
+constexpr int kDTile = kSThreads * kDItems;
+
+__device__ __forceinline__ SegVal seg_add(SegVal a, SegVal b) {
+    SegVal r;
+    r.v = b.f ? b.v : a.v + b.v;
+    r.f = a.f | b.f;
+    return r;
+}
+// Ordered exclusive prefix over the CTA's threads; *total: the whole CTA's.
+// sm: kSWarps values, free again after the next __syncthreads.
+__device__ __forceinline__ SegVal seg_block(SegVal v, SegVal *sm, SegVal *total) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    SegVal inc = v;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        SegVal o;
+        o.v = ::__shfl_up_sync(0xffffffffu, inc.v, d);
+        o.f = ::__shfl_up_sync(0xffffffffu, inc.f, d);
+        if (lane >= d) inc = seg_add(o, inc);
+    }
+    if (lane == 31) sm[w] = inc;
+    SegVal ex;
+    ex.v = ::__shfl_up_sync(0xffffffffu, inc.v, 1);
+    ex.f = ::__shfl_up_sync(0xffffffffu, inc.f, 1);
+    if (lane == 0) ex = SegVal{0, 0};
+    __syncthreads();
+    SegVal pre{0, 0}, all{0, 0};
+#pragma unroll
+    for (int i = 0; i < kSWarps; i++) {
+        if (i == w) pre = all;
+        all = seg_add(all, sm[i]);
+    }
+    *total = all;
+    return seg_add(pre, ex);
+}
+
+// A round's state, the same in every CTA.
+struct DRound {
+    int round, G;  // G: CTAs taking part
+    unsigned stamp;
+    int64_t na, nacc, nsmall;  // live edges; accepted ones of large and of small groups
+    bool odd;  // the live list changes sides every round
+};
+#define D_LIST                                                       \
+    const int32_t *act = w.odd ? a.act2 : a.act;                     \
+    int32_t *ecu = w.odd ? a.ecu2 : a.ecu, *ecv = w.odd ? a.ecv2 : a.ecv; \
+    const int64_t na = w.na;                                         \
+    (void)act, (void)ecu, (void)ecv
+#define D_STRIDE \
+    const int64_t gsize = (int64_t)w.G * kSThreads, g0 = (int64_t)blockIdx.x * kSThreads + threadIdx.x
+
+// The steps of a round, each a function of its own so that each gets the
+// registers it needs.
+// Every live edge offers its rank to both super-vertices; the slots are read
+// just before (not ahead for several edges): they only fall, and most offers
+// to a large super-vertex cannot win once a few have been made.
+__device__ __forceinline__ void d_bid(const DArgs &a, const DRound &w) {
+    D_STRIDE;
+    const int32_t *act = w.odd ? a.act2 : a.act;
+    int32_t *ecu = w.odd ? a.ecu2 : a.ecu, *ecv = w.odd ? a.ecv2 : a.ecv;
+    const int64_t na = w.na;
+    for (int64_t j = g0; j < na; j += gsize) {
+        const unsigned long long key = rkey(w.stamp, act[j]);
         int cu = ecu[j], cv = ecv[j];
-        if (!flag[j]) {
-            int64_t at = j - pos[j];
-            act2[at] = act[j];
-            ecu2[at] = svpar[cu];
-            ecv2[at] = svpar[cv];
+        if (w.round > 0) {  // labels move one hop after a round's merges
+            cu = a.svpar[cu];
+            cv = a.svpar[cv];
+            ecu[j] = cu;
+            ecv[j] = cv;
+        }
+        if (key < a.minr[cu]) atomicMin(&a.minr[cu], key);
+        if (key < a.minr[cv]) atomicMin(&a.minr[cv], key);
+    }
+}
+__device__ __forceinline__ void d_ptr(const DArgs &a, const DRound &w) {
+    D_LIST;
+    D_STRIDE;
+    const unsigned stamp = w.stamp;
+    // pointers (a mutual pair points both ends at its smaller label)
+    for (int64_t j0 = g0; j0 < na; j0 += gsize * kDItems) {
+        int s[kDItems], cu[kDItems], cv[kDItems];
+        bool pu[kDItems], pv[kDItems];
+#pragma unroll
+        for (int q = 0; q < kDItems; q++) {
+            const int64_t j = j0 + q * gsize;
+            s[q] = -1;
+            if (j >= na) continue;
+            s[q] = act[j];
+            cu[q] = ecu[j];
+            cv[q] = ecv[j];
+        }
+#pragma unroll
+        for (int q = 0; q < kDItems; q++) {
+            if (s[q] < 0) continue;
+            pu[q] = rval(a.minr[cu[q]], stamp) == s[q];
+            pv[q] = rval(a.minr[cv[q]], stamp) == s[q];
+        }
+#pragma unroll
+        for (int q = 0; q < kDItems; q++) {
+            if (s[q] < 0) continue;
+            if (pu[q] && pv[q]) {
+                const int r = cu[q] < cv[q] ? cu[q] : cv[q];
+                a.gp[cu[q]] = r;
+                a.gp[cv[q]] = r;
+            } else {
+                if (pu[q]) a.gp[cu[q]] = cv[q];
+                if (pv[q]) a.gp[cv[q]] = cu[q];
+            }
+            a.st[j0 + q * gsize] = (unsigned char)((pu[q] ? 1 : 0) | (pv[q] ? 2 : 0));
+        }
+    }
+}
+__device__ __forceinline__ void d_jump(const DArgs &a, const DRound &w) {
+    D_LIST;
+    D_STRIDE;
+    // every pointer to its tree's root
+    for (int64_t j = g0; j < na; j += gsize) {
+        const int st = a.st[j];
+        if (!st) continue;
+#pragma unroll
+        for (int side = 0; side < 2; side++) {
+            if (!((st >> side) & 1)) continue;
+            const int c = side ? ecv[j] : ecu[j];
+            int r = a.gp[c];
+            for (int it = 0; it < kMaxWalk; it++) {  // bounded: pointer trees
+                const int rr = *(volatile int32_t *)(a.gp + r);
+                if (rr == r) break;
+                r = rr;
+                atomicExch(a.gp + c, r);  // (not a store: see d_alloc)
+            }
+        }
+    }
+}
+__device__ __forceinline__ void d_tau(const DArgs &a, const DRound &w) {
+    D_LIST;
+    D_STRIDE;
+    const unsigned stamp = w.stamp;
+    // tau: the smallest non-pointer edge touching each tree
+    for (int64_t j = g0; j < na; j += gsize) {
+        if (a.st[j]) continue;
+        const int gu = a.gp[ecu[j]], gv = a.gp[ecv[j]];
+        const unsigned long long key = rkey(stamp, act[j]);
+        if (key < a.tau[gu]) atomicMin(&a.tau[gu], key);
+        if (key < a.tau[gv]) atomicMin(&a.tau[gv], key);
+    }
+}
+// A place in cnt[g] for every lane with `take`. Two groups of the warp (the
+// first lane's, then the first left's) take theirs with one atomic each, so a
+// very large group does not serialise on its counter; the others one by one.
+__device__ __forceinline__ int group_place(bool take, int g, int *cnt) {
+    unsigned left = __ballot_sync(0xffffffffu, take);
+    int place = 0;
+    const unsigned lt = (1u << lane_id()) - 1u;
+#pragma unroll
+    for (int i = 0; i < 2; i++) {
+        if (!left) return place;
+        const int lead = __ffs(left) - 1;
+        const int lg = ::__shfl_sync(0xffffffffu, g, lead);
+        const unsigned same = left & __ballot_sync(0xffffffffu, g == lg);
+        int base = 0;
+        if ((int)lane_id() == lead) base = atomicAdd(&cnt[lg], __popc(same));
+        base = ::__shfl_sync(0xffffffffu, base, lead);
+        if ((same >> lane_id()) & 1u) place = base + __popc(same & lt);
+        left &= ~same;
+    }
+    if ((left >> lane_id()) & 1u) place = atomicAdd(&cnt[g], 1);
+    return place;
+}
+
+// Accept the pointer edges below their tree's tau; each takes a place in its
+// group, and every CTA counts the edges it keeps.
+__device__ __forceinline__ void d_accept(const DArgs &a, const DRound &w) {
+    __shared__ int s_int[kSWarps];
+    D_LIST;
+    const int tid = threadIdx.x, me = blockIdx.x, G = w.G;
+    const int64_t tiles = (na + kDTile - 1) / kDTile;
+    const int64_t t0 = tiles * me / G, t1 = tiles * (me + 1) / G;
+    const int64_t j1 = t1 * kDTile < na ? t1 * kDTile : na;
+    int cnt = 0;
+    for (int64_t b = t0 * kDTile; b < j1; b += kDTile) {  // CTA-uniform
+        const int64_t jb = b + tid;
+        int s[kDItems], g[kDItems];
+        unsigned char st[kDItems];
+#pragma unroll
+        for (int q = 0; q < kDItems; q++) {
+            const int64_t j = jb + q * kSThreads;
+            st[q] = j < j1 ? a.st[j] : 0;
+            cnt += j < j1;
+            if (st[q]) {
+                s[q] = act[j];
+                g[q] = ecu[j];
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < kDItems; q++)
+            if (st[q]) g[q] = a.gp[g[q]];
+#pragma unroll
+        for (int q = 0; q < kDItems; q++) {
+            const bool acc = st[q] && s[q] < rval(a.tau[g[q]], w.stamp);
+            const int place = group_place(acc, acc ? g[q] : -1, a.gcnt);
+            if (!acc) continue;
+            const int64_t j = jb + q * kSThreads;
+            a.st[j] = st[q] | 4;
+            a.slot[j] = place;
+            cnt--;
+        }
+    }
+    for (int d = 16; d > 0; d >>= 1) cnt += ::__shfl_xor_sync(0xffffffffu, cnt, d);
+    if ((tid & 31) == 0) s_int[tid >> 5] = cnt;
+    __syncthreads();
+    if (tid == 0) {
+        int all = 0;
+        for (int i = 0; i < kSWarps; i++) all += s_int[i];
+        a.ccnt[me] = (unsigned)all;
+    }
+}
+
+// Every group's stretch of the accepted edges, taken by its mutual edge (the
+// one edge that is both ends' pointer, smallest of its group).
+__device__ __forceinline__ void d_alloc(const DArgs &a, const DRound &w) {
+    D_LIST;
+    const int64_t tile = (int64_t)kSThreads * kDItems;
+    for (int64_t base = (int64_t)blockIdx.x * tile; base < na; base += (int64_t)w.G * tile) {  // CTA-uniform
+        // step by step for all items, so that their loads overlap
+        int g[kDItems], gu[kDItems], gv[kDItems], c[kDItems];
+        unsigned need = 0;
+        unsigned char st[kDItems];
+#pragma unroll
+        for (int q = 0; q < kDItems; q++) {
+            const int64_t j = base + q * kSThreads + threadIdx.x;
+            st[q] = j < na ? a.st[j] : 0;
+        }
+#pragma unroll
+        for (int q = 0; q < kDItems; q++) {
+            const int64_t j = base + q * kSThreads + threadIdx.x;
+            gu[q] = gv[q] = -1;
+            if (st[q] == 7) {
+                gu[q] = ecu[j];
+                gv[q] = ecv[j];
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < kDItems; q++) {
+            g[q] = gu[q] < gv[q] ? gu[q] : gv[q];  // the tree's root
+            c[q] = 0;
+            // read and cleared in one: a load and a store here, among other CTAs'
+            // loads of the same lines, takes 8 times as long (0.84 against 0.1 ms
+            // for 16M edges)
+            if (g[q] >= 0) c[q] = atomicExch(&a.gcnt[g[q]], 0);
+        }
+#pragma unroll
+        for (int q = 0; q < kDItems; q++)
+            if (c[q] <= kDSmall) need += (unsigned)c[q];
+        long long at = cta_reserve_count(need, a.tot + (w.round & 1));
+#pragma unroll
+        for (int q = 0; q < kDItems; q++) {
+            if (g[q] < 0) continue;
+            const bool small = c[q] <= kDSmall;
+            a.gseg[g[q]] = make_int2(small ? (int)at : -1, c[q]);
+            if (small) at += c[q];
         }
     }
 }
 
-__global__ void k_d_split(const int2 *__restrict__ lab, int64_t n, int32_t *__restrict__ la,
-                          int32_t *__restrict__ lb) {
-    for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n;
-         s += (int64_t)gridDim.x * blockDim.x) {
-        const int2 r = lab[s];
-        la[s] = r.x;
-        lb[s] = r.y;
+// The accepted edges to their groups' stretches (those of large groups as
+// (group, rank) keys to the sort), the kept ones on to the next round in order.
+// Returns how many are kept.
+__device__ __forceinline__ int64_t d_emit(const DArgs &a, const DRound &w) {
+    __shared__ SegVal s_seg[kSWarps];
+    __shared__ int s_int[kSWarps];
+    D_LIST;
+    const int tid = threadIdx.x, me = blockIdx.x, G = w.G;
+    const int64_t tiles = (na + kDTile - 1) / kDTile;
+    const int64_t t0 = tiles * me / G, t1 = tiles * (me + 1) / G;
+    int64_t kept, pos;
+    {
+        unsigned before = 0, all = 0;
+        for (int i = tid; i < G; i += kSThreads) {
+            const unsigned c = a.ccnt[i];
+            all += c;
+            if (i < me) before += c;
+        }
+        for (int d = 16; d > 0; d >>= 1) {
+            before += ::__shfl_xor_sync(0xffffffffu, before, d);
+            all += ::__shfl_xor_sync(0xffffffffu, all, d);
+        }
+        if ((tid & 31) == 0) s_seg[tid >> 5] = SegVal{(long long)before, (int)all};
+        __syncthreads();
+        unsigned long long b = 0, t = 0;
+        for (int i = 0; i < kSWarps; i++) {
+            b += (unsigned long long)s_seg[i].v;
+            t += (unsigned)s_seg[i].f;
+        }
+        kept = (int64_t)t;
+        pos = (int64_t)b;
     }
+    int32_t *act2 = w.odd ? a.act : a.act2, *ecu2 = w.odd ? a.ecu : a.ecu2, *ecv2 = w.odd ? a.ecv : a.ecv2;
+    for (int64_t t = t0; t < t1; t++) {
+        const int64_t j = t * kDTile + tid * kDItems;
+        int s[kDItems], cu[kDItems], cv[kDItems], sl[kDItems];
+        unsigned char st[kDItems];
+        if (j + kDItems <= na) {
+            const int4 x = *(const int4 *)(act + j), y = *(const int4 *)(ecu + j), z = *(const int4 *)(ecv + j),
+                       l = *(const int4 *)(a.slot + j);
+            const uchar4 f = *(const uchar4 *)(a.st + j);
+            s[0] = x.x, s[1] = x.y, s[2] = x.z, s[3] = x.w;
+            cu[0] = y.x, cu[1] = y.y, cu[2] = y.z, cu[3] = y.w;
+            cv[0] = z.x, cv[1] = z.y, cv[2] = z.z, cv[3] = z.w;
+            sl[0] = l.x, sl[1] = l.y, sl[2] = l.z, sl[3] = l.w;
+            st[0] = f.x, st[1] = f.y, st[2] = f.z, st[3] = f.w;
+        } else {
+#pragma unroll
+            for (int q = 0; q < kDItems; q++) {
+                const bool in = j + q < na;
+                s[q] = in ? act[j + q] : -1;
+                cu[q] = in ? ecu[j + q] : 0;
+                cv[q] = in ? ecv[j + q] : 0;
+                sl[q] = in ? a.slot[j + q] : 0;
+                st[q] = in ? a.st[j + q] : 0;
+            }
+        }
+        int cnt = 0;
+#pragma unroll
+        for (int q = 0; q < kDItems; q++) cnt += s[q] >= 0 && !(st[q] & 4);
+        __syncthreads();  // s_int and s_seg are free again
+        int64_t at = pos + sort_block_exclusive(cnt, s_int);
+        int g[kDItems];
+        int2 sg[kDItems];
+        unsigned large = 0;
+#pragma unroll
+        for (int q = 0; q < kDItems; q++) g[q] = s[q] >= 0 && (st[q] & 4) ? a.gp[cu[q]] : -1;
+#pragma unroll
+        for (int q = 0; q < kDItems; q++) {
+            sg[q] = g[q] >= 0 ? a.gseg[g[q]] : make_int2(0, 0);
+            large += sg[q].x < 0;
+        }
+        long long lx = 0;
+        if (__syncthreads_or(large)) lx = cta_reserve_count(large, a.tot + 2 + (w.round & 1));
+#pragma unroll
+        for (int q = 0; q < kDItems; q++) {
+            if (s[q] < 0) continue;
+            if (g[q] < 0) {
+                act2[at] = s[q];
+                ecu2[at] = cu[q];
+                ecv2[at] = cv[q];
+                at++;
+                continue;
+            }
+            const bool mutual = (st[q] & 3) == 3;
+            int Y = (st[q] & 1) ? cu[q] : cv[q], O = (st[q] & 1) ? cv[q] : cu[q];
+            if (mutual && Y == g[q]) {  // the pair's other end, so that the root's own label needs no change
+                Y = O;
+                O = g[q];
+            }
+            if (sg[q].x >= 0) {
+                const SvRec ry = a.sv[Y];
+                int add = (int)ry.size, ro = -1;
+                if (mutual) {
+                    const SvRec o = a.sv[O];
+                    add += (int)o.size;
+                    ro = o.root;
+                }
+                const int x = sg[q].x + sl[q];
+                a.segA[x] = make_int2(s[q], add);
+                a.segB[x] = make_int4(Y, g[q], ry.root, ro);
+                a.segC[x] = sg[q];
+            } else {
+                a.sort.ka[lx] = ((unsigned long long)(unsigned)g[q] << a.sbits) | (unsigned)s[q];
+                a.sort.va[lx] = ((unsigned long long)(unsigned)Y << 32) | (unsigned)O;
+                lx++;
+            }
+        }
+        int tot = 0;
+        for (int i = 0; i < kSWarps; i++) tot += s_int[i];
+        pos += tot;
+    }
+    return kept;
+}
+
+// The chains of the small groups: an edge finds the edges before and after it
+// among its group's few, and the leaves below.
+__device__ __forceinline__ void d_small(const DArgs &a, const DRound &w, int64_t n) {
+    D_STRIDE;
+    for (int64_t x = g0; x < n; x += gsize) {
+        const int2 c = a.segC[x];
+        const int4 e = a.segB[x];
+        const int2 me = a.segA[x];
+        int prev = -1, next = INT_MAX, size = me.y;
+        for (int i = 0; i < c.y; i++) {
+            const int2 o = a.segA[c.x + i];
+            if (o.x < me.x) {
+                size += o.y;
+                if (o.x > prev) prev = o.x;
+            } else if (o.x > me.x && o.x < next) {
+                next = o.x;
+            }
+        }
+        const int node = (int)(a.E + me.x);
+        const int n1 = prev < 0 ? e.w : (int)(a.E + prev), n2 = e.z;
+        DRow *r = a.row + me.x;
+        *(int4 *)r = make_int4(n1 < n2 ? n1 : n2, n1 < n2 ? n2 : n1, next == INT_MAX ? -1 : (int)(a.E + next), 0);
+        *(longlong2 *)((char *)r + 16) = make_longlong2(size, 0);
+        if (n2 < a.E) a.parent[n2] = node;
+        else a.row[n2 - a.E].parent = node;
+        if (prev < 0) {
+            if (n1 < a.E) a.parent[n1] = node;
+            else a.row[n1 - a.E].parent = node;
+        }
+        a.svpar[e.x] = e.y;
+        if (next == INT_MAX) a.sv[e.y] = SvRec{size, node, 0};
+    }
+}
+
+__device__ __forceinline__ void d_chain(const DArgs &a, const DRound &w, const unsigned long long *__restrict__ key, const unsigned long long *__restrict__ val) {
+    __shared__ SegVal s_seg[kSWarps];
+    const int tid = threadIdx.x, me = blockIdx.x, G = w.G;
+    const int64_t nacc = w.nacc, ct = (nacc + kDTile - 1) / kDTile;
+    const int64_t c0 = ct * me / G, c1 = ct * (me + 1) / G;
+    const unsigned long long smask = (1ull << a.sbits) - 1ull;
+    // the chains: g_1 joins the mutual pair, g_k joins g_{k-1} with the
+    // super-vertex whose pointer it is
+    SegVal agg{0, 0};
+    for (int64_t t = c0; t < c1; t++) {
+        const int64_t x0 = t * kDTile + tid * kDItems;
+        unsigned long long k[kDItems], v[kDItems];
+        unsigned long long kp = x0 > 0 && x0 < nacc ? key[x0 - 1] : ~0ull;
+#pragma unroll
+        for (int q = 0; q < kDItems; q++) {
+            const bool in = x0 + q < nacc;
+            k[q] = in ? key[x0 + q] : 0;
+            v[q] = in ? val[x0 + q] : 0;
+        }
+        SvRec y[kDItems];
+#pragma unroll
+        for (int q = 0; q < kDItems; q++)
+            if (x0 + q < nacc) y[q] = a.sv[v[q] >> 32];
+        SegVal mine{0, 0};
+#pragma unroll
+        for (int q = 0; q < kDItems; q++) {
+            const int64_t x = x0 + q;
+            if (x >= nacc) continue;
+            const bool h = x == 0 || (kp >> a.sbits) != (k[q] >> a.sbits);
+            int n1;
+            long long add = y[q].size;
+            if (h) {
+                const SvRec o = a.sv[v[q] & 0xffffffffull];
+                n1 = o.root;
+                add += o.size;
+            } else {
+                n1 = (int)(a.E + (int64_t)(kp & smask));
+            }
+            a.kids[x] = make_int2(n1, y[q].root);
+            a.contrib[x] = (add << 1) | (h ? 1 : 0);
+            mine = seg_add(mine, SegVal{add, h ? 1 : 0});
+            kp = k[q];
+        }
+        SegVal tot;
+        __syncthreads();  // s_seg is free again
+        seg_block(mine, s_seg, &tot);
+        agg = seg_add(agg, tot);
+    }
+    if (tid == 0) a.cagg[me] = agg;
+}
+__device__ __forceinline__ void d_rows(const DArgs &a, const DRound &w, const unsigned long long *__restrict__ key, const unsigned long long *__restrict__ val) {
+    __shared__ SegVal s_seg[kSWarps];
+    const int tid = threadIdx.x, me = blockIdx.x, G = w.G;
+    const int64_t nacc = w.nacc, ct = (nacc + kDTile - 1) / kDTile;
+    const int64_t c0 = ct * me / G, c1 = ct * (me + 1) / G;
+    const unsigned long long smask = (1ull << a.sbits) - 1ull;
+    // sizes along the chains, rows, and the merged super-vertices
+    SegVal run{0, 0};
+    for (int i0 = 0; i0 < me; i0 += kSThreads) {
+        SegVal v = i0 + tid < me ? a.cagg[i0 + tid] : SegVal{0, 0};
+        SegVal tot;
+        __syncthreads();
+        seg_block(v, s_seg, &tot);
+        run = seg_add(run, tot);
+    }
+    for (int64_t t = c0; t < c1; t++) {
+        const int64_t x0 = t * kDTile + tid * kDItems;
+        unsigned long long k[kDItems + 1], v[kDItems];
+        long long cb[kDItems];
+        int2 kid[kDItems];
+        SegVal mine{0, 0};
+#pragma unroll
+        for (int q = 0; q < kDItems; q++) {
+            const bool in = x0 + q < nacc;
+            k[q] = in ? key[x0 + q] : ~0ull;
+            v[q] = in ? val[x0 + q] : 0;
+            cb[q] = in ? a.contrib[x0 + q] : 0;
+            if (in) kid[q] = a.kids[x0 + q];
+        }
+        k[kDItems] = x0 + kDItems < nacc ? key[x0 + kDItems] : ~0ull;
+#pragma unroll
+        for (int q = 0; q < kDItems; q++)
+            if (x0 + q < nacc) mine = seg_add(mine, SegVal{cb[q] >> 1, (int)(cb[q] & 1)});
+        SegVal tot;
+        __syncthreads();  // s_seg is free again
+        SegVal pre = seg_add(run, seg_block(mine, s_seg, &tot));
+        run = seg_add(run, tot);
+#pragma unroll
+        for (int q = 0; q < kDItems; q++) {
+            const int64_t x = x0 + q;
+            if (x >= nacc) continue;
+            const bool h = cb[q] & 1;
+            pre = seg_add(pre, SegVal{cb[q] >> 1, h ? 1 : 0});
+            const int grp = (int)(k[q] >> a.sbits), s = (int)(k[q] & smask);
+            const bool tail = x == nacc - 1 || (k[q + 1] >> a.sbits) != (k[q] >> a.sbits);
+            const int node = (int)(a.E + s), n1 = kid[q].x, n2 = kid[q].y;
+            DRow *r = a.row + s;
+            *(int4 *)r = make_int4(n1 < n2 ? n1 : n2, n1 < n2 ? n2 : n1,
+                                   tail ? -1 : (int)(a.E + (int64_t)(k[q + 1] & smask)), 0);
+            *(longlong2 *)((char *)r + 16) = make_longlong2(pre.v, 0);
+            // the children's parent (a chain's merge below knows already)
+            if (n2 < a.E) a.parent[n2] = node;
+            else a.row[n2 - a.E].parent = node;
+            a.svpar[v[q] >> 32] = grp;
+            if (h) {
+                if (n1 < a.E) a.parent[n1] = node;
+                else a.row[n1 - a.E].parent = node;
+                a.svpar[v[q] & 0xffffffffull] = grp;
+            }
+            if (tail) a.sv[grp] = SvRec{pre.v, node, 0};
+        }
+    }
+}
+// Large rounds: every step a kernel of its own, at the occupancy its
+// registers allow.
+#define D_KERNEL(name, call)                                                                          \
+    __global__ void __launch_bounds__(kSThreads, 2) k_d_##name(const __grid_constant__ DArgs a,       \
+                                                               const __grid_constant__ DRound w) { call; }
+D_KERNEL(bid, d_bid(a, w))
+D_KERNEL(ptr, d_ptr(a, w))
+D_KERNEL(jump, d_jump(a, w))
+D_KERNEL(tau, d_tau(a, w))
+D_KERNEL(accept, d_accept(a, w))
+D_KERNEL(alloc, d_alloc(a, w))
+D_KERNEL(emit, const int64_t n = d_emit(a, w); if (blockIdx.x == 0 && threadIdx.x == 0) a.state[2] = (int)n)
+D_KERNEL(small, d_small(a, w, w.nsmall))
+#undef D_KERNEL
+__global__ void __launch_bounds__(kSThreads, 2) k_d_chain(const __grid_constant__ DArgs a, const __grid_constant__ DRound w,
+                                                       const unsigned long long *key, const unsigned long long *val) {
+    d_chain(a, w, key, val);
+}
+__global__ void __launch_bounds__(kSThreads, 2) k_d_rows(const __grid_constant__ DArgs a, const __grid_constant__ DRound w,
+                                                      const unsigned long long *key, const unsigned long long *val) {
+    d_rows(a, w, key, val);
+}
+
+// The same steps inside the cooperative kernel, as calls so that each keeps
+// its own registers.
+__device__ __noinline__ void dc_bid(const DArgs &a, const DRound &w) { d_bid(a, w); }
+__device__ __noinline__ void dc_ptr(const DArgs &a, const DRound &w) { d_ptr(a, w); }
+__device__ __noinline__ void dc_jump(const DArgs &a, const DRound &w) { d_jump(a, w); }
+__device__ __noinline__ void dc_tau(const DArgs &a, const DRound &w) { d_tau(a, w); }
+__device__ __noinline__ void dc_accept(const DArgs &a, const DRound &w) { d_accept(a, w); }
+__device__ __noinline__ void dc_alloc(const DArgs &a, const DRound &w) { d_alloc(a, w); }
+__device__ __noinline__ void dc_small(const DArgs &a, const DRound &w) { d_small(a, w, w.nsmall); }
+__device__ __noinline__ int64_t dc_emit(const DArgs &a, const DRound &w) { return d_emit(a, w); }
+__device__ __noinline__ void dc_chain(const DArgs &a, const DRound &w, const unsigned long long *key,
+                                      const unsigned long long *val) { d_chain(a, w, key, val); }
+__device__ __noinline__ void dc_rows(const DArgs &a, const DRound &w, const unsigned long long *key,
+                                     const unsigned long long *val) { d_rows(a, w, key, val); }
+__device__ __noinline__ bool dc_sort(const DArgs &a, int64_t n, int bits, int most, unsigned long long *sm, GridBar &bar) {
+    return sort_run<true>(a.sort, n, 0, bits, most, sort_smem<true>(sm), bar);
+}
+#undef D_LIST
+#undef D_STRIDE
+
+// Middle rounds in one cooperative kernel: no launch and no host read between
+// the steps, from the round the host stops at until at most kTailMax edges
+// are live.
+__global__ void __launch_bounds__(kSThreads, 2) k_d_rounds(const __grid_constant__ DArgs a, const __grid_constant__ DRound w0) {
+    extern __shared__ __align__(16) unsigned long long d_sm[];
+    GridBar bar(a.bar, a.err);
+    DRound w = w0;
+    w.G = gridDim.x;
+    int error = 0;
+    for (; w.na > kTailMax; w.round++) {
+        if (w.round >= a.max_rounds) {
+            error = 1;
+            break;
+        }
+        w.odd = w.round & 1;
+        w.stamp = kStampTop - (unsigned)w.round;
+        dc_bid(a, w);
+        if (!bar.sync()) return;
+        dc_ptr(a, w);
+        if (!bar.sync()) return;
+        dc_jump(a, w);
+        if (!bar.sync()) return;
+        dc_tau(a, w);
+        if (!bar.sync()) return;
+        dc_accept(a, w);
+        if (!bar.sync()) return;
+        dc_alloc(a, w);
+        if (!bar.sync()) return;
+        const int64_t kept = dc_emit(a, w);
+        if (kept == w.na) {  // cannot be: every round accepts each tree's mutual edge
+            error = 2;
+            break;
+        }
+        if (!bar.sync()) return;
+        volatile unsigned long long *tot = a.tot;
+        w.nsmall = (int64_t)tot[w.round & 1];
+        w.nacc = (int64_t)tot[2 + (w.round & 1)];
+        if (blockIdx.x == 0 && threadIdx.x == 0) tot[(w.round & 1) ^ 1] = tot[2 + ((w.round & 1) ^ 1)] = 0;
+        dc_small(a, w);
+        if (w.nacc > 0) {
+            // each large group's chain in rank order
+            const int kbits = a.lb + a.sbits, most = w.nacc > kSNarrow ? kSBits - 1 : kSBits;
+            if (!dc_sort(a, w.nacc, kbits, most, d_sm, bar)) return;
+            if (!bar.sync()) return;
+            const bool in_b = sort_in_b(w.nacc, kbits, most);
+            const unsigned long long *key = in_b ? a.sort.kb : a.sort.ka, *val = in_b ? a.sort.vb : a.sort.va;
+            dc_chain(a, w, key, val);
+            if (!bar.sync()) return;
+            dc_rows(a, w, key, val);
+        }
+        if (!bar.sync()) return;
+        w.na = kept;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.state[0] = w.round;
+        a.state[1] = error;
+        a.state[2] = (int)w.na;
+    }
+    bar.finish();
 }
 
 // ------------------------------------------------ one-CTA tail of the rounds
@@ -275,33 +790,47 @@ __global__ void k_d_split(const int2 *__restrict__ lab, int64_t n, int32_t *__re
 // bitonic network, and no count read on the host between rounds. The output
 // orders of acceptance and keep come from shared counters: the sort orders
 // the accepted edges, and the live list's order changes no result.
-constexpr int kTailMax = 8192;
 constexpr int kTailThreads = 1024;
 constexpr size_t kTailSmem = (size_t)kTailMax * 16 + kTailMax;
 
-__device__ __forceinline__ SegVal tail_seg(SegVal a, SegVal b) {
-    SegVal r;
-    r.v = b.f ? b.v : a.v + b.v;
-    r.f = a.f | b.f;
-    return r;
-}
-
 __global__ void __launch_bounds__(kTailThreads) k_d_tail(
-    int32_t *act, int32_t *act2, int32_t *ecu, int32_t *ecu2, int32_t *ecv, int32_t *ecv2, int64_t na0, int64_t E,
-    int sbits, unsigned round0, unsigned max_rounds, unsigned long long *minr, unsigned long long *tau, int32_t *gp,
-    SvRec *sv, int32_t *svpar, int2 *lab, int32_t *parent, int64_t *lsize, int *status) {
+    const __grid_constant__ DArgs a) {
     extern __shared__ unsigned long long tsm[];
     unsigned long long *skey = tsm, *sval = tsm + kTailMax;
     unsigned char *sflag = (unsigned char *)(tsm + 2 * kTailMax);
     __shared__ int s_nacc, s_nkeep;
     __shared__ SegVal s_warp[kTailThreads / 32];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const unsigned long long smask = (1ull << sbits) - 1ull;
-    int na = (int)na0;
+    if (a.state[1]) return;  // an error of the rounds before
+    const unsigned round0 = (unsigned)a.state[0];
+    int na = a.state[2];
     unsigned round = round0;
+    const int64_t E = a.E;
+    const int sbits = a.sbits;
+    const unsigned long long smask = (1ull << sbits) - 1ull;
+    unsigned long long *minr = a.minr, *tau = a.tau;
+    int32_t *gp = a.gp, *svpar = a.svpar;
+    SvRec *sv = a.sv;
+    DRow *row = a.row;
+    const bool odd = round0 & 1;
+    int32_t *act = odd ? a.act2 : a.act, *act2 = odd ? a.act : a.act2;
+    int32_t *ecu = odd ? a.ecu2 : a.ecu, *ecu2 = odd ? a.ecu : a.ecu2;
+    int32_t *ecv = odd ? a.ecv2 : a.ecv, *ecv2 = odd ? a.ecv : a.ecv2;
+    auto set_parent = [&](int c, int node) {
+        if (c < E) a.parent[c] = node;
+        else row[c - E].parent = node;
+    };
+    for (int j = tid; j < na; j += kTailThreads) {
+        if (round0 > 0) {  // the hop after the last round's merges
+            ecu[j] = svpar[ecu[j]];
+            ecv[j] = svpar[ecv[j]];
+        }
+        row[act[j]].parent = -1;
+    }
+    __syncthreads();
     while (na > 0) {
-        if (round - round0 >= max_rounds) {
-            if (tid == 0) status[1] = 1;
+        if (round >= (unsigned)a.max_rounds) {
+            if (tid == 0) a.state[1] = 1;
             return;
         }
         const unsigned stamp = kStampTop - round;
@@ -375,7 +904,7 @@ __global__ void __launch_bounds__(kTailThreads) k_d_tail(
         __syncthreads();
         const int nacc = s_nacc;
         if (nacc == 0) {  // every round accepts each tree's mutual edge
-            if (tid == 0) status[1] = 2;
+            if (tid == 0) a.state[1] = 2;
             return;
         }
         int N = 1;
@@ -425,9 +954,10 @@ __global__ void __launch_bounds__(kTailThreads) k_d_tail(
                 c2 = ry.root;
                 add[q] = ry.size;
             }
-            lab[s] = c1 < c2 ? make_int2(c1, c2) : make_int2(c2, c1);
-            parent[c1] = (int32_t)(E + s);
-            parent[c2] = (int32_t)(E + s);
+            row[s].a = c1 < c2 ? c1 : c2;
+            row[s].b = c1 < c2 ? c2 : c1;
+            set_parent(c1, (int)(E + s));
+            set_parent(c2, (int)(E + s));
             hd[q] = h;
         }
         // sizes along each chain: a segmented inclusive sum over the runs
@@ -439,14 +969,14 @@ __global__ void __launch_bounds__(kTailThreads) k_d_tail(
             SegVal it;
             it.v = add[q];
             it.f = hd[q];
-            agg = tail_seg(agg, it);
+            agg = seg_add(agg, it);
         }
         SegVal inc = agg;
         for (int d = 1; d < 32; d <<= 1) {
             SegVal o;
             o.v = ::__shfl_up_sync(0xffffffffu, inc.v, d);
             o.f = ::__shfl_up_sync(0xffffffffu, inc.f, d);
-            if (lane >= d) inc = tail_seg(o, inc);
+            if (lane >= d) inc = seg_add(o, inc);
         }
         if (lane == 31) s_warp[wid] = inc;
         __syncthreads();  // also orders the chains' reads of sv before the writes below
@@ -456,7 +986,7 @@ __global__ void __launch_bounds__(kTailThreads) k_d_tail(
                 SegVal o;
                 o.v = ::__shfl_up_sync(0xffffffffu, w.v, d);
                 o.f = ::__shfl_up_sync(0xffffffffu, w.f, d);
-                if (lane >= d) w = tail_seg(o, w);
+                if (lane >= d) w = seg_add(o, w);
             }
             s_warp[lane] = w;
         }
@@ -470,7 +1000,7 @@ __global__ void __launch_bounds__(kTailThreads) k_d_tail(
                 ex.v = 0;
                 ex.f = 0;
             }
-            if (wid > 0) ex = lane == 0 ? s_warp[wid - 1] : tail_seg(s_warp[wid - 1], ex);
+            if (wid > 0) ex = lane == 0 ? s_warp[wid - 1] : seg_add(s_warp[wid - 1], ex);
             run = ex;
         }
 #pragma unroll
@@ -480,11 +1010,11 @@ __global__ void __launch_bounds__(kTailThreads) k_d_tail(
             SegVal it;
             it.v = add[q];
             it.f = hd[q];
-            run = tail_seg(run, it);
+            run = seg_add(run, it);
             const unsigned long long k = skey[x], vv = sval[x];
             const unsigned long long G = k >> sbits;
             const int s = (int)(k & smask);
-            lsize[s] = run.v;
+            row[s].size = run.v;
             svpar[(int)(vv >> 32)] = (int32_t)G;
             svpar[(int)(vv & 0xffffffffu)] = (int32_t)G;
             if (x == nacc - 1 || (skey[x + 1] >> sbits) != G) sv[G] = SvRec{run.v, (int32_t)(E + s), 0};
@@ -512,7 +1042,7 @@ __global__ void __launch_bounds__(kTailThreads) k_d_tail(
         round++;
         __syncthreads();
     }
-    if (tid == 0) status[0] = (int)(round - round0);
+    if (tid == 0) a.state[0] = (int)round;
 }
 
 void plan_dendro(Arena &ws, const Problem &p, Dendro &o) {
@@ -524,13 +1054,18 @@ void plan_dendro(Arena &ws, const Problem &p, Dendro &o) {
 
 struct DScratch {
     int32_t *svpar, *gp, *act, *act2, *ecu, *ecv, *ecu2, *ecv2;
+    unsigned char *st;
     SvRec *sv;
-    int *tstat;  // one-CTA tail: [0] rounds run, [1] error
-    int2 *lab;  // rows (a, b) side by side; split into the two outputs at the end
+    int *state;
+    DRow *row;
     unsigned long long *minr, *tau;  // round-stamped slots (see rkey)
-    int *flag, *head;
-    long long *pos, *contrib, *csum, *scan_tmp;
-    SegVal *seg_tmp;
+    int *gcnt;
+    int2 *gseg, *segA, *segC, *kids;
+    int4 *segB;
+    int32_t *slot;
+    long long *contrib;
+    unsigned *ccnt;
+    SegVal *cagg;
     unsigned long long *k1, *k2, *v1, *v2;
     void *radix;
 };
@@ -539,8 +1074,8 @@ static DScratch carve_dendro(Arena &a, const Problem &p) {
     int64_t E = p.E;
     s.svpar = a.take<int32_t>(E);
     s.sv = a.take<SvRec>(E);
-    s.tstat = a.take<int>(2);
-    s.lab = a.take<int2>(E);
+    s.state = a.take<int>(12);  // state[4], then tot[4] as 64-bit words
+    s.row = a.take<DRow>(E);
     s.minr = a.take<unsigned long long>(E);
     s.tau = a.take<unsigned long long>(E);
     s.gp = a.take<int32_t>(E);
@@ -550,13 +1085,18 @@ static DScratch carve_dendro(Arena &a, const Problem &p) {
     s.ecv = a.take<int32_t>(E);
     s.ecu2 = a.take<int32_t>(E);
     s.ecv2 = a.take<int32_t>(E);
-    s.flag = a.take<int>(E + 1);
-    s.head = a.take<int>(E + 1);
-    s.pos = a.take<long long>(E + 1);
-    s.contrib = a.take<long long>(E + 1);
-    s.csum = a.take<long long>(E + 1);
-    s.scan_tmp = a.take<long long>(scan_scratch_elems(E + 1));
-    s.seg_tmp = a.take<SegVal>(scan_scratch_elems(E + 1));
+    s.st = a.take<unsigned char>(E);
+    s.gcnt = a.take<int>(E);
+    s.gseg = a.take<int2>(E);
+    s.slot = a.take<int32_t>(E);
+    s.segA = a.take<int2>(E);
+    s.segB = a.take<int4>(E);
+    s.segC = a.take<int2>(E);
+    s.kids = a.take<int2>(E);
+    s.contrib = a.take<long long>(E);
+    const int64_t ctas = sort_ranges_of(E, kSRanges);
+    s.ccnt = a.take<unsigned>(ctas);
+    s.cagg = a.take<SegVal>(ctas);
     s.k1 = a.take<unsigned long long>(E);
     s.k2 = a.take<unsigned long long>(E);
     s.v1 = a.take<unsigned long long>(E);
@@ -577,7 +1117,7 @@ dgec_status stage_dendro(Ctx *c, const Problem &p, const Csr &g, const Msf &m, D
     if (E == 0) return DGEC_OK;
     Arena a(scratch, SIZE_MAX);
     DScratch s = carve_dendro(a, p);
-    TK(c, "k_d_init", k_d_init<<<grid_for(E + n, kBlock, kStreamCap), kBlock, 0, st>>>(
+    TK(c, "k_d_init", k_d_init<<<grid_for(E, kBlock, kStreamCap), kBlock, 0, st>>>(
                           E, n, m.ru, m.rv, g.orig_of, s.svpar, s.sv, s.minr, s.tau,
                           o.parent, s.act, s.ecu, s.ecv));
     const int lb = p.idbits > 0 ? p.idbits : 1;
@@ -590,65 +1130,82 @@ dgec_status stage_dendro(Ctx *c, const Problem &p, const Csr &g, const Msf &m, D
         TK(c, "k_d_order_act", k_d_order_act<<<gn, kBlock, 0, st>>>(in_b ? s.k2 : s.k1, n, sbits, m.rv, s.act,
                                                                s.ecu, s.ecv));
     }
-    int64_t na = n;
-    int32_t *act = s.act, *act2 = s.act2, *ecu = s.ecu, *ecv = s.ecv, *ecu2 = s.ecu2, *ecv2 = s.ecv2;
-    for (int64_t round = 0; na > 0; round++) {
-        if (round >= (1 << 16))
-            return set_err(c, DGEC_ERR_TIMEOUT, "dendrogram rounds exceeded %d", 1 << 16);
-        if (na <= kTailMax) {  // the rest in one CTA, one launch
-            CU_TRY(c, cudaFuncSetAttribute(k_d_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmem));
-            CU_TRY(c, cudaMemsetAsync(s.tstat, 0, 2 * sizeof(int), st));
-            TK(c, "k_d_tail", k_d_tail<<<1, kTailThreads, kTailSmem, st>>>(
-                                  act, act2, ecu, ecu2, ecv, ecv2, na, E, sbits, (unsigned)round,
-                                  (unsigned)((1 << 16) - round), s.minr, s.tau, s.gp, s.sv, s.svpar, s.lab,
-                                  o.parent, o.size, s.tstat));
-            int64_t ts;
-            DG_TRY(read_counters(c, (const int64_t *)s.tstat, 1, &ts));
-            const int done_rounds = (int)(ts & 0xffffffff), err = (int)(ts >> 32);
-            if (err == 1) return set_err(c, DGEC_ERR_TIMEOUT, "dendrogram rounds exceeded %d", 1 << 16);
-            if (err) return set_err(c, DGEC_ERR_INTERNAL, "dendrogram round accepted no edge");
-            o.rounds = round + done_rounds;
-            break;
+    if (n > 0) {
+        DArgs d{E, n, lb, sbits, s.act, s.act2, s.ecu, s.ecu2, s.ecv, s.ecv2, s.st, s.minr, s.tau, s.gp, s.svpar, s.sv,
+                s.gcnt, s.gseg, s.slot, s.segA, s.segB, s.segC, (unsigned long long *)(s.state + 4), s.kids, s.contrib,
+                s.row, o.parent,
+                sort_args(c, RadixBuffers{s.k1, s.k2, s.v1, s.v2}, n, 0, lb + sbits, s.radix, E), s.ccnt, s.cagg,
+                s.state, 1 << 16, c->bar, c->bar_err};
+        DRound w{0, 0, kStampTop, n, 0, 0, false};
+        CU_TRY(c, cudaMemsetAsync(s.state, 0, sizeof(int) * 12, st));
+        CU_TRY(c, cudaMemsetAsync(s.gcnt, 0, sizeof(int) * E, st));
+        const int most = (int)sort_ranges_of(E, kSRanges);  // CTAs the per-CTA counts have room for
+        for (; w.na > kDLarge; w.round++) {
+            if (w.round >= d.max_rounds)
+                return set_err(c, DGEC_ERR_TIMEOUT, "dendrogram rounds exceeded %d", d.max_rounds);
+            w.odd = w.round & 1;
+            w.stamp = kStampTop - (unsigned)w.round;
+            const int wide = (int)std::min<int64_t>(cdiv(w.na, kSThreads), c->stream_ctas);
+            const int few = (int)std::min<int64_t>(std::min<int64_t>(cdiv(w.na, kDTile), 4 * (int64_t)c->num_sms), most);
+            w.G = wide;
+            TK(c, "k_d_bid", k_d_bid<<<wide, kSThreads, 0, st>>>(d, w));
+            w.G = (int)std::min<int64_t>(cdiv(w.na, kDTile), c->stream_ctas);
+            TK(c, "k_d_ptr", k_d_ptr<<<w.G, kSThreads, 0, st>>>(d, w));
+            w.G = wide;
+            TK(c, "k_d_gjump", k_d_jump<<<wide, kSThreads, 0, st>>>(d, w));
+            TK(c, "k_d_tau", k_d_tau<<<wide, kSThreads, 0, st>>>(d, w));
+            w.G = few;
+            TK(c, "k_d_accept", k_d_accept<<<few, kSThreads, 0, st>>>(d, w));
+            w.G = (int)std::min<int64_t>(cdiv(w.na, kDTile), c->stream_ctas);
+            TK(c, "k_d_alloc", k_d_alloc<<<w.G, kSThreads, 0, st>>>(d, w));
+            w.G = few;
+            TK(c, "k_d_emit", k_d_emit<<<few, kSThreads, 0, st>>>(d, w));
+            int64_t h[6];  // state, then tot
+            DG_TRY(read_counters(c, (const int64_t *)s.state, 6, h));
+            const int64_t kept = (int)(h[1] & 0xffffffff);
+            if (kept == w.na) return set_err(c, DGEC_ERR_INTERNAL, "dendrogram round accepted no edge");
+            w.nsmall = h[2 + (w.round & 1)];
+            w.nacc = h[4 + (w.round & 1)];
+            CU_TRY(c, cudaMemsetAsync(d.tot, 0, 4 * sizeof(unsigned long long), st));
+            if (w.nsmall > 0) {
+                w.G = (int)std::min<int64_t>(cdiv(w.nsmall, kSThreads), c->stream_ctas);
+                TK(c, "k_d_small", k_d_small<<<w.G, kSThreads, 0, st>>>(d, w));
+            }
+            if (w.nacc > 0) {
+                bool in_b;
+                DG_TRY(radix_sort(c, RadixBuffers{s.k1, s.k2, s.v1, s.v2}, w.nacc, 0, lb + sbits, s.radix, &in_b));
+                const unsigned long long *key = in_b ? s.k2 : s.k1, *val = in_b ? s.v2 : s.v1;
+                w.G = (int)std::min<int64_t>(std::min<int64_t>(cdiv(w.nacc, kDTile), 4 * (int64_t)c->num_sms), most);
+                TK(c, "k_d_chain", k_d_chain<<<w.G, kSThreads, 0, st>>>(d, w, key, val));
+                TK(c, "k_d_rows", k_d_rows<<<w.G, kSThreads, 0, st>>>(d, w, key, val));
+            }
+            w.na = kept;
         }
-        const int g = grid_for(na, kBlock, kStreamCap);
-        const unsigned stamp = kStampTop - (unsigned)round;
-        TK(c, "k_d_bid", k_d_bid<<<g, kBlock, 0, st>>>(act, na, ecu, ecv, s.minr, stamp));
-        TK(c, "k_d_ptr", k_d_ptr<<<g, kBlock, 0, st>>>(act, na, ecu, ecv, s.minr, stamp, s.gp));
-        TK(c, "k_d_gjump", k_d_gjump<<<g, kBlock, 0, st>>>(act, na, ecu, ecv, s.minr, stamp, s.gp));
-        TK(c, "k_d_tau", k_d_tau<<<g, kBlock, 0, st>>>(act, na, ecu, ecv, s.minr, stamp, s.gp, s.tau));
-        TK(c, "k_d_accept", k_d_accept<<<grid_for(na + 1, kBlock, kStreamCap), kBlock, 0, st>>>(
-                                act, na, ecu, ecv, s.minr, stamp, s.gp, s.tau, s.flag));
-        DG_TRY(exclusive_scan_i32(c, s.flag, s.pos, na + 1, s.scan_tmp));
-        int64_t nacc;
-        DG_TRY(read_counters(c, (const int64_t *)(s.pos + na), 1, &nacc));
-        if (nacc <= 0) return set_err(c, DGEC_ERR_INTERNAL, "dendrogram round accepted no edge");
-        TK(c, "k_d_emit", k_d_emit<<<g, kBlock, 0, st>>>(act, na, ecu, ecv, s.minr, stamp, s.gp, s.flag, s.pos, sbits,
-                                                         s.k1, s.v1));
-        bool in_b;
-        DG_TRY(radix_sort(c, RadixBuffers{s.k1, s.k2, s.v1, s.v2}, nacc, 0, lb + sbits, s.radix, &in_b));
-        unsigned long long *key = in_b ? s.k2 : s.k1, *val = in_b ? s.v2 : s.v1;
-        const int ga = grid_for(nacc, kBlock, kStreamCap);
-        TK(c, "k_d_chain", k_d_chain<<<ga, kBlock, 0, st>>>(key, val, nacc, E, sbits, s.sv, s.lab,
-                                                           o.parent, s.contrib, s.head));
-        DG_TRY(segmented_inclusive_sum(c, s.contrib, s.head, s.csum, nacc, s.seg_tmp));
-        TK(c, "k_d_sizes", k_d_sizes<<<ga, kBlock, 0, st>>>(key, val, nacc, E, sbits, s.csum, o.size, s.svpar,
-                                                           s.sv));
-        TK(c, "k_d_keep", k_d_keep<<<g, kBlock, 0, st>>>(act, na, s.flag, s.pos, act2, ecu, ecv, ecu2, ecv2,
-                                                         s.svpar));
-        na -= nacc;
-        int32_t *t = act;
-        act = act2;
-        act2 = t;
-        t = ecu;
-        ecu = ecu2;
-        ecu2 = t;
-        t = ecv;
-        ecv = ecv2;
-        ecv2 = t;
-        o.rounds = round + 1;
+        {
+            const size_t smem = sort_smem_bytes<true>();
+            int grid = 1;
+            DG_TRY(coop_grid(c, kCoopDendro, (const void *)k_d_rounds, kSThreads, smem, &grid));
+            grid = w.na > kTailMax ? std::min(sort_ranges_of(w.na, grid), most) : 1;
+            void *args[] = {&d, &w};
+            cudaError_t e;
+            TK(c, "k_d_rounds", e = cudaLaunchCooperativeKernel((const void *)k_d_rounds, dim3((unsigned)grid),
+                                                                dim3(kSThreads), args, smem, st));
+            if (e != cudaSuccess) return set_err(c, DGEC_ERR_CUDA, "k_d_rounds launch: %s", cudaGetErrorString(e));
+        }
+        CU_TRY(c, cudaFuncSetAttribute(k_d_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmem));
+        TK(c, "k_d_tail", k_d_tail<<<1, kTailThreads, kTailSmem, st>>>(d));
     }
     if (n > 0)
-        TK(c, "k_d_split", k_d_split<<<grid_for(n, kBlock, kStreamCap), kBlock, 0, st>>>(s.lab, n, o.a, o.b));
+        TK(c, "k_d_split", k_d_split<<<grid_for(n, kBlock, kStreamCap), kBlock, 0, st>>>(s.row, n, o.a, o.b, o.size,
+                                                                                    o.parent + E));
+    if (n > 0) {
+        int64_t ts;
+        DG_TRY(read_counters(c, (const int64_t *)s.state, 1, &ts));
+        const int err = (int)(ts >> 32);
+        if (err == 1) return set_err(c, DGEC_ERR_TIMEOUT, "dendrogram rounds exceeded %d", 1 << 16);
+        if (err) return set_err(c, DGEC_ERR_INTERNAL, "dendrogram round accepted no edge");
+        o.rounds = (int)(ts & 0xffffffff);
+    }
     return DGEC_OK;
 }
 
