@@ -122,7 +122,7 @@ __global__ void k_c_top(int64_t n, int64_t off, Sel sel, int32_t *ptr, unsigned 
             const int rr = ptr[r];
             if (rr == r) break;
             r = rr;
-            ptr[x] = r;
+            atomicExch(ptr + x, r);  // not a store: other CTAs read these lines meanwhile
         }
         cut |= it == kTopWalk;
     }
@@ -553,7 +553,7 @@ __global__ void __launch_bounds__(256, 4) k_e_tree(Eom e) {
             while ((int)(v >> 32) >= 0 && it < kTopWalk) {
                 const unsigned long long u = *(volatile unsigned long long *)(e.slot + (v >> 32));
                 v = (u & 0xffffffff00000000ull) | ((int)(unsigned)u >= 0 ? (unsigned)u : (unsigned)v);
-                *(volatile unsigned long long *)(e.slot + c) = v;
+                atomicExch(e.slot + c, v);  // not a store: other CTAs read these lines meanwhile
                 it++;
             }
             if ((int)(v >> 32) >= 0) {

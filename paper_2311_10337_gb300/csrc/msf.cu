@@ -343,7 +343,7 @@ __global__ void k_m_jump(const int32_t *roots, int64_t nr, int32_t *par) {
             int rr = par[r];
             if (rr == r) break;
             r = rr;
-            par[x] = r;
+            atomicExch(par + x, r);  // not a store: other CTAs read these lines meanwhile
         }
     }
 }
@@ -556,7 +556,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_m_forest(MsfArgs a) {
                     const int rr = a.par[r];
                     if (rr == r) break;
                     r = rr;
-                    a.par[xs[q]] = r;
+                    atomicExch(a.par + xs[q], r);  // not a store: other CTAs read these lines meanwhile
                 }
             }
             long long at = cta_reserve_count(__popc(keep), a.cnt + 2 + (round & 1));
