@@ -145,7 +145,7 @@ struct DArgs {
 // edges, 34 with the large rounds apart); below, its barriers (about 2 us)
 // replace launches and a host read (3M edges: 2.18 ms with the line at 2^19, 2.22
 // at 2^20, 2.78 at 2^22).
-constexpr int kTailMax = 8192;
+constexpr int kTailMax = 4096;
 constexpr int64_t kDLarge = int64_t(1) << 19;
 // Groups of at most this many accepted edges skip the sort: each edge scans
 // its group (316,229 edges: 1.08 ms for the stage at 16, 0.92 at 32, 0.87 at 64
@@ -784,121 +784,158 @@ __global__ void __launch_bounds__(kSThreads, 2) k_d_rounds(const __grid_constant
 
 // ------------------------------------------------ one-CTA tail of the rounds
 // Once at most kTailMax forest edges are live, one CTA runs every remaining
-// round: the same steps as the kernels above (bids, pointers, jumps, tau,
-// acceptance, chains, sizes, keep), separated by barriers instead of
-// launches, the accepted edges sorted by (group, rank) in shared memory by a
-// bitonic network, and no count read on the host between rounds. The output
-// orders of acceptance and keep come from shared counters: the sort orders
-// the accepted edges, and the live list's order changes no result.
+// round in shared memory: the live edges, and for the super-vertices at their
+// ends -- renamed 0 .. 2 kTailMax - 1 through gcnt, which is zero between
+// rounds -- the slots, pointers, sizes and roots. Only the rows and parents go
+// out. The same steps as above; the accepted edges are sorted by (group, rank)
+// by a bitonic network, the live list's order changes no result. Bound by
+// the steps' CTA barriers and the network (with the arrays in global memory a
+// round took 41 us, nearly all of it L2 latency).
 constexpr int kTailThreads = 1024;
-constexpr size_t kTailSmem = (size_t)kTailMax * 16 + kTailMax;
+constexpr int kTailPer = kTailMax / kTailThreads;  // edges a thread holds
+constexpr int kTailLabels = 2 * kTailMax;
+constexpr size_t kTailSmem = (size_t)kTailLabels * (4 + 4 + 4 + 4 + 2) + (size_t)kTailMax * (4 + 2 + 2 + 1);
 
-__global__ void __launch_bounds__(kTailThreads) k_d_tail(
-    const __grid_constant__ DArgs a) {
-    extern __shared__ unsigned long long tsm[];
-    unsigned long long *skey = tsm, *sval = tsm + kTailMax;
-    unsigned char *sflag = (unsigned char *)(tsm + 2 * kTailMax);
-    __shared__ int s_nacc, s_nkeep;
+__global__ void __launch_bounds__(kTailThreads) k_d_tail(const __grid_constant__ DArgs a) {
+    extern __shared__ __align__(16) unsigned char tsm[];
+    unsigned *minr = (unsigned *)tsm;                         // [labels] smallest live rank; the sort's keys once the
+    unsigned long long *skey = (unsigned long long *)tsm;     //   pointers are known: (group << 32) | rank
+    unsigned *tau = minr + kTailLabels;                       // [labels]
+    unsigned short *sown = (unsigned short *)(tau);           // the sort's values, once tau is used: the pointers' owners
+    int *size = (int *)(tau + kTailLabels), *root = size + kTailLabels;  // [labels]
+    int *rank = root + kTailLabels;                           // [edges]
+    unsigned short *gp = (unsigned short *)(rank + kTailMax); // [labels] pointer, then its tree's root; kMerged: merged into it
+    unsigned short *lu = gp + kTailLabels, *lv = lu + kTailMax;  // [edges] labels
+    unsigned char *st = (unsigned char *)(lv + kTailMax);     // [edges] bit 0/1: it is the pointer of lu/lv
+    constexpr unsigned short kMerged = 0x8000;
+    static_assert(kTailLabels <= kMerged, "labels in 15 bits");
+    __shared__ int s_nlab, s_nacc, s_nkeep;
     __shared__ SegVal s_warp[kTailThreads / 32];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     if (a.state[1]) return;  // an error of the rounds before
-    const unsigned round0 = (unsigned)a.state[0];
     int na = a.state[2];
-    unsigned round = round0;
-    const int64_t E = a.E;
-    const int sbits = a.sbits;
-    const unsigned long long smask = (1ull << sbits) - 1ull;
-    unsigned long long *minr = a.minr, *tau = a.tau;
-    int32_t *gp = a.gp, *svpar = a.svpar;
-    SvRec *sv = a.sv;
-    DRow *row = a.row;
-    const bool odd = round0 & 1;
-    int32_t *act = odd ? a.act2 : a.act, *act2 = odd ? a.act : a.act2;
-    int32_t *ecu = odd ? a.ecu2 : a.ecu, *ecu2 = odd ? a.ecu : a.ecu2;
-    int32_t *ecv = odd ? a.ecv2 : a.ecv, *ecv2 = odd ? a.ecv : a.ecv2;
-    auto set_parent = [&](int c, int node) {
-        if (c < E) a.parent[c] = node;
-        else row[c - E].parent = node;
-    };
-    for (int j = tid; j < na; j += kTailThreads) {
-        if (round0 > 0) {  // the hop after the last round's merges
-            ecu[j] = svpar[ecu[j]];
-            ecv[j] = svpar[ecv[j]];
+    int round = a.state[0];
+    if (na == 0) return;
+    const int E = (int)a.E;
+    {  // in: edges, renamed labels, their sizes and roots
+        const bool odd = round & 1;
+        const int32_t *act = odd ? a.act2 : a.act, *ecu = odd ? a.ecu2 : a.ecu, *ecv = odd ? a.ecv2 : a.ecv;
+        if (tid == 0) s_nlab = 0;
+        __syncthreads();
+        int c[2 * kTailPer], id[2 * kTailPer];
+#pragma unroll
+        for (int q = 0; q < kTailPer; q++) {
+            const int j = tid + q * kTailThreads;
+            c[2 * q] = c[2 * q + 1] = -1;
+            if (j >= na) continue;
+            rank[j] = act[j];
+            c[2 * q] = ecu[j];
+            c[2 * q + 1] = ecv[j];
         }
-        row[act[j]].parent = -1;
+        if (round > 0) {  // the hop after the last round's merges
+#pragma unroll
+            for (int q = 0; q < 2 * kTailPer; q++)
+                if (c[q] >= 0) c[q] = a.svpar[c[q]];
+        }
+#pragma unroll
+        for (int q = 0; q < 2 * kTailPer; q++)  // one edge end names each label
+            id[q] = c[q] >= 0 && atomicExch(&a.gcnt[c[q]], 1) == 0 ? atomicAdd(&s_nlab, 1) : -1;
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 2 * kTailPer; q++) {
+            if (id[q] < 0) continue;
+            atomicExch(&a.gcnt[c[q]], id[q] + 2);
+            const SvRec r = a.sv[c[q]];
+            size[id[q]] = (int)r.size;
+            root[id[q]] = r.root;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kTailPer; q++) {
+            const int j = tid + q * kTailThreads;
+            if (j >= na) continue;
+            lu[j] = (unsigned short)(*(volatile int *)&a.gcnt[c[2 * q]] - 2);
+            lv[j] = (unsigned short)(*(volatile int *)&a.gcnt[c[2 * q + 1]] - 2);
+        }
     }
     __syncthreads();
+    const int nlab = s_nlab;
     while (na > 0) {
-        if (round >= (unsigned)a.max_rounds) {
+        if (round >= a.max_rounds) {
             if (tid == 0) a.state[1] = 1;
             return;
         }
-        const unsigned stamp = kStampTop - round;
-        // bids: every live edge offers its rank to both super-vertices
+        for (int c = tid; c < nlab; c += kTailThreads) minr[c] = tau[c] = ~0u;
+        if (tid == 0) s_nacc = s_nkeep = 0;
+        __syncthreads();
+        // every live edge offers its rank to both super-vertices
         for (int j = tid; j < na; j += kTailThreads) {
-            const unsigned long long key = rkey(stamp, act[j]);
-            const int cu = ecu[j], cv = ecv[j];
-            if (key < minr[cu]) atomicMin(&minr[cu], key);
-            if (key < minr[cv]) atomicMin(&minr[cv], key);
-        }
-        if (tid == 0) {
-            s_nacc = 0;
-            s_nkeep = 0;
+            const unsigned s = (unsigned)rank[j];
+            if (s < minr[lu[j]]) atomicMin(&minr[lu[j]], s);
+            if (s < minr[lv[j]]) atomicMin(&minr[lv[j]], s);
         }
         __syncthreads();
         // pointers (a mutual pair points both ends at its smaller label)
         for (int j = tid; j < na; j += kTailThreads) {
-            const int s = act[j], cu = ecu[j], cv = ecv[j];
-            const bool pu = rval(minr[cu], stamp) == s, pv = rval(minr[cv], stamp) == s;
+            const unsigned s = (unsigned)rank[j];
+            const unsigned short cu = lu[j], cv = lv[j];
+            const bool pu = minr[cu] == s, pv = minr[cv] == s;
             if (pu && pv) {
-                const int r = cu < cv ? cu : cv;
+                const unsigned short r = cu < cv ? cu : cv;
                 gp[cu] = r;
                 gp[cv] = r;
             } else {
                 if (pu) gp[cu] = cv;
                 if (pv) gp[cv] = cu;
             }
+            st[j] = (unsigned char)((pu ? 1 : 0) | (pv ? 2 : 0));
         }
         __syncthreads();
         // every pointer to its tree's root
         for (int j = tid; j < na; j += kTailThreads) {
-            const int s = act[j];
             for (int side = 0; side < 2; side++) {
-                const int c = side ? ecv[j] : ecu[j];
-                if (rval(minr[c], stamp) != s) continue;
+                if (!((st[j] >> side) & 1)) continue;
+                const int c = side ? lv[j] : lu[j];
                 int r = gp[c];
-                for (int it = 0; it < kMaxWalk; it++) {
-                    const int rr = *(volatile int32_t *)(gp + r);
+                for (int it = 0; it < kTailLabels; it++) {  // bounded: pointer trees
+                    const int rr = *(volatile unsigned short *)(gp + r);
                     if (rr == r) break;
                     r = rr;
-                    *(volatile int32_t *)(gp + c) = r;
+                    *(volatile unsigned short *)(gp + c) = (unsigned short)r;
                 }
             }
         }
         __syncthreads();
         // tau: the smallest non-pointer edge touching each tree
         for (int j = tid; j < na; j += kTailThreads) {
-            const int s = act[j], cu = ecu[j], cv = ecv[j];
-            if (rval(minr[cu], stamp) != s && rval(minr[cv], stamp) != s) {
-                const int gu = gp[cu], gv = gp[cv];
-                const unsigned long long key = rkey(stamp, s);
-                if (key < tau[gu]) atomicMin(&tau[gu], key);
-                if (key < tau[gv]) atomicMin(&tau[gv], key);
-            }
+            if (st[j]) continue;
+            const unsigned s = (unsigned)rank[j];
+            const int gu = gp[lu[j]], gv = gp[lv[j]];
+            if (s < tau[gu]) atomicMin(&tau[gu], s);
+            if (s < tau[gv]) atomicMin(&tau[gv], s);
         }
         __syncthreads();
-        // accept the pointer edges below their tree's tau; emit (group, rank)
-        for (int j = tid; j < na; j += kTailThreads) {
-            const int s = act[j], cu = ecu[j], cv = ecv[j];
-            const bool own_u = rval(minr[cu], stamp) == s, own_v = rval(minr[cv], stamp) == s;
+        // accept the pointer edges below their tree's tau (minr's place takes the
+        // keys); what is kept waits in registers
+        int ks[kTailPer], at[kTailPer];
+        unsigned kl[kTailPer];
+        unsigned short own[kTailPer];
+#pragma unroll
+        for (int q = 0; q < kTailPer; q++) {
+            const int j = tid + q * kTailThreads;
+            ks[q] = at[q] = -1;
+            if (j >= na) continue;
+            const int s = rank[j];
+            const unsigned short cu = lu[j], cv = lv[j];
             const int G = gp[cu];
-            const bool acc = (own_u || own_v) && s < rval(tau[G], stamp);
-            sflag[j] = acc;
-            if (acc) {
-                const int at = atomicAdd(&s_nacc, 1);
-                const unsigned Y = (unsigned)(own_u ? cu : cv), O = (unsigned)(own_u ? cv : cu);
-                skey[at] = ((unsigned long long)G << sbits) | (unsigned long long)s;
-                sval[at] = ((unsigned long long)Y << 32) | O;
+            if (st[j] && (unsigned)s < tau[G]) {
+                at[q] = atomicAdd(&s_nacc, 1);
+                own[q] = (st[j] & 1) ? cu : cv;
+                if (st[j] == 3 && own[q] == G) own[q] = cv;  // the pair's end that is not the root
+                skey[at[q]] = ((unsigned long long)(unsigned)G << 32) | (unsigned)s;
+            } else {
+                ks[q] = s;
+                kl[q] = (unsigned)cu | ((unsigned)cv << 16);
             }
         }
         __syncthreads();
@@ -910,67 +947,51 @@ __global__ void __launch_bounds__(kTailThreads) k_d_tail(
         int N = 1;
         while (N < nacc) N <<= 1;
         for (int i = nacc + tid; i < N; i += kTailThreads) skey[i] = ~0ull;  // padding sorts last
+#pragma unroll
+        for (int q = 0; q < kTailPer; q++)
+            if (at[q] >= 0) sown[at[q]] = own[q];
         __syncthreads();
-        for (int size = 2; size <= N; size <<= 1) {
-            for (int stride = size >> 1; stride > 0; stride >>= 1) {
+        for (int sz = 2; sz <= N; sz <<= 1) {
+            for (int stride = sz >> 1; stride > 0; stride >>= 1) {
                 for (int i = tid; i < (N >> 1); i += kTailThreads) {
-                    const int lo = 2 * stride * (i / stride) + (i % stride), hi = lo + stride;
-                    const bool up = (lo & size) == 0;
+                    const int lo = 2 * i - (i & (stride - 1)), hi = lo + stride;
+                    const bool up = (lo & sz) == 0;
                     const unsigned long long ka = skey[lo], kb = skey[hi];
                     if ((ka > kb) == up) {
                         skey[lo] = kb;
                         skey[hi] = ka;
-                        const unsigned long long t = sval[lo];
-                        sval[lo] = sval[hi];
-                        sval[hi] = t;
+                        const unsigned short t = sown[lo];
+                        sown[lo] = sown[hi];
+                        sown[hi] = t;
                     }
                 }
                 __syncthreads();
             }
         }
-        // chains: each thread a run of up to 8 consecutive sorted edges
-        const int C = (nacc + kTailThreads - 1) / kTailThreads;  // <= kTailMax / kTailThreads
+        // chains: each thread a run of consecutive sorted edges
+        const int C = (nacc + kTailThreads - 1) / kTailThreads;  // <= kTailPer
         const int x0 = tid * C;
-        long long add[kTailMax / kTailThreads];
-        int hd[kTailMax / kTailThreads];
+        int add[kTailPer], n1[kTailPer], n2[kTailPer];
+        bool hd[kTailPer];
+        SegVal agg{0, 0};
 #pragma unroll
-        for (int q = 0; q < kTailMax / kTailThreads; q++) {
+        for (int q = 0; q < kTailPer; q++) {
             const int x = x0 + q;
-            add[q] = 0;
-            hd[q] = 0;
             if (q >= C || x >= nacc) continue;
-            const unsigned long long k = skey[x], vv = sval[x];
-            const int s = (int)(k & smask), Y = (int)(vv >> 32), O = (int)(vv & 0xffffffffu);
-            const bool h = x == 0 || (skey[x - 1] >> sbits) != (k >> sbits);
-            const SvRec ry = sv[Y];
-            int c1, c2;
-            if (h) {
-                const SvRec ro = sv[O];
-                c1 = ry.root;
-                c2 = ro.root;
-                add[q] = ry.size + ro.size;
+            const unsigned long long k = skey[x];
+            const int G = (int)(k >> 32), Y = sown[x];
+            hd[q] = x == 0 || (int)(skey[x - 1] >> 32) != G;
+            n2[q] = root[Y];
+            add[q] = size[Y];
+            if (hd[q]) {  // the mutual pair: its other end is the tree's root
+                n1[q] = root[G];
+                add[q] += size[G];
             } else {
-                c1 = (int)(E + (int64_t)(skey[x - 1] & smask));
-                c2 = ry.root;
-                add[q] = ry.size;
+                n1[q] = E + (int)(unsigned)skey[x - 1];
             }
-            row[s].a = c1 < c2 ? c1 : c2;
-            row[s].b = c1 < c2 ? c2 : c1;
-            set_parent(c1, (int)(E + s));
-            set_parent(c2, (int)(E + s));
-            hd[q] = h;
+            agg = seg_add(agg, SegVal{add[q], hd[q] ? 1 : 0});
         }
         // sizes along each chain: a segmented inclusive sum over the runs
-        SegVal agg;
-        agg.v = 0;
-        agg.f = 0;
-#pragma unroll
-        for (int q = 0; q < kTailMax / kTailThreads; q++) {
-            SegVal it;
-            it.v = add[q];
-            it.f = hd[q];
-            agg = seg_add(agg, it);
-        }
         SegVal inc = agg;
         for (int d = 1; d < 32; d <<= 1) {
             SegVal o;
@@ -979,70 +1000,54 @@ __global__ void __launch_bounds__(kTailThreads) k_d_tail(
             if (lane >= d) inc = seg_add(o, inc);
         }
         if (lane == 31) s_warp[wid] = inc;
-        __syncthreads();  // also orders the chains' reads of sv before the writes below
-        if (wid == 0) {
-            SegVal w = s_warp[lane];
-            for (int d = 1; d < 32; d <<= 1) {
-                SegVal o;
-                o.v = ::__shfl_up_sync(0xffffffffu, w.v, d);
-                o.f = ::__shfl_up_sync(0xffffffffu, w.f, d);
-                if (lane >= d) w = seg_add(o, w);
-            }
-            s_warp[lane] = w;
-        }
-        __syncthreads();
-        SegVal run;
-        {
-            SegVal ex;
-            ex.v = ::__shfl_up_sync(0xffffffffu, inc.v, 1);
-            ex.f = ::__shfl_up_sync(0xffffffffu, inc.f, 1);
-            if (lane == 0) {
-                ex.v = 0;
-                ex.f = 0;
-            }
-            if (wid > 0) ex = lane == 0 ? s_warp[wid - 1] : seg_add(s_warp[wid - 1], ex);
-            run = ex;
-        }
+        SegVal ex;
+        ex.v = ::__shfl_up_sync(0xffffffffu, inc.v, 1);
+        ex.f = ::__shfl_up_sync(0xffffffffu, inc.f, 1);
+        if (lane == 0) ex = SegVal{0, 0};
+        __syncthreads();  // also orders the chains' reads of size and root before the writes below
+        SegVal run{0, 0};
+        for (int i = 0; i < wid; i++) run = seg_add(run, s_warp[i]);
+        run = seg_add(run, ex);
 #pragma unroll
-        for (int q = 0; q < kTailMax / kTailThreads; q++) {
+        for (int q = 0; q < kTailPer; q++) {
             const int x = x0 + q;
             if (q >= C || x >= nacc) continue;
-            SegVal it;
-            it.v = add[q];
-            it.f = hd[q];
-            run = seg_add(run, it);
-            const unsigned long long k = skey[x], vv = sval[x];
-            const unsigned long long G = k >> sbits;
-            const int s = (int)(k & smask);
-            row[s].size = run.v;
-            svpar[(int)(vv >> 32)] = (int32_t)G;
-            svpar[(int)(vv & 0xffffffffu)] = (int32_t)G;
-            if (x == nacc - 1 || (skey[x + 1] >> sbits) != G) sv[G] = SvRec{run.v, (int32_t)(E + s), 0};
+            run = seg_add(run, SegVal{add[q], hd[q] ? 1 : 0});
+            const unsigned long long k = skey[x];
+            const int G = (int)(k >> 32), s = (int)(unsigned)k, node = E + s;
+            const bool tail = x == nacc - 1 || (int)(skey[x + 1] >> 32) != G;
+            DRow *r = a.row + s;
+            *(int4 *)r = make_int4(min(n1[q], n2[q]), max(n1[q], n2[q]), tail ? -1 : E + (int)(unsigned)skey[x + 1], 0);
+            *(longlong2 *)((char *)r + 16) = make_longlong2(run.v, 0);
+            if (n2[q] < E) a.parent[n2[q]] = node;
+            else a.row[n2[q] - E].parent = node;
+            if (hd[q]) {
+                if (n1[q] < E) a.parent[n1[q]] = node;
+                else a.row[n1[q] - E].parent = node;
+            }
+            gp[sown[x]] |= kMerged;
+            if (tail) {
+                size[G] = (int)run.v;
+                root[G] = node;
+            }
         }
         __syncthreads();
         // the edges not accepted stay live, their labels moved one hop
-        for (int j = tid; j < na; j += kTailThreads) {
-            if (sflag[j]) continue;
-            const int at = atomicAdd(&s_nkeep, 1);
-            act2[at] = act[j];
-            ecu2[at] = svpar[ecu[j]];
-            ecv2[at] = svpar[ecv[j]];
+#pragma unroll
+        for (int q = 0; q < kTailPer; q++) {
+            if (ks[q] < 0) continue;
+            const int i = atomicAdd(&s_nkeep, 1);
+            const unsigned short cu = (unsigned short)kl[q], cv = (unsigned short)(kl[q] >> 16);
+            rank[i] = ks[q];
+            lu[i] = (gp[cu] & kMerged) ? gp[cu] & (kMerged - 1) : cu;
+            lv[i] = (gp[cv] & kMerged) ? gp[cv] & (kMerged - 1) : cv;
         }
         __syncthreads();
         na = s_nkeep;
-        int32_t *t = act;
-        act = act2;
-        act2 = t;
-        t = ecu;
-        ecu = ecu2;
-        ecu2 = t;
-        t = ecv;
-        ecv = ecv2;
-        ecv2 = t;
         round++;
         __syncthreads();
     }
-    if (tid == 0) a.state[0] = (int)round;
+    if (tid == 0) a.state[0] = round;
 }
 
 void plan_dendro(Arena &ws, const Problem &p, Dendro &o) {
