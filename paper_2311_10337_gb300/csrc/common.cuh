@@ -266,6 +266,38 @@ __device__ __forceinline__ long long cta_reserve_count(unsigned cnt, unsigned lo
     return slot;
 }
 
+// Two compactions with one atomicAdd per CTA: thread i asks for a_i and b_i
+// slots (below 2^16 a CTA each); the low and the high word of `counter` count
+// them, and the first slots of its runs come back the same way.
+__device__ __forceinline__ unsigned long long cta_reserve_pair(unsigned a, unsigned b, unsigned long long *counter) {
+    __shared__ unsigned s_warp[32];
+    __shared__ unsigned long long s_base;
+    const int w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+    const unsigned own = a | (b << 16);
+    unsigned inc = own;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const unsigned o = __shfl_up_sync(0xffffffffu, inc, d);
+        if ((int)lane_id() >= d) inc += o;
+    }
+    if (lane_id() == 31) s_warp[w] = inc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned tot = 0;
+        for (int i = 0; i < nw; i++) {
+            const unsigned c = s_warp[i];
+            s_warp[i] = tot;
+            tot += c;
+        }
+        s_base = tot ? atomicAdd(counter, (unsigned long long)(tot & 0xffffu) | ((unsigned long long)(tot >> 16) << 32)) : 0ull;
+    }
+    __syncthreads();
+    const unsigned pre = s_warp[w] + inc - own;
+    const unsigned long long slot = s_base + ((unsigned long long)(pre & 0xffffu) | ((unsigned long long)(pre >> 16) << 32));
+    __syncthreads();
+    return slot;
+}
+
 // 128-bit unsigned add into (hi, lo) words; exact and order independent.
 __device__ __forceinline__ void atomic_add_u128(unsigned long long *hi,
                                                 unsigned long long *lo,

@@ -402,11 +402,12 @@ struct MsfArgs {
     const int64_t *w;
     const int32_t *rank_of;
     int32_t *par, *roots, *roots2, *bp;
-    ulonglong2 *slot;       // best key bid at each root (all ones: none)
+    ulonglong2 *slot, *slot2;  // best key bid at each root (all ones: none), one for each round parity
     int2 *la, *lb;          // live edges: labels
     ulonglong2 *ka, *kb;    // live edges: keys without the label
     FEdge *fe;
-    unsigned long long *cnt;  // [0], [1] live edges, [2], [3] roots, [4] forest edges, [5] error; zeroed before
+    unsigned long long *cnt;  // [0], [1] live edges, [2], [3] (next roots << 32) | forest edges of the round,
+                              // [4] forest edges, [5] error; all but [4] zeroed before
     int ib, lbits;            // bits of an original id, of the label in a key (0: none)
     unsigned *bar, *err;
 };
@@ -429,20 +430,40 @@ __device__ __forceinline__ u128 cas_u128(ulonglong2 *p, u128 cmp, u128 val) {
         : "memory");
     return ((u128)hi << 64) | lo;
 }
-// Minimum into a slot. The read before skips bids that cannot win (most, at a
-// large component). It trusts the high word alone, which only falls: the two
-// words of the read need not belong together, so where the high words tie, a
-// swap of the value for itself reads it whole.
-__device__ __forceinline__ void bid_u128(ulonglong2 *slot, u128 key) {
-    const ulonglong2 seen = *slot;
-    if ((unsigned long long)(key >> 64) > seen.y) return;
-    u128 cur = as_u128(seen);
-    if (key >= cur) cur = cas_u128(slot, cur, cur);
-    while (key < cur) {
-        const u128 old = cas_u128(slot, cur, key);
-        if (old == cur) return;
-        cur = old;
+// Minima of two keys into two slots, their reads and their swaps in flight
+// together. The read before skips bids that cannot win (most, at a large
+// component). It trusts the high word alone, which only falls: the two words
+// of the read need not belong together, so where the high words tie, a swap
+// of the value for itself reads it whole.
+__device__ __forceinline__ void bid_u128(ulonglong2 *sa, u128 ka, ulonglong2 *sb, u128 kb) {
+    const ulonglong2 pa = *sa, pb = *sb;
+    bool ga = (unsigned long long)(ka >> 64) <= pa.y, gb = (unsigned long long)(kb >> 64) <= pb.y;
+    u128 ca = as_u128(pa), cb = as_u128(pb), oa = 0, ob = 0;
+    if (ga) oa = cas_u128(sa, ca, ka < ca ? ka : ca);
+    if (gb) ob = cas_u128(sb, cb, kb < cb ? kb : cb);
+    // a swap that took place wrote the smaller of the two; else go on from the value it met
+    if (ga && oa != ca)
+        for (ca = oa; ka < ca; ca = oa)
+            if ((oa = cas_u128(sa, ca, ka)) == ca) break;
+    if (gb && ob != cb)
+        for (cb = ob; kb < cb; cb = ob)
+            if ((ob = cas_u128(sb, cb, kb)) == cb) break;
+}
+
+// The root above label x after the hooks; x's own pointer is moved there when
+// the way was longer than one step (by an exchange, not a store: other CTAs
+// read these lines meanwhile).
+__device__ __forceinline__ int new_root(int32_t *par, int x) {
+    const int p = par[x];
+    int r = p;
+    for (int it = 0; it < kMaxWalk; it++) {  // bounded: pointers form a forest
+        const int rr = par[r];
+        if (rr == r) break;
+        r = rr;
+        if ((it & 7) == 7) atomicExch(par + x, r);
     }
+    if (r != p) atomicExch(par + x, r);
+    return r;
 }
 
 // Borůvka, all rounds in one cooperative kernel. A root's slot takes the
@@ -452,12 +473,12 @@ __device__ __forceinline__ void bid_u128(ulonglong2 *slot, u128 key) {
 // not fit -- w bits + 3 id bits > 127 -- the label is left out and a pass over
 // the live edges tells each root its winner's other end.) Per round:
 //   hook:   each root follows its best edge; a mutual pair keeps the smaller
-//           label as root; every forest edge is appended once;
-//   jump:   the old roots walk to their new root; those that stayed roots are
-//           the next round's, their slots cleared;
-//   filter: labels move one hop, edges inside one component are dropped, the
-//           rest is compacted and bids again.
-constexpr int kRes = 4;          // items a thread has in flight between slot reservations
+//           label as root, which is next round's list; every forest edge is
+//           appended once;
+//   filter: every live edge's labels walk to their new roots (leaving
+//           shortcuts), edges inside one component are dropped, the rest is
+//           compacted and bids again, in the slots the hooks have cleared.
+constexpr int kRes = 1;          // items a thread handles between slot reservations (20,000 edges: 0.15 ms at 1, 0.19 at 2, 0.34 at 4)
 __global__ void __launch_bounds__(kBlock, 4) k_m_forest(MsfArgs a) {
     GridBar bar(a.bar, a.err);
     const int64_t gsize = (int64_t)gridDim.x * blockDim.x, g0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -478,11 +499,11 @@ __global__ void __launch_bounds__(kBlock, 4) k_m_forest(MsfArgs a) {
     for (int64_t x = g0; x < a.n0; x += gsize) {
         const int cu = a.ru[x], cv = a.rv[x];
         const u128 key = pack(x);
-        bid_u128(a.slot + cu, key | (lb ? (unsigned)cv : 0u));
-        bid_u128(a.slot + cv, key | (lb ? (unsigned)cu : 0u));
+        bid_u128(a.slot + cu, key | (lb ? (unsigned)cv : 0u), a.slot + cv, key | (lb ? (unsigned)cu : 0u));
     }
     if (!bar.sync()) return;
-    int64_t n = a.n0, nr = a.nr0;
+    int64_t n = a.n0, nr = a.nr0, nfe = (int64_t)a.cnt[4];
+    ulonglong2 *slot = a.slot, *slot2 = a.slot2;
     const int32_t *roots = a.roots0;
     int32_t *rout = a.roots, *rnext = a.roots2;
     int2 *lin = a.la, *lout = a.lb;
@@ -496,15 +517,15 @@ __global__ void __launch_bounds__(kBlock, 4) k_m_forest(MsfArgs a) {
             for (int64_t x = g0; x < n; x += gsize) {
                 const int2 l = round ? lin[x] : make_int2(a.ru[x], a.rv[x]);
                 const u128 key = round ? as_u128(kin[x]) : pack(x);
-                if (as_u128(a.slot[l.x]) == key) a.bp[l.x] = l.y;
-                if (as_u128(a.slot[l.y]) == key) a.bp[l.y] = l.x;
+                if (as_u128(slot[l.x]) == key) a.bp[l.x] = l.y;
+                if (as_u128(slot[l.y]) == key) a.bp[l.y] = l.x;
             }
             if (!bar.sync()) return;
         }
         for (int64_t base = (int64_t)blockIdx.x * tile; base < nr; base += gsize * kRes) {  // CTA-uniform
             int xs[kRes], ps[kRes];
             u128 key[kRes];
-            unsigned emit = 0;
+            unsigned emit = 0, stay = 0;
 #pragma unroll
             for (int q = 0; q < kRes; q++) {
                 const int64_t ix = base + (int64_t)q * blockDim.x + threadIdx.x;
@@ -512,20 +533,26 @@ __global__ void __launch_bounds__(kBlock, 4) k_m_forest(MsfArgs a) {
             }
 #pragma unroll
             for (int q = 0; q < kRes; q++) {
-                key[q] = xs[q] >= 0 ? as_u128(a.slot[xs[q]]) : none;
+                key[q] = xs[q] >= 0 ? as_u128(slot[xs[q]]) : none;
                 ps[q] = -1;
                 if (key[q] != none) ps[q] = lb ? (int)((unsigned)key[q] & lmask) : a.bp[xs[q]];
             }
 #pragma unroll
             for (int q = 0; q < kRes; q++) {
                 if (ps[q] < 0) continue;  // no edge left: par[x] stays x
-                const bool mutual = (as_u128(a.slot[ps[q]]) >> lb) == (key[q] >> lb);
+                const bool mutual = (as_u128(slot[ps[q]]) >> lb) == (key[q] >> lb);
                 if (!mutual || xs[q] < ps[q]) emit |= 1u << q;
                 if (!mutual || xs[q] > ps[q]) a.par[xs[q]] = ps[q];
+                else stay |= 1u << q;
             }
-            long long at = cta_reserve_count(__popc(emit), a.cnt + 4);
+            const unsigned long long at2 = cta_reserve_pair(__popc(emit), __popc(stay), a.cnt + 2 + (round & 1));
+            int64_t at = nfe + (int64_t)(unsigned)at2, rat = (int64_t)(at2 >> 32);
 #pragma unroll
             for (int q = 0; q < kRes; q++) {
+                if ((stay >> q) & 1u) {
+                    slot2[xs[q]] = as_pair(none);
+                    rout[rat++] = xs[q];
+                }
                 if (!((emit >> q) & 1u)) continue;
                 const u128 k = key[q] >> lb;
                 FEdge f;
@@ -539,36 +566,11 @@ __global__ void __launch_bounds__(kBlock, 4) k_m_forest(MsfArgs a) {
         }
         if (lead) a.cnt[round & 1] = 0;  // the live count written in this round's filter
         if (!bar.sync()) return;
-        for (int64_t base = (int64_t)blockIdx.x * tile; base < nr; base += gsize * kRes) {  // CTA-uniform
-            int xs[kRes];
-            unsigned keep = 0;
-#pragma unroll
-            for (int q = 0; q < kRes; q++) {
-                const int64_t ix = base + (int64_t)q * blockDim.x + threadIdx.x;
-                xs[q] = ix < nr ? (roots ? roots[ix] : (int)ix) : -1;
-                if (xs[q] < 0) continue;
-                int r = a.par[xs[q]];
-                if (r == xs[q]) {
-                    if (as_u128(a.slot[r]) != none) keep |= 1u << q;
-                    continue;
-                }
-                for (int it = 0; it < kMaxWalk; it++) {  // bounded: pointers form a forest
-                    const int rr = a.par[r];
-                    if (rr == r) break;
-                    r = rr;
-                    atomicExch(a.par + xs[q], r);  // not a store: other CTAs read these lines meanwhile
-                }
-            }
-            long long at = cta_reserve_count(__popc(keep), a.cnt + 2 + (round & 1));
-#pragma unroll
-            for (int q = 0; q < kRes; q++) {
-                if (!((keep >> q) & 1u)) continue;
-                a.slot[xs[q]] = as_pair(none);
-                rout[at++] = xs[q];
-            }
+        {
+            const unsigned long long c = *(volatile unsigned long long *)(a.cnt + 2 + (round & 1));
+            nr = (int64_t)(c >> 32);
+            nfe += (int64_t)(unsigned)c;
         }
-        if (!bar.sync()) return;
-        nr = (int64_t) * (volatile unsigned long long *)(a.cnt + 2 + (round & 1));
         for (int64_t base = (int64_t)blockIdx.x * tile; base < n; base += gsize * kRes) {  // CTA-uniform
             int ca[kRes], cb[kRes];
             unsigned keep = 0;
@@ -578,8 +580,8 @@ __global__ void __launch_bounds__(kBlock, 4) k_m_forest(MsfArgs a) {
                 ca[q] = cb[q] = 0;
                 if (x < n) {
                     const int2 l = round ? lin[x] : make_int2(a.ru[x], a.rv[x]);
-                    ca[q] = a.par[l.x];
-                    cb[q] = a.par[l.y];
+                    ca[q] = new_root(a.par, l.x);
+                    cb[q] = new_root(a.par, l.y);
                     if (ca[q] != cb[q]) keep |= 1u << q;
                 }
             }
@@ -592,8 +594,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_m_forest(MsfArgs a) {
                 lout[at] = make_int2(ca[q], cb[q]);
                 kout[at] = as_pair(key);
                 at++;
-                bid_u128(a.slot + ca[q], key | (lb ? (unsigned)cb[q] : 0u));
-                bid_u128(a.slot + cb[q], key | (lb ? (unsigned)ca[q] : 0u));
+                bid_u128(slot2 + ca[q], key | (lb ? (unsigned)cb[q] : 0u), slot2 + cb[q], key | (lb ? (unsigned)ca[q] : 0u));
             }
         }
         if (lead) a.cnt[2 + ((round & 1) ^ 1)] = 0;
@@ -611,8 +612,12 @@ __global__ void __launch_bounds__(kBlock, 4) k_m_forest(MsfArgs a) {
             ulonglong2 *tk = kin;
             kin = kout;
             kout = tk;
+            tk = slot;
+            slot = slot2;
+            slot2 = tk;
         }
     }
+    if (lead) a.cnt[4] = (unsigned long long)nfe;
     bar.finish();
 }
 
@@ -705,11 +710,10 @@ void plan_msf(Arena &ws, const Problem &p, Msf &o) {
 
 // Live edges above which the host launches every step of a round by itself:
 // the 64-bit bids in three passes at full occupancy beat the one 128-bit pass
-// there (100M hub edges, 190M links: 25.4 against 28.6 ms for all rounds; 50M
-// edges 17.4 against 18.8), while below, the launches and the host's read of
-// every round cost more than they save (316,229 edges: 0.93 -> 0.61 ms for the
-// stage, 20,000: 0.60 -> 0.48, 3M: 2.4 -> 2.1; the line measured flat from 2^20 to
-// 2^24).
+// there (100M hub edges, 190M links: the stage takes 40.0 ms, 54.9 with every
+// round in the cooperative kernel; 10M edges 5.3 against 6.5), while below, the
+// launches and the host's read of every round cost more than they save (3M
+// edges 2.07 ms, 2.17 with the line at 2^24).
 constexpr int64_t kMLarge = int64_t(1) << 22;
 // One side of the live edges: 24 bytes each, as five columns in the large
 // rounds, as labels and keys in the cooperative kernel.
@@ -735,7 +739,7 @@ static LiveSide carve_side(Arena &a, int64_t S) {
 struct MsfScratch {
     int32_t *par, *roots, *roots2, *bp, *win;
     LiveSide side[2];
-    ulonglong2 *slot;
+    ulonglong2 *slot, *slot2;
     FEdge *fe;
     unsigned long long *cnt;
     unsigned long long *k1, *k2, *v1, *v2;
@@ -752,6 +756,7 @@ static MsfScratch carve_msf(Arena &a, const Problem &p) {
     s.side[0] = carve_side(a, S);
     s.side[1] = carve_side(a, S);
     s.slot = a.take<ulonglong2>(E);
+    s.slot2 = a.take<ulonglong2>(E);
     s.fe = a.take<FEdge>(E);
     s.cnt = a.take<unsigned long long>(8);
     s.k1 = a.take<unsigned long long>(E);
@@ -820,7 +825,7 @@ dgec_status stage_msf(Ctx *c, const Problem &p, const Csr &g, const Skel &sk, Ms
         // the kernel's first filter writes lb/kb: not the side its edges come from
         const LiveSide &in = s.side[which ^ 1], &out = s.side[which];
         MsfArgs f{nr, n, roots0, ccu, ccv, cu, cv, cw, g.rank_of, s.par, roots0 ? roots2 : roots, roots0 ? roots : roots2,
-                  s.bp, s.slot, in.lab, out.lab, in.key, out.key, s.fe, s.cnt, p.idbits,
+                  s.bp, s.slot, s.slot2, in.lab, out.lab, in.key, out.key, s.fe, s.cnt, p.idbits,
                   p.tbits + 3 * p.idbits <= 127 ? p.idbits : 0, c->bar, c->bar_err};
         int grid = 1;
         DG_TRY(coop_grid(c, kCoopMsf, (const void *)k_m_forest, kBlock, 0, &grid));
