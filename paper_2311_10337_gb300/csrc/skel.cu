@@ -149,6 +149,70 @@ __device__ __forceinline__ bool cand_less(const Cand &a, const Cand &b) {
     return a.w < b.w || (a.w == b.w && a.id < b.id);
 }
 
+// A packed candidate (w << 32 | id) of the forms for spans below 2^32.
+__device__ __forceinline__ long long cand_w(unsigned long long c) { return (long long)(c >> 32); }
+__device__ __forceinline__ unsigned cand_id(unsigned long long c) { return (unsigned)c; }
+__device__ __forceinline__ bool cand_none(unsigned long long c) { return c == 0xFFFFFFFFFFFFFFFFull; }
+__device__ __forceinline__ long long cand_w(const Cand &c) { return c.w; }
+__device__ __forceinline__ unsigned cand_id(const Cand &c) { return (unsigned)c.id; }
+__device__ __forceinline__ bool cand_none(const Cand &c) { return c.id == INT_MAX; }
+
+// The edge's row and core distance from its 2K sorted candidates: the first k
+// distinct ones within dmax. A node on both sides (a reciprocal concurrent
+// edge) stands twice in a row; there is one unless triples repeat, so the row
+// is the first candidates with one place left out, picked in registers and
+// written as 16-byte words: single 4-byte stores made 8 write requests of a
+// row's one sector at k = 8, and picking the places while storing kept 22 more
+// registers (k_knn_succ<8> at 100M hub edges 16.1 ms so, 6.3 ms with the words;
+// 50M edges 8.0 and 3.1).
+template <int K, class C>
+__device__ __forceinline__ void knn_write(const C (&c)[2 * K], int k, int64_t e0, long long dmax, int32_t *row,
+                                          int64_t *core) {
+    int dups = 0, d = 2 * K;
+#pragma unroll
+    for (int x = 2 * K - 1; x > 0; x--) {
+        if (!cand_none(c[x]) && cand_id(c[x]) == cand_id(c[x - 1])) {
+            dups++;
+            d = x;
+        }
+    }
+    if (dups <= 1) {
+        int32_t out[K];
+        long long last = LLONG_MAX;
+#pragma unroll
+        for (int x = 0; x < K; x++) {
+            const C &y = x >= d ? c[x + 1] : c[x];
+            const bool ok = !cand_none(y) && cand_w(y) <= dmax;
+            out[x] = ok ? (int32_t)((int64_t)cand_id(y) - e0) : -1;
+            if (x == k - 1 && ok) last = cand_w(y);
+        }
+        if (k == K && ((uintptr_t)row & 15) == 0) {
+#pragma unroll
+            for (int x = 0; x < K; x += 4)
+                *reinterpret_cast<int4 *>(row + x) = make_int4(out[x], out[x + 1], out[x + 2], out[x + 3]);
+        } else {
+#pragma unroll
+            for (int x = 0; x < K; x++)
+                if (x < k) row[x] = out[x];
+        }
+        *core = last;
+        return;
+    }
+    int cnt = 0;
+    long long last = LLONG_MAX;
+#pragma unroll
+    for (int x = 0; x < 2 * K; x++) {
+        const bool again = x > 0 && cand_id(c[x]) == cand_id(c[x - 1]);
+        if (!cand_none(c[x]) && !again && cnt < k && cand_w(c[x]) <= dmax) {
+            row[cnt] = (int32_t)((int64_t)cand_id(c[x]) - e0);
+            last = cand_w(c[x]);
+            cnt++;
+        }
+    }
+    for (int x = cnt; x < k; x++) row[x] = -1;
+    *core = cnt == k ? last : LLONG_MAX;
+}
+
 template <int K>
 __global__ void __launch_bounds__(256) k_knn(const int64_t *t, const int32_t *orig_of, int64_t E,
                                              const int64_t *out_t, const int32_t *out_id,
@@ -230,20 +294,7 @@ __global__ void __launch_bounds__(256) k_knn(const int64_t *t, const int32_t *or
                 }
             }
         }
-        int cnt = 0;
-        long long last_w = LLONG_MAX;
-        int prev = -1;
-#pragma unroll
-        for (int x = 0; x < N; x++) {
-            if (c[x].id != INT_MAX && c[x].id != prev && cnt < k && c[x].w <= dmax) {
-                row[cnt] = (int32_t)(c[x].id - e0);
-                last_w = c[x].w;
-                cnt++;
-            }
-            prev = c[x].id;
-        }
-        for (int x = cnt; x < k; x++) row[x] = -1;
-        core[e] = cnt == k ? last_w : LLONG_MAX;
+        knn_write<K>(c, k, e0, dmax, row, core + e);
     }
 }
 
@@ -328,22 +379,7 @@ __global__ void __launch_bounds__(256, K <= 8 ? 3 : 1) k_knn32(const int64_t *t,
                 }
             }
         }
-        int cnt = 0;
-        long long last_w = LLONG_MAX;
-        unsigned prev = 0xFFFFFFFFu;
-#pragma unroll
-        for (int x = 0; x < N; x++) {
-            const unsigned id = (unsigned)c[x];
-            const long long w = (long long)(c[x] >> 32);
-            if (c[x] != kNone && id != prev && cnt < k && w <= dmax) {
-                row[cnt] = (int32_t)((int64_t)id - e0);
-                last_w = w;
-                cnt++;
-            }
-            prev = id;
-        }
-        for (int x = cnt; x < k; x++) row[x] = -1;
-        core[e] = cnt == k ? last_w : LLONG_MAX;
+        knn_write<K>(c, k, e0, dmax, row, core + e);
     }
 }
 
@@ -460,22 +496,7 @@ __global__ void __launch_bounds__(256, K <= 8 ? 3 : 1) k_knn_succ(
                 }
             }
         }
-        int cnt = 0;
-        long long last_w = LLONG_MAX;
-        unsigned prev = 0xFFFFFFFFu;
-#pragma unroll
-        for (int u = 0; u < N; u++) {
-            const unsigned id = (unsigned)c[u];
-            const long long w = (long long)(c[u] >> 32);
-            if (c[u] != kNone && id != prev && cnt < k && w <= dmax) {
-                row[cnt] = (int32_t)((int64_t)id - e0);
-                last_w = w;
-                cnt++;
-            }
-            prev = id;
-        }
-        for (int u = cnt; u < k; u++) row[u] = -1;
-        core[e] = cnt == k ? last_w : LLONG_MAX;
+        knn_write<K>(c, k, e0, dmax, row, core + e);
     }
 }
 
