@@ -159,17 +159,26 @@ static dgec_status jump_to_fixed(Ctx *c, int64_t n, int64_t off, Sel sel, int32_
 __global__ void k_c_cpar(Gview gv, const int32_t *__restrict__ parent, const int32_t *__restrict__ up,
                          const int *__restrict__ isrep, const int64_t *__restrict__ size,
                          int32_t *__restrict__ cpar, unsigned long long *__restrict__ nbs) {
-    const int64_t E = gv.E;
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < E + gv.n;
-         x += (int64_t)gridDim.x * blockDim.x) {
-        if (x >= E && !isrep[x - E]) continue;
-        int P = parent[x];
-        int64_t cp = P < 0 ? gv.R0 + graph_of(gv, x) : E + up[P - E];
-        cpar[x] = (int32_t)cp;
-        if (x >= E) {
-            const int64_t sz = size[x - E];
-            if (sz >= gv.gM[graph_of(gv, x)]) atomicAdd(&nbs[cp - E], (1ull << 32) | (unsigned long long)sz);
+    const int64_t E = gv.E, total = E + gv.n;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t base = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; base < total;
+         base += stride) {  // warp-uniform
+        const int64_t x = base + lane_id();
+        bool big = false;
+        int64_t cp = E;
+        unsigned sz = 0;
+        if (x < total && (x < E || isrep[x - E])) {
+            const int P = parent[x];
+            cp = P < 0 ? gv.R0 + graph_of(gv, x) : E + up[P - E];
+            cpar[x] = (int32_t)cp;
+            if (x >= E) {
+                sz = (unsigned)size[x - E];
+                big = (int64_t)sz >= gv.gM[graph_of(gv, x)];
+            }
         }
+        // (merges of equal weight collapse: a parent can have very many big
+        // children; one atomic a child took 7.5 ms at 100M hub edges, 3.8 by key)
+        warp_add_count_size(big, (int)(cp - E), sz, nbs);
     }
 }
 
@@ -280,7 +289,7 @@ __global__ void k_c_nrec(Gview gv, const int *isrep, const int64_t *size, const 
             }
             if (write) rec[s] = r;
         }
-        warp_add_u96(0xffffffffu, has, K, val, st_hi, st_lo);
+        warp_add_u96(has, K, val, st_hi, st_lo);
     }
 }
 
@@ -298,20 +307,30 @@ __global__ void k_c_points(Gview gv, const int32_t *__restrict__ cpar, const Nod
     }
 }
 
-// A child cluster's points leave the parent P at P's death: P gains
-// (death - birth) * (total size of its child clusters). The sizes are summed
-// here per cluster index (plain adds, no returned value, so the many
-// components under a virtual root do not wait on one hot address), over the
-// compacted cluster list; the product is taken when the stabilities are
-// gathered.
-__global__ void k_c_child_size(int64_t ncl, Gview gv, const int32_t *__restrict__ clist,
-                               const int32_t *__restrict__ cparent, const int32_t *__restrict__ cidx,
-                               const int64_t *__restrict__ size, unsigned long long *csz) {
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < ncl;
-         c += (int64_t)gridDim.x * blockDim.x) {
-        const int K = clist[c];
-        if (K >= gv.R0) continue;
-        atomicAdd(&csz[cidx[cparent[K]]], (unsigned long long)size[K - gv.E]);
+// Every cluster's parent as a cluster index, and per parent the number of its
+// child clusters and their total size, (count << 32) + size: the child
+// clusters' points leave the parent P at P's death, so P gains (death - birth)
+// * (that size), a product taken when the stabilities are gathered.
+__global__ void k_c_kids(int64_t ncl, Gview gv, const int32_t *__restrict__ clist,
+                         const int32_t *__restrict__ cparent, const int32_t *__restrict__ cidx,
+                         const int64_t *__restrict__ size, int32_t *__restrict__ par, unsigned long long *kids) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t base = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; base < ncl;
+         base += stride) {  // warp-uniform
+        const int64_t c = base + lane_id();
+        int p = -1;
+        unsigned sz = 0;
+        bool add = false;
+        if (c < ncl) {
+            const int K = clist[c];
+            if (K < gv.R0) {
+                p = cidx[cparent[K]];
+                sz = (unsigned)size[K - gv.E];
+                add = true;
+            }
+            par[c] = p;
+        }
+        warp_add_count_size(add, p, sz, kids);
     }
 }
 
@@ -332,11 +351,11 @@ struct Eom {
     int64_t ncl;
     int64_t root0;  // clusters [root0, ncl) are the virtual roots (never selected, nothing reads their sums)
     int64_t R0;     // node ids >= R0 are virtual roots
-    const int32_t *clist, *cidx, *cparent;  // cparent by node id
-    int32_t *par;                            // compact parent, -1 root
+    const int32_t *clist, *cparent;  // cparent by node id
+    const int32_t *par;                      // compact parent, -1 root
     int *pending, *done, *fin;
     u128 *stab, *S, *Fa, *Fc, *Fa2, *Fc2;
-    const unsigned long long *csz;        // total size of the child clusters (0: none)
+    const unsigned long long *kids;       // (child clusters << 32) + their total size (0: none)
     unsigned long long *acc_hi, *acc_lo;  // sum of the children's S
     int32_t *ucand, *nxt, *nxt2, *al, *al2;
     unsigned long long *slot;  // (next ancestor << 32) | highest selected on the way there
@@ -349,16 +368,14 @@ __global__ void k_e_init(Eom e, const unsigned long long *st_hi, const unsigned 
                          const unsigned long long *cbirth, const unsigned long long *cdeath) {
     for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < e.ncl;
          c += (int64_t)gridDim.x * blockDim.x) {
-        int node = e.clist[c];
-        int pn = e.cparent[node];
-        e.par[c] = pn < 0 ? -1 : e.cidx[pn];
-        const unsigned long long kids = e.csz[c];
-        const u128 from_kids = kids ? (u128)(cdeath[node] - cbirth[node]) * kids : (u128)0;
+        const int node = e.clist[c];
+        const unsigned long long kids = e.kids[c];
+        const u128 from_kids = kids ? (u128)(cdeath[node] - cbirth[node]) * (kids & 0xffffffffull) : (u128)0;
         e.stab[c] = (((u128)st_hi[node] << 64) | st_lo[node]) + from_kids;
+        e.pending[c] = (int)(kids >> 32);
         e.done[c] = 0;
         e.acc_hi[c] = 0;
         e.acc_lo[c] = 0;
-        if (pn >= 0 && pn < e.R0) atomicAdd(&e.pending[e.par[c]], 1);
     }
 }
 
@@ -417,7 +434,7 @@ __global__ void __launch_bounds__(256, 4) k_e_tree(Eom e) {
     const int64_t gsize = (int64_t)gridDim.x * blockDim.x, g0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
     for (int64_t c = g0; c < e.root0; c += gsize)
-        if (e.csz[c] == 0) e_walk(e, (int)c);  // no child cluster
+        if (e.kids[c] == 0) e_walk(e, (int)c);  // no child cluster
     if (!bar.sync()) return;
     int32_t *al = e.al, *al2 = e.al2;
     int64_t nact = e.root0;
@@ -751,9 +768,10 @@ dgec_status stage_condense(Ctx *c, const Problem &p, const Msf &m, const Dendro 
     unsigned long long *nbs = reinterpret_cast<unsigned long long *>(s.cpos);
     CU_TRY(c, cudaMemsetAsync(nbs, 0, sizeof(unsigned long long) * (n + p.G), st));
     CU_TRY(c, cudaMemsetAsync(s.isc + E, 0, sizeof(int) * (n + p.G + 1), st));
-    CU_TRY(c, cudaMemsetAsync(s.cdeath, 0, sizeof(unsigned long long) * N, st));
-    CU_TRY(c, cudaMemsetAsync(s.st_hi, 0, sizeof(unsigned long long) * N, st));
-    CU_TRY(c, cudaMemsetAsync(s.st_lo, 0, sizeof(unsigned long long) * N, st));
+    // (a cluster is a merge or a virtual root, never a leaf)
+    CU_TRY(c, cudaMemsetAsync(s.cdeath + E, 0, sizeof(unsigned long long) * (n + p.G), st));
+    CU_TRY(c, cudaMemsetAsync(s.st_hi + E, 0, sizeof(unsigned long long) * (n + p.G), st));
+    CU_TRY(c, cudaMemsetAsync(s.st_lo + E, 0, sizeof(unsigned long long) * (n + p.G), st));
     if (n > 0) {
         TK(c, "k_c_up", k_c_up<<<gn, kBlock, 0, st>>>(E, n, d.parent, m.w, s.up, s.isrep));
         DG_TRY(jump_to_fixed(c, n, 0, SelAll{}, s.up, s.jflag));
@@ -775,15 +793,14 @@ dgec_status stage_condense(Ctx *c, const Problem &p, const Msf &m, const Dendro 
     TK(c, "k_c_compact", k_c_compact<<<gn, kBlock, 0, st>>>(E, n + p.G, s.isc + E, s.cpos, s.clist, s.cidx));
     o.n_cl = ncl;
     CU_TRY(c, cudaMemsetAsync(s.csz, 0, sizeof(unsigned long long) * (ncl + 1), st));
-    TK(c, "k_c_child_size", k_c_child_size<<<grid_for(ncl, kBlock, kStreamCap), kBlock, 0, st>>>(
-                                ncl, gv, s.clist, s.cparent, s.cidx, d.size, s.csz));
+    TK(c, "k_c_kids", k_c_kids<<<grid_for(ncl, kBlock, kStreamCap), kBlock, 0, st>>>(ncl, gv, s.clist, s.cparent, s.cidx,
+                                                                                d.size, s.par, s.csz));
     // ---- excess of mass over the cluster tree
     Eom e;
     e.ncl = ncl;
     e.root0 = ncl - p.G;  // every virtual root is a cluster, and their node ids are the last
     e.R0 = E + n;
     e.clist = s.clist;
-    e.cidx = s.cidx;
     e.cparent = s.cparent;
     e.par = s.par;
     e.pending = s.pending;
@@ -795,7 +812,7 @@ dgec_status stage_condense(Ctx *c, const Problem &p, const Msf &m, const Dendro 
     e.Fc = s.Fc;
     e.Fa2 = s.Fa2;
     e.Fc2 = s.Fc2;
-    e.csz = s.csz;
+    e.kids = s.csz;
     e.acc_hi = s.acc_hi;
     e.acc_lo = s.acc_lo;
     e.ucand = s.ucand;
@@ -809,7 +826,6 @@ dgec_status stage_condense(Ctx *c, const Problem &p, const Msf &m, const Dendro 
     e.bar = c->bar;
     e.err = c->bar_err;
     const int gc = grid_for(ncl + 1, kBlock, kStreamCap);
-    CU_TRY(c, cudaMemsetAsync(s.pending, 0, sizeof(int) * (ncl + 1), st));
     CU_TRY(c, cudaMemsetAsync(s.cnt, 0, 8 * sizeof(unsigned long long), st));
     TK(c, "k_e_init", k_e_init<<<gc, kBlock, 0, st>>>(e, s.st_hi, s.st_lo, s.cbirth, s.cdeath));
     {
