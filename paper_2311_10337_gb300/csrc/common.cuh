@@ -209,6 +209,16 @@ __device__ __forceinline__ int warp_agg_inc(int *counter, int key, unsigned acti
     return base + __popc(lt);
 }
 
+// One 32-byte sector (32-byte aligned) in one request: two 16-byte stores of
+// a scattered record are two half-written sectors to L2.
+__device__ __forceinline__ void store_sector(void *p, unsigned long long a, unsigned long long b, unsigned long long c,
+                                             unsigned long long d) {
+    asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(p), "l"(a), "l"(b), "l"(c), "l"(d) : "memory");
+}
+__device__ __forceinline__ unsigned long long pack_i32(int lo, int hi) {
+    return (unsigned long long)(unsigned)lo | ((unsigned long long)(unsigned)hi << 32);
+}
+
 // Stream compaction slot through ONE atomicAdd per CTA: threads with
 // `take` get consecutive slots of `counter` (order within the CTA follows
 // thread order). Every thread of the CTA must call it the same number of

@@ -552,8 +552,8 @@ __device__ __forceinline__ void d_small(const DArgs &a, const DRound &w, int64_t
         const int node = (int)(a.E + me.x);
         const int n1 = prev < 0 ? e.w : (int)(a.E + prev), n2 = e.z;
         DRow *r = a.row + me.x;
-        *(int4 *)r = make_int4(n1 < n2 ? n1 : n2, n1 < n2 ? n2 : n1, next == INT_MAX ? -1 : (int)(a.E + next), 0);
-        *(longlong2 *)((char *)r + 16) = make_longlong2(size, 0);
+        store_sector(r, pack_i32(n1 < n2 ? n1 : n2, n1 < n2 ? n2 : n1),
+                     pack_i32(next == INT_MAX ? -1 : (int)(a.E + next), 0), (unsigned long long)size, 0ull);
         if (n2 < a.E) a.parent[n2] = node;
         else a.row[n2 - a.E].parent = node;
         if (prev < 0) {
@@ -662,9 +662,8 @@ __device__ __forceinline__ void d_rows(const DArgs &a, const DRound &w, const un
             const bool tail = x == nacc - 1 || (k[q + 1] >> a.sbits) != (k[q] >> a.sbits);
             const int node = (int)(a.E + s), n1 = kid[q].x, n2 = kid[q].y;
             DRow *r = a.row + s;
-            *(int4 *)r = make_int4(n1 < n2 ? n1 : n2, n1 < n2 ? n2 : n1,
-                                   tail ? -1 : (int)(a.E + (int64_t)(k[q + 1] & smask)), 0);
-            *(longlong2 *)((char *)r + 16) = make_longlong2(pre.v, 0);
+            store_sector(r, pack_i32(n1 < n2 ? n1 : n2, n1 < n2 ? n2 : n1),
+                         pack_i32(tail ? -1 : (int)(a.E + (int64_t)(k[q + 1] & smask)), 0), (unsigned long long)pre.v, 0ull);
             // the children's parent (a chain's merge below knows already)
             if (n2 < a.E) a.parent[n2] = node;
             else a.row[n2 - a.E].parent = node;
@@ -1017,8 +1016,8 @@ __global__ void __launch_bounds__(kTailThreads) k_d_tail(const __grid_constant__
             const int G = (int)(k >> 32), s = (int)(unsigned)k, node = E + s;
             const bool tail = x == nacc - 1 || (int)(skey[x + 1] >> 32) != G;
             DRow *r = a.row + s;
-            *(int4 *)r = make_int4(min(n1[q], n2[q]), max(n1[q], n2[q]), tail ? -1 : E + (int)(unsigned)skey[x + 1], 0);
-            *(longlong2 *)((char *)r + 16) = make_longlong2(run.v, 0);
+            store_sector(r, pack_i32(min(n1[q], n2[q]), max(n1[q], n2[q])),
+                         pack_i32(tail ? -1 : E + (int)(unsigned)skey[x + 1], 0), (unsigned long long)run.v, 0ull);
             if (n2[q] < E) a.parent[n2[q]] = node;
             else a.row[n2[q] - E].parent = node;
             if (hd[q]) {

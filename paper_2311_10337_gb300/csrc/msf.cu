@@ -18,12 +18,15 @@ namespace dgec {
 constexpr unsigned long long kMax64 = 0xFFFFFFFFFFFFFFFFull;
 
 // A forest edge as the rounds append it: original ends (u < v), internal
-// ends, weight. One 24-byte record, so that the gathers by sorted index
-// after the rounds touch one sector per edge.
-struct FEdge {
+// ends, weight. One 32-byte record, so that it is written and gathered (by
+// sorted index, after the rounds) as one sector.
+struct __align__(32) FEdge {
     int32_t u, v, ru, rv;
-    int64_t w;
+    int64_t w, pad;
 };
+__device__ __forceinline__ void put_fedge(FEdge *p, int u, int v, int ru, int rv, int64_t w) {
+    store_sector(p, pack_i32(u, v), pack_i32(ru, rv), (unsigned long long)w, 0ull);
+}
 
 // Drop edges inside one component; compact the rest; bid w. In the first
 // round every node is its own component, so the label reads are skipped.
@@ -322,13 +325,7 @@ __global__ void k_m_hook(const int32_t *__restrict__ roots, int64_t nr, const un
         for (int q = 0; q < kRes8; q++) {
             if (!((emit >> q) & 1u)) continue;
             const int a = u[wx[q]], b = v[wx[q]];
-            FEdge f;
-            f.u = a;
-            f.v = b;
-            f.ru = rank_of[a];
-            f.rv = rank_of[b];
-            f.w = w[wx[q]];
-            fe[at++] = f;
+            put_fedge(fe + at++, a, b, rank_of[a], rank_of[b], w[wx[q]]);
         }
     }
 }
@@ -555,13 +552,8 @@ __global__ void __launch_bounds__(kBlock, 4) k_m_forest(MsfArgs a) {
                 }
                 if (!((emit >> q) & 1u)) continue;
                 const u128 k = key[q] >> lb;
-                FEdge f;
-                f.v = (int32_t)((unsigned)k & imask);
-                f.u = (int32_t)((unsigned)(k >> ib) & imask);
-                f.w = (int64_t)(unsigned long long)(k >> (2 * ib));
-                f.ru = a.rank_of[f.u];
-                f.rv = a.rank_of[f.v];
-                a.fe[at++] = f;
+                const int u = (int)((unsigned)(k >> ib) & imask), v = (int)((unsigned)k & imask);
+                put_fedge(a.fe + at++, u, v, a.rank_of[u], a.rank_of[v], (int64_t)(unsigned long long)(k >> (2 * ib)));
             }
         }
         if (lead) a.cnt[round & 1] = 0;  // the live count written in this round's filter
@@ -693,7 +685,18 @@ __global__ void k_gather_msf(const unsigned long long *idx, unsigned long long i
                              int32_t *u, int32_t *v, int32_t *ru, int32_t *rv, int64_t *w) {
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n;
          x += (int64_t)gridDim.x * blockDim.x) {
-        const FEdge f = fe[idx[x] & imask];
+        FEdge f;
+        {
+            unsigned long long q0, q1, q2, q3;
+            asm volatile("ld.global.v4.b64 {%0, %1, %2, %3}, [%4];"
+                         : "=l"(q0), "=l"(q1), "=l"(q2), "=l"(q3)
+                         : "l"(fe + (idx[x] & imask)));
+            f.u = (int32_t)q0;
+            f.v = (int32_t)(q0 >> 32);
+            f.ru = (int32_t)q1;
+            f.rv = (int32_t)(q1 >> 32);
+            f.w = (int64_t)q2;
+        }
         u[x] = f.u;
         v[x] = f.v;
         ru[x] = f.ru;

@@ -186,7 +186,12 @@ __device__ __forceinline__ void knn_write(const C (&c)[2 * K], int k, int64_t e0
             out[x] = ok ? (int32_t)((int64_t)cand_id(y) - e0) : -1;
             if (x == k - 1 && ok) last = cand_w(y);
         }
-        if (k == K && ((uintptr_t)row & 15) == 0) {
+        if (K >= 8 && k == K && ((uintptr_t)row & 31) == 0) {
+#pragma unroll
+            for (int x = 0; x + 8 <= K; x += 8)
+                store_sector(row + x, pack_i32(out[x], out[x + 1]), pack_i32(out[x + 2], out[x + 3]),
+                             pack_i32(out[x + 4], out[x + 5]), pack_i32(out[x + 6], out[x + 7]));
+        } else if (k == K && ((uintptr_t)row & 15) == 0) {
 #pragma unroll
             for (int x = 0; x < K; x += 4)
                 *reinterpret_cast<int4 *>(row + x) = make_int4(out[x], out[x + 1], out[x + 2], out[x + 3]);
@@ -437,7 +442,7 @@ __global__ void __launch_bounds__(256) k_knn_pred(int64_t E, const unsigned long
         }
         ulonglong2 *dstp = half + (int64_t)y * (K / 2);
 #pragma unroll
-        for (int u = 0; u < K / 2; u++) dstp[u] = make_ulonglong2(c[2 * u], c[2 * u + 1]);
+        for (int u = 0; u < K; u += 4) store_sector(dstp + u / 2, c[u], c[u + 1], c[u + 2], c[u + 3]);
     }
 }
 
