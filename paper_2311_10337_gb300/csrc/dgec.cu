@@ -156,10 +156,29 @@ __global__ void k_localize(int64_t n, int64_t E, const int32_t *mu, const int32_
     }
 }
 
-// Per-graph tables, staged through host arrays, one copy each.
+// One graph's tables, from the launch's own arguments.
+__global__ void k_one_table(int64_t E, int64_t V, int32_t k, int32_t M, int64_t *eoff, int64_t *voff,
+                            int64_t *knn_off, int32_t *gk, int32_t *gM) {
+    eoff[0] = voff[0] = knn_off[0] = 0;
+    eoff[1] = E;
+    voff[1] = V;
+    knn_off[1] = E * k;
+    gk[0] = k;
+    gM[0] = M;
+}
+
+// Per-graph tables, staged through host arrays, one copy each. A single
+// graph's come as kernel arguments: five copies from pageable memory and the
+// wait before the staging is freed cost 24 us of a 0.8 ms call more than the launch.
 dgec_status upload_tables(Ctx *c, const HostBatch &hb, int64_t *eoff, int64_t *voff, int64_t *knn_off,
                           int32_t *gk, int32_t *gM) {
     int G = hb.G;
+    if (G == 1) {
+        TK(c, "k_one_table", k_one_table<<<1, 1, 0, c->stream>>>(hb.eoff[1], hb.nv[0], hb.k[0], hb.M[0], eoff, voff,
+                                                                 knn_off, gk, gM));
+        CU_TRY(c, cudaGetLastError());
+        return DGEC_OK;
+    }
     int64_t *hv = (int64_t *)malloc(sizeof(int64_t) * (3 * (size_t)(G + 1)));
     if (!hv) return set_err(c, DGEC_ERR_OOM, "host memory");
     int64_t *hvoff = hv, *hknn = hv + (G + 1), *heoff = hv + 2 * (G + 1);

@@ -643,16 +643,24 @@ class Server:
             pass
 
 
+def _typed(ws):
+    """The workspace's bytes as int32 and as int64, to slice the result arrays
+    from (each starts on a 256-byte boundary): one tensor operation an array."""
+    import torch
+    b = ws.narrow(0, 0, ws.numel() // 8 * 8)
+    return {torch.int32: b.view(torch.int32), torch.int64: b.view(torch.int64)}
+
+
 class Output:
     """Device-resident results of one run, as torch views of the workspace."""
 
-    _SPEC = {  # name -> (dtype, length expression)
-        "out_off": ("int64", "V+1"), "in_off": ("int64", "V+1"),
+    _SPEC = {  # name -> (dtype, length: a key of the sizes made from the result)
+        "out_off": ("int64", "V1"), "in_off": ("int64", "V1"),
         "out_t": ("int64", "E"), "in_t": ("int64", "E"),
         "out_id": ("int32", "E"), "in_id": ("int32", "E"),
         "pos_out": ("int32", "E"), "pos_in": ("int32", "E"),
         "sk_u": ("int32", "nsk"), "sk_v": ("int32", "nsk"), "sk_w": ("int64", "nsk"),
-        "knn_id": ("int32", "E*k"), "core": ("int64", "E"),
+        "knn_id": ("int32", "Ek"), "core": ("int64", "E"),
         "mst_u": ("int32", "nmst"), "mst_v": ("int32", "nmst"), "mst_w": ("int64", "nmst"),
         "link_a": ("int32", "nmst"), "link_b": ("int32", "nmst"), "link_size": ("int64", "nmst"),
         "fall_cluster": ("int32", "E"), "fall_lambda": ("uint64", "E"),
@@ -669,19 +677,20 @@ class Output:
         self.n_mst = int(res.n_mst)
         self.n_condensed = int(res.n_condensed)
         self.n_clusters = int(res.n_clusters)
-        env = dict(E=E, V=V, k=k, nsk=self.n_skeleton, nmst=self.n_mst, ncl=self.n_condensed)
+        env = {"E": E, "V1": int(V) + 1, "Ek": E * int(k), "nsk": self.n_skeleton, "nmst": self.n_mst,
+               "ncl": self.n_condensed}
         base = ws.data_ptr()
         dts = {"int32": (torch.int32, 4), "int64": (torch.int64, 8), "uint64": (torch.int64, 8)}
+        typed = _typed(ws)
         self._raw = {}
-        for name, (dt, expr) in self._SPEC.items():
+        for name, (dt, length) in self._SPEC.items():
             ptr = getattr(res, name)
-            n = int(eval(expr, {}, env))
+            n = env[length]
             tdt, sz = dts[dt]
             if n == 0 or ptr is None:
                 self._raw[name] = (torch.empty(0, dtype=tdt, device=ws.device), dt)
                 continue
-            off = ptr - base
-            self._raw[name] = (ws[off:off + n * sz].view(tdt), dt)
+            self._raw[name] = (typed[tdt].narrow(0, (ptr - base) // sz, n), dt)
         self.E, self.V, self.k = E, V, k
 
     def tensor(self, name):
