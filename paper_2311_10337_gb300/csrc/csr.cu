@@ -48,43 +48,22 @@ __global__ void k_egraph(const int64_t *eoff, int G, int64_t E, int32_t *egraph)
     }
 }
 
-// Validates ids against each edge's own graph and counts degrees under
-// global vertex ids (local id + the graph's vertex offset).
+// Validates ids against each edge's own graph; smallest and largest time.
 __global__ void k_count(const int32_t *src, const int32_t *dst, const int64_t *t, int64_t E,
-                        const int32_t *egraph, const int64_t *voff, int *deg_out, int *deg_in,
-                        long long *flags) {
+                        const int32_t *egraph, const int64_t *voff, long long *flags) {
     __shared__ long long smin[kBlock / 32], smax[kBlock / 32];
     long long tmin = LLONG_MAX, tmax = LLONG_MIN;
     int bad = 0, loops = 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    // warp-aligned grid-stride loop so warp_agg_inc sees whole warps
-    const int64_t warp_global = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = stride >> 5;
-    for (int64_t wb = warp_global * 32; wb < E; wb += nwarps * 32) {
-        int64_t e = wb + lane_id();
-        bool ok = e < E;
-        int s = ok ? src[e] : 0, d = ok ? dst[e] : 0;
-        int64_t vo = 0, nv = 0;
-        if (ok) {
-            int g = egraph[e];
-            vo = voff[g];
-            nv = voff[g + 1] - vo;
-        }
-        bool vs = ok && s >= 0 && s < nv && d >= 0 && d < nv;
-        if (ok && !vs) bad++;
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < E; e += stride) {
+        const int s = src[e], d = dst[e], g = egraph[e];
+        const int64_t nv = voff[g + 1] - voff[g];
+        const bool vs = s >= 0 && s < nv && d >= 0 && d < nv;
+        if (!vs) bad++;
         if (vs && s == d) loops++;
-        if (ok) {
-            long long x = t[e];
-            tmin = x < tmin ? x : tmin;
-            tmax = x > tmax ? x : tmax;
-        }
-        if (deg_out) {  // degrees only when the caller wants them
-            unsigned act = __ballot_sync(0xffffffffu, vs);
-            if (vs) {
-                warp_agg_inc(deg_out, (int)(s + vo), act);
-                warp_agg_inc(deg_in, (int)(d + vo), act);
-            }
-        }
+        const long long x = t[e];
+        tmin = x < tmin ? x : tmin;
+        tmax = x > tmax ? x : tmax;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -572,7 +551,7 @@ dgec_status stage_csr(Ctx *c, Problem &p, Csr &o, void *scratch) {
         if (p.G == 1) CU_TRY(c, cudaMemsetAsync(p.egraph, 0, sizeof(int32_t) * E, st));
         else TK(c, "k_egraph", k_egraph<<<grid_for(E, kBlock, kStreamCap), kBlock, 0, st>>>(p.eoff, p.G, E, p.egraph));
         TK(c, "k_count", k_count<<<grid_for(E, kBlock, (int64_t)c->num_sms * 16), kBlock, 0, st>>>(
-                             p.src, p.dst, p.t, E, p.egraph, p.voff, nullptr, nullptr, s.flags));
+                             p.src, p.dst, p.t, E, p.egraph, p.voff, s.flags));
     }
     int64_t f[4];
     DG_TRY(read_counters(c, (const int64_t *)s.flags, 4, f));

@@ -1073,6 +1073,15 @@ struct DScratch {
     unsigned long long *k1, *k2, *v1, *v2;
     void *radix;
 };
+// CTAs of the middle rounds: one for each 512 live edges, so that a thread
+// has no chain of bids and loads one after another, but at most one an SM (a
+// second CTA on some SMs makes every phase wait for those). 20,000 edges: 0.24
+// ms at one CTA per 4,096 edges, 0.154 so; 317,000: 0.49, 0.51 with 192 CTAs, 0.45 with 152.
+constexpr int kMidEdges = 512, kMidCtas = 152;
+// CTAs the per-CTA counts have room for.
+static int chunk_ctas(int64_t E) {
+    return std::max(sort_ranges_of(E, kSRanges), (int)std::min<int64_t>(cdiv(E, kMidEdges), kMidCtas));
+}
 static DScratch carve_dendro(Arena &a, const Problem &p) {
     DScratch s;
     int64_t E = p.E;
@@ -1098,7 +1107,7 @@ static DScratch carve_dendro(Arena &a, const Problem &p) {
     s.segC = a.take<int2>(E);
     s.kids = a.take<int2>(E);
     s.contrib = a.take<long long>(E);
-    const int64_t ctas = sort_ranges_of(E, kSRanges);
+    const int64_t ctas = chunk_ctas(E);
     s.ccnt = a.take<unsigned>(ctas);
     s.cagg = a.take<SegVal>(ctas);
     s.k1 = a.take<unsigned long long>(E);
@@ -1143,7 +1152,7 @@ dgec_status stage_dendro(Ctx *c, const Problem &p, const Csr &g, const Msf &m, D
         DRound w{0, 0, kStampTop, n, 0, 0, false};
         CU_TRY(c, cudaMemsetAsync(s.state, 0, sizeof(int) * 12, st));
         CU_TRY(c, cudaMemsetAsync(s.gcnt, 0, sizeof(int) * E, st));
-        const int most = (int)sort_ranges_of(E, kSRanges);  // CTAs the per-CTA counts have room for
+        const int most = chunk_ctas(E);
         for (; w.na > kDLarge; w.round++) {
             if (w.round >= d.max_rounds)
                 return set_err(c, DGEC_ERR_TIMEOUT, "dendrogram rounds exceeded %d", d.max_rounds);
@@ -1189,7 +1198,7 @@ dgec_status stage_dendro(Ctx *c, const Problem &p, const Csr &g, const Msf &m, D
             const size_t smem = sort_smem_bytes<true>();
             int grid = 1;
             DG_TRY(coop_grid(c, kCoopDendro, (const void *)k_d_rounds, kSThreads, smem, &grid));
-            grid = w.na > kTailMax ? std::min(sort_ranges_of(w.na, grid), most) : 1;
+            grid = w.na > kTailMax ? (int)std::min<int64_t>(std::min(grid, kMidCtas), cdiv(w.na, kMidEdges)) : 1;
             void *args[] = {&d, &w};
             cudaError_t e;
             TK(c, "k_d_rounds", e = cudaLaunchCooperativeKernel((const void *)k_d_rounds, dim3((unsigned)grid),

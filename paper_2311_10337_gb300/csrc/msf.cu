@@ -773,14 +773,16 @@ static MsfScratch carve_msf(Arena &a, const Problem &p) {
     s.win = a.take<int32_t>(E);
     s.side[0] = carve_side(a, S);
     s.side[1] = carve_side(a, S);
-    s.slot = a.take<ulonglong2>(E);
-    s.slot2 = a.take<ulonglong2>(E);
+    const int64_t Er = (E + 31) / 32 * 32;
+    s.slot = a.take<ulonglong2>(Er);
+    s.slot2 = a.take<ulonglong2>(Er);
     s.fe = a.take<FEdge>(E);
     s.cnt = a.take<unsigned long long>(8);
-    s.k1 = a.take<unsigned long long>(E);
-    s.k2 = a.take<unsigned long long>(E);
-    s.v1 = a.take<unsigned long long>(E);
-    s.v2 = a.take<unsigned long long>(E);
+    // the sorts after the rounds, when no bid is read any more
+    s.k1 = (unsigned long long *)s.slot;
+    s.k2 = s.k1 + Er;
+    s.v1 = (unsigned long long *)s.slot2;
+    s.v2 = s.v1 + Er;
     s.radix = a.take<char>(radix_scratch_bytes(E));
     return s;
 }
