@@ -864,7 +864,7 @@ dgec_status stage_condense(Ctx *c, const Problem &p, const Msf &m, const Dendro 
     {
         int grid = 1;
         DG_TRY(coop_grid(c, kCoopEom, (const void *)k_e_tree, kBlock, 0, &grid));
-        const int64_t want = cdiv(ncl, 2 * kBlock);
+        const int64_t want = cdiv(ncl, kBlock);  // (two clusters a thread: 0.070 ms instead of 0.058 at 20,000 edges)
         DG_TRY(coop_launch(c, "k_e_tree", (const void *)k_e_tree, want < grid ? (int)want : grid, kBlock, 0, e));
     }
     TK(c, "k_e_labels", k_e_labels<<<gE, kBlock, 0, st>>>(E, o.fall_cluster, s.cidx, s.H, o.labels, s.minmem));

@@ -114,7 +114,7 @@ __device__ __forceinline__ int64_t warp_edge_of(const int64_t *off, int64_t E, i
 // vertex's segment as key r = rank_of[e]; the slot remembers the vertex.
 // The warp finds its first member's e together, then each lane searches the
 // few offsets up to the last member's. Bound by the scattered writes and the
-// places' atomics (10M members of 5M hyperedges: 0.55 ms; a search of all
+// places' atomics (5M directed hyperedges: 0.55 ms; a search of all
 // offsets in every lane: 0.63).
 __global__ void k_h_scatter(const int64_t *off, int64_t E, const int32_t *vert, int64_t M,
                             const int32_t *rank_of, const int64_t *voff, int *cur,

@@ -6,8 +6,9 @@
 // bids its key into both, each component hooks along its winning edge, a
 // mutual pair keeps the smaller label as root, labels are pointer-jumped to
 // their roots, and edges inside one component are dropped while the survivors
-// are compacted for the next round. The pipeline's form is k_m_forest; the
-// kernels before it serve dgec_msf_static.
+// are compacted for the next round. The pipeline's forms are the k_m_*
+// rounds while many edges live and k_m_forest after that; the kernels before
+// them serve dgec_msf_static.
 #include <utility>
 
 #include "coop.cuh"

@@ -15,30 +15,6 @@ dgec_status exclusive_scan_i64(Ctx *c, const long long *in, long long *out, int6
         c, LoadPtr<long long>{in}, StorePtr<long long>{out}, n, SumI64{}, 0ll, false, scratch);
 }
 
-struct LoadSeg {
-    const long long *v;
-    const int *h;
-    __device__ __forceinline__ SegVal operator()(int64_t i) const {
-        SegVal s;
-        s.v = v[i];
-        s.f = h[i];
-        return s;
-    }
-};
-struct StoreSeg {
-    long long *o;
-    __device__ __forceinline__ void operator()(int64_t i, SegVal s) const { o[i] = s.v; }
-};
-
-dgec_status segmented_inclusive_sum(Ctx *c, const long long *v, const int *head, long long *out,
-                                    int64_t n, SegVal *scratch) {
-    SegVal id;
-    id.v = 0;
-    id.f = 0;
-    return device_scan<SegVal, SegSumOp, LoadSeg, StoreSeg>(c, LoadSeg{v, head}, StoreSeg{out}, n,
-                                                            SegSumOp{}, id, true, scratch);
-}
-
 // ------------------------------------------------------------ radix sort
 // What bounds it: up to some 100,000 keys the launch and the two barriers of a
 // pass; in L2's reach the latency of a tile's chain (load, ballots, counter

@@ -50,23 +50,6 @@ struct SegVal {
     long long v;
     int f;
 };
-struct SegSumOp {
-    __device__ __forceinline__ SegVal operator()(SegVal a, SegVal b) const {
-        SegVal r;
-        r.v = b.f ? b.v : a.v + b.v;
-        r.f = a.f | b.f;
-        return r;
-    }
-};
-
-// SegVal shuffles word by word (found by argument-dependent lookup from
-// the scan templates above).
-__device__ __forceinline__ SegVal __shfl_up_sync(unsigned m, SegVal x, unsigned d) {
-    SegVal r;
-    r.v = ::__shfl_up_sync(m, x.v, d);
-    r.f = ::__shfl_up_sync(m, x.f, d);
-    return r;
-}
 
 // ----------------------------------------------------- device-wide scans
 // Three passes: per-tile aggregates, scan of aggregates (recursive), tile
@@ -165,9 +148,6 @@ dgec_status device_scan(Ctx *c, Load ld, Store st, int64_t n, Op op, T identity,
 dgec_status exclusive_scan_i32(Ctx *c, const int *in, long long *out, int64_t n, long long *scratch);
 dgec_status exclusive_scan_i64(Ctx *c, const long long *in, long long *out, int64_t n,
                                long long *scratch);
-// Inclusive segmented sum: out[i] = sum of v over [segment start .. i].
-dgec_status segmented_inclusive_sum(Ctx *c, const long long *v, const int *head, long long *out,
-                                    int64_t n, SegVal *scratch);
 
 // ------------------------------------------------------------ radix sort
 // Stable LSD radix sort on key bits [begin_bit, end_bit), 8 bits a pass.

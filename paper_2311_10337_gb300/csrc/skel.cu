@@ -161,7 +161,7 @@ __device__ __forceinline__ bool cand_none(const Cand &c) { return c.id == INT_MA
 // distinct ones within dmax. A node on both sides (a reciprocal concurrent
 // edge) stands twice in a row; there is one unless triples repeat, so the row
 // is the first candidates with one place left out, picked in registers and
-// written as 16-byte words: single 4-byte stores made 8 write requests of a
+// written as 32- or 16-byte words: single 4-byte stores made 8 write requests of a
 // row's one sector at k = 8, and picking the places while storing kept 22 more
 // registers (k_knn_succ<8> at 100M hub edges 16.1 ms so, 6.3 ms with the words;
 // 50M edges 8.0 and 3.1).
