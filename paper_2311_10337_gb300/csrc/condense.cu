@@ -84,8 +84,13 @@ struct SelBigRep {  // big kept merges (the nodes whose cluster link is set)
 // One pass of start-compressing walks, in descending index order: parents
 // have larger ids than their children, so ancestors tend to be resolved
 // first and later walks stop after a few steps. A walk that exceeds
-// kTopWalk steps stores the ancestor it reached and flags *moved.
-constexpr int kTopWalk = 1 << 12;
+// kTopWalk steps stores the ancestor it reached and flags *moved. The limit
+// bounds what a long run of equal weights costs, whose first walkers meet
+// only pointers as short as their own: 60M edges at one threshold take 188 ms
+// with walks of up to 4,096 steps, 39 with 512 and the rounds (1.7) behind
+// them; times of 60M edges in whole days 114 and 34. With 256 those take 23 and
+// 21 ms, but 100M hub edges then need the rounds (0.5 ms), with 512 they do not.
+constexpr int kTopWalk = 512;
 template <class Sel>
 __global__ void k_c_top(int64_t n, int64_t off, Sel sel, int32_t *ptr, unsigned long long *moved) {
     bool cut = false;
