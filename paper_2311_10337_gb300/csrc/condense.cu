@@ -112,42 +112,23 @@ __global__ void k_c_top(int64_t n, int64_t off, Sel sel, int32_t *ptr, unsigned 
     if (__syncthreads_or(cut) && threadIdx.x == 0) atomicOr(moved, 1ull);
 }
 
-// In-place pointer jumping over the pointers `Sel` picks, ptr[x] =
-// ptr[ptr[x]], in rounds until none moves: nothing to do unless *moved says
-// that a walk was cut short. Pointers only move to ancestors and fixed
-// points are never written, so reading a neighbour's new or old value is
-// equally valid, and every distance to the fixed point at least halves per
-// round. moved[1 .. 3] are the rounds' flags in turn, zero at the start.
-constexpr int kJumpRounds = 64;  // halvings of any distance below 2^31, twice over
+// The pointers `Sel` picks, as jump_rounds takes them.
+template <class Sel>
+struct SelItem {
+    int64_t off;
+    Sel sel;
+    __device__ __forceinline__ int64_t operator()(int64_t s) const { return sel(s) ? off + s : -1; }
+};
+// The jumping rounds: nothing to do unless *moved says that a walk was cut
+// short. moved[1 .. 3] are their flags, zero at the start.
 template <class Sel>
 __global__ void __launch_bounds__(kBlock) k_c_jump(int64_t n, int64_t off, Sel sel, int32_t *ptr,
                                                    unsigned long long *moved, unsigned *barw, unsigned *err) {
     if (moved[0] == 0) return;  // the same for every CTA: written before this launch
     GridBar bar(barw, err);
-    bool more = true;
-    for (int it = 0; more; it++) {
-        unsigned long long *f = moved + 1 + it % 3;
-        if (it == kJumpRounds) {
-            if (threadIdx.x == 0) *(volatile unsigned *)err = 1u;
-            break;
-        }
-        if (blockIdx.x == 0 && threadIdx.x == 0) moved[1 + (it + 1) % 3] = 0;  // last read before the barrier behind us
-        bool any = false;
-        for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n;
-             s += (int64_t)gridDim.x * blockDim.x) {
-            if (!sel(s)) continue;
-            const int64_t x = off + s;
-            const int p = *(volatile int32_t *)(ptr + x);
-            const int pp = *(volatile int32_t *)(ptr + p);
-            if (pp != p) {
-                *(volatile int32_t *)(ptr + x) = pp;
-                any = true;
-            }
-        }
-        if (__syncthreads_or(any) && threadIdx.x == 0) atomicOr(f, 1ull);
-        if (!bar.sync()) return;
-        more = *(volatile unsigned long long *)f != 0;
-    }
+    const JumpEnd e = jump_rounds(bar, n, SelItem<Sel>{off, sel}, ptr, moved + 1);
+    if (e == kJumpBarrier) return;
+    if (e == kJumpBound && threadIdx.x == 0) *(volatile unsigned *)err = 1u;
     bar.finish();
 }
 

@@ -61,4 +61,39 @@ struct GridBar {
     }
 };
 
+// In-place pointer jumping, ptr[x] = ptr[ptr[x]], over the n pointers x =
+// item(i) (negative: none), in rounds until none moves. Pointers only move to
+// ancestors and fixed points are never written, so reading a neighbour's new
+// or old value is equally valid, and every distance to the fixed point at
+// least halves per round. flag[0 .. 2] are the rounds' flags in turn; flag[0]
+// is zero at the start and at the end.
+constexpr int kJumpRounds = 64;  // halvings of any distance below 2^31, twice over
+enum JumpEnd { kJumpDone, kJumpBarrier, kJumpBound };
+template <class Item>
+__device__ __forceinline__ JumpEnd jump_rounds(GridBar &bar, int64_t n, const Item &item, int32_t *ptr,
+                                               unsigned long long *flag) {
+    for (int it = 0; it < kJumpRounds; it++) {
+        unsigned long long *f = flag + it % 3;
+        if (blockIdx.x == 0 && threadIdx.x == 0) flag[(it + 1) % 3] = 0;  // last read before the barrier behind us
+        bool any = false;
+        for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+            const int64_t x = item(i);
+            if (x < 0) continue;
+            const int p = *(volatile int32_t *)(ptr + x);
+            const int pp = *(volatile int32_t *)(ptr + p);
+            if (pp != p) {
+                *(volatile int32_t *)(ptr + x) = pp;
+                any = true;
+            }
+        }
+        if (__syncthreads_or(any) && threadIdx.x == 0) atomicOr(f, 1ull);
+        if (!bar.sync()) return kJumpBarrier;
+        if (*(volatile unsigned long long *)f == 0) {
+            if (blockIdx.x == 0 && threadIdx.x == 0) flag[0] = 0;  // (already zero where others still read it)
+            return kJumpDone;
+        }
+    }
+    return kJumpBound;
+}
+
 }  // namespace dgec

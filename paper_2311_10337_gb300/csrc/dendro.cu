@@ -124,7 +124,8 @@ struct DArgs {
     int2 *segA;      // (rank, leaves the edge adds)
     int4 *segB;      // (pointer's owner, group, owner's root, the mutual pair's other root or -1)
     int2 *segC;      // its group's (first place, edges)
-    unsigned long long *tot;  // [0], [1] places of small groups taken (by round parity), [2], [3] edges of large groups
+    unsigned long long *tot;  // [0], [1] places of small groups taken (by round parity), [2], [3] edges of large groups,
+                              // [4] a walk of d_jump was cut, [5 .. 7] flags of the jumping rounds
     // accepted edges of large groups, sorted by (group, rank)
     int2 *kids;          // the nodes the edge merges
     long long *contrib;  // (leaves it adds << 1) | first of its chain
@@ -264,10 +265,20 @@ __device__ __forceinline__ void d_ptr(const DArgs &a, const DRound &w) {
         }
     }
 }
+// Every pointer to its tree's root, by walks that shorten their own pointer as
+// they go. Walks are cut after kDWalk steps, and jump_rounds finishes the rest:
+// on a long chain the threads running meet only pointers as short as their
+// own, and the last of them walks all of it. A path whose gaps fall, with all
+// walks whole / cut at 512 / 256 / 128 / 64 steps: 400,000 edges 167 / 1.3 / 0.82
+// / 0.56 / 0.42 ms in the middle rounds, 3M edges 4.4 s / 6.2 / 2.5 / 1.4 / 0.6
+// ms in this step. At 128 no walk of 100M hub edges is cut, at 64 they pay 2.8 ms
+// for the rounds; asking whether any was cut costs them 0.07 ms in 12 launches
+// and the walks 3.56 ms instead of 3.40.
+constexpr int kDWalk = 128;
 __device__ __forceinline__ void d_jump(const DArgs &a, const DRound &w) {
     D_LIST;
     D_STRIDE;
-    // every pointer to its tree's root
+    bool cut = false;
     for (int64_t j = g0; j < na; j += gsize) {
         const int st = a.st[j];
         if (!st) continue;
@@ -276,14 +287,30 @@ __device__ __forceinline__ void d_jump(const DArgs &a, const DRound &w) {
             if (!((st >> side) & 1)) continue;
             const int c = side ? ecv[j] : ecu[j];
             int r = a.gp[c];
-            for (int it = 0; it < kMaxWalk; it++) {  // bounded: pointer trees
+            int it = 0;
+            for (; it < kDWalk; it++) {
                 const int rr = *(volatile int32_t *)(a.gp + r);
                 if (rr == r) break;
                 r = rr;
                 atomicExch(a.gp + c, r);  // (not a store: see d_alloc)
             }
+            cut |= it == kDWalk;
         }
     }
+    if (__syncthreads_or(cut) && threadIdx.x == 0) atomicOr(a.tot + 4, 1ull);
+}
+// The pointers of the live edges' ends, as jump_rounds takes them.
+struct DItem {
+    const unsigned char *st;
+    const int32_t *ecu, *ecv;
+    __device__ __forceinline__ int64_t operator()(int64_t i) const {
+        const int64_t j = i >> 1;
+        if (!((st[j] >> (i & 1)) & 1)) return -1;
+        return (i & 1) ? ecv[j] : ecu[j];
+    }
+};
+__device__ __forceinline__ JumpEnd d_settle(const DArgs &a, const DRound &w, GridBar &bar) {
+    return jump_rounds(bar, 2 * w.na, DItem{a.st, w.odd ? a.ecu2 : a.ecu, w.odd ? a.ecv2 : a.ecv}, a.gp, a.tot + 5);
 }
 __device__ __forceinline__ void d_tau(const DArgs &a, const DRound &w) {
     D_LIST;
@@ -700,11 +727,22 @@ __global__ void __launch_bounds__(kSThreads, 2) k_d_rows(const __grid_constant__
     d_rows(a, w, key, val);
 }
 
+// What d_jump left of a large round's walks: nothing unless one was cut.
+__global__ void __launch_bounds__(kSThreads, 2) k_d_settle(const __grid_constant__ DArgs a, const __grid_constant__ DRound w) {
+    if (a.tot[4] == 0) return;  // the same for every CTA: written before this launch
+    GridBar bar(a.bar, a.err);
+    const JumpEnd e = d_settle(a, w, bar);
+    if (e == kJumpBarrier) return;
+    if (e == kJumpBound && threadIdx.x == 0) *(volatile unsigned *)a.err = 1u;
+    bar.finish();
+}
+
 // The same steps inside the cooperative kernel, as calls so that each keeps
 // its own registers.
 __device__ __noinline__ void dc_bid(const DArgs &a, const DRound &w) { d_bid(a, w); }
 __device__ __noinline__ void dc_ptr(const DArgs &a, const DRound &w) { d_ptr(a, w); }
 __device__ __noinline__ void dc_jump(const DArgs &a, const DRound &w) { d_jump(a, w); }
+__device__ __noinline__ JumpEnd dc_settle(const DArgs &a, const DRound &w, GridBar &bar) { return d_settle(a, w, bar); }
 __device__ __noinline__ void dc_tau(const DArgs &a, const DRound &w) { d_tau(a, w); }
 __device__ __noinline__ void dc_accept(const DArgs &a, const DRound &w) { d_accept(a, w); }
 __device__ __noinline__ void dc_alloc(const DArgs &a, const DRound &w) { d_alloc(a, w); }
@@ -742,8 +780,17 @@ __global__ void __launch_bounds__(kSThreads, 2) k_d_rounds(const __grid_constant
         if (!bar.sync()) return;
         dc_jump(a, w);
         if (!bar.sync()) return;
+        if (*(volatile unsigned long long *)(a.tot + 4)) {
+            const JumpEnd e = dc_settle(a, w, bar);
+            if (e == kJumpBarrier) return;
+            if (e == kJumpBound) {
+                error = 3;
+                break;
+            }
+        }
         dc_tau(a, w);
         if (!bar.sync()) return;
+        if (blockIdx.x == 0 && threadIdx.x == 0) a.tot[4] = 0;  // every CTA has read it
         dc_accept(a, w);
         if (!bar.sync()) return;
         dc_alloc(a, w);
@@ -1087,7 +1134,7 @@ static DScratch carve_dendro(Arena &a, const Problem &p) {
     int64_t E = p.E;
     s.svpar = a.take<int32_t>(E);
     s.sv = a.take<SvRec>(E);
-    s.state = a.take<int>(12);  // state[4], then tot[4] as 64-bit words
+    s.state = a.take<int>(20);  // state[4], then tot[8] as 64-bit words
     s.row = a.take<DRow>(E);
     s.minr = a.take<unsigned long long>(E);
     s.tau = a.take<unsigned long long>(E);
@@ -1150,7 +1197,7 @@ dgec_status stage_dendro(Ctx *c, const Problem &p, const Csr &g, const Msf &m, D
                 sort_args(c, RadixBuffers{s.k1, s.k2, s.v1, s.v2}, n, 0, lb + sbits, s.radix, E), s.ccnt, s.cagg,
                 s.state, 1 << 16, c->bar, c->bar_err};
         DRound w{0, 0, kStampTop, n, 0, 0, false};
-        CU_TRY(c, cudaMemsetAsync(s.state, 0, sizeof(int) * 12, st));
+        CU_TRY(c, cudaMemsetAsync(s.state, 0, sizeof(int) * 20, st));
         CU_TRY(c, cudaMemsetAsync(s.gcnt, 0, sizeof(int) * E, st));
         const int most = chunk_ctas(E);
         for (; w.na > kDLarge; w.round++) {
@@ -1166,6 +1213,15 @@ dgec_status stage_dendro(Ctx *c, const Problem &p, const Csr &g, const Msf &m, D
             TK(c, "k_d_ptr", k_d_ptr<<<w.G, kSThreads, 0, st>>>(d, w));
             w.G = wide;
             TK(c, "k_d_gjump", k_d_jump<<<wide, kSThreads, 0, st>>>(d, w));
+            DG_TRY(coop_grid(c, kCoopDJump, (const void *)k_d_settle, kSThreads, 0, &w.G));
+            {
+                void *args[] = {&d, &w};
+                cudaError_t e;
+                TK(c, "k_d_settle", e = cudaLaunchCooperativeKernel((const void *)k_d_settle, dim3((unsigned)w.G),
+                                                                    dim3(kSThreads), args, 0, st));
+                if (e != cudaSuccess) return set_err(c, DGEC_ERR_CUDA, "k_d_settle launch: %s", cudaGetErrorString(e));
+            }
+            w.G = wide;
             TK(c, "k_d_tau", k_d_tau<<<wide, kSThreads, 0, st>>>(d, w));
             w.G = few;
             TK(c, "k_d_accept", k_d_accept<<<few, kSThreads, 0, st>>>(d, w));
@@ -1179,7 +1235,7 @@ dgec_status stage_dendro(Ctx *c, const Problem &p, const Csr &g, const Msf &m, D
             if (kept == w.na) return set_err(c, DGEC_ERR_INTERNAL, "dendrogram round accepted no edge");
             w.nsmall = h[2 + (w.round & 1)];
             w.nacc = h[4 + (w.round & 1)];
-            CU_TRY(c, cudaMemsetAsync(d.tot, 0, 4 * sizeof(unsigned long long), st));
+            CU_TRY(c, cudaMemsetAsync(d.tot, 0, 8 * sizeof(unsigned long long), st));
             if (w.nsmall > 0) {
                 w.G = (int)std::min<int64_t>(cdiv(w.nsmall, kSThreads), c->stream_ctas);
                 TK(c, "k_d_small", k_d_small<<<w.G, kSThreads, 0, st>>>(d, w));
@@ -1216,6 +1272,7 @@ dgec_status stage_dendro(Ctx *c, const Problem &p, const Csr &g, const Msf &m, D
         DG_TRY(read_counters(c, (const int64_t *)s.state, 1, &ts));
         const int err = (int)(ts >> 32);
         if (err == 1) return set_err(c, DGEC_ERR_TIMEOUT, "dendrogram rounds exceeded %d", 1 << 16);
+        if (err == 3) return set_err(c, DGEC_ERR_TIMEOUT, "dendrogram pointers not settled in %d rounds", kJumpRounds);
         if (err) return set_err(c, DGEC_ERR_INTERNAL, "dendrogram round accepted no edge");
         o.rounds = (int)(ts & 0xffffffff);
     }

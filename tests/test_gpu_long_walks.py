@@ -2,9 +2,10 @@
 pointers as short as their own must not take time by the length of the chain.
 Each test compares a stage with another of the same call or of a call on as
 many edges without long chains, on the device's own clock."""
+import numpy as np
 import pytest
 
-from gpu_helpers import ctx
+from gpu_helpers import compare_all, ctx
 
 pytestmark = pytest.mark.gpu
 
@@ -35,3 +36,34 @@ def test_one_run_of_equal_weights():
     s = _stages(lambda: ctx().run_levels(src, dst, t, V, [1 << 20], 5))
     ctx().ws = None  # tens of GB: not kept for the tests after
     assert s["D2 condense and labels"] < 5 * s["A incidence lists"]
+
+
+def _path(n, rising):
+    """A relay of n + 1 edges whose gaps rise or fall, so that in the first
+    round every edge points to its neighbour on one side: one chain. Edge ids
+    in random order."""
+    gaps = 2 + np.arange(n, dtype=np.int64)
+    t = np.concatenate([[0], np.cumsum(gaps if rising else gaps[::-1])])
+    p = np.random.default_rng(n).permutation(n + 1)
+    a = np.arange(n + 1, dtype=np.int32)
+    return a[p], a[p] + 1, t[p], n + 2
+
+
+def _path_stages(n, rising):
+    import torch
+    src, dst, t, V = _path(n, rising)
+    e = [torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in (src, dst, t)]
+    return _stages(lambda: ctx().run(*e, V, 2, 2))
+
+
+@pytest.mark.parametrize("n", [400_000, 2_000_000])  # middle rounds; a large round
+def test_dendrogram_of_a_path(n):
+    fall, rise = _path_stages(n, False), _path_stages(n, True)
+    assert fall["D1 dendrogram"] < 8 * rise["D1 dendrogram"]
+
+
+@pytest.mark.parametrize("n", [100_000, 600_000])
+def test_paths_equal_the_oracle(n):
+    src, dst, t, V = _path(n, False)
+    q = np.arange(0, n, n // 100).astype(np.int32)
+    compare_all(src, dst, t, V, 2, 2, knn_query=q)
