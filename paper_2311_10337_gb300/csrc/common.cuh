@@ -44,7 +44,7 @@ struct StageTimer {
 };
 
 // Cooperative kernels whose resident-CTA count a context remembers.
-enum CoopKernel { kCoopSortK, kCoopSortKV, kCoopEom, kCoopMsf, kCoopDendro, kCoopDJump, kCoopJumpAll, kCoopJumpBig, kCoopCount };
+enum CoopKernel { kCoopSortK, kCoopSortKV, kCoopEom, kCoopMsf, kCoopMJump, kCoopMLabels, kCoopDendro, kCoopDJump, kCoopJumpAll, kCoopJumpBig, kCoopCount };
 
 struct Ctx {
     int device = 0;

@@ -9,6 +9,7 @@
 // are compacted for the next round. The pipeline's forms are the k_m_*
 // rounds while many edges live and k_m_forest after that; the kernels before
 // them serve dgec_msf_static.
+#include <algorithm>
 #include <utility>
 
 #include "coop.cuh"
@@ -343,19 +344,45 @@ __global__ void k_m_hook(const int32_t *__restrict__ roots, int64_t nr, const un
     }
 }
 
-// Roots walk to their new root (own pointer compressed on the way).
-__global__ void k_m_jump(const int32_t *roots, int64_t nr, int32_t *par) {
+// Roots walk to their new root (own pointer compressed on the way). Walks are
+// cut after kMWalk steps and left to k_m_settle: on a long chain the threads
+// running meet only pointers as short as their own, and the last of them walks
+// all of it. A path of 3M edges whose gaps fall took 1.3 s in k_m_forest; with
+// walks cut at 256 / 128 / 64 steps it and k_m_labels take 1.2 / 0.93 / 0.77 ms.
+// At 256 steps hardly a walk of 100M hub edges is cut (k_m_settle 0.04 to 0.15 ms
+// in 7 rounds, 0.25 at 64).
+constexpr int kMWalk = 256;
+__global__ void k_m_jump(const int32_t *roots, int64_t nr, int32_t *par, unsigned long long *cut) {
+    bool any = false;
     for (int64_t ix = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; ix < nr;
          ix += (int64_t)gridDim.x * blockDim.x) {
         int x = roots[ix];
         int r = par[x];
-        for (int it = 0; it < kMaxWalk; it++) {
+        int it = 0;
+        for (; it < kMWalk; it++) {
             int rr = par[r];
             if (rr == r) break;
             r = rr;
             atomicExch(par + x, r);  // not a store: other CTAs read these lines meanwhile
         }
+        any |= it == kMWalk;
     }
+    if (__syncthreads_or(any) && threadIdx.x == 0) atomicOr(cut, 1ull);
+}
+struct RootItem {
+    const int32_t *roots;
+    __device__ __forceinline__ int64_t operator()(int64_t i) const { return roots[i]; }
+};
+// Jumping rounds for the walks that were cut (cut[1 .. 3]: their flags): nothing
+// to do unless one was.
+__global__ void __launch_bounds__(kBlock) k_m_settle(const int32_t *roots, int64_t nr, int32_t *par, unsigned long long *cut,
+                                                     unsigned *barw, unsigned *err) {
+    if (cut[0] == 0) return;  // the same for every CTA: written before this launch
+    GridBar bar(barw, err);
+    const JumpEnd e = jump_rounds(bar, nr, RootItem{roots}, par, cut + 1);
+    if (e == kJumpBarrier) return;
+    if (e == kJumpBound && threadIdx.x == 0) *(volatile unsigned *)err = 1u;
+    bar.finish();
 }
 
 // Next round's roots (old roots that stayed roots); every old root's bid
@@ -417,7 +444,8 @@ struct MsfArgs {
     ulonglong2 *ka, *kb;    // live edges: keys without the label
     FEdge *fe;
     unsigned long long *cnt;  // [0], [1] live edges, [2], [3] (next roots << 32) | forest edges of the round,
-                              // [4] forest edges, [5] error; all but [4] zeroed before
+                              // [4] forest edges, [5] error, [6] a walk was cut; if so [7] rounds begun, [8] the
+                              // last one's live edges, [9] next roots; all but [4] zeroed before
     int ib, lbits;            // bits of an original id, of the label in a key (0: none)
     unsigned *bar, *err;
 };
@@ -462,15 +490,20 @@ __device__ __forceinline__ void bid_u128(ulonglong2 *sa, u128 ka, ulonglong2 *sb
 
 // The root above label x after the hooks; x's own pointer is moved there when
 // the way was longer than one step (by an exchange, not a store: other CTAs
-// read these lines meanwhile).
-__device__ __forceinline__ int new_root(int32_t *par, int x) {
+// read these lines meanwhile). A walk is cut after kMWalk steps, which *cut
+// then says; what is returned is an ancestor short of the root.
+__device__ __forceinline__ int new_root(int32_t *par, int x, unsigned long long *cut) {
     const int p = par[x];
     int r = p;
-    for (int it = 0; it < kMaxWalk; it++) {  // bounded: pointers form a forest
+    for (int it = 0;; it++) {
         const int rr = par[r];
         if (rr == r) break;
         r = rr;
         if ((it & 7) == 7) atomicExch(par + x, r);
+        if (it == kMWalk) {
+            *(volatile unsigned long long *)cut = 1;
+            break;
+        }
     }
     if (r != p) atomicExch(par + x, r);
     return r;
@@ -488,6 +521,10 @@ __device__ __forceinline__ int new_root(int32_t *par, int x) {
 //   filter: every live edge's labels walk to their new roots (leaving
 //           shortcuts), edges inside one component are dropped, the rest is
 //           compacted and bids again, in the slots the hooks have cleared.
+// If a walk of the filter was cut, the kernel stops there, k_m_labels settles
+// the pointers by jumping rounds and does the filter, and the rounds start
+// again from its edges (the jumping rounds as a call in here: 0.82 instead of
+// 0.65 ms for the last rounds of 20M edges, for the registers).
 constexpr int kRes = 1;          // items a thread handles between slot reservations (20,000 edges: 0.15 ms at 1, 0.19 at 2, 0.34 at 4)
 __global__ void __launch_bounds__(kBlock, 4) k_m_forest(MsfArgs a) {
     GridBar bar(a.bar, a.err);
@@ -585,8 +622,8 @@ __global__ void __launch_bounds__(kBlock, 4) k_m_forest(MsfArgs a) {
                 ca[q] = cb[q] = 0;
                 if (x < n) {
                     const int2 l = round ? lin[x] : make_int2(a.ru[x], a.rv[x]);
-                    ca[q] = new_root(a.par, l.x);
-                    cb[q] = new_root(a.par, l.y);
+                    ca[q] = new_root(a.par, l.x, a.cnt + 6);
+                    cb[q] = new_root(a.par, l.y, a.cnt + 6);
                     if (ca[q] != cb[q]) keep |= 1u << q;
                 }
             }
@@ -604,8 +641,17 @@ __global__ void __launch_bounds__(kBlock, 4) k_m_forest(MsfArgs a) {
         }
         if (lead) a.cnt[2 + ((round & 1) ^ 1)] = 0;
         if (!bar.sync()) return;
-        n = (int64_t) * (volatile unsigned long long *)(a.cnt + (round & 1));
-        if (n == 0) break;
+        const int64_t left = (int64_t) * (volatile unsigned long long *)(a.cnt + (round & 1));
+        if (left == 0) break;
+        if (*(volatile unsigned long long *)(a.cnt + 6)) {  // this round's filter is void: its input is what goes on
+            if (lead) {
+                a.cnt[7] = (unsigned long long)round + 1;
+                a.cnt[8] = (unsigned long long)n;
+                a.cnt[9] = (unsigned long long)nr;
+            }
+            break;
+        }
+        n = left;
         {
             int32_t *t = rout;
             roots = rout;
@@ -623,6 +669,64 @@ __global__ void __launch_bounds__(kBlock, 4) k_m_forest(MsfArgs a) {
         }
     }
     if (lead) a.cnt[4] = (unsigned long long)nfe;
+    bar.finish();
+}
+
+// After k_m_forest stopped at a filter: the pointers of the n live edges'
+// labels settle by jumping rounds, and the edges between two components go out
+// as columns. cnt: [0] edges out, [1 .. 3] flags of the jumping rounds, zero
+// at the start. Labels and keys as k_m_forest keeps them, or (lab null) columns.
+struct MLabels {
+    int64_t n;
+    const int2 *lab;
+    const ulonglong2 *key;
+    const int32_t *ru, *rv, *u, *v;
+    const int64_t *w;
+    int32_t *par;
+    int32_t *cu2, *cv2, *u2, *v2;
+    int64_t *w2;
+    unsigned long long *cnt;
+    int ib, lbits;
+    unsigned *bar, *err;
+};
+struct LabelItem {
+    const int2 *lab;
+    const int32_t *ru, *rv;
+    __device__ __forceinline__ int64_t operator()(int64_t i) const {
+        const int64_t x = i >> 1;
+        if (lab) return (i & 1) ? lab[x].y : lab[x].x;
+        return (i & 1) ? rv[x] : ru[x];
+    }
+};
+__global__ void __launch_bounds__(kBlock) k_m_labels(MLabels a) {
+    GridBar bar(a.bar, a.err);
+    const JumpEnd e = jump_rounds(bar, 2 * a.n, LabelItem{a.lab, a.ru, a.rv}, a.par, a.cnt + 1);
+    if (e == kJumpBarrier) return;
+    if (e == kJumpBound && threadIdx.x == 0) *(volatile unsigned *)a.err = 1u;
+    const unsigned imask = (unsigned)((1ull << a.ib) - 1ull);
+    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < a.n; base += (int64_t)gridDim.x * blockDim.x) {  // CTA-uniform
+        const int64_t x = base + threadIdx.x;
+        int ca = 0, cb = 0;
+        if (x < a.n) {
+            const int2 l = a.lab ? a.lab[x] : make_int2(a.ru[x], a.rv[x]);
+            ca = *(volatile int32_t *)(a.par + l.x);
+            cb = *(volatile int32_t *)(a.par + l.y);
+        }
+        const long long at = cta_reserve(ca != cb, a.cnt);
+        if (ca == cb) continue;
+        a.cu2[at] = ca;
+        a.cv2[at] = cb;
+        if (a.lab) {
+            const u128 k = as_u128(a.key[x]) >> a.lbits;
+            a.u2[at] = (int)((unsigned)(k >> a.ib) & imask);
+            a.v2[at] = (int)((unsigned)k & imask);
+            a.w2[at] = (int64_t)(unsigned long long)(k >> (2 * a.ib));
+        } else {
+            a.u2[at] = a.u[x];
+            a.v2[at] = a.v[x];
+            a.w2[at] = a.w[x];
+        }
+    }
     bar.finish();
 }
 
@@ -778,7 +882,7 @@ static MsfScratch carve_msf(Arena &a, const Problem &p) {
     s.slot = a.take<ulonglong2>(Er);
     s.slot2 = a.take<ulonglong2>(Er);
     s.fe = a.take<FEdge>(E);
-    s.cnt = a.take<unsigned long long>(8);
+    s.cnt = a.take<unsigned long long>(12);
     // the sorts after the rounds, when no bid is read any more
     s.k1 = (unsigned long long *)s.slot;
     s.k2 = s.k1 + Er;
@@ -801,7 +905,7 @@ dgec_status stage_msf(Ctx *c, const Problem &p, const Csr &g, const Skel &sk, Ms
     if (E == 0 || sk.n == 0) return DGEC_OK;
     Arena a(scratch, SIZE_MAX);
     MsfScratch s = carve_msf(a, p);
-    CU_TRY(c, cudaMemsetAsync(s.cnt, 0, 8 * sizeof(unsigned long long), st));
+    CU_TRY(c, cudaMemsetAsync(s.cnt, 0, 12 * sizeof(unsigned long long), st));
     // live edges: (cu, cv) component labels, (u, v) original ends, w; the
     // first round reads the skeleton itself (labels = internal ids)
     const int32_t *ccu = sk.ru, *ccv = sk.rv, *cu = sk.u, *cv = sk.v, *roots0 = nullptr;
@@ -821,7 +925,19 @@ dgec_status stage_msf(Ctx *c, const Problem &p, const Csr &g, const Skel &sk, Ms
             TK(c, "k_m_claim", k_m_claim<<<gn, kBlock, 0, st>>>(ccu, ccv, cu, cv, n, buv, s.bp, s.win));
             TK(c, "k_m_hook", k_m_hook<<<grk, kBlock, 0, st>>>(roots, nr, bw, buv, s.bp, s.win, cu, cv, cw, g.rank_of,
                                                             round == 0 ? g.orig_of : nullptr, s.par, s.fe, s.cnt + 4));
-            TK(c, "k_m_jump", k_m_jump<<<gr, kBlock, 0, st>>>(roots, nr, s.par));
+            CU_TRY(c, cudaMemsetAsync(s.cnt, 0, 4 * sizeof(unsigned long long), st));
+            TK(c, "k_m_jump", k_m_jump<<<gr, kBlock, 0, st>>>(roots, nr, s.par, s.cnt));
+            {
+                int grid = 1;
+                DG_TRY(coop_grid(c, kCoopMJump, (const void *)k_m_settle, kBlock, 0, &grid));
+                unsigned long long *cut = s.cnt;
+                void *args[] = {&roots, &nr, &s.par, &cut, &c->bar, &c->bar_err};
+                cudaError_t e;
+                TK(c, "k_m_settle", e = cudaLaunchCooperativeKernel((const void *)k_m_settle,
+                                                                    dim3((unsigned)std::min(gr, grid)), dim3(kBlock), args,
+                                                                    0, st));
+                if (e != cudaSuccess) return set_err(c, DGEC_ERR_CUDA, "k_m_settle launch: %s", cudaGetErrorString(e));
+            }
             CU_TRY(c, cudaMemsetAsync(s.cnt, 0, 4 * sizeof(unsigned long long), st));
             TK(c, "k_m_next_roots", k_m_next_roots<<<grk, kBlock, 0, st>>>(roots, nr, s.par, bw, buv, roots2, s.cnt + 1));
             std::swap(roots, roots2);
@@ -842,21 +958,48 @@ dgec_status stage_msf(Ctx *c, const Problem &p, const Csr &g, const Skel &sk, Ms
         roots0 = roots;
         CU_TRY(c, cudaMemsetAsync(s.cnt, 0, 4 * sizeof(unsigned long long), st));
     }
-    if (n > 0) {
+    int64_t m = 0;
+    if (n == 0) DG_TRY(read_counters(c, (const int64_t *)(s.cnt + 4), 1, &m));
+    const int lbits = p.tbits + 3 * p.idbits <= 127 ? p.idbits : 0;
+    for (int starts = 0; n > 0; starts++) {
+        if (starts >= 64) return set_err(c, DGEC_ERR_TIMEOUT, "Boruvka did not finish in 64 starts");
         // the kernel's first filter writes lb/kb: not the side its edges come from
         const LiveSide &in = s.side[which ^ 1], &out = s.side[which];
         MsfArgs f{nr, n, roots0, ccu, ccv, cu, cv, cw, g.rank_of, s.par, roots0 ? roots2 : roots, roots0 ? roots : roots2,
-                  s.bp, s.slot, s.slot2, in.lab, out.lab, in.key, out.key, s.fe, s.cnt, p.idbits,
-                  p.tbits + 3 * p.idbits <= 127 ? p.idbits : 0, c->bar, c->bar_err};
+                  s.bp, s.slot, s.slot2, in.lab, out.lab, in.key, out.key, s.fe, s.cnt, p.idbits, lbits, c->bar, c->bar_err};
         int grid = 1;
         DG_TRY(coop_grid(c, kCoopMsf, (const void *)k_m_forest, kBlock, 0, &grid));
         const int64_t want = cdiv(n > nr ? n : nr, kBlock * kRes);
         DG_TRY(coop_launch(c, "k_m_forest", (const void *)k_m_forest, want < grid ? (int)want : grid, kBlock, 0, f));
+        int64_t h[6];
+        DG_TRY(read_counters(c, (const int64_t *)(s.cnt + 4), 6, h));
+        if (h[1]) return set_err(c, DGEC_ERR_TIMEOUT, "Boruvka did not finish in 64 rounds");
+        m = h[0];
+        if (h[3] == 0) break;
+        // a filter's walk was cut: its input's labels settle, and the rounds go on from there
+        const int64_t round = h[3] - 1;
+        const bool odd = round & 1;  // an odd round reads the side `out`, the others (but the first) `in`
+        const LiveSide &from = odd ? out : in, &to = round == 0 ? out : odd ? in : out;
+        n = h[4];
+        nr = h[5];
+        roots = odd ? f.roots2 : f.roots;
+        roots2 = odd ? f.roots : f.roots2;
+        roots0 = roots;
+        CU_TRY(c, cudaMemsetAsync(s.cnt, 0, 4 * sizeof(unsigned long long), st));
+        CU_TRY(c, cudaMemsetAsync(s.cnt + 5, 0, 5 * sizeof(unsigned long long), st));
+        DG_TRY(coop_grid(c, kCoopMLabels, (const void *)k_m_labels, kBlock, 0, &grid));
+        DG_TRY(coop_launch(c, "k_m_labels", (const void *)k_m_labels, (int)std::min<int64_t>(grid, cdiv(n, kBlock)), kBlock, 0,
+                           MLabels{n, round ? from.lab : nullptr, from.key, ccu, ccv, cu, cv, cw, s.par, to.cu, to.cv, to.u,
+                                   to.v, to.w, s.cnt, p.idbits, lbits, c->bar, c->bar_err}));
+        DG_TRY(read_counters(c, (const int64_t *)s.cnt, 1, &n));
+        CU_TRY(c, cudaMemsetAsync(s.cnt, 0, 4 * sizeof(unsigned long long), st));
+        ccu = to.cu;
+        ccv = to.cv;
+        cu = to.u;
+        cv = to.v;
+        cw = to.w;
+        which = &to == &s.side[0] ? 1 : 0;
     }
-    int64_t h[2];
-    DG_TRY(read_counters(c, (const int64_t *)(s.cnt + 4), 2, h));
-    if (h[1]) return set_err(c, DGEC_ERR_TIMEOUT, "Boruvka did not finish in 64 rounds");
-    const int64_t m = h[0];
     o.n = m;
     if (m == 0) return DGEC_OK;
     // order by (w, u, v): stable radix by the packed original ends, then by w,

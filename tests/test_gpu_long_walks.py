@@ -62,6 +62,41 @@ def test_dendrogram_of_a_path(n):
     assert fall["D1 dendrogram"] < 8 * rise["D1 dendrogram"]
 
 
+@pytest.mark.parametrize("n", [400_000, 2_000_000])
+def test_forest_of_a_path(n):
+    fall, rise = _path_stages(n, False), _path_stages(n, True)
+    assert fall["C spanning forest"] < 8 * rise["C spanning forest"]
+
+
+@pytest.mark.parametrize("n", [1_000_000, 5_000_000])  # cooperative rounds alone; a large round first
+def test_long_paths_merge_from_the_last(n):
+    import torch
+    src, dst, t, V = _path(n, False)
+    out = ctx().run(*(torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in (src, dst, t)), V, 2, 2)
+    assert np.array_equal(out.numpy("mst_w"), 2 + np.arange(n))
+    assert np.array_equal(out.numpy("link_size"), 2 + np.arange(n))
+    assert out.n_mst == n
+
+
+def _chain_of_chains(m):
+    """m relay chains of falling gaps, joined end to end by longer ones that
+    fall too: after the first round a long chain of components is left."""
+    gaps = np.concatenate([np.append(2 + np.arange(8)[::-1], 1000 + m - i) for i in range(m)])[:-1]
+    t = np.concatenate([[0], np.cumsum(gaps)])
+    p = np.random.default_rng(m).permutation(len(t))
+    a = np.arange(len(t), dtype=np.int32)
+    return a[p], a[p] + 1, t[p], len(t) + 1
+
+
+@pytest.mark.parametrize("shift", [0, 27])  # with and without labels in the bids
+def test_walks_cut_in_a_later_round(shift):
+    src, dst, t, V = _chain_of_chains(240_000)
+    t = t << shift
+    assert (int(t.max()).bit_length() + 3 * (len(t) - 1).bit_length() > 127) == (shift > 0)
+    q = np.arange(0, len(t), 50_000).astype(np.int32)
+    compare_all(src, dst, t, V, 2, 2, knn_query=q)
+
+
 @pytest.mark.parametrize("n", [100_000, 600_000])
 def test_paths_equal_the_oracle(n):
     src, dst, t, V = _path(n, False)
