@@ -468,15 +468,34 @@ __device__ __forceinline__ u128 cas_u128(ulonglong2 *p, u128 cmp, u128 val) {
         : "memory");
     return ((u128)hi << 64) | lo;
 }
+// A slot as one value (a plain 16-byte read may mix words of two writes).
+__device__ __forceinline__ u128 whole_u128(const ulonglong2 *p) {
+    unsigned long long lo, hi;
+    asm volatile(
+        "{\n\t.reg .b128 o;\n\t"
+        "ld.relaxed.gpu.global.b128 o, [%2];\n\t"
+        "mov.b128 {%0, %1}, o;\n\t}"
+        : "=l"(lo), "=l"(hi)
+        : "l"(p)
+        : "memory");
+    return ((u128)hi << 64) | lo;
+}
 // Minima of two keys into two slots, their reads and their swaps in flight
 // together. The read before skips bids that cannot win (most, at a large
 // component). It trusts the high word alone, which only falls: the two words
 // of the read need not belong together, so where the high words tie, a swap
-// of the value for itself reads it whole.
+// of the value for itself reads it whole. FIRST: every label is a node, and
+// very many edges of one weight can meet at one of them, whose swaps would wait
+// for one another; there a bid that seems lost reads the slot whole instead
+// (3M in-edges of one time: k_m_forest 1.28 ms with swaps alone, 0.43 so;
+// in every round 0.40, but 2M mixed edges then 1.02 ms instead of 0.99).
+template <bool FIRST>
 __device__ __forceinline__ void bid_u128(ulonglong2 *sa, u128 ka, ulonglong2 *sb, u128 kb) {
     const ulonglong2 pa = *sa, pb = *sb;
     bool ga = (unsigned long long)(ka >> 64) <= pa.y, gb = (unsigned long long)(kb >> 64) <= pb.y;
     u128 ca = as_u128(pa), cb = as_u128(pb), oa = 0, ob = 0;
+    if (FIRST && ga && ka >= ca) ga = ka < (ca = whole_u128(sa));
+    if (FIRST && gb && kb >= cb) gb = kb < (cb = whole_u128(sb));
     if (ga) oa = cas_u128(sa, ca, ka < ca ? ka : ca);
     if (gb) ob = cas_u128(sb, cb, kb < cb ? kb : cb);
     // a swap that took place wrote the smaller of the two; else go on from the value it met
@@ -546,7 +565,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_m_forest(MsfArgs a) {
     for (int64_t x = g0; x < a.n0; x += gsize) {
         const int cu = a.ru[x], cv = a.rv[x];
         const u128 key = pack(x);
-        bid_u128(a.slot + cu, key | (lb ? (unsigned)cv : 0u), a.slot + cv, key | (lb ? (unsigned)cu : 0u));
+        bid_u128<true>(a.slot + cu, key | (lb ? (unsigned)cv : 0u), a.slot + cv, key | (lb ? (unsigned)cu : 0u));
     }
     if (!bar.sync()) return;
     int64_t n = a.n0, nr = a.nr0, nfe = (int64_t)a.cnt[4];
@@ -636,7 +655,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_m_forest(MsfArgs a) {
                 lout[at] = make_int2(ca[q], cb[q]);
                 kout[at] = as_pair(key);
                 at++;
-                bid_u128(slot2 + ca[q], key | (lb ? (unsigned)cb[q] : 0u), slot2 + cb[q], key | (lb ? (unsigned)ca[q] : 0u));
+                bid_u128<false>(slot2 + ca[q], key | (lb ? (unsigned)cb[q] : 0u), slot2 + cb[q], key | (lb ? (unsigned)ca[q] : 0u));
             }
         }
         if (lead) a.cnt[2 + ((round & 1) ^ 1)] = 0;

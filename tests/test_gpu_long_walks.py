@@ -1,5 +1,6 @@
-"""Pointer walks on the longest chains: a stage whose walkers meet only
-pointers as short as their own must not take time by the length of the chain.
+"""Inputs on which one address or one chain holds everything up: pointer
+walks on the longest chains, whose walkers meet only pointers as short as their
+own, and edges of one weight at one vertex, whose bids meet at one slot.
 Each test compares a stage with another of the same call or of a call on as
 many edges without long chains, on the device's own clock."""
 import numpy as np
@@ -102,3 +103,23 @@ def test_paths_equal_the_oracle(n):
     src, dst, t, V = _path(n, False)
     q = np.arange(0, n, n // 100).astype(np.int32)
     compare_all(src, dst, t, V, 2, 2, knn_query=q)
+
+
+def test_bids_of_one_weight_at_one_vertex():
+    """A vertex that millions of edges reach at one time before it sends: all
+    of them bid the same weight there. The forest of as many edges at distinct
+    times has the same edges and more digits to sort."""
+    import torch
+    m = 3_000_000
+    src = torch.arange(1, m + 2, dtype=torch.int32, device="cuda")
+    src[m] = 0
+    dst = torch.zeros(m + 1, dtype=torch.int32, device="cuda")
+    dst[m] = m + 1
+    one = torch.zeros(m + 1, dtype=torch.int64, device="cuda")
+    g = torch.Generator(device="cuda")
+    g.manual_seed(2)
+    many = torch.zeros(m + 1, dtype=torch.int64, device="cuda")
+    many[:m] = torch.randperm(m, generator=g, device="cuda")
+    one[m] = many[m] = m + 5
+    a, b = (_stages(lambda: ctx().run(src, dst, t, m + 2, 4, 5), 6)["C spanning forest"] for t in (one, many))
+    assert a < b
