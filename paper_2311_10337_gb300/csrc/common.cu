@@ -25,15 +25,20 @@ dgec_status read_counters(Ctx *c, const int64_t *d, int n, int64_t *host) {
 }
 
 dgec_status coop_begin(Ctx *c, unsigned *bar) {
-    c->bar = bar;
-    *(volatile unsigned *)c->bar_err = 0u;
+    c->bar.word = bar;
+    c->coop_launches = 0;
+    *(volatile unsigned *)c->bar.err = 0u;
     CU_TRY(c, cudaMemsetAsync(bar, 0, sizeof(unsigned) * kBarWords, c->stream));
     return DGEC_OK;
 }
 
 dgec_status coop_check(Ctx *c) {
-    if (*(volatile unsigned *)c->bar_err) return set_err(c, DGEC_ERR_TIMEOUT, "a grid barrier gave up");
-    return DGEC_OK;
+    switch (*(volatile unsigned *)c->bar.err) {
+        case 0: return DGEC_OK;
+        case kStopJump: return set_err(c, DGEC_ERR_TIMEOUT, "pointer jumping did not settle");
+        case kStopEom: return set_err(c, DGEC_ERR_TIMEOUT, "the EOM pass exceeded its round bound");
+        default: return set_err(c, DGEC_ERR_TIMEOUT, "a grid barrier gave up");
+    }
 }
 
 dgec_status coop_grid(Ctx *c, CoopKernel which, const void *fn, int threads, size_t smem, int *grid) {

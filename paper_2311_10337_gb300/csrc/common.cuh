@@ -46,6 +46,19 @@ struct StageTimer {
 // Cooperative kernels whose resident-CTA count a context remembers.
 enum CoopKernel { kCoopSortK, kCoopSortKV, kCoopEom, kCoopMsf, kCoopMJump, kCoopMLabels, kCoopDendro, kCoopDJump, kCoopJumpAll, kCoopJumpBig, kCoopCount };
 
+// What the grid barriers of a call share. `word` (in the call's workspace, zeroed
+// once a call): [0] arrivals, [1] exits, [2] the call's stop word. Once a
+// cooperative kernel gives up it writes its StopCode there and to *err
+// (host-mapped). Until the host reads that, the kernels behind it still run:
+// those that follow what it left as indices return when the stop word is set,
+// and so does every cooperative kernel.
+enum StopCode : unsigned { kStopBarrier = 1, kStopJump = 2, kStopEom = 3 };
+struct BarRef {
+    unsigned *word = nullptr;
+    unsigned *err = nullptr;
+    unsigned polls = 0;  // polls before a barrier gives up
+};
+
 struct Ctx {
     int device = 0;
     int knn_block = 128;           // launch configuration (dgec_set_launch_config)
@@ -59,14 +72,22 @@ struct Ctx {
     KernelTimer *kt = nullptr;
     StageTimer stages;
     int coop_ctas[kCoopCount] = {};  // CTAs of each cooperative kernel the device holds at once; 0 = not asked yet
-    unsigned *bar = nullptr;         // barrier words of the current call (in its workspace)
-    unsigned *bar_err = nullptr;     // host-mapped: 1 once a grid barrier gave up
+    BarRef bar;                      // of the current call
+    unsigned bar_polls = 1u << 24;   // bounds of the waits (dgec_set_limits)
+    int bar_from = 0;
+    int coop_launches = 0;           // of the current call
+    BarRef next_bar() {              // for the next cooperative launch
+        BarRef b = bar;
+        b.polls = coop_launches++ >= bar_from ? bar_polls : 1u << 24;
+        return b;
+    }
+    const unsigned *stop() const { return bar.word + 2; }
 };
 
 // The current call's barrier words, zeroed on its stream.
 constexpr int kBarWords = 64;
 dgec_status coop_begin(Ctx *c, unsigned *bar);
-// DGEC_ERR_TIMEOUT if a grid barrier gave up (after a stream synchronisation).
+// DGEC_ERR_TIMEOUT if a cooperative kernel gave up (after a stream synchronisation).
 dgec_status coop_check(Ctx *c);
 // How many CTAs of the kernel fit on the device at once (also raises its
 // dynamic shared memory limit).
@@ -190,6 +211,9 @@ dgec_status read_counters(Ctx *c, const int64_t *d, int n, int64_t *host);
 // ---------------------------------------------------------------- device
 
 __device__ __forceinline__ unsigned lane_id() { return threadIdx.x & 31; }
+
+// A cooperative kernel of this call has given up (see BarRef).
+__device__ __forceinline__ bool stopped(const unsigned *stop) { return *stop != 0; }
 
 // Warp-aggregated increment of counter[key] by 1 per lane; returns this
 // lane's slot (old value + rank among lanes with the same key). All lanes

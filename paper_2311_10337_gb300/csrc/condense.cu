@@ -92,7 +92,8 @@ struct SelBigRep {  // big kept merges (the nodes whose cluster link is set)
 // 21 ms, but 100M hub edges then need the rounds (0.5 ms), with 512 they do not.
 constexpr int kTopWalk = 512;
 template <class Sel>
-__global__ void k_c_top(int64_t n, int64_t off, Sel sel, int32_t *ptr, unsigned long long *moved) {
+__global__ void k_c_top(const unsigned *stop, int64_t n, int64_t off, Sel sel, int32_t *ptr, unsigned long long *moved) {
+    if (stopped(stop)) return;
     bool cut = false;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n;
          t += (int64_t)gridDim.x * blockDim.x) {
@@ -123,12 +124,13 @@ struct SelItem {
 // short. moved[1 .. 3] are their flags, zero at the start.
 template <class Sel>
 __global__ void __launch_bounds__(kBlock) k_c_jump(int64_t n, int64_t off, Sel sel, int32_t *ptr,
-                                                   unsigned long long *moved, unsigned *barw, unsigned *err) {
+                                                   unsigned long long *moved, BarRef ref) {
     if (moved[0] == 0) return;  // the same for every CTA: written before this launch
-    GridBar bar(barw, err);
+    GridBar bar(ref);
+    if (bar.stopped()) return;
     const JumpEnd e = jump_rounds(bar, n, SelItem<Sel>{off, sel}, ptr, moved + 1);
     if (e == kJumpBarrier) return;
-    if (e == kJumpBound && threadIdx.x == 0) *(volatile unsigned *)err = 1u;
+    if (e == kJumpBound && threadIdx.x == 0) bar.stop(kStopJump);
     bar.finish();
 }
 
@@ -141,11 +143,12 @@ static dgec_status jump_to_fixed(Ctx *c, CoopKernel which, int64_t n, int64_t of
                                  unsigned long long *moved) {
     if (n <= 0) return DGEC_OK;
     const int g = grid_for(n, kBlock, kStreamCap);
-    TK(c, "k_c_top", k_c_top<Sel><<<g, kBlock, 0, c->stream>>>(n, off, sel, ptr, moved));
+    TK(c, "k_c_top", k_c_top<Sel><<<g, kBlock, 0, c->stream>>>(c->stop(), n, off, sel, ptr, moved));
     int grid = 1;
     const void *fn = (const void *)k_c_jump<Sel>;
     DG_TRY(coop_grid(c, which, fn, kBlock, 0, &grid));
-    void *args[] = {&n, &off, &sel, &ptr, &moved, &c->bar, &c->bar_err};
+    BarRef ref = c->next_bar();
+    void *args[] = {&n, &off, &sel, &ptr, &moved, &ref};
     cudaError_t e;
     TK(c, "k_c_jump", e = cudaLaunchCooperativeKernel(fn, dim3((unsigned)(g < grid ? g : grid)), dim3(kBlock), args, 0,
                                                       c->stream));
@@ -188,8 +191,9 @@ __global__ void k_c_cpar(Gview gv, const int32_t *__restrict__ parent, const int
 // link: a big kept merge continues its parent's cluster when it is the
 // parent's only big child, else it starts a cluster (link to itself);
 // virtual roots link to themselves.
-__global__ void k_c_link(Gview gv, const int *isrep, const int64_t *size, const int32_t *cpar,
+__global__ void k_c_link(const unsigned *stop, Gview gv, const int *isrep, const int64_t *size, const int32_t *cpar,
                          const unsigned long long *nbs, int32_t *link) {
+    if (stopped(stop)) return;
     const int64_t E = gv.E, n = gv.n;
     for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n + gv.G;
          s += (int64_t)gridDim.x * blockDim.x) {
@@ -205,10 +209,11 @@ __global__ void k_c_link(Gview gv, const int *isrep, const int64_t *size, const 
 
 
 // cluster records, indexed by node id
-__global__ void k_c_clusters(Gview gv, const int *isrep, const int64_t *size, const int64_t *w,
+__global__ void k_c_clusters(const unsigned *stop, Gview gv, const int *isrep, const int64_t *size, const int64_t *w,
                              const int32_t *cpar, const unsigned long long *nbs, const int32_t *link, int *isc,
                              unsigned long long *cbirth, unsigned long long *cdeath,
                              int32_t *cparent) {
+    if (stopped(stop)) return;
     const int64_t E = gv.E, n = gv.n;
     for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n + gv.G;
          s += (int64_t)gridDim.x * blockDim.x) {
@@ -250,10 +255,11 @@ struct __align__(32) NodeRec {
 // = size(X) minus the sizes of X's big children (the points under its small
 // children, which walk up to X): one exact 128-bit add per node, summed per
 // warp and cluster, instead of one per point.
-__global__ void k_c_nrec(Gview gv, const int *isrep, const int64_t *size, const int64_t *w,
+__global__ void k_c_nrec(const unsigned *stop, Gview gv, const int *isrep, const int64_t *size, const int64_t *w,
                          const int32_t *cpar, const int32_t *link, const unsigned long long *cbirth,
                          const unsigned long long *__restrict__ nbs, NodeRec *rec, unsigned long long *st_hi,
                          unsigned long long *st_lo) {
+    if (stopped(stop)) return;
     const int64_t E = gv.E, n = gv.n, total = n + gv.G;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t base = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; base < total;
@@ -298,8 +304,9 @@ __global__ void k_c_nrec(Gview gv, const int *isrep, const int64_t *size, const 
 
 // where each point leaves: the lowest kept ancestor of size >= M (its
 // stability share is counted per node above)
-__global__ void k_c_points(Gview gv, const int32_t *__restrict__ cpar, const NodeRec *__restrict__ rec,
+__global__ void k_c_points(const unsigned *stop, Gview gv, const int32_t *__restrict__ cpar, const NodeRec *__restrict__ rec,
                            int32_t *__restrict__ fall_cluster, uint64_t *__restrict__ fall_lambda) {
+    if (stopped(stop)) return;
     const int64_t E = gv.E;
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < E;
          p += (int64_t)gridDim.x * blockDim.x) {
@@ -370,8 +377,8 @@ struct Eom {
     int32_t *ucand, *nxt, *nxt2, *al, *al2;
     unsigned long long *slot;  // (next ancestor << 32) | highest selected on the way there
     int32_t *H;                // highest selected ancestor-or-self, -1
-    unsigned long long *cnt;   // [0], [1] open clusters, [2..4] flags, [5] error; zeroed before the kernel
-    unsigned *bar, *err;
+    unsigned long long *cnt;   // [0], [1] open clusters, [2..4] flags; zeroed before the kernel
+    BarRef bar;
 };
 
 __global__ void k_e_init(Eom e, const unsigned long long *st_hi, const unsigned long long *st_lo,
@@ -440,7 +447,8 @@ __device__ __forceinline__ void e_walk(const Eom &e, int c) {
 // for 0.55 at 20,000 edges, 0.63 for 2.7 at 10M, 4.7 for about 15 at 100M hub
 // edges.
 __global__ void __launch_bounds__(256, 4) k_e_tree(Eom e) {
-    GridBar bar(e.bar, e.err);
+    GridBar bar(e.bar);
+    if (bar.stopped()) return;
     const int64_t gsize = (int64_t)gridDim.x * blockDim.x, g0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
     for (int64_t c = g0; c < e.root0; c += gsize)
@@ -450,8 +458,8 @@ __global__ void __launch_bounds__(256, 4) k_e_tree(Eom e) {
     int64_t nact = e.root0;
     for (int phase = 0;; phase++) {
         if (phase > 4096) {
-            if (lead) e.cnt[5] = 1;
-            break;
+            if (lead) bar.stop(kStopEom);
+            return;
         }
         // the open clusters; each tells a parent that waits for it alone
         for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < nact; base += gsize) {  // CTA-uniform
@@ -568,8 +576,8 @@ __global__ void __launch_bounds__(256, 4) k_e_tree(Eom e) {
     if (!bar.sync()) return;
     for (int round = 0;; round++) {
         if (round > 4096) {
-            if (lead) e.cnt[5] = 2;
-            break;
+            if (lead) bar.stop(kStopEom);
+            return;
         }
         bool cut = false;
         for (int64_t t = g0; t < e.ncl; t += gsize) {
@@ -598,8 +606,9 @@ __global__ void __launch_bounds__(256, 4) k_e_tree(Eom e) {
     bar.finish();
 }
 
-__global__ void k_e_labels(int64_t E, const int32_t *fall_cluster, const int32_t *cidx,
+__global__ void k_e_labels(const unsigned *stop, int64_t E, const int32_t *fall_cluster, const int32_t *cidx,
                            const int32_t *H, int32_t *lab, int *minmem) {
+    if (stopped(stop)) return;
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < E;
          p += (int64_t)gridDim.x * blockDim.x) {
         int L = H[cidx[fall_cluster[p]]];
@@ -626,8 +635,9 @@ __global__ void k_e_final_emit(int64_t ncl, const int *flag, const long long *po
 
 // Final clusters sorted by smallest member (a global edge id, so graphs
 // come in order); a cluster's label is its position within its graph.
-__global__ void k_e_gstart(int64_t nf, const unsigned long long *key, const int32_t *egraph,
+__global__ void k_e_gstart(const unsigned *stop, int64_t nf, const unsigned long long *key, const int32_t *egraph,
                            int64_t *gstart, int32_t *gcount) {
+    if (stopped(stop)) return;
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < nf;
          x += (int64_t)gridDim.x * blockDim.x) {
         int g = egraph[key[x]];
@@ -639,8 +649,9 @@ __global__ void k_e_gcount(int G, const int64_t *gstart, int32_t *gcount) {
     for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x)
         if (gcount[g] > 0) gcount[g] -= (int32_t)gstart[g];
 }
-__global__ void k_e_rank(int64_t nf, const unsigned long long *key, const unsigned long long *v,
+__global__ void k_e_rank(const unsigned *stop, int64_t nf, const unsigned long long *key, const unsigned long long *v,
                          const int32_t *egraph, const int64_t *gstart, int32_t *rank) {
+    if (stopped(stop)) return;
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < nf;
          x += (int64_t)gridDim.x * blockDim.x)
         rank[v[x]] = (int32_t)(x - gstart[egraph[key[x]]]);
@@ -797,15 +808,15 @@ dgec_status stage_condense(Ctx *c, const Problem &p, const Msf &m, const Dendro 
         DG_TRY(jump_to_fixed(c, kCoopJumpAll, n, 0, SelAll{}, s.up, s.jflag));
     }
     TK(c, "k_c_cpar", k_c_cpar<<<gN, kBlock, 0, st>>>(gv, d.parent, s.up, s.isrep, d.size, s.cpar, nbs));
-    TK(c, "k_c_link", k_c_link<<<gn, kBlock, 0, st>>>(gv, s.isrep, d.size, s.cpar, nbs, s.link));
+    TK(c, "k_c_link", k_c_link<<<gn, kBlock, 0, st>>>(c->stop(), gv, s.isrep, d.size, s.cpar, nbs, s.link));
     DG_TRY(jump_to_fixed(c, kCoopJumpBig, n, E, SelBigRep{gv, s.isrep, d.size}, s.link, s.jflag + 4));
-    TK(c, "k_c_clusters", k_c_clusters<<<gn, kBlock, 0, st>>>(gv, s.isrep, d.size, m.w, s.cpar, nbs, s.link,
+    TK(c, "k_c_clusters", k_c_clusters<<<gn, kBlock, 0, st>>>(c->stop(), gv, s.isrep, d.size, m.w, s.cpar, nbs, s.link,
                                                              s.isc, s.cbirth, s.cdeath, s.cparent));
     // the node records live in the EOM phase's Fa and Fc arrays (adjacent, not in use yet)
     NodeRec *nrec = reinterpret_cast<NodeRec *>(s.Fa);
-    TK(c, "k_c_nrec", k_c_nrec<<<gn, kBlock, 0, st>>>(gv, s.isrep, d.size, m.w, s.cpar, s.link, s.cbirth, nbs,
+    TK(c, "k_c_nrec", k_c_nrec<<<gn, kBlock, 0, st>>>(c->stop(), gv, s.isrep, d.size, m.w, s.cpar, s.link, s.cbirth, nbs,
                                                      nrec, s.st_hi, s.st_lo));
-    TK(c, "k_c_points", k_c_points<<<gE, kBlock, 0, st>>>(gv, s.cpar, nrec, o.fall_cluster, o.fall_lambda));
+    TK(c, "k_c_points", k_c_points<<<gE, kBlock, 0, st>>>(c->stop(), gv, s.cpar, nrec, o.fall_cluster, o.fall_lambda));
     // cluster flags of node ids E .. N (the last one a zero sentinel)
     DG_TRY(exclusive_scan_i32(c, s.isc + E, s.cpos, n + p.G + 1, s.scan_tmp));
     int64_t ncl;
@@ -843,23 +854,20 @@ dgec_status stage_condense(Ctx *c, const Problem &p, const Msf &m, const Dendro 
     e.slot = s.k1;
     e.H = s.H;
     e.cnt = s.cnt;
-    e.bar = c->bar;
-    e.err = c->bar_err;
     const int gc = grid_for(ncl + 1, kBlock, kStreamCap);
     TK(c, "k_e_init", k_e_init<<<gc, kBlock, 0, st>>>(e, s.st_hi, s.st_lo, s.cbirth, s.cdeath));
     {
         int grid = 1;
+        e.bar = c->next_bar();
         DG_TRY(coop_grid(c, kCoopEom, (const void *)k_e_tree, kBlock, 0, &grid));
         const int64_t want = cdiv(ncl, kBlock);  // (two clusters a thread: 0.070 ms instead of 0.058 at 20,000 edges)
         DG_TRY(coop_launch(c, "k_e_tree", (const void *)k_e_tree, want < grid ? (int)want : grid, kBlock, 0, e));
     }
-    TK(c, "k_e_labels", k_e_labels<<<gE, kBlock, 0, st>>>(E, o.fall_cluster, s.cidx, s.H, o.labels, s.minmem));
+    TK(c, "k_e_labels", k_e_labels<<<gE, kBlock, 0, st>>>(c->stop(), E, o.fall_cluster, s.cidx, s.H, o.labels, s.minmem));
     TK(c, "k_e_final_keys", k_e_final_keys<<<gc, kBlock, 0, st>>>(ncl, s.H, s.minmem, s.flag));
     DG_TRY(exclusive_scan_i32(c, s.flag, s.cpos, ncl + 1, s.scan_tmp));
     int64_t nf;
-    CU_TRY(c, cudaMemcpyAsync(c->h_pinned + 8, s.cnt + 5, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     DG_TRY(read_counters(c, (const int64_t *)(s.cpos + ncl), 1, &nf));
-    if (c->h_pinned[8]) return set_err(c, DGEC_ERR_TIMEOUT, "the EOM pass exceeded its round bound");
     o.n_clusters = (int32_t)nf;
     if (nf > 0) {
         TK(c, "k_e_final_emit", k_e_final_emit<<<gc, kBlock, 0, st>>>(ncl, s.flag, s.cpos, s.minmem, s.k1, s.v1));
@@ -868,9 +876,9 @@ dgec_status stage_condense(Ctx *c, const Problem &p, const Msf &m, const Dendro 
                           s.radix, &in_b));
         unsigned long long *kk = in_b ? s.k2 : s.k1, *vv = in_b ? s.v2 : s.v1;
         const int gf = grid_for(nf, kBlock, kStreamCap);
-        TK(c, "k_e_gstart", k_e_gstart<<<gf, kBlock, 0, st>>>(nf, kk, p.egraph, s.gstart, o.gclusters));
+        TK(c, "k_e_gstart", k_e_gstart<<<gf, kBlock, 0, st>>>(c->stop(), nf, kk, p.egraph, s.gstart, o.gclusters));
         TK(c, "k_e_gcount", k_e_gcount<<<grid_for(p.G), kBlock, 0, st>>>(p.G, s.gstart, o.gclusters));
-        TK(c, "k_e_rank", k_e_rank<<<gf, kBlock, 0, st>>>(nf, kk, vv, p.egraph, s.gstart, s.rank));
+        TK(c, "k_e_rank", k_e_rank<<<gf, kBlock, 0, st>>>(c->stop(), nf, kk, vv, p.egraph, s.gstart, s.rank));
         TK(c, "k_e_relabel", k_e_relabel<<<gE, kBlock, 0, st>>>(E, s.rank, o.labels));
     }
     TK(c, "k_e_out", k_e_out<<<gc, kBlock, 0, st>>>(e, gv, d.size, s.cbirth, s.cdeath, s.H, o.cl_id, o.cl_parent,

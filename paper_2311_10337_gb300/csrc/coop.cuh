@@ -1,51 +1,46 @@
 // Cooperative building blocks: a grid barrier for kernels whose CTAs are all
-// resident (launched through coop_launch), and the stable LSD radix sort as
-// one such kernel.
+// resident (cooperative launches), and pointer jumping inside such a kernel.
 #pragma once
 
 #include "common.cuh"
 
 namespace dgec {
 
-// The barrier words of a call (kBarWords of them): [0] arrivals, [1] exits.
-// Zeroed once per call; the last CTA out of a kernel leaves them zero again.
-
-// Polls before a barrier gives up (about a microsecond each). CTAs of a
-// cooperative launch are co-resident, so this only bounds the wait should
-// that ever not hold.
-constexpr unsigned kBarPolls = 1u << 24;
-
 // Barrier over every CTA of a cooperative launch. Arrivals count up without
-// a reset between barriers (compared by signed difference). A barrier that
-// gives up writes 1 to *err (host-mapped memory) and returns false in every
-// thread of its CTA; the kernel must then return at once (the other CTAs
-// give up likewise).
+// a reset between barriers (compared by signed difference). CTAs of a
+// cooperative launch are co-resident, so the limit on the polls (about a
+// microsecond each) only bounds the wait should that ever not hold. A barrier
+// that gives up writes the stop word (see BarRef) and returns false in every
+// thread of its CTA; the kernel must then return at once. The other CTAs find
+// the stop word or their own limit at the next barrier, which cannot complete,
+// so no CTA goes on to read what the missing one has not written.
 struct GridBar {
-    unsigned *word;
-    unsigned *err;
-    unsigned nblk, target;  // nblk = 1 once one CTA goes on alone
-    __device__ __forceinline__ GridBar(unsigned *w, unsigned *e) : word(w), err(e), nblk(gridDim.x), target(0) {}
+    BarRef ref;
+    unsigned target;
+    __device__ __forceinline__ explicit GridBar(const BarRef &r) : ref(r), target(0) {}
+    // A kernel of the call has given up before: return at once, without finish().
+    __device__ __forceinline__ bool stopped() const { return __syncthreads_or(*(volatile unsigned *)(ref.word + 2) != 0); }
+    __device__ __forceinline__ void stop(StopCode code) {  // one thread or more
+        *(volatile unsigned *)ref.err = code;
+        *(volatile unsigned *)(ref.word + 2) = code;
+    }
     __device__ __forceinline__ bool sync() {
-        if (nblk == 1) {
-            __syncthreads();
-            return true;
-        }
         __syncthreads();
+        if (gridDim.x == 1) return true;
         bool bad = false;
-        target += nblk;
+        target += gridDim.x;
         if (threadIdx.x == 0) {
             __threadfence();
-            atomicAdd(word, 1u);
-            unsigned polls = 0;
-            for (;;) {
-                unsigned v;
-                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(word) : "memory");
-                if ((int)(v - target) >= 0) break;
-                if (++polls > kBarPolls) {
+            atomicAdd(ref.word, 1u);
+            for (unsigned polls = 0;; polls++) {
+                if (polls >= ref.polls || ((polls & 1023) == 1023 && *(volatile unsigned *)(ref.word + 2))) {
                     bad = true;
-                    *(volatile unsigned *)err = 1u;
+                    stop(kStopBarrier);
                     break;
                 }
+                unsigned v;
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ref.word) : "memory");
+                if ((int)(v - target) >= 0) break;
             }
             __threadfence();
         }
@@ -54,9 +49,9 @@ struct GridBar {
     // every CTA calls this after its last barrier
     __device__ __forceinline__ void finish() {
         if (gridDim.x == 1 || threadIdx.x != 0) return;
-        if (atomicAdd(word + 1, 1u) == gridDim.x - 1) {
-            word[0] = 0u;
-            word[1] = 0u;
+        if (atomicAdd(ref.word + 1, 1u) == gridDim.x - 1) {
+            ref.word[0] = 0u;
+            ref.word[1] = 0u;
         }
     }
 };

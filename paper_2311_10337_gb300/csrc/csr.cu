@@ -110,9 +110,10 @@ struct TE {
 // rank r = position of edge (t, id) in the global order; time-ordered
 // copies of the inputs for the later stages. The sort carried each edge's
 // (src, dst) pair, in global vertex ids, as its value.
-__global__ void k_rank_init(const unsigned long long *ks, const unsigned long long *vs, int64_t E,
+__global__ void k_rank_init(const unsigned *stop, const unsigned long long *ks, const unsigned long long *vs, int64_t E,
                             long long tmin, int idbits, int32_t *orig_of, int32_t *rank_of, int32_t *isrc,
                             int32_t *idst, int64_t *it, TE *te) {
+    if (stopped(stop)) return;
     const unsigned long long idmask = (1ull << idbits) - 1ull;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < E;
          r += (int64_t)gridDim.x * blockDim.x) {
@@ -129,10 +130,11 @@ __global__ void k_rank_init(const unsigned long long *ks, const unsigned long lo
 }
 
 // the same from a (t - tmin) key sorted with the edge id as its value
-__global__ void k_rank_init_kv(const unsigned long long *ks, const unsigned long long *vs, int64_t E,
+__global__ void k_rank_init_kv(const unsigned *stop, const unsigned long long *ks, const unsigned long long *vs, int64_t E,
                                long long tmin, const int32_t *src, const int32_t *dst,
                                const int32_t *egraph, const int64_t *voff, int G, int32_t *orig_of,
                                int32_t *rank_of, int32_t *isrc, int32_t *idst, int64_t *it, TE *te) {
+    if (stopped(stop)) return;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < E;
          r += (int64_t)gridDim.x * blockDim.x) {
         int32_t e = (int32_t)vs[r];
@@ -193,8 +195,9 @@ __global__ void k_mkeys(const int32_t *isrc, const int32_t *idst, const int *fla
     }
 }
 // out_off[v] = out-items before v's segment; in_off[v] = in-items before it
-__global__ void k_moff_split(const int64_t *moff, const int32_t *oidx, int64_t V, int64_t *out_off,
+__global__ void k_moff_split(const unsigned *stop, const int64_t *moff, const int32_t *oidx, int64_t V, int64_t *out_off,
                              int64_t *in_off) {
+    if (stopped(stop)) return;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v <= V;
          v += (int64_t)gridDim.x * blockDim.x) {
         const int64_t m = moff[v];
@@ -205,13 +208,14 @@ __global__ void k_moff_split(const int64_t *moff, const int32_t *oidx, int64_t V
 }
 // Every item of the merged lists goes to its slot in the out- or in-list
 // arrays; its rank in the other list is its position difference.
-__global__ void k_munpack(const unsigned long long *key, const unsigned long long *val, long long tmin,
+__global__ void k_munpack(const unsigned *stop, const unsigned long long *key, const unsigned long long *val, long long tmin,
                           int64_t n2, int cb, const int64_t *moff,
                           const int32_t *oidx, const int64_t *out_off, const TE *te, int64_t *out_t,
                           int32_t *out_id, int32_t *out_r, int4 *outrk, int32_t *pos_out, int64_t *in_t,
                           int32_t *in_id, int32_t *in_r, int32_t *pos_in, unsigned char *in_head,
                           int2 *inrk, int2 *in_va, int2 *out_vb, unsigned long long *out_key,
                           unsigned long long *in_key) {
+    if (stopped(stop)) return;
     const unsigned long long cmask = (1ull << cb) - 1ull;
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n2;
          x += (int64_t)gridDim.x * blockDim.x) {
@@ -370,9 +374,10 @@ __global__ void k_hub_gather(const unsigned long long *keys, const int64_t *off,
 }
 
 // After sorting by (hub, key): element j goes back to its hub's segment.
-__global__ void k_hub_scatter(const unsigned long long *hub_of, const unsigned long long *key_of,
+__global__ void k_hub_scatter(const unsigned *stop, const unsigned long long *hub_of, const unsigned long long *key_of,
                               int64_t n, const int64_t *off, const int *list,
                               const long long *hoff, unsigned long long *keys) {
+    if (stopped(stop)) return;
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n;
          j += (int64_t)gridDim.x * blockDim.x) {
         int h = (int)hub_of[j];
@@ -381,7 +386,8 @@ __global__ void k_hub_scatter(const unsigned long long *hub_of, const unsigned l
 }
 
 // off[v] = first sorted position whose vertex (key >> idbits) is >= v, for v in [0, V]
-__global__ void k_voffsets(const unsigned long long *key, int64_t E, int64_t V, int idbits, int64_t *off) {
+__global__ void k_voffsets(const unsigned *stop, const unsigned long long *key, int64_t E, int64_t V, int idbits, int64_t *off) {
+    if (stopped(stop)) return;
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x <= E;
          x += (int64_t)gridDim.x * blockDim.x) {
         const int64_t v = x < E ? (int64_t)(key[x] >> idbits) : V;
@@ -481,6 +487,7 @@ dgec_status sort_segments(Ctx *c, int64_t V, unsigned long long *keys, const int
         memcpy(tmp, c->h_pinned, sizeof(tmp));
         for (int q = 0; q < 4; q++) h[q] = tmp[q];
     }
+    DG_TRY(coop_check(c));
     if (h[0]) {
         TK(c, "k_sort_warp", k_sort_warp<<<grid_for(h[0] * 32), kBlock, 0, st>>>(keys, off, s.bin_list, (int)h[0]));
     }
@@ -511,7 +518,7 @@ dgec_status sort_segments(Ctx *c, int64_t V, unsigned long long *keys, const int
         if (hb == 0) hb = 1;
         DG_TRY(radix_sort(c, rb2, tot, 0, hb, s.radix, &in_b));
         unsigned long long *hub_of = in_b ? v1o : v1, *key_of = in_b ? k1o : k1;
-        TK(c, "k_hub_scatter", k_hub_scatter<<<grid_for(tot, kBlock, kStreamCap), kBlock, 0, st>>>(hub_of, key_of, tot, off, hl, hstart,
+        TK(c, "k_hub_scatter", k_hub_scatter<<<grid_for(tot, kBlock, kStreamCap), kBlock, 0, st>>>(c->stop(), hub_of, key_of, tot, off, hl, hstart,
                                                                        keys));
     }
     return DGEC_OK;
@@ -577,7 +584,7 @@ dgec_status stage_csr(Ctx *c, Problem &p, Csr &o, void *scratch) {
         bool in_b;
         DG_TRY(radix_sort(c, RadixBuffers{s.mk, s.mk2, s.mk + E, s.mk2 + E}, E, p.idbits, p.idbits + p.tbits,
                           s.radix, &in_b));
-        TK(c, "k_rank_init", k_rank_init<<<gEE, kBlock, 0, st>>>(in_b ? s.mk2 : s.mk, in_b ? s.mk2 + E : s.mk + E, E,
+        TK(c, "k_rank_init", k_rank_init<<<gEE, kBlock, 0, st>>>(c->stop(), in_b ? s.mk2 : s.mk, in_b ? s.mk2 + E : s.mk + E, E,
                                                                 p.tmin, p.idbits, o.orig_of, o.rank_of, o.isrc, o.idst,
                                                                 o.it, p.tbits <= 32 ? nullptr : s.te));
     } else {
@@ -586,7 +593,7 @@ dgec_status stage_csr(Ctx *c, Problem &p, Csr &o, void *scratch) {
         bool in_b;
         DG_TRY(radix_sort(c, RadixBuffers{s.mk, s.mk2, s.mk + E, s.mk2 + E}, E, 0, p.tbits, s.radix, &in_b));
         TK(c, "k_rank_init_kv", k_rank_init_kv<<<gEE, kBlock, 0, st>>>(
-                                    in_b ? s.mk2 : s.mk, in_b ? s.mk2 + E : s.mk + E, E, p.tmin, p.src, p.dst,
+                           c->stop(), in_b ? s.mk2 : s.mk, in_b ? s.mk2 + E : s.mk + E, E, p.tmin, p.src, p.dst,
                                     p.egraph, p.voff, p.G, o.orig_of, o.rank_of, o.isrc, o.idst, o.it, s.te));
     }
     // time groups of the r order, then the incidence items in (t, in-before-out, r) order
@@ -604,15 +611,15 @@ dgec_status stage_csr(Ctx *c, Problem &p, Csr &o, void *scratch) {
                       cb + vbits, s.radix, &in_b));
     const unsigned long long *key = in_b ? s.mk2 : s.mk;
     const unsigned long long *mval = carry ? (in_b ? s.mv2 : s.mv) : nullptr;
-    TK(c, "k_voffsets", k_voffsets<<<grid_for(2 * E + 1, kBlock, kStreamCap), kBlock, 0, st>>>(key, 2 * E, V, cb, s.moff));
+    TK(c, "k_voffsets", k_voffsets<<<grid_for(2 * E + 1, kBlock, kStreamCap), kBlock, 0, st>>>(c->stop(), key, 2 * E, V, cb, s.moff));
     DG_TRY((device_scan<long long, SumI64, LoadOutBit, StoreI32>(c, LoadOutBit{key, 2 * E}, StoreI32{s.oidx},
                                                                  2 * E + 1, SumI64{}, 0ll, false, s.scan_tmp)));
-    TK(c, "k_moff_split", k_moff_split<<<grid_for(V + 1, kBlock, kStreamCap), kBlock, 0, st>>>(s.moff, s.oidx, V, o.out_off,
+    TK(c, "k_moff_split", k_moff_split<<<grid_for(V + 1, kBlock, kStreamCap), kBlock, 0, st>>>(c->stop(), s.moff, s.oidx, V, o.out_off,
                                                                                         o.in_off));
     // the per-edge kNN forms read the window places by r; the list-order form and the skeleton do not
     const bool rk = p.knn && p.knn_form != 2;
     TK(c, "k_munpack", k_munpack<<<grid_for(2 * E, kBlock, kStreamCap), kBlock, 0, st>>>(
-                           key, mval, p.tmin, 2 * E, cb, s.moff, s.oidx, o.out_off, s.te, o.out_t, o.out_id,
+                           c->stop(), key, mval, p.tmin, 2 * E, cb, s.moff, s.oidx, o.out_off, s.te, o.out_t, o.out_id,
                            o.out_r, rk ? o.outrk : nullptr,
                            o.pos_out, o.in_t, o.in_id, o.in_r, o.pos_in, s.in_head, rk ? o.inrk : nullptr, o.in_va,
                            o.out_vb, o.out_key, o.in_key));

@@ -77,8 +77,9 @@ __global__ void k_d_order_keys(const int32_t *ru, int64_t n, int sbits, unsigned
          x += (int64_t)gridDim.x * blockDim.x)
         k[x] = ((unsigned long long)(unsigned)ru[x] << sbits) | (unsigned long long)x;
 }
-__global__ void k_d_order_act(const unsigned long long *k, int64_t n, int sbits, const int32_t *rv,
+__global__ void k_d_order_act(const unsigned *stop, const unsigned long long *k, int64_t n, int sbits, const int32_t *rv,
                               int32_t *act, int32_t *ecu, int32_t *ecv) {
+    if (stopped(stop)) return;
     const unsigned long long smask = (1ull << sbits) - 1ull;
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n;
          j += (int64_t)gridDim.x * blockDim.x) {
@@ -136,7 +137,7 @@ struct DArgs {
     SegVal *cagg;        // [CTAs] chain sum over each CTA's chunk
     int *state;          // [0] rounds run, [1] error, [2] live edges (accepted ones after a large round's emit)
     int max_rounds;
-    unsigned *bar, *err;
+    BarRef bar;
 };
 
 // The last rounds (k_d_tail) take over at this many live edges; above
@@ -708,7 +709,10 @@ __device__ __forceinline__ void d_rows(const DArgs &a, const DRound &w, const un
 // registers allow.
 #define D_KERNEL(name, call)                                                                          \
     __global__ void __launch_bounds__(kSThreads, 2) k_d_##name(const __grid_constant__ DArgs a,       \
-                                                               const __grid_constant__ DRound w) { call; }
+                                                               const __grid_constant__ DRound w) { \
+        if (stopped(a.bar.word + 2)) return;                                                              \
+        call;                                                                                             \
+    }
 D_KERNEL(bid, d_bid(a, w))
 D_KERNEL(ptr, d_ptr(a, w))
 D_KERNEL(jump, d_jump(a, w))
@@ -720,20 +724,23 @@ D_KERNEL(small, d_small(a, w, w.nsmall))
 #undef D_KERNEL
 __global__ void __launch_bounds__(kSThreads, 2) k_d_chain(const __grid_constant__ DArgs a, const __grid_constant__ DRound w,
                                                        const unsigned long long *key, const unsigned long long *val) {
+    if (stopped(a.bar.word + 2)) return;
     d_chain(a, w, key, val);
 }
 __global__ void __launch_bounds__(kSThreads, 2) k_d_rows(const __grid_constant__ DArgs a, const __grid_constant__ DRound w,
-                                                      const unsigned long long *key, const unsigned long long *val) {
+                                                       const unsigned long long *key, const unsigned long long *val) {
+    if (stopped(a.bar.word + 2)) return;
     d_rows(a, w, key, val);
 }
 
 // What d_jump left of a large round's walks: nothing unless one was cut.
 __global__ void __launch_bounds__(kSThreads, 2) k_d_settle(const __grid_constant__ DArgs a, const __grid_constant__ DRound w) {
     if (a.tot[4] == 0) return;  // the same for every CTA: written before this launch
-    GridBar bar(a.bar, a.err);
+    GridBar bar(a.bar);
+    if (bar.stopped()) return;
     const JumpEnd e = d_settle(a, w, bar);
     if (e == kJumpBarrier) return;
-    if (e == kJumpBound && threadIdx.x == 0) *(volatile unsigned *)a.err = 1u;
+    if (e == kJumpBound && threadIdx.x == 0) bar.stop(kStopJump);
     bar.finish();
 }
 
@@ -763,7 +770,8 @@ __device__ __noinline__ bool dc_sort(const DArgs &a, int64_t n, int bits, int mo
 // are live.
 __global__ void __launch_bounds__(kSThreads, 2) k_d_rounds(const __grid_constant__ DArgs a, const __grid_constant__ DRound w0) {
     extern __shared__ __align__(16) unsigned long long d_sm[];
-    GridBar bar(a.bar, a.err);
+    GridBar bar(a.bar);
+    if (bar.stopped()) return;
     DRound w = w0;
     w.G = gridDim.x;
     int error = 0;
@@ -784,8 +792,8 @@ __global__ void __launch_bounds__(kSThreads, 2) k_d_rounds(const __grid_constant
             const JumpEnd e = dc_settle(a, w, bar);
             if (e == kJumpBarrier) return;
             if (e == kJumpBound) {
-                error = 3;
-                break;
+                if (threadIdx.x == 0) bar.stop(kStopJump);
+                return;
             }
         }
         dc_tau(a, w);
@@ -858,7 +866,7 @@ __global__ void __launch_bounds__(kTailThreads) k_d_tail(const __grid_constant__
     __shared__ int s_nlab, s_nacc, s_nkeep;
     __shared__ SegVal s_warp[kTailThreads / 32];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    if (a.state[1]) return;  // an error of the rounds before
+    if (stopped(a.bar.word + 2) || a.state[1] || a.state[2] > kTailMax) return;  // the rounds before did not end
     int na = a.state[2];
     int round = a.state[0];
     if (na == 0) return;
@@ -1187,7 +1195,7 @@ dgec_status stage_dendro(Ctx *c, const Problem &p, const Csr &g, const Msf &m, D
         TK(c, "k_d_order_keys", k_d_order_keys<<<gn, kBlock, 0, st>>>(m.ru, n, sbits, s.k1));
         bool in_b;
         DG_TRY(radix_sort(c, RadixBuffers{s.k1, s.k2, nullptr, nullptr}, n, sbits, sbits + lb, s.radix, &in_b));
-        TK(c, "k_d_order_act", k_d_order_act<<<gn, kBlock, 0, st>>>(in_b ? s.k2 : s.k1, n, sbits, m.rv, s.act,
+        TK(c, "k_d_order_act", k_d_order_act<<<gn, kBlock, 0, st>>>(c->stop(), in_b ? s.k2 : s.k1, n, sbits, m.rv, s.act,
                                                                s.ecu, s.ecv));
     }
     if (n > 0) {
@@ -1195,7 +1203,7 @@ dgec_status stage_dendro(Ctx *c, const Problem &p, const Csr &g, const Msf &m, D
                 s.gcnt, s.gseg, s.slot, s.segA, s.segB, s.segC, (unsigned long long *)(s.state + 4), s.kids, s.contrib,
                 s.row, o.parent,
                 sort_args(c, RadixBuffers{s.k1, s.k2, s.v1, s.v2}, n, 0, lb + sbits, s.radix, E), s.ccnt, s.cagg,
-                s.state, 1 << 16, c->bar, c->bar_err};
+                s.state, 1 << 16, c->bar};
         DRound w{0, 0, kStampTop, n, 0, 0, false};
         CU_TRY(c, cudaMemsetAsync(s.state, 0, sizeof(int) * 20, st));
         CU_TRY(c, cudaMemsetAsync(s.gcnt, 0, sizeof(int) * E, st));
@@ -1215,6 +1223,7 @@ dgec_status stage_dendro(Ctx *c, const Problem &p, const Csr &g, const Msf &m, D
             TK(c, "k_d_gjump", k_d_jump<<<wide, kSThreads, 0, st>>>(d, w));
             DG_TRY(coop_grid(c, kCoopDJump, (const void *)k_d_settle, kSThreads, 0, &w.G));
             {
+                d.bar = c->next_bar();
                 void *args[] = {&d, &w};
                 cudaError_t e;
                 TK(c, "k_d_settle", e = cudaLaunchCooperativeKernel((const void *)k_d_settle, dim3((unsigned)w.G),
@@ -1255,6 +1264,7 @@ dgec_status stage_dendro(Ctx *c, const Problem &p, const Csr &g, const Msf &m, D
             int grid = 1;
             DG_TRY(coop_grid(c, kCoopDendro, (const void *)k_d_rounds, kSThreads, smem, &grid));
             grid = w.na > kTailMax ? (int)std::min<int64_t>(std::min(grid, kMidCtas), cdiv(w.na, kMidEdges)) : 1;
+            d.bar = c->next_bar();
             void *args[] = {&d, &w};
             cudaError_t e;
             TK(c, "k_d_rounds", e = cudaLaunchCooperativeKernel((const void *)k_d_rounds, dim3((unsigned)grid),
@@ -1272,7 +1282,6 @@ dgec_status stage_dendro(Ctx *c, const Problem &p, const Csr &g, const Msf &m, D
         DG_TRY(read_counters(c, (const int64_t *)s.state, 1, &ts));
         const int err = (int)(ts >> 32);
         if (err == 1) return set_err(c, DGEC_ERR_TIMEOUT, "dendrogram rounds exceeded %d", 1 << 16);
-        if (err == 3) return set_err(c, DGEC_ERR_TIMEOUT, "dendrogram pointers not settled in %d rounds", kJumpRounds);
         if (err) return set_err(c, DGEC_ERR_INTERNAL, "dendrogram round accepted no edge");
         o.rounds = (int)(ts & 0xffffffff);
     }

@@ -385,7 +385,7 @@ dgec_status dgec_create(dgec_ctx **out, int device) {
     cudaError_t e = cudaSetDevice(device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device);
     if (e == cudaSuccess) e = cudaMallocHost((void **)&c->h_pinned, 4096);
-    if (e == cudaSuccess) c->bar_err = (unsigned *)(c->h_pinned + 511);  // last word pair of the 4 KB, read and written by kernels too
+    if (e == cudaSuccess) c->bar.err = (unsigned *)(c->h_pinned + 511);  // last word pair of the 4 KB, written by kernels
     c->kt = new (std::nothrow) KernelTimer();
     if (e != cudaSuccess || !c->kt) {
         if (c->h_pinned) cudaFreeHost(c->h_pinned);
@@ -475,6 +475,15 @@ dgec_status dgec_get_launch_config(const dgec_ctx *x, dgec_launch_config *cfg) {
     cfg->knn_block = x->c.knn_block;
     cfg->stream_ctas = (int32_t)x->c.stream_ctas;
     cfg->knn_packed = x->c.knn_packed;
+    return DGEC_OK;
+}
+
+dgec_status dgec_set_limits(dgec_ctx *x, const dgec_limits *limits) {
+    if (!x || !limits) return DGEC_ERR_INVALID_ARG;
+    if (limits->barrier_polls < 0 || limits->barrier_from < 0)
+        return set_err(&x->c, DGEC_ERR_INVALID_ARG, "limits must not be negative");
+    x->c.bar_polls = (unsigned)limits->barrier_polls;
+    x->c.bar_from = limits->barrier_from;
     return DGEC_OK;
 }
 

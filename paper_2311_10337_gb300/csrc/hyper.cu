@@ -83,8 +83,9 @@ __global__ void k_h_pack(const int64_t *t, int64_t E, long long tmin, int idbits
         k[e] = ((unsigned long long)(t[e] - tmin) << idbits) | (unsigned long long)e;
 }
 
-__global__ void k_h_rank_init(const unsigned long long *ks, int64_t E, long long tmin, int idbits,
+__global__ void k_h_rank_init(const unsigned *stop, const unsigned long long *ks, int64_t E, long long tmin, int idbits,
                               int32_t *orig_of, int32_t *rank_of, int64_t *it) {
+    if (stopped(stop)) return;
     const unsigned long long mask = (1ull << idbits) - 1ull;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < E;
          r += (int64_t)gridDim.x * blockDim.x) {
@@ -241,8 +242,9 @@ __global__ void k_h_uflag(const unsigned long long *lk, int64_t L, int *flag) {
         flag[x] = x < L && lk[x] != ~0ull && (x == 0 || lk[x] != lk[x - 1]);
 }
 
-__global__ void k_h_links(const unsigned long long *lk, int64_t L, const int *flag, const long long *pos,
+__global__ void k_h_links(const unsigned *stop, const unsigned long long *lk, int64_t L, const int *flag, const long long *pos,
                           int idbits, const int32_t *orig_of, const int64_t *it, Skel sk) {
+    if (stopped(stop)) return;
     const unsigned long long mask = (1ull << idbits) - 1ull;
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < L;
          x += (int64_t)gridDim.x * blockDim.x) {
@@ -374,7 +376,7 @@ dgec_status stage_hyper(Ctx *c, Problem &p, const HyperProblem &h, Csr &g, Hyper
         bool in_b;
         DG_TRY(radix_sort(c, RadixBuffers{s.k1, s.k2, nullptr, nullptr}, E, p.idbits, p.idbits + p.tbits, s.radix,
                           &in_b));
-        TK(c, "k_h_rank_init", k_h_rank_init<<<gE, kBlock, 0, st>>>(in_b ? s.k2 : s.k1, E, p.tmin, p.idbits,
+        TK(c, "k_h_rank_init", k_h_rank_init<<<gE, kBlock, 0, st>>>(c->stop(), in_b ? s.k2 : s.k1, E, p.tmin, p.idbits,
                                                                    g.orig_of, g.rank_of, g.it));
     }
     DG_TRY(build_lists(c, h, h.s_off, h.s_vert, h.Ms, s.deg_s, g, p.idbits, S, s));
@@ -404,7 +406,7 @@ dgec_status stage_hyper(Ctx *c, Problem &p, const HyperProblem &h, Csr &g, Hyper
     const unsigned long long *lk = in_b ? s.k2 : s.k1;
     TK(c, "k_h_uflag", k_h_uflag<<<grid_for(L + 1, kBlock, kStreamCap), kBlock, 0, st>>>(lk, L, s.flag));
     DG_TRY(exclusive_scan_i32(c, s.flag, s.pos, L + 1, s.scan_tmp));
-    TK(c, "k_h_links", k_h_links<<<grid_for(L, kBlock, kStreamCap), kBlock, 0, st>>>(lk, L, s.flag, s.pos, p.idbits,
+    TK(c, "k_h_links", k_h_links<<<grid_for(L, kBlock, kStreamCap), kBlock, 0, st>>>(c->stop(), lk, L, s.flag, s.pos, p.idbits,
                                                                                g.orig_of, g.it, sk));
     int64_t n;
     DG_TRY(read_counters(c, (const int64_t *)(s.pos + L), 1, &n));

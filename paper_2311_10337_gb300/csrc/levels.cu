@@ -58,7 +58,8 @@ __global__ void k_lv_keys(const int64_t *w, const int32_t *ru, const int32_t *rv
 }
 
 // boff[b] = first sorted position with bucket >= b, for b in [0, q + 1].
-__global__ void k_lv_bounds(const unsigned long long *key, int64_t n, int q, int64_t *boff) {
+__global__ void k_lv_bounds(const unsigned *stop, const unsigned long long *key, int64_t n, int q, int64_t *boff) {
+    if (stopped(stop)) return;
     for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s <= n;
          s += (int64_t)gridDim.x * blockDim.x) {
         int b = s < n ? (int)key[s] : q + 1;
@@ -109,10 +110,11 @@ __device__ __forceinline__ int uf_root(int32_t *par, int x) {
 // Unite the bucket of level l. Roots hooked here get merge_level = l (under
 // their original id) and go to the level's list (one reservation per CTA);
 // the CTA-uniform loop keeps every thread in the reservation.
-__global__ void __launch_bounds__(kBlock) k_lv_hook(const unsigned long long *val, const int64_t *boff,
+__global__ void __launch_bounds__(kBlock) k_lv_hook(const unsigned *stop, const unsigned long long *val, const int64_t *boff,
                                                     int l, const int32_t *orig_of, int32_t *par,
                                                     int32_t *mlevel, int32_t *list, unsigned long long *tot,
                                                     int *err) {
+    if (stopped(stop)) return;
     const int64_t lo = boff[l], hi = boff[l + 1];
     for (int64_t base = lo + (int64_t)blockIdx.x * blockDim.x; base < hi;
          base += (int64_t)gridDim.x * blockDim.x) {
@@ -203,8 +205,9 @@ __global__ void k_lv_row_keys(int64_t E, const int32_t *mlevel, unsigned long lo
         key[x] = ((unsigned long long)(mlevel[x] + 1) << 32) | (unsigned long long)x;
 }
 
-__global__ void k_lv_rows(const unsigned long long *key, int64_t first, int64_t n, const int32_t *mparent,
+__global__ void k_lv_rows(const unsigned *stop, const unsigned long long *key, int64_t first, int64_t n, const int32_t *mparent,
                           const int32_t *rank_of, const int64_t *omega, Msf m) {
+    if (stopped(stop)) return;
     for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n;
          s += (int64_t)gridDim.x * blockDim.x) {
         const unsigned long long k = key[first + s];
@@ -291,11 +294,11 @@ dgec_status stage_levels(Ctx *c, const Problem &p, const Csr &g, const Skel &sk,
         bool in_b;
         DG_TRY(radix_sort(c, RadixBuffers{s.k1, s.k2, s.v1, s.v2}, n, 0, bits_for(q), s.radix, &in_b));
         const unsigned long long *key = in_b ? s.k2 : s.k1, *val = in_b ? s.v2 : s.v1;
-        TK(c, "k_lv_bounds", k_lv_bounds<<<grid_for(n + 1, kBlock, kStreamCap), kBlock, 0, st>>>(key, n, q, s.boff));
+        TK(c, "k_lv_bounds", k_lv_bounds<<<grid_for(n + 1, kBlock, kStreamCap), kBlock, 0, st>>>(c->stop(), key, n, q, s.boff));
         // hook kernels read their bucket bounds on the device: no host round trip per level
         const int gh = c->num_sms * 8;
         for (int l = 0; l < q; l++) {
-            TK(c, "k_lv_hook", k_lv_hook<<<gh, kBlock, 0, st>>>(val, s.boff, l, g.orig_of, s.par, o.mlevel, s.list,
+            TK(c, "k_lv_hook", k_lv_hook<<<gh, kBlock, 0, st>>>(c->stop(), val, s.boff, l, g.orig_of, s.par, o.mlevel, s.list,
                                                                s.tot, s.err));
             TK(c, "k_lv_parent", k_lv_parent<<<gh, kBlock, 0, st>>>(s.list, s.snap, s.tot, l, g.orig_of, s.par,
                                                                    o.mparent, s.err));
@@ -337,7 +340,7 @@ dgec_status build_level_rows(Ctx *c, const Problem &p, const Csr &g, Levels &o, 
     DG_TRY(radix_sort(c, RadixBuffers{s.k1, s.k2, nullptr, nullptr}, E, 32, 32 + bits_for(o.q), s.radix, &in_b));
     const unsigned long long *key = in_b ? s.k2 : s.k1;
     TK(c, "k_lv_rows", k_lv_rows<<<grid_for(o.rows.n > 0 ? o.rows.n : 1, kBlock, kStreamCap), kBlock, 0, st>>>(
-                           key, E - o.rows.n, o.rows.n, o.mparent, g.rank_of, o.omega, o.rows));
+                           c->stop(), key, E - o.rows.n, o.rows.n, o.mparent, g.rank_of, o.omega, o.rows));
     return DGEC_OK;
 }
 

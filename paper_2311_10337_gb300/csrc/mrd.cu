@@ -48,8 +48,9 @@ __device__ __forceinline__ long long mrd_weight(unsigned long long kk, int idbit
     return m;
 }
 
-__global__ void k_mrd_flag(const unsigned long long *key, int64_t L, int idbits, const int32_t *orig_of,
+__global__ void k_mrd_flag(const unsigned *stop, const unsigned long long *key, int64_t L, int idbits, const int32_t *orig_of,
                            const int64_t *it, const int64_t *core, int *flag) {
+    if (stopped(stop)) return;
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x <= L;
          x += (int64_t)gridDim.x * blockDim.x) {
         int f = 0;
@@ -61,8 +62,9 @@ __global__ void k_mrd_flag(const unsigned long long *key, int64_t L, int idbits,
     }
 }
 
-__global__ void k_mrd_emit(const unsigned long long *key, int64_t L, const int *flag, const long long *pos,
+__global__ void k_mrd_emit(const unsigned *stop, const unsigned long long *key, int64_t L, const int *flag, const long long *pos,
                            int idbits, const int32_t *orig_of, const int64_t *it, const int64_t *core, Skel h) {
+    if (stopped(stop)) return;
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < L;
          x += (int64_t)gridDim.x * blockDim.x) {
         if (!flag[x]) continue;
@@ -126,10 +128,10 @@ dgec_status stage_mrd(Ctx *c, const Problem &p, const Csr &g, const Skel &sk, Sk
     bool in_b;
     DG_TRY(radix_sort(c, RadixBuffers{s.k1, s.k2, nullptr, nullptr}, L, 0, 2 * p.idbits, s.radix, &in_b));
     const unsigned long long *key = in_b ? s.k2 : s.k1;
-    TK(c, "k_mrd_flag", k_mrd_flag<<<grid_for(L + 1, kBlock, kStreamCap), kBlock, 0, st>>>(key, L, p.idbits, g.orig_of,
+    TK(c, "k_mrd_flag", k_mrd_flag<<<grid_for(L + 1, kBlock, kStreamCap), kBlock, 0, st>>>(c->stop(), key, L, p.idbits, g.orig_of,
                                                                                     g.it, sk.core, s.flag));
     DG_TRY(exclusive_scan_i32(c, s.flag, s.pos, L + 1, s.scan_tmp));
-    TK(c, "k_mrd_emit", k_mrd_emit<<<gL, kBlock, 0, st>>>(key, L, s.flag, s.pos, p.idbits, g.orig_of, g.it, sk.core,
+    TK(c, "k_mrd_emit", k_mrd_emit<<<gL, kBlock, 0, st>>>(c->stop(), key, L, s.flag, s.pos, p.idbits, g.orig_of, g.it, sk.core,
                                                          h));
     int64_t n;
     DG_TRY(read_counters(c, (const int64_t *)(s.pos + L), 1, &n));

@@ -376,12 +376,13 @@ struct RootItem {
 // Jumping rounds for the walks that were cut (cut[1 .. 3]: their flags): nothing
 // to do unless one was.
 __global__ void __launch_bounds__(kBlock) k_m_settle(const int32_t *roots, int64_t nr, int32_t *par, unsigned long long *cut,
-                                                     unsigned *barw, unsigned *err) {
+                                                     BarRef ref) {
     if (cut[0] == 0) return;  // the same for every CTA: written before this launch
-    GridBar bar(barw, err);
+    GridBar bar(ref);
+    if (bar.stopped()) return;
     const JumpEnd e = jump_rounds(bar, nr, RootItem{roots}, par, cut + 1);
     if (e == kJumpBarrier) return;
-    if (e == kJumpBound && threadIdx.x == 0) *(volatile unsigned *)err = 1u;
+    if (e == kJumpBound && threadIdx.x == 0) bar.stop(kStopJump);
     bar.finish();
 }
 
@@ -447,7 +448,7 @@ struct MsfArgs {
                               // [4] forest edges, [5] error, [6] a walk was cut; if so [7] rounds begun, [8] the
                               // last one's live edges, [9] next roots; all but [4] zeroed before
     int ib, lbits;            // bits of an original id, of the label in a key (0: none)
-    unsigned *bar, *err;
+    BarRef bar;
 };
 
 __device__ __forceinline__ u128 as_u128(ulonglong2 x) { return ((u128)x.y << 64) | x.x; }
@@ -546,7 +547,8 @@ __device__ __forceinline__ int new_root(int32_t *par, int x, unsigned long long 
 // 0.65 ms for the last rounds of 20M edges, for the registers).
 constexpr int kRes = 1;          // items a thread handles between slot reservations (20,000 edges: 0.15 ms at 1, 0.19 at 2, 0.34 at 4)
 __global__ void __launch_bounds__(kBlock, 4) k_m_forest(MsfArgs a) {
-    GridBar bar(a.bar, a.err);
+    GridBar bar(a.bar);
+    if (bar.stopped()) return;
     const int64_t gsize = (int64_t)gridDim.x * blockDim.x, g0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t tile = (int64_t)blockDim.x * kRes;
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
@@ -706,7 +708,7 @@ struct MLabels {
     int64_t *w2;
     unsigned long long *cnt;
     int ib, lbits;
-    unsigned *bar, *err;
+    BarRef bar;
 };
 struct LabelItem {
     const int2 *lab;
@@ -718,10 +720,11 @@ struct LabelItem {
     }
 };
 __global__ void __launch_bounds__(kBlock) k_m_labels(MLabels a) {
-    GridBar bar(a.bar, a.err);
+    GridBar bar(a.bar);
+    if (bar.stopped()) return;
     const JumpEnd e = jump_rounds(bar, 2 * a.n, LabelItem{a.lab, a.ru, a.rv}, a.par, a.cnt + 1);
     if (e == kJumpBarrier) return;
-    if (e == kJumpBound && threadIdx.x == 0) *(volatile unsigned *)a.err = 1u;
+    if (e == kJumpBound && threadIdx.x == 0) bar.stop(kStopJump);
     const unsigned imask = (unsigned)((1ull << a.ib) - 1ull);
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < a.n; base += (int64_t)gridDim.x * blockDim.x) {  // CTA-uniform
         const int64_t x = base + threadIdx.x;
@@ -758,8 +761,9 @@ __global__ void k_pack_uv_idx(const FEdge *fe, int64_t n, int idbits, unsigned l
     }
 }
 
-__global__ void k_gather_w(const FEdge *fe, const unsigned long long *idx, int64_t n,
+__global__ void k_gather_w(const unsigned *stop, const FEdge *fe, const unsigned long long *idx, int64_t n,
                            unsigned long long *k, unsigned long long *val) {
+    if (stopped(stop)) return;
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n;
          x += (int64_t)gridDim.x * blockDim.x) {
         unsigned long long i = idx[x];
@@ -772,15 +776,17 @@ __global__ void k_gather_w(const FEdge *fe, const unsigned long long *idx, int64
 // edge index rides in the low 32 bits, which the passes do not sort on, so
 // the order stays that of the previous sort among equal w (LSD stability)
 // and each pass moves 8 bytes an edge instead of 16.
-__global__ void k_gather_w32(const FEdge *fe, const unsigned long long *idx, int64_t n, unsigned long long *k) {
+__global__ void k_gather_w32(const unsigned *stop, const FEdge *fe, const unsigned long long *idx, int64_t n, unsigned long long *k) {
+    if (stopped(stop)) return;
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n;
          x += (int64_t)gridDim.x * blockDim.x) {
         const unsigned long long i = idx[x];
         k[x] = ((unsigned long long)fe[i].w << 32) | i;
     }
 }
-__global__ void k_gather_graph32(const FEdge *fe, const int32_t *egraph, const unsigned long long *kin, int64_t n,
+__global__ void k_gather_graph32(const unsigned *stop, const FEdge *fe, const int32_t *egraph, const unsigned long long *kin, int64_t n,
                                  unsigned long long *k) {
+    if (stopped(stop)) return;
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n;
          x += (int64_t)gridDim.x * blockDim.x) {
         const unsigned long long i = kin[x] & 0xffffffffull;
@@ -789,8 +795,9 @@ __global__ void k_gather_graph32(const FEdge *fe, const int32_t *egraph, const u
 }
 
 // graph of each sorted forest edge, as a sort key (graph-major output)
-__global__ void k_gather_graph(const FEdge *fe, const int32_t *egraph, const unsigned long long *idx,
+__global__ void k_gather_graph(const unsigned *stop, const FEdge *fe, const int32_t *egraph, const unsigned long long *idx,
                                int64_t n, unsigned long long *k, unsigned long long *val) {
+    if (stopped(stop)) return;
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n;
          x += (int64_t)gridDim.x * blockDim.x) {
         unsigned long long i = idx[x];
@@ -800,8 +807,9 @@ __global__ void k_gather_graph(const FEdge *fe, const int32_t *egraph, const uns
 }
 
 // goff[g] = first row of graph g in the graph-major forest (binary search)
-__global__ void k_graph_offsets(const int32_t *u, const int32_t *egraph, int64_t n, int G,
+__global__ void k_graph_offsets(const unsigned *stop, const int32_t *u, const int32_t *egraph, int64_t n, int G,
                                 int64_t *goff) {
+    if (stopped(stop)) return;
     for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g <= G;
          g += (int64_t)gridDim.x * blockDim.x) {
         int64_t lo = 0, hi = n;  // first row whose graph >= g
@@ -817,8 +825,9 @@ __global__ void k_graph_offsets(const int32_t *u, const int32_t *egraph, int64_t
 // one graph: no search (its 20 or more dependent reads take 10 to 18 us)
 __global__ void k_one_offset(int64_t *goff, int64_t n) { goff[1] = n; }
 
-__global__ void k_gather_msf(const unsigned long long *idx, unsigned long long imask, int64_t n, const FEdge *fe,
+__global__ void k_gather_msf(const unsigned *stop, const unsigned long long *idx, unsigned long long imask, int64_t n, const FEdge *fe,
                              int32_t *u, int32_t *v, int32_t *ru, int32_t *rv, int64_t *w) {
+    if (stopped(stop)) return;
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n;
          x += (int64_t)gridDim.x * blockDim.x) {
         FEdge f;
@@ -950,7 +959,8 @@ dgec_status stage_msf(Ctx *c, const Problem &p, const Csr &g, const Skel &sk, Ms
                 int grid = 1;
                 DG_TRY(coop_grid(c, kCoopMJump, (const void *)k_m_settle, kBlock, 0, &grid));
                 unsigned long long *cut = s.cnt;
-                void *args[] = {&roots, &nr, &s.par, &cut, &c->bar, &c->bar_err};
+                BarRef ref = c->next_bar();
+                void *args[] = {&roots, &nr, &s.par, &cut, &ref};
                 cudaError_t e;
                 TK(c, "k_m_settle", e = cudaLaunchCooperativeKernel((const void *)k_m_settle,
                                                                     dim3((unsigned)std::min(gr, grid)), dim3(kBlock), args,
@@ -985,7 +995,7 @@ dgec_status stage_msf(Ctx *c, const Problem &p, const Csr &g, const Skel &sk, Ms
         // the kernel's first filter writes lb/kb: not the side its edges come from
         const LiveSide &in = s.side[which ^ 1], &out = s.side[which];
         MsfArgs f{nr, n, roots0, ccu, ccv, cu, cv, cw, g.rank_of, s.par, roots0 ? roots2 : roots, roots0 ? roots : roots2,
-                  s.bp, s.slot, s.slot2, in.lab, out.lab, in.key, out.key, s.fe, s.cnt, p.idbits, lbits, c->bar, c->bar_err};
+                  s.bp, s.slot, s.slot2, in.lab, out.lab, in.key, out.key, s.fe, s.cnt, p.idbits, lbits, c->next_bar()};
         int grid = 1;
         DG_TRY(coop_grid(c, kCoopMsf, (const void *)k_m_forest, kBlock, 0, &grid));
         const int64_t want = cdiv(n > nr ? n : nr, kBlock * kRes);
@@ -1009,7 +1019,7 @@ dgec_status stage_msf(Ctx *c, const Problem &p, const Csr &g, const Skel &sk, Ms
         DG_TRY(coop_grid(c, kCoopMLabels, (const void *)k_m_labels, kBlock, 0, &grid));
         DG_TRY(coop_launch(c, "k_m_labels", (const void *)k_m_labels, (int)std::min<int64_t>(grid, cdiv(n, kBlock)), kBlock, 0,
                            MLabels{n, round ? from.lab : nullptr, from.key, ccu, ccv, cu, cv, cw, s.par, to.cu, to.cv, to.u,
-                                   to.v, to.w, s.cnt, p.idbits, lbits, c->bar, c->bar_err}));
+                                   to.v, to.w, s.cnt, p.idbits, lbits, c->next_bar()}));
         DG_TRY(read_counters(c, (const int64_t *)s.cnt, 1, &n));
         CU_TRY(c, cudaMemsetAsync(s.cnt, 0, 4 * sizeof(unsigned long long), st));
         ccu = to.cu;
@@ -1032,26 +1042,26 @@ dgec_status stage_msf(Ctx *c, const Problem &p, const Csr &g, const Skel &sk, Ms
                       s.radix, &in_b));
     if (in_b) cur = 1 - cur;
     if (p.tbits <= 32) {
-        TK(c, "k_gather_w", k_gather_w32<<<gm, kBlock, 0, st>>>(s.fe, Vb[cur], m, K[1 - cur]));
+        TK(c, "k_gather_w", k_gather_w32<<<gm, kBlock, 0, st>>>(c->stop(), s.fe, Vb[cur], m, K[1 - cur]));
         cur = 1 - cur;
         DG_TRY(radix_sort(c, RadixBuffers{K[cur], K[1 - cur], nullptr, nullptr}, m, 32,
                           32 + (p.tbits > 0 ? p.tbits : 1), s.radix, &in_b));
         if (in_b) cur = 1 - cur;
         if (p.G > 1) {
-            TK(c, "k_gather_graph", k_gather_graph32<<<gm, kBlock, 0, st>>>(s.fe, p.egraph, K[cur], m, K[1 - cur]));
+            TK(c, "k_gather_graph", k_gather_graph32<<<gm, kBlock, 0, st>>>(c->stop(), s.fe, p.egraph, K[cur], m, K[1 - cur]));
             cur = 1 - cur;
             DG_TRY(radix_sort(c, RadixBuffers{K[cur], K[1 - cur], nullptr, nullptr}, m, 32,
                               32 + bits_for((uint64_t)(p.G - 1)), s.radix, &in_b));
             if (in_b) cur = 1 - cur;
         }
     } else {
-    TK(c, "k_gather_w", k_gather_w<<<gm, kBlock, 0, st>>>(s.fe, Vb[cur], m, K[1 - cur], Vb[1 - cur]));
+    TK(c, "k_gather_w", k_gather_w<<<gm, kBlock, 0, st>>>(c->stop(), s.fe, Vb[cur], m, K[1 - cur], Vb[1 - cur]));
     cur = 1 - cur;
     DG_TRY(radix_sort(c, RadixBuffers{K[cur], K[1 - cur], Vb[cur], Vb[1 - cur]}, m, 0,
                       p.tbits > 0 ? p.tbits : 1, s.radix, &in_b));
     if (in_b) cur = 1 - cur;
     if (p.G > 1) {
-        TK(c, "k_gather_graph", k_gather_graph<<<gm, kBlock, 0, st>>>(s.fe, p.egraph, Vb[cur], m, K[1 - cur],
+        TK(c, "k_gather_graph", k_gather_graph<<<gm, kBlock, 0, st>>>(c->stop(), s.fe, p.egraph, Vb[cur], m, K[1 - cur],
                                                                      Vb[1 - cur]));
         cur = 1 - cur;
         DG_TRY(radix_sort(c, RadixBuffers{K[cur], K[1 - cur], Vb[cur], Vb[1 - cur]}, m, 0,
@@ -1061,10 +1071,10 @@ dgec_status stage_msf(Ctx *c, const Problem &p, const Csr &g, const Skel &sk, Ms
     }
     const bool low32 = p.tbits <= 32;  // the index is the sorted key's low word
     const unsigned long long *fin = low32 ? K[cur] : Vb[cur];
-    TK(c, "k_gather_msf", k_gather_msf<<<gm, kBlock, 0, st>>>(fin, low32 ? 0xffffffffull : ~0ull, m, s.fe, o.u,
+    TK(c, "k_gather_msf", k_gather_msf<<<gm, kBlock, 0, st>>>(c->stop(), fin, low32 ? 0xffffffffull : ~0ull, m, s.fe, o.u,
                                                               o.v, o.ru, o.rv, o.w));
     if (p.G == 1) TK(c, "k_graph_offsets", k_one_offset<<<1, 1, 0, st>>>(o.goff, m));
-    else TK(c, "k_graph_offsets", k_graph_offsets<<<grid_for(p.G + 1), kBlock, 0, st>>>(o.u, p.egraph, m, p.G, o.goff));
+    else TK(c, "k_graph_offsets", k_graph_offsets<<<grid_for(p.G + 1), kBlock, 0, st>>>(c->stop(), o.u, p.egraph, m, p.G, o.goff));
     return DGEC_OK;
 }
 

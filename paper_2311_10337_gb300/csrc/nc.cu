@@ -44,8 +44,9 @@ __global__ void k_nc_flag(const unsigned long long *key, int64_t L, int *flag) {
         flag[x] = x < L && key[x] != ~0ull && (x == 0 || key[x] != key[x - 1]);
 }
 
-__global__ void k_nc_emit(const unsigned long long *key, int64_t L, const int *flag, const long long *pos, int idbits,
+__global__ void k_nc_emit(const unsigned *stop, const unsigned long long *key, int64_t L, const int *flag, const long long *pos, int idbits,
                           const int32_t *rank_of, const int64_t *t, Skel h) {
+    if (stopped(stop)) return;
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < L;
          x += (int64_t)gridDim.x * blockDim.x) {
         if (!flag[x]) continue;
@@ -168,7 +169,7 @@ dgec_status stage_nc(Ctx *c, const Problem &p, const Csr &g, const Skel &s1, con
     const unsigned long long *key = in_b ? s.k2 : s.k1;
     TK(c, "k_nc_flag", k_nc_flag<<<grid_for(L + 1, kBlock, kStreamCap), kBlock, 0, st>>>(key, L, s.flag));
     DG_TRY(exclusive_scan_i32(c, s.flag, s.pos, L + 1, s.scan_tmp));
-    TK(c, "k_nc_emit", k_nc_emit<<<gL, kBlock, 0, st>>>(key, L, s.flag, s.pos, p.idbits, g.rank_of, p.t, h));
+    TK(c, "k_nc_emit", k_nc_emit<<<gL, kBlock, 0, st>>>(c->stop(), key, L, s.flag, s.pos, p.idbits, g.rank_of, p.t, h));
     int64_t n;
     DG_TRY(read_counters(c, (const int64_t *)(s.pos + L), 1, &n));
     h.n = n;

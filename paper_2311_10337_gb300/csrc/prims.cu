@@ -29,7 +29,8 @@ template <bool VALS>
 __global__ void __launch_bounds__(kSThreads, 2) k_radix_sort(SortArgs a) {
     extern __shared__ __align__(16) unsigned long long sort_sm[];
     const SortSmem s = sort_smem<VALS>(sort_sm);
-    GridBar bar(a.bar, a.err);
+    GridBar bar(a.bar);
+    if (bar.stopped()) return;
     if (sort_run<VALS>(a, a.n, a.begin_bit, a.end_bit, a.most, s, bar)) bar.finish();
 }
 
@@ -42,7 +43,7 @@ SortArgs sort_args(Ctx *c, RadixBuffers buf, int64_t n, int begin_bit, int end_b
     unsigned *w = (unsigned *)scratch;
     const size_t R = (size_t)sort_ranges_of(cap, kSRanges) * kSBins;
     return SortArgs{buf.ka, buf.kb, buf.va, buf.vb, n, begin_bit, end_bit, buf.va && n > kSNarrow ? kSBits - 1 : kSBits,
-                    w, w + R, w + 2 * R, w + 2 * R + kSBins, c->bar, c->bar_err};
+                    w, w + R, w + 2 * R, w + 2 * R + kSBins, c->next_bar()};
 }
 
 template <bool VALS>

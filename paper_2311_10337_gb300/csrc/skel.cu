@@ -61,8 +61,9 @@ struct LinkRec {
 // Type 1, over the in-list slots: the in-edge e at slot x of vertex j (its
 // p_x) links to q_{a_x}, the first out-edge of j not before it. a is
 // nondecreasing along j's in-list, so the partners are read nearly in order.
-__global__ void k_links_in(SkView g, const int2 *in_va, const int64_t *out_t, const int64_t *in_t, int64_t E,
+__global__ void k_links_in(const unsigned *stop, SkView g, const int2 *in_va, const int64_t *out_t, const int64_t *in_t, int64_t E,
                            int64_t dmax, LinkRec *rec) {
+    if (stopped(stop)) return;
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < E;
          x += (int64_t)gridDim.x * blockDim.x) {
         const int2 va = in_va[x];
@@ -83,8 +84,9 @@ __global__ void k_links_in(SkView g, const int2 *in_va, const int64_t *out_t, co
 // Type 2, over the out-list slots: the out-edge e at slot y of vertex i (its
 // q_m, m >= 1) links to p_{b_{m-1} - 1}, where b_{m-1} is the b of the
 // out-edge in slot y - 1; b is nondecreasing along i's out-list.
-__global__ void k_links_out(SkView g, const int2 *out_vb, const int64_t *out_t, const int64_t *in_t,
+__global__ void k_links_out(const unsigned *stop, SkView g, const int2 *out_vb, const int64_t *out_t, const int64_t *in_t,
                             int64_t E, int64_t dmax, LinkRec *rec) {
+    if (stopped(stop)) return;
     for (int64_t y = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; y < E;
          y += (int64_t)gridDim.x * blockDim.x) {
         const int i = out_vb[y].x, e = g.out_id[y];
@@ -109,8 +111,9 @@ struct LoadKeep {
     __device__ __forceinline__ long long operator()(int64_t i) const { return i < n ? rec[i].keep : 0; }
 };
 
-__global__ void k_compact_links(const LinkRec *rec, const long long *pos, int64_t E, const int32_t *orig_of,
+__global__ void k_compact_links(const unsigned *stop, const LinkRec *rec, const long long *pos, int64_t E, const int32_t *orig_of,
                                 int32_t *ru, int32_t *rv, int32_t *u, int32_t *v, int64_t *w) {
+    if (stopped(stop)) return;
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < 2 * E;
          x += (int64_t)gridDim.x * blockDim.x) {
         const LinkRec l = rec[x];
@@ -219,7 +222,7 @@ __device__ __forceinline__ void knn_write(const C (&c)[2 * K], int k, int64_t e0
 }
 
 template <int K>
-__global__ void __launch_bounds__(256) k_knn(const int64_t *t, const int32_t *orig_of, int64_t E,
+__global__ void __launch_bounds__(256) k_knn(const unsigned *stop, const int64_t *t, const int32_t *orig_of, int64_t E,
                                              const int64_t *out_t, const int32_t *out_id,
                                              const int64_t *in_t, const int32_t *in_id,
                                              const int32_t *in_gs, const int4 *outrk, const int2 *inrk,
@@ -227,6 +230,7 @@ __global__ void __launch_bounds__(256) k_knn(const int64_t *t, const int32_t *or
                                              const int32_t *egraph, const int64_t *eoff,
                                              const int32_t *gk, const int64_t *knn_off, int64_t dmax,
                                              int32_t *knn, int64_t *core) {
+    if (stopped(stop)) return;
     constexpr int N = 2 * K;
     // r runs over internal ids (src, dst, t are the r-ordered copies); the
     // neighbour lists are written under the original id, with original ids
@@ -311,7 +315,7 @@ __global__ void __launch_bounds__(256) k_knn(const int64_t *t, const int32_t *or
 // compare a step) and the kernel keeps more warps resident to hide its
 // gathers' latency.
 template <int K>
-__global__ void __launch_bounds__(256, K <= 8 ? 3 : 1) k_knn32(const int64_t *t, long long tmin,
+__global__ void __launch_bounds__(256, K <= 8 ? 3 : 1) k_knn32(const unsigned *stop, const int64_t *t, long long tmin,
                                                const int32_t *orig_of, int64_t E,
                                                const unsigned long long *__restrict__ out_key,
                                                const unsigned long long *__restrict__ in_key,
@@ -320,6 +324,7 @@ __global__ void __launch_bounds__(256, K <= 8 ? 3 : 1) k_knn32(const int64_t *t,
                                                const int32_t *egraph, const int64_t *eoff,
                                                const int32_t *gk, const int64_t *knn_off, int64_t dmax,
                                                int32_t *knn, int64_t *core) {
+    if (stopped(stop)) return;
     constexpr int N = 2 * K;
     constexpr unsigned long long kNone = 0xFFFFFFFFFFFFFFFFull;
     constexpr unsigned long long kLo = 0xFFFFFFFFull;
@@ -403,13 +408,14 @@ __global__ void __launch_bounds__(256, K <= 8 ? 3 : 1) k_knn32(const int64_t *t,
 // The per-edge form above reads both windows at scattered places, several
 // sectors each, and its warps wait on them.
 template <int K>
-__global__ void __launch_bounds__(256) k_knn_pred(int64_t E, const unsigned long long *__restrict__ out_key,
+__global__ void __launch_bounds__(256) k_knn_pred(const unsigned *stop, int64_t E, const unsigned long long *__restrict__ out_key,
                                                   const int2 *__restrict__ out_vb,
                                                   const int64_t *__restrict__ in_off,
                                                   const unsigned long long *__restrict__ in_key,
                                                   const int32_t *__restrict__ in_gs,
                                                   const int32_t *__restrict__ pos_in,
                                                   ulonglong2 *__restrict__ half) {
+    if (stopped(stop)) return;
     constexpr unsigned long long kNone = 0xFFFFFFFFFFFFFFFFull;
     constexpr unsigned long long kLo = 0xFFFFFFFFull;
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < E;
@@ -448,10 +454,12 @@ __global__ void __launch_bounds__(256) k_knn_pred(int64_t E, const unsigned long
 
 template <int K>
 __global__ void __launch_bounds__(256, K <= 8 ? 3 : 1) k_knn_succ(
+    const unsigned *stop,
     int64_t E, const unsigned long long *__restrict__ in_key, const int2 *__restrict__ in_va,
     const int64_t *__restrict__ out_off, const unsigned long long *__restrict__ out_key,
     const ulonglong2 *__restrict__ half, int G, const int32_t *egraph, const int64_t *eoff,
     const int32_t *gk, const int64_t *knn_off, int64_t dmax, int32_t *knn, int64_t *core) {
+    if (stopped(stop)) return;
     constexpr int N = 2 * K;
     constexpr unsigned long long kNone = 0xFFFFFFFFFFFFFFFFull;
     constexpr unsigned long long kLo = 0xFFFFFFFFull;
@@ -547,16 +555,16 @@ dgec_status stage_skeleton(Ctx *c, const Problem &p, const Csr &g, Skel &o, void
     const int kb = c->knn_block;
     int grid = grid_for(E, kb, 1 << 20);
 #define KNN_ARGS                                                                                   \
-    g.it, g.orig_of, E, g.out_t, g.out_id, g.in_t, g.in_id, g.in_gs, g.outrk, g.inrk, p.G, p.egraph, p.eoff, \
+    c->stop(), g.it, g.orig_of, E, g.out_t, g.out_id, g.in_t, g.in_id, g.in_gs, g.outrk, g.inrk, p.G, p.egraph, p.eoff, \
         p.gk, p.knn_off, p.dmax, o.knn, o.core
 #define KNN32_ARGS                                                                                 \
-    g.it, p.tmin, g.orig_of, E, g.out_key, g.in_key, g.in_gs, g.outrk, g.inrk, p.G, p.egraph, p.eoff, p.gk, \
+    c->stop(), g.it, p.tmin, g.orig_of, E, g.out_key, g.in_key, g.in_gs, g.outrk, g.inrk, p.G, p.egraph, p.eoff, p.gk, \
         p.knn_off, p.dmax, o.knn, o.core
     if (p.knn && p.knn_form == 2) {  // packed keys, in list order (two passes)
         const int gl = grid_for(E, kb, 1 << 20);
-#define KNN_PRED_ARGS E, g.out_key, g.out_vb, g.in_off, g.in_key, g.in_gs, g.pos_in, s.half
+#define KNN_PRED_ARGS c->stop(), E, g.out_key, g.out_vb, g.in_off, g.in_key, g.in_gs, g.pos_in, s.half
 #define KNN_SUCC_ARGS \
-    E, g.in_key, g.in_va, g.out_off, g.out_key, s.half, p.G, p.egraph, p.eoff, p.gk, p.knn_off, p.dmax, o.knn, o.core
+    c->stop(), E, g.in_key, g.in_va, g.out_off, g.out_key, s.half, p.G, p.egraph, p.eoff, p.gk, p.knn_off, p.dmax, o.knn, o.core
         switch (knn_kpad(p.k)) {
         case 4:
             TK(c, "k_knn_pred", k_knn_pred<4><<<gl, kb, 0, st>>>(KNN_PRED_ARGS));
@@ -586,13 +594,13 @@ dgec_status stage_skeleton(Ctx *c, const Problem &p, const Csr &g, Skel &o, void
 #undef KNN32_ARGS
     SkView v{g.isrc, g.idst, g.out_off, g.in_off, g.out_r, g.in_r, g.orig_of, g.pos_out, g.pos_in, g.in_va, g.out_vb};
     TK(c, "k_links_in", k_links_in<<<grid_for(E, kBlock, kStreamCap), kBlock, 0, st>>>(
-                            v, g.in_va, g.out_t, g.in_t, E, p.dmax, s.rec));
+                           c->stop(), v, g.in_va, g.out_t, g.in_t, E, p.dmax, s.rec));
     TK(c, "k_links_out", k_links_out<<<grid_for(E, kBlock, kStreamCap), kBlock, 0, st>>>(
-                             v, g.out_vb, g.out_t, g.in_t, E, p.dmax, s.rec));
+                           c->stop(), v, g.out_vb, g.out_t, g.in_t, E, p.dmax, s.rec));
     DG_TRY((device_scan<long long, SumI64, LoadKeep, StorePtr<long long>>(
         c, LoadKeep{s.rec, 2 * E}, StorePtr<long long>{s.pos}, 2 * E + 1, SumI64{}, 0ll, false, s.scan_tmp)));
     TK(c, "k_compact_links", k_compact_links<<<grid_for(2 * E, kBlock, kStreamCap), kBlock, 0, st>>>(
-                                 s.rec, s.pos, E, g.orig_of, o.ru, o.rv, o.u, o.v, o.w));
+                           c->stop(), s.rec, s.pos, E, g.orig_of, o.ru, o.rv, o.u, o.v, o.w));
     int64_t n;
     DG_TRY(read_counters(c, (const int64_t *)(s.pos + 2 * E), 1, &n));
     o.n = n;

@@ -164,7 +164,7 @@ struct SortArgs {
     unsigned *rtot, *rpre;  // [CTAs][digits]: digit counts of each CTA's range of tiles, and those of the ranges before
     unsigned *total;        // [digits]
     unsigned *tile;         // [tiles][digits]: keys of the digit in the range's tiles before
-    unsigned *bar, *err;
+    BarRef bar;
 };
 
 // First places of the calling thread's digits: the keys of smaller digits

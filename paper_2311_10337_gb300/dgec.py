@@ -25,7 +25,7 @@ STATUS = {0: "DGEC_OK", 1: "DGEC_ERR_INVALID_ARG", 2: "DGEC_ERR_VERTEX_RANGE",
 EXPORTS = ["dgec_create", "dgec_destroy", "dgec_last_error", "dgec_status_string",
            "dgec_workspace_size", "dgec_run", "dgec_run_host", "dgec_last_launch_count",
            "dgec_set_kernel_timing", "dgec_kernel_timing", "dgec_stage_timing", "dgec_set_launch_config",
-           "dgec_get_launch_config", "dgec_msf_static",
+           "dgec_get_launch_config", "dgec_set_limits", "dgec_msf_static",
            "dgec_batch_workspace_size", "dgec_run_batch", "dgec_server_create", "dgec_submit",
            "dgec_wait", "dgec_server_lane_capacity", "dgec_server_destroy",
            "dgec_levels_workspace_size", "dgec_run_levels", "dgec_hyper_workspace_size",
@@ -38,6 +38,10 @@ MAX_LEVELS = 64
 class LaunchConfig(ctypes.Structure):
     _fields_ = [("knn_block", ctypes.c_int32), ("stream_ctas", ctypes.c_int32),
                 ("knn_packed", ctypes.c_int32)]
+
+
+class Limits(ctypes.Structure):
+    _fields_ = [("barrier_polls", ctypes.c_int32), ("barrier_from", ctypes.c_int32)]
 
 
 class DgecError(RuntimeError):
@@ -148,6 +152,7 @@ def load(path: str = LIB_PATH):
                                     ctypes.POINTER(ctypes.c_double)]
     L.dgec_set_launch_config.argtypes = [_P, ctypes.POINTER(LaunchConfig)]
     L.dgec_get_launch_config.argtypes = [_P, ctypes.POINTER(LaunchConfig)]
+    L.dgec_set_limits.argtypes = [_P, ctypes.POINTER(Limits)]
     I64A = ctypes.POINTER(ctypes.c_int64)
     I32A = ctypes.POINTER(ctypes.c_int32)
     L.dgec_batch_workspace_size.argtypes = [ctypes.c_int32, I64A, I32A, I32A, I32A,
@@ -339,6 +344,13 @@ class Context:
         c = LaunchConfig()
         self._check(self.L.dgec_get_launch_config(self.h, ctypes.byref(c)))
         return int(c.knn_block), int(c.stream_ctas), int(c.knn_packed)
+
+    def set_limits(self, barrier_polls: int = 1 << 24, barrier_from: int = 0):
+        """Bounds of the waits inside the calls on this context: how often a
+        grid barrier polls before its call ends with DGEC_ERR_TIMEOUT, from
+        the call's cooperative launch `barrier_from` on."""
+        lim = Limits(barrier_polls, barrier_from)
+        self._check(self.L.dgec_set_limits(self.h, ctypes.byref(lim)))
 
     def stage_timing(self) -> list:
         """[(stage name, device ms)] of the last completed call, in order."""
