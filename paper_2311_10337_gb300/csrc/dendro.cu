@@ -21,6 +21,7 @@
 // dendrogram height.
 #include <algorithm>
 
+#include "grids.h"
 #include "sort_dev.cuh"
 #include "stages.cuh"
 
@@ -1128,15 +1129,8 @@ struct DScratch {
     unsigned long long *k1, *k2, *v1, *v2;
     void *radix;
 };
-// CTAs of the middle rounds: one for each 512 live edges, so that a thread
-// has no chain of bids and loads one after another, but at most one an SM (a
-// second CTA on some SMs makes every phase wait for those). 20,000 edges: 0.24
-// ms at one CTA per 4,096 edges, 0.154 so; 317,000: 0.49, 0.51 with 192 CTAs, 0.45 with 152.
-constexpr int kMidEdges = 512, kMidCtas = 152;
-// CTAs the per-CTA counts have room for.
-static int chunk_ctas(int64_t E) {
-    return std::max(sort_ranges_of(E, kSRanges), (int)std::min<int64_t>(cdiv(E, kMidEdges), kMidCtas));
-}
+// CTAs the per-CTA counts have room for, whatever the device.
+static int chunk_room(int64_t E) { return std::max(sort_ranges_of(E, kSRanges), mid_ctas(E, kSRanges, kSRanges)); }
 static DScratch carve_dendro(Arena &a, const Problem &p) {
     DScratch s;
     int64_t E = p.E;
@@ -1162,7 +1156,7 @@ static DScratch carve_dendro(Arena &a, const Problem &p) {
     s.segC = a.take<int2>(E);
     s.kids = a.take<int2>(E);
     s.contrib = a.take<long long>(E);
-    const int64_t ctas = chunk_ctas(E);
+    const int64_t ctas = chunk_room(E);
     s.ccnt = a.take<unsigned>(ctas);
     s.cagg = a.take<SegVal>(ctas);
     s.k1 = a.take<unsigned long long>(E);
@@ -1207,7 +1201,7 @@ dgec_status stage_dendro(Ctx *c, const Problem &p, const Csr &g, const Msf &m, D
         DRound w{0, 0, kStampTop, n, 0, 0, false};
         CU_TRY(c, cudaMemsetAsync(s.state, 0, sizeof(int) * 20, st));
         CU_TRY(c, cudaMemsetAsync(s.gcnt, 0, sizeof(int) * E, st));
-        const int most = chunk_ctas(E);
+        const int most = std::max(sort_ranges_of(E, kSRanges), mid_ctas(E, c->num_sms, kSRanges));
         for (; w.na > kDLarge; w.round++) {
             if (w.round >= d.max_rounds)
                 return set_err(c, DGEC_ERR_TIMEOUT, "dendrogram rounds exceeded %d", d.max_rounds);
@@ -1263,7 +1257,7 @@ dgec_status stage_dendro(Ctx *c, const Problem &p, const Csr &g, const Msf &m, D
             const size_t smem = sort_smem_bytes<true>();
             int grid = 1;
             DG_TRY(coop_grid(c, kCoopDendro, (const void *)k_d_rounds, kSThreads, smem, &grid));
-            grid = w.na > kTailMax ? (int)std::min<int64_t>(std::min(grid, kMidCtas), cdiv(w.na, kMidEdges)) : 1;
+            grid = w.na > kTailMax ? std::min(grid, mid_ctas(w.na, c->num_sms, most)) : 1;
             d.bar = c->next_bar();
             void *args[] = {&d, &w};
             cudaError_t e;
