@@ -1,7 +1,8 @@
 """Dendrogram rounds over every form they take: the last rounds in one CTA (at
-most 8,192 live edges), the middle rounds in one cooperative kernel, large
+most 4,096 live edges), the middle rounds in one cooperative kernel, large
 rounds (above 524,288) as separate launches, and in each both group sizes (up
-to 128 accepted edges an edge scans its group, above they are sorted)."""
+to 128 accepted edges an edge scans its group, above they are sorted). The
+exact lines between the forms are in test_gpu_dendro_lines.py."""
 import numpy as np
 import pytest
 
