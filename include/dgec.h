@@ -294,17 +294,21 @@ typedef struct {
 dgec_status dgec_set_launch_config(dgec_ctx *ctx, const dgec_launch_config *cfg);
 dgec_status dgec_get_launch_config(const dgec_ctx *ctx, dgec_launch_config *cfg);
 
-/* Bounds of the waits inside the calls made on ctx (results do not depend on
- * them). Several kernels of a call are cooperative: their CTAs wait for one
+/* Bounds of the waits and walks inside the calls made on ctx (results do not
+ * depend on them). Several kernels of a call are cooperative: their CTAs wait for one
  * another at grid barriers, which the device completes as long as all CTAs are
  * resident. A barrier polls at most barrier_polls times (about a microsecond
  * each; 0 gives up at once; default 2^24) in the call's cooperative launches
  * from number barrier_from on (counted from 0; default 0), the default bound
  * before. A call whose barrier gave up returns DGEC_ERR_TIMEOUT; ctx and its
- * workspace can be used again. Negative values give DGEC_ERR_INVALID_ARG. */
+ * workspace can be used again. A thread follows at most walk_steps pointers
+ * (default INT32_MAX; each kernel's own limit of 128 to 512 applies if it is
+ * smaller) before its walk is left to passes that halve every distance.
+ * Negative values, and 0 steps, give DGEC_ERR_INVALID_ARG. */
 typedef struct {
     int32_t barrier_polls;
     int32_t barrier_from;
+    int32_t walk_steps;
 } dgec_limits;
 dgec_status dgec_set_limits(dgec_ctx *ctx, const dgec_limits *limits);
 

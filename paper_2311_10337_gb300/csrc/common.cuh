@@ -75,12 +75,15 @@ struct Ctx {
     BarRef bar;                      // of the current call
     unsigned bar_polls = 1u << 24;   // bounds of the waits (dgec_set_limits)
     int bar_from = 0;
+    int walk_steps = INT32_MAX;      // bounds every walk below its kernel's own limit
     int coop_launches = 0;           // of the current call
     BarRef next_bar() {              // for the next cooperative launch
         BarRef b = bar;
         b.polls = coop_launches++ >= bar_from ? bar_polls : 1u << 24;
         return b;
     }
+    int walk(int own) const { return own < walk_steps ? own : walk_steps; }
+    bool own_walk(int own) const { return own <= walk_steps; }
     const unsigned *stop() const { return bar.word + 2; }
 };
 

@@ -91,9 +91,13 @@ struct SelBigRep {  // big kept merges (the nodes whose cluster link is set)
 // them; times of 60M edges in whole days 114 and 34. With 256 those take 23 and
 // 21 ms, but 100M hub edges then need the rounds (0.5 ms), with 512 they do not.
 constexpr int kTopWalk = 512;
-template <class Sel>
-__global__ void k_c_top(const unsigned *stop, int64_t n, int64_t off, Sel sel, int32_t *ptr, unsigned long long *moved) {
+// OWN: the limit is kTopWalk, known when the loop is compiled (read from the
+// arguments, the walks of 20M edges take 0.63 ms instead of 0.32).
+template <bool OWN, class Sel>
+__global__ void k_c_top(const unsigned *stop, int64_t n, int64_t off, Sel sel, int32_t *ptr, int steps,
+                        unsigned long long *moved) {
     if (stopped(stop)) return;
+    const int limit = OWN ? kTopWalk : steps;
     bool cut = false;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n;
          t += (int64_t)gridDim.x * blockDim.x) {
@@ -102,13 +106,13 @@ __global__ void k_c_top(const unsigned *stop, int64_t n, int64_t off, Sel sel, i
         const int64_t x = off + s;
         int r = ptr[x];
         int it = 0;
-        for (; it < kTopWalk; it++) {
+        for (; it < limit; it++) {
             const int rr = ptr[r];
             if (rr == r) break;
             r = rr;
             atomicExch(ptr + x, r);  // not a store: other CTAs read these lines meanwhile
         }
-        cut |= it == kTopWalk;
+        cut |= it == limit;
     }
     if (__syncthreads_or(cut) && threadIdx.x == 0) atomicOr(moved, 1ull);
 }
@@ -143,7 +147,10 @@ static dgec_status jump_to_fixed(Ctx *c, CoopKernel which, int64_t n, int64_t of
                                  unsigned long long *moved) {
     if (n <= 0) return DGEC_OK;
     const int g = grid_for(n, kBlock, kStreamCap);
-    TK(c, "k_c_top", k_c_top<Sel><<<g, kBlock, 0, c->stream>>>(c->stop(), n, off, sel, ptr, moved));
+    if (c->own_walk(kTopWalk))
+        TK(c, "k_c_top", k_c_top<true, Sel><<<g, kBlock, 0, c->stream>>>(c->stop(), n, off, sel, ptr, kTopWalk, moved));
+    else
+        TK(c, "k_c_top", k_c_top<false, Sel><<<g, kBlock, 0, c->stream>>>(c->stop(), n, off, sel, ptr, c->walk_steps, moved));
     int grid = 1;
     const void *fn = (const void *)k_c_jump<Sel>;
     DG_TRY(coop_grid(c, which, fn, kBlock, 0, &grid));
@@ -378,6 +385,7 @@ struct Eom {
     unsigned long long *slot;  // (next ancestor << 32) | highest selected on the way there
     int32_t *H;                // highest selected ancestor-or-self, -1
     unsigned long long *cnt;   // [0], [1] open clusters, [2..4] flags; zeroed before the kernel
+    int walk;                  // limit of a walk
     BarRef bar;
 };
 
@@ -438,7 +446,7 @@ __device__ __forceinline__ void e_walk(const Eom &e, int c) {
 //      is open; a phase at least halves the spines' branchings.
 //   3. Walks toward the root that leave a (next, highest selected) shortcut
 //      in their slot, in descending order, so the clusters near the root
-//      finish first and later walks are short; a walk cut at kTopWalk steps
+//      finish first and later walks are short; a walk cut at e.walk steps
 //      is taken up again in another round.
 // What bounds it: the random 8 and 16-byte accesses of the walks' reports at
 // large trees, the barriers (about 2 us each) of the contraction at small ones.
@@ -585,7 +593,7 @@ __global__ void __launch_bounds__(256, 4) k_e_tree(Eom e) {
             if (e.fin[c]) continue;
             unsigned long long v = e.slot[c];
             int it = 0;
-            while ((int)(v >> 32) >= 0 && it < kTopWalk) {
+            while ((int)(v >> 32) >= 0 && it < e.walk) {
                 const unsigned long long u = *(volatile unsigned long long *)(e.slot + (v >> 32));
                 v = (u & 0xffffffff00000000ull) | ((int)(unsigned)u >= 0 ? (unsigned)u : (unsigned)v);
                 atomicExch(e.slot + c, v);  // not a store: other CTAs read these lines meanwhile
@@ -859,6 +867,7 @@ dgec_status stage_condense(Ctx *c, const Problem &p, const Msf &m, const Dendro 
     {
         int grid = 1;
         e.bar = c->next_bar();
+        e.walk = c->walk(kTopWalk);
         DG_TRY(coop_grid(c, kCoopEom, (const void *)k_e_tree, kBlock, 0, &grid));
         const int64_t want = cdiv(ncl, kBlock);  // (two clusters a thread: 0.070 ms instead of 0.058 at 20,000 edges)
         DG_TRY(coop_launch(c, "k_e_tree", (const void *)k_e_tree, want < grid ? (int)want : grid, kBlock, 0, e));

@@ -137,7 +137,7 @@ struct DArgs {
     unsigned *ccnt;      // [CTAs] accepted edges of each CTA's chunk
     SegVal *cagg;        // [CTAs] chain sum over each CTA's chunk
     int *state;          // [0] rounds run, [1] error, [2] live edges (accepted ones after a large round's emit)
-    int max_rounds;
+    int max_rounds, walk;
     BarRef bar;
 };
 
@@ -277,7 +277,10 @@ __device__ __forceinline__ void d_ptr(const DArgs &a, const DRound &w) {
 // for the rounds; asking whether any was cut costs them 0.07 ms in 12 launches
 // and the walks 3.56 ms instead of 3.40.
 constexpr int kDWalk = 128;
+// OWN: the limit is kDWalk, known when the loop is compiled.
+template <bool OWN>
 __device__ __forceinline__ void d_jump(const DArgs &a, const DRound &w) {
+    const int limit = OWN ? kDWalk : a.walk;
     D_LIST;
     D_STRIDE;
     bool cut = false;
@@ -290,13 +293,13 @@ __device__ __forceinline__ void d_jump(const DArgs &a, const DRound &w) {
             const int c = side ? ecv[j] : ecu[j];
             int r = a.gp[c];
             int it = 0;
-            for (; it < kDWalk; it++) {
+            for (; it < limit; it++) {
                 const int rr = *(volatile int32_t *)(a.gp + r);
                 if (rr == r) break;
                 r = rr;
                 atomicExch(a.gp + c, r);  // (not a store: see d_alloc)
             }
-            cut |= it == kDWalk;
+            cut |= it == limit;
         }
     }
     if (__syncthreads_or(cut) && threadIdx.x == 0) atomicOr(a.tot + 4, 1ull);
@@ -716,7 +719,8 @@ __device__ __forceinline__ void d_rows(const DArgs &a, const DRound &w, const un
     }
 D_KERNEL(bid, d_bid(a, w))
 D_KERNEL(ptr, d_ptr(a, w))
-D_KERNEL(jump, d_jump(a, w))
+D_KERNEL(jump, d_jump<true>(a, w))
+D_KERNEL(jump_n, d_jump<false>(a, w))
 D_KERNEL(tau, d_tau(a, w))
 D_KERNEL(accept, d_accept(a, w))
 D_KERNEL(alloc, d_alloc(a, w))
@@ -749,7 +753,8 @@ __global__ void __launch_bounds__(kSThreads, 2) k_d_settle(const __grid_constant
 // its own registers.
 __device__ __noinline__ void dc_bid(const DArgs &a, const DRound &w) { d_bid(a, w); }
 __device__ __noinline__ void dc_ptr(const DArgs &a, const DRound &w) { d_ptr(a, w); }
-__device__ __noinline__ void dc_jump(const DArgs &a, const DRound &w) { d_jump(a, w); }
+template <bool OWN>
+__device__ __noinline__ void dc_jump(const DArgs &a, const DRound &w) { d_jump<OWN>(a, w); }
 __device__ __noinline__ JumpEnd dc_settle(const DArgs &a, const DRound &w, GridBar &bar) { return d_settle(a, w, bar); }
 __device__ __noinline__ void dc_tau(const DArgs &a, const DRound &w) { d_tau(a, w); }
 __device__ __noinline__ void dc_accept(const DArgs &a, const DRound &w) { d_accept(a, w); }
@@ -787,7 +792,8 @@ __global__ void __launch_bounds__(kSThreads, 2) k_d_rounds(const __grid_constant
         if (!bar.sync()) return;
         dc_ptr(a, w);
         if (!bar.sync()) return;
-        dc_jump(a, w);
+        if (a.walk == kDWalk) dc_jump<true>(a, w);
+        else dc_jump<false>(a, w);
         if (!bar.sync()) return;
         if (*(volatile unsigned long long *)(a.tot + 4)) {
             const JumpEnd e = dc_settle(a, w, bar);
@@ -1197,7 +1203,7 @@ dgec_status stage_dendro(Ctx *c, const Problem &p, const Csr &g, const Msf &m, D
                 s.gcnt, s.gseg, s.slot, s.segA, s.segB, s.segC, (unsigned long long *)(s.state + 4), s.kids, s.contrib,
                 s.row, o.parent,
                 sort_args(c, RadixBuffers{s.k1, s.k2, s.v1, s.v2}, n, 0, lb + sbits, s.radix, E), s.ccnt, s.cagg,
-                s.state, 1 << 16, c->bar};
+                s.state, 1 << 16, c->walk(kDWalk), c->bar};
         DRound w{0, 0, kStampTop, n, 0, 0, false};
         CU_TRY(c, cudaMemsetAsync(s.state, 0, sizeof(int) * 20, st));
         CU_TRY(c, cudaMemsetAsync(s.gcnt, 0, sizeof(int) * E, st));
@@ -1214,7 +1220,8 @@ dgec_status stage_dendro(Ctx *c, const Problem &p, const Csr &g, const Msf &m, D
             w.G = (int)std::min<int64_t>(cdiv(w.na, kDTile), c->stream_ctas);
             TK(c, "k_d_ptr", k_d_ptr<<<w.G, kSThreads, 0, st>>>(d, w));
             w.G = wide;
-            TK(c, "k_d_gjump", k_d_jump<<<wide, kSThreads, 0, st>>>(d, w));
+            if (d.walk == kDWalk) TK(c, "k_d_gjump", k_d_jump<<<wide, kSThreads, 0, st>>>(d, w));
+            else TK(c, "k_d_gjump", k_d_jump_n<<<wide, kSThreads, 0, st>>>(d, w));
             DG_TRY(coop_grid(c, kCoopDJump, (const void *)k_d_settle, kSThreads, 0, &w.G));
             {
                 d.bar = c->next_bar();

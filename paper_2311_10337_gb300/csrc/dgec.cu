@@ -480,10 +480,11 @@ dgec_status dgec_get_launch_config(const dgec_ctx *x, dgec_launch_config *cfg) {
 
 dgec_status dgec_set_limits(dgec_ctx *x, const dgec_limits *limits) {
     if (!x || !limits) return DGEC_ERR_INVALID_ARG;
-    if (limits->barrier_polls < 0 || limits->barrier_from < 0)
-        return set_err(&x->c, DGEC_ERR_INVALID_ARG, "limits must not be negative");
+    if (limits->barrier_polls < 0 || limits->barrier_from < 0 || limits->walk_steps < 1)
+        return set_err(&x->c, DGEC_ERR_INVALID_ARG, "limits must not be negative, walk_steps at least 1");
     x->c.bar_polls = (unsigned)limits->barrier_polls;
     x->c.bar_from = limits->barrier_from;
+    x->c.walk_steps = limits->walk_steps;
     return DGEC_OK;
 }
 

@@ -352,20 +352,23 @@ __global__ void k_m_hook(const int32_t *__restrict__ roots, int64_t nr, const un
 // At 256 steps hardly a walk of 100M hub edges is cut (k_m_settle 0.04 to 0.15 ms
 // in 7 rounds, 0.25 at 64).
 constexpr int kMWalk = 256;
-__global__ void k_m_jump(const int32_t *roots, int64_t nr, int32_t *par, unsigned long long *cut) {
+// OWN: the limit is kMWalk, known when the loop is compiled.
+template <bool OWN>
+__global__ void k_m_jump(const int32_t *roots, int64_t nr, int32_t *par, int steps, unsigned long long *cut) {
+    const int limit = OWN ? kMWalk : steps;
     bool any = false;
     for (int64_t ix = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; ix < nr;
          ix += (int64_t)gridDim.x * blockDim.x) {
         int x = roots[ix];
         int r = par[x];
         int it = 0;
-        for (; it < kMWalk; it++) {
+        for (; it < limit; it++) {
             int rr = par[r];
             if (rr == r) break;
             r = rr;
             atomicExch(par + x, r);  // not a store: other CTAs read these lines meanwhile
         }
-        any |= it == kMWalk;
+        any |= it == limit;
     }
     if (__syncthreads_or(any) && threadIdx.x == 0) atomicOr(cut, 1ull);
 }
@@ -448,6 +451,7 @@ struct MsfArgs {
                               // [4] forest edges, [5] error, [6] a walk was cut; if so [7] rounds begun, [8] the
                               // last one's live edges, [9] next roots; all but [4] zeroed before
     int ib, lbits;            // bits of an original id, of the label in a key (0: none)
+    int walk;                 // limit of a walk
     BarRef bar;
 };
 
@@ -510,9 +514,9 @@ __device__ __forceinline__ void bid_u128(ulonglong2 *sa, u128 ka, ulonglong2 *sb
 
 // The root above label x after the hooks; x's own pointer is moved there when
 // the way was longer than one step (by an exchange, not a store: other CTAs
-// read these lines meanwhile). A walk is cut after kMWalk steps, which *cut
+// read these lines meanwhile). A walk is cut after `limit` steps, which *cut
 // then says; what is returned is an ancestor short of the root.
-__device__ __forceinline__ int new_root(int32_t *par, int x, unsigned long long *cut) {
+__device__ __forceinline__ int new_root(int32_t *par, int x, int limit, unsigned long long *cut) {
     const int p = par[x];
     int r = p;
     for (int it = 0;; it++) {
@@ -520,7 +524,7 @@ __device__ __forceinline__ int new_root(int32_t *par, int x, unsigned long long 
         if (rr == r) break;
         r = rr;
         if ((it & 7) == 7) atomicExch(par + x, r);
-        if (it == kMWalk) {
+        if (it == limit) {
             *(volatile unsigned long long *)cut = 1;
             break;
         }
@@ -643,8 +647,8 @@ __global__ void __launch_bounds__(kBlock, 4) k_m_forest(MsfArgs a) {
                 ca[q] = cb[q] = 0;
                 if (x < n) {
                     const int2 l = round ? lin[x] : make_int2(a.ru[x], a.rv[x]);
-                    ca[q] = new_root(a.par, l.x, a.cnt + 6);
-                    cb[q] = new_root(a.par, l.y, a.cnt + 6);
+                    ca[q] = new_root(a.par, l.x, a.walk, a.cnt + 6);
+                    cb[q] = new_root(a.par, l.y, a.walk, a.cnt + 6);
                     if (ca[q] != cb[q]) keep |= 1u << q;
                 }
             }
@@ -954,7 +958,8 @@ dgec_status stage_msf(Ctx *c, const Problem &p, const Csr &g, const Skel &sk, Ms
             TK(c, "k_m_hook", k_m_hook<<<grk, kBlock, 0, st>>>(roots, nr, bw, buv, s.bp, s.win, cu, cv, cw, g.rank_of,
                                                             round == 0 ? g.orig_of : nullptr, s.par, s.fe, s.cnt + 4));
             CU_TRY(c, cudaMemsetAsync(s.cnt, 0, 4 * sizeof(unsigned long long), st));
-            TK(c, "k_m_jump", k_m_jump<<<gr, kBlock, 0, st>>>(roots, nr, s.par, s.cnt));
+            if (c->own_walk(kMWalk)) TK(c, "k_m_jump", k_m_jump<true><<<gr, kBlock, 0, st>>>(roots, nr, s.par, kMWalk, s.cnt));
+            else TK(c, "k_m_jump", k_m_jump<false><<<gr, kBlock, 0, st>>>(roots, nr, s.par, c->walk_steps, s.cnt));
             {
                 int grid = 1;
                 DG_TRY(coop_grid(c, kCoopMJump, (const void *)k_m_settle, kBlock, 0, &grid));
@@ -995,7 +1000,7 @@ dgec_status stage_msf(Ctx *c, const Problem &p, const Csr &g, const Skel &sk, Ms
         // the kernel's first filter writes lb/kb: not the side its edges come from
         const LiveSide &in = s.side[which ^ 1], &out = s.side[which];
         MsfArgs f{nr, n, roots0, ccu, ccv, cu, cv, cw, g.rank_of, s.par, roots0 ? roots2 : roots, roots0 ? roots : roots2,
-                  s.bp, s.slot, s.slot2, in.lab, out.lab, in.key, out.key, s.fe, s.cnt, p.idbits, lbits, c->next_bar()};
+                  s.bp, s.slot, s.slot2, in.lab, out.lab, in.key, out.key, s.fe, s.cnt, p.idbits, lbits, c->walk(kMWalk), c->next_bar()};
         int grid = 1;
         DG_TRY(coop_grid(c, kCoopMsf, (const void *)k_m_forest, kBlock, 0, &grid));
         const int64_t want = cdiv(n > nr ? n : nr, kBlock * kRes);

@@ -41,7 +41,7 @@ class LaunchConfig(ctypes.Structure):
 
 
 class Limits(ctypes.Structure):
-    _fields_ = [("barrier_polls", ctypes.c_int32), ("barrier_from", ctypes.c_int32)]
+    _fields_ = [("barrier_polls", ctypes.c_int32), ("barrier_from", ctypes.c_int32), ("walk_steps", ctypes.c_int32)]
 
 
 class DgecError(RuntimeError):
@@ -345,11 +345,13 @@ class Context:
         self._check(self.L.dgec_get_launch_config(self.h, ctypes.byref(c)))
         return int(c.knn_block), int(c.stream_ctas), int(c.knn_packed)
 
-    def set_limits(self, barrier_polls: int = 1 << 24, barrier_from: int = 0):
-        """Bounds of the waits inside the calls on this context: how often a
-        grid barrier polls before its call ends with DGEC_ERR_TIMEOUT, from
-        the call's cooperative launch `barrier_from` on."""
-        lim = Limits(barrier_polls, barrier_from)
+    def set_limits(self, barrier_polls: int = 1 << 24, barrier_from: int = 0, walk_steps: int = 2**31 - 1):
+        """Bounds of the waits and walks inside the calls on this context: how
+        often a grid barrier polls before its call ends with
+        DGEC_ERR_TIMEOUT, from the call's cooperative launch `barrier_from`
+        on; how many pointers a thread follows before its walk is left to
+        jumping passes."""
+        lim = Limits(barrier_polls, barrier_from, walk_steps)
         self._check(self.L.dgec_set_limits(self.h, ctypes.byref(lim)))
 
     def stage_timing(self) -> list:

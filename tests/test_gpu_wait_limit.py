@@ -110,7 +110,7 @@ def test_every_barrier_can_give_up(name):
 
 def test_bad_limits_are_rejected():
     from paper_2311_10337_gb300 import dgec
-    for polls, first in ((-1, 0), (1, -1)):
+    for polls, first, steps in ((-1, 0, 1), (1, -1, 1), (1, 0, 0), (1, 0, -5)):
         with pytest.raises(dgec.DgecError) as e:
-            ctx().set_limits(polls, first)
+            ctx().set_limits(polls, first, steps)
         assert e.value.status == 1
