@@ -766,7 +766,7 @@ __device__ __noinline__ void dc_chain(const DArgs &a, const DRound &w, const uns
 __device__ __noinline__ void dc_rows(const DArgs &a, const DRound &w, const unsigned long long *key,
                                      const unsigned long long *val) { d_rows(a, w, key, val); }
 __device__ __noinline__ bool dc_sort(const DArgs &a, int64_t n, int bits, int most, unsigned long long *sm, GridBar &bar) {
-    return sort_run<true>(a.sort, n, 0, bits, most, sort_smem<true>(sm), bar);
+    return sort_run<SortWide, true>(a.sort, n, 0, bits, most, sort_smem<SortWide, true>(sm), bar);
 }
 #undef D_LIST
 #undef D_STRIDE
@@ -823,10 +823,10 @@ __global__ void __launch_bounds__(kSThreads, 2) k_d_rounds(const __grid_constant
         dc_small(a, w);
         if (w.nacc > 0) {
             // each large group's chain in rank order
-            const int kbits = a.lb + a.sbits, most = w.nacc > kSNarrow ? kSBits - 1 : kSBits;
-            if (!dc_sort(a, w.nacc, kbits, most, d_sm, bar)) return;
+            const int kbits = a.lb + a.sbits;
+            if (!dc_sort(a, w.nacc, kbits, kSBits, d_sm, bar)) return;
             if (!bar.sync()) return;
-            const bool in_b = sort_in_b(w.nacc, kbits, most);
+            const bool in_b = sort_in_b(w.nacc, kbits, kSBits);
             const unsigned long long *key = in_b ? a.sort.kb : a.sort.ka, *val = in_b ? a.sort.vb : a.sort.va;
             dc_chain(a, w, key, val);
             if (!bar.sync()) return;
@@ -1261,7 +1261,7 @@ dgec_status stage_dendro(Ctx *c, const Problem &p, const Csr &g, const Msf &m, D
             w.na = kept;
         }
         {
-            const size_t smem = sort_smem_bytes<true>();
+            const size_t smem = sort_smem_bytes<SortWide, true>();
             int grid = 1;
             DG_TRY(coop_grid(c, kCoopDendro, (const void *)k_d_rounds, kSThreads, smem, &grid));
             grid = w.na > kTailMax ? std::min(grid, mid_ctas(w.na, c->num_sms, most)) : 1;
