@@ -47,7 +47,8 @@ struct StageTimer {
 enum CoopKernel { kCoopSortK, kCoopSortKV, kCoopSortNarrowK, kCoopSortNarrowKV, kCoopEom, kCoopMsf, kCoopMJump, kCoopMLabels, kCoopDendro, kCoopDJump, kCoopJumpAll, kCoopJumpBig, kCoopCount };
 
 // What the grid barriers of a call share. `word` (in the call's workspace, zeroed
-// once a call): [0] arrivals, [1] exits, [2] the call's stop word. Once a
+// once a call): [0] arrivals, [1] exits, [2] the call's stop word, [32] the next
+// tile of a sort's pass. Once a
 // cooperative kernel gives up it writes its StopCode there and to *err
 // (host-mapped). Until the host reads that, the kernels behind it still run:
 // those that follow what it left as indices return when the stop word is set,

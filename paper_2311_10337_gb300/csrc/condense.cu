@@ -625,7 +625,7 @@ __global__ void k_e_labels(const unsigned *stop, int64_t E, const int32_t *fall_
     }
 }
 
-__global__ void k_e_final_keys(int64_t ncl, const int32_t *H, const int *minmem, int *flag) {
+__global__ void k_e_final_keys(int64_t ncl, const int32_t *H, int *flag) {
     for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c <= ncl;
          c += (int64_t)gridDim.x * blockDim.x)
         flag[c] = (c < ncl && H[c] == (int32_t)c) ? 1 : 0;
@@ -873,7 +873,7 @@ dgec_status stage_condense(Ctx *c, const Problem &p, const Msf &m, const Dendro 
         DG_TRY(coop_launch(c, "k_e_tree", (const void *)k_e_tree, want < grid ? (int)want : grid, kBlock, 0, e));
     }
     TK(c, "k_e_labels", k_e_labels<<<gE, kBlock, 0, st>>>(c->stop(), E, o.fall_cluster, s.cidx, s.H, o.labels, s.minmem));
-    TK(c, "k_e_final_keys", k_e_final_keys<<<gc, kBlock, 0, st>>>(ncl, s.H, s.minmem, s.flag));
+    TK(c, "k_e_final_keys", k_e_final_keys<<<gc, kBlock, 0, st>>>(ncl, s.H, s.flag));
     DG_TRY(exclusive_scan_i32(c, s.flag, s.cpos, ncl + 1, s.scan_tmp));
     int64_t nf;
     DG_TRY(read_counters(c, (const int64_t *)(s.cpos + ncl), 1, &nf));

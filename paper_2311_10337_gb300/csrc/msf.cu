@@ -434,8 +434,6 @@ __global__ void k_m_init(int64_t E, int32_t *par, int32_t *roots, unsigned long 
 
 typedef unsigned __int128 u128;
 
-// A live edge after the first round: the labels of the components at its
-// ends, and its packed key.
 struct MsfArgs {
     int64_t nr0, n0;
     const int32_t *roots0;           // the roots to begin with (null: 0 .. nr0-1)

@@ -150,7 +150,7 @@ dgec_status exclusive_scan_i64(Ctx *c, const long long *in, long long *out, int6
                                long long *scratch);
 
 // ------------------------------------------------------------ radix sort
-// Stable LSD radix sort on key bits [begin_bit, end_bit), 8 bits a pass.
+// Stable LSD radix sort on key bits [begin_bit, end_bit), digits of up to 9 bits.
 // keys/vals are sorted between (a) and (b) buffers; on return *in_b tells
 // which buffer holds the result. vals may be null.
 struct RadixBuffers {
