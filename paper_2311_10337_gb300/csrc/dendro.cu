@@ -1223,6 +1223,7 @@ dgec_status stage_dendro(Ctx *c, const Problem &p, const Csr &g, const Msf &m, D
             if (d.walk == kDWalk) TK(c, "k_d_gjump", k_d_jump<<<wide, kSThreads, 0, st>>>(d, w));
             else TK(c, "k_d_gjump", k_d_jump_n<<<wide, kSThreads, 0, st>>>(d, w));
             DG_TRY(coop_grid(c, kCoopDJump, (const void *)k_d_settle, kSThreads, 0, &w.G));
+            w.G = std::min(w.G, c->num_sms);  // hardly ever with work to do: no more than it takes
             {
                 d.bar = c->next_bar();
                 void *args[] = {&d, &w};

@@ -966,7 +966,7 @@ dgec_status stage_msf(Ctx *c, const Problem &p, const Csr &g, const Skel &sk, Ms
                 void *args[] = {&roots, &nr, &s.par, &cut, &ref};
                 cudaError_t e;
                 TK(c, "k_m_settle", e = cudaLaunchCooperativeKernel((const void *)k_m_settle,
-                                                                    dim3((unsigned)std::min(gr, grid)), dim3(kBlock), args,
+                                                                    dim3((unsigned)std::min({gr, grid, c->num_sms})), dim3(kBlock), args,
                                                                     0, st));
                 if (e != cudaSuccess) return set_err(c, DGEC_ERR_CUDA, "k_m_settle launch: %s", cudaGetErrorString(e));
             }
