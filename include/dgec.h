@@ -302,7 +302,7 @@ dgec_status dgec_get_launch_config(const dgec_ctx *ctx, dgec_launch_config *cfg)
  * from number barrier_from on (counted from 0; default 0), the default bound
  * before. A call whose barrier gave up returns DGEC_ERR_TIMEOUT; ctx and its
  * workspace can be used again. A thread follows at most walk_steps pointers
- * (default INT32_MAX; each kernel's own limit of 128 to 512 applies if it is
+ * (default INT32_MAX; each kernel's own limit of 64 or 256 applies if it is
  * smaller) before its walk is left to passes that halve every distance.
  * Negative values, and 0 steps, give DGEC_ERR_INVALID_ARG. */
 typedef struct {

@@ -44,7 +44,7 @@ struct StageTimer {
 };
 
 // Cooperative kernels whose resident-CTA count a context remembers.
-enum CoopKernel { kCoopSortK, kCoopSortKV, kCoopSortNarrowK, kCoopSortNarrowKV, kCoopEom, kCoopMsf, kCoopMJump, kCoopMLabels, kCoopDendro, kCoopDJump, kCoopJumpAll, kCoopJumpBig, kCoopCount };
+enum CoopKernel { kCoopSortK, kCoopSortKV, kCoopSortNarrowK, kCoopSortNarrowKV, kCoopEom, kCoopMsf, kCoopMJump, kCoopMLabels, kCoopDendro, kCoopDJump, kCoopCJump, kCoopCount };
 
 // What the grid barriers of a call share. `word` (in the call's workspace, zeroed
 // once a call): [0] arrivals, [1] exits, [2] the call's stop word, [32] the next

@@ -84,21 +84,21 @@ struct SelBigRep {  // big kept merges (the nodes whose cluster link is set)
 // One pass of start-compressing walks, in descending index order: parents
 // have larger ids than their children, so ancestors tend to be resolved
 // first and later walks stop after a few steps. A walk that exceeds
-// kTopWalk steps stores the ancestor it reached and flags *moved. The limit
-// bounds what a long run of equal weights costs, whose first walkers meet
-// only pointers as short as their own: 60M edges at one threshold take 188 ms
-// with walks of up to 4,096 steps, 39 with 512 and the rounds (1.7) behind
-// them; times of 60M edges in whole days 114 and 34. With 256 those take 23 and
-// 21 ms, but 100M hub edges then need the rounds (0.5 ms), with 512 they do not.
-constexpr int kTopWalk = 512;
+// kTopWalk steps stores the ancestor it reached and goes to the list of cut
+// walks (*cut: their number). The limit bounds what a long run of equal weights
+// costs, whose first walkers meet only pointers as short as their own: this
+// stage on 60M edges at one threshold, walks of up to 4,096 / 256 / 128 / 64 steps:
+// 190 / 16.8 / 10.7 / 8.9 ms; 60M edges with times in whole days 92.6 / 14.3 / 11.5 /
+// 10.2. 200M hub edges, whose few long walks the rounds finish in 0.05 ms, 51.4 ms
+// at 4,096 and 51.3 at 64.
+constexpr int kTopWalk = 64;
 // OWN: the limit is kTopWalk, known when the loop is compiled (read from the
 // arguments, the walks of 20M edges take 0.63 ms instead of 0.32).
 template <bool OWN, class Sel>
-__global__ void k_c_top(const unsigned *stop, int64_t n, int64_t off, Sel sel, int32_t *ptr, int steps,
-                        unsigned long long *moved) {
+__global__ void k_c_top(const unsigned *stop, int64_t n, int64_t off, Sel sel, int32_t *ptr, int steps, int32_t *list,
+                        unsigned long long *cut) {
     if (stopped(stop)) return;
     const int limit = OWN ? kTopWalk : steps;
-    bool cut = false;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n;
          t += (int64_t)gridDim.x * blockDim.x) {
         const int64_t s = n - 1 - t;
@@ -112,27 +112,18 @@ __global__ void k_c_top(const unsigned *stop, int64_t n, int64_t off, Sel sel, i
             r = rr;
             atomicExch(ptr + x, r);  // not a store: other CTAs read these lines meanwhile
         }
-        cut |= it == limit;
+        if (it == limit) list_cut(list, cut, (int)x);
     }
-    if (__syncthreads_or(cut) && threadIdx.x == 0) atomicOr(moved, 1ull);
 }
 
-// The pointers `Sel` picks, as jump_rounds takes them.
-template <class Sel>
-struct SelItem {
-    int64_t off;
-    Sel sel;
-    __device__ __forceinline__ int64_t operator()(int64_t s) const { return sel(s) ? off + s : -1; }
-};
-// The jumping rounds: nothing to do unless *moved says that a walk was cut
-// short. moved[1 .. 3] are their flags, zero at the start.
-template <class Sel>
-__global__ void __launch_bounds__(kBlock) k_c_jump(int64_t n, int64_t off, Sel sel, int32_t *ptr,
-                                                   unsigned long long *moved, BarRef ref) {
-    if (moved[0] == 0) return;  // the same for every CTA: written before this launch
+// The cut walks' pointers to their fixed points. cut[1 .. 3]: the rounds'
+// flags, zero at the start.
+__global__ void __launch_bounds__(kBlock) k_c_jump(const int32_t *list, int32_t *ptr, unsigned long long *cut, BarRef ref) {
+    const int64_t n = (int64_t)cut[0];
+    if (n == 0) return;  // the same for every CTA: written before this launch
     GridBar bar(ref);
     if (bar.stopped()) return;
-    const JumpEnd e = jump_rounds(bar, n, SelItem<Sel>{off, sel}, ptr, moved + 1);
+    const JumpEnd e = jump_rounds(bar, n, ListItem{list}, ptr, cut + 1);
     if (e == kJumpBarrier) return;
     if (e == kJumpBound && threadIdx.x == 0) bar.stop(kStopJump);
     bar.finish();
@@ -143,22 +134,21 @@ __global__ void __launch_bounds__(kBlock) k_c_jump(int64_t n, int64_t off, Sel s
 // host whether to launch them cost a call two waits; with the memsets that
 // k_c_zero took over, this stage took 0.20 ms instead of 0.16 at 1,000 edges.)
 template <class Sel>
-static dgec_status jump_to_fixed(Ctx *c, CoopKernel which, int64_t n, int64_t off, Sel sel, int32_t *ptr,
-                                 unsigned long long *moved) {
+static dgec_status jump_to_fixed(Ctx *c, int64_t n, int64_t off, Sel sel, int32_t *ptr, int32_t *list,
+                                 unsigned long long *cut) {
     if (n <= 0) return DGEC_OK;
     const int g = grid_for(n, kBlock, kStreamCap);
     if (c->own_walk(kTopWalk))
-        TK(c, "k_c_top", k_c_top<true, Sel><<<g, kBlock, 0, c->stream>>>(c->stop(), n, off, sel, ptr, kTopWalk, moved));
+        TK(c, "k_c_top", k_c_top<true, Sel><<<g, kBlock, 0, c->stream>>>(c->stop(), n, off, sel, ptr, kTopWalk, list, cut));
     else
-        TK(c, "k_c_top", k_c_top<false, Sel><<<g, kBlock, 0, c->stream>>>(c->stop(), n, off, sel, ptr, c->walk_steps, moved));
+        TK(c, "k_c_top", k_c_top<false, Sel><<<g, kBlock, 0, c->stream>>>(c->stop(), n, off, sel, ptr, c->walk_steps, list, cut));
     int grid = 1;
-    const void *fn = (const void *)k_c_jump<Sel>;
-    DG_TRY(coop_grid(c, which, fn, kBlock, 0, &grid));
+    DG_TRY(coop_grid(c, kCoopCJump, (const void *)k_c_jump, kBlock, 0, &grid));
     BarRef ref = c->next_bar();
-    void *args[] = {&n, &off, &sel, &ptr, &moved, &ref};
+    void *args[] = {&list, &ptr, &cut, &ref};
     cudaError_t e;
-    TK(c, "k_c_jump", e = cudaLaunchCooperativeKernel(fn, dim3((unsigned)(g < grid ? g : grid)), dim3(kBlock), args, 0,
-                                                      c->stream));
+    TK(c, "k_c_jump", e = cudaLaunchCooperativeKernel((const void *)k_c_jump, dim3((unsigned)(g < grid ? g : grid)),
+                                                      dim3(kBlock), args, 0, c->stream));
     if (e != cudaSuccess) return set_err(c, DGEC_ERR_CUDA, "k_c_jump launch: %s", cudaGetErrorString(e));
     return DGEC_OK;
 }
@@ -811,13 +801,14 @@ dgec_status stage_condense(Ctx *c, const Problem &p, const Msf &m, const Dendro 
     unsigned long long *nbs = reinterpret_cast<unsigned long long *>(s.cpos);
     TK(c, "k_c_zero", k_c_zero<<<gn, kBlock, 0, st>>>(n + p.G, p.G, nbs, s.isc + E, s.cdeath + E, s.st_hi + E, s.st_lo + E,
                                                      o.gclusters, s.cnt, s.jflag));
+    // (the lists of cut walks lie in al1, which the EOM pass takes later)
     if (n > 0) {
         TK(c, "k_c_up", k_c_up<<<gn, kBlock, 0, st>>>(E, n, d.parent, m.w, s.up, s.isrep));
-        DG_TRY(jump_to_fixed(c, kCoopJumpAll, n, 0, SelAll{}, s.up, s.jflag));
+        DG_TRY(jump_to_fixed(c, n, 0, SelAll{}, s.up, s.al1, s.jflag));
     }
     TK(c, "k_c_cpar", k_c_cpar<<<gN, kBlock, 0, st>>>(gv, d.parent, s.up, s.isrep, d.size, s.cpar, nbs));
     TK(c, "k_c_link", k_c_link<<<gn, kBlock, 0, st>>>(c->stop(), gv, s.isrep, d.size, s.cpar, nbs, s.link));
-    DG_TRY(jump_to_fixed(c, kCoopJumpBig, n, E, SelBigRep{gv, s.isrep, d.size}, s.link, s.jflag + 4));
+    DG_TRY(jump_to_fixed(c, n, E, SelBigRep{gv, s.isrep, d.size}, s.link, s.al1, s.jflag + 4));
     TK(c, "k_c_clusters", k_c_clusters<<<gn, kBlock, 0, st>>>(c->stop(), gv, s.isrep, d.size, m.w, s.cpar, nbs, s.link,
                                                              s.isc, s.cbirth, s.cdeath, s.cparent));
     // the node records live in the EOM phase's Fa and Fc arrays (adjacent, not in use yet)

@@ -127,7 +127,7 @@ struct DArgs {
     int4 *segB;      // (pointer's owner, group, owner's root, the mutual pair's other root or -1)
     int2 *segC;      // its group's (first place, edges)
     unsigned long long *tot;  // [0], [1] places of small groups taken (by round parity), [2], [3] edges of large groups,
-                              // [4] a walk of d_jump was cut, [5 .. 7] flags of the jumping rounds
+                              // [4] cut walks of d_jump, [5 .. 7] flags of the jumping rounds
     // accepted edges of large groups, sorted by (group, rank)
     int2 *kids;          // the nodes the edge merges
     long long *contrib;  // (leaves it adds << 1) | first of its chain
@@ -268,22 +268,20 @@ __device__ __forceinline__ void d_ptr(const DArgs &a, const DRound &w) {
     }
 }
 // Every pointer to its tree's root, by walks that shorten their own pointer as
-// they go. Walks are cut after kDWalk steps, and jump_rounds finishes the rest:
+// they go. Walks are cut after kDWalk steps, and jump_rounds finishes those:
 // on a long chain the threads running meet only pointers as short as their
-// own, and the last of them walks all of it. A path whose gaps fall, with all
-// walks whole / cut at 512 / 256 / 128 / 64 steps: 400,000 edges 167 / 1.3 / 0.82
-// / 0.56 / 0.42 ms in the middle rounds, 3M edges 4.4 s / 6.2 / 2.5 / 1.4 / 0.6
-// ms in this step. At 128 no walk of 100M hub edges is cut, at 64 they pay 2.8 ms
-// for the rounds; asking whether any was cut costs them 0.07 ms in 12 launches
-// and the walks 3.56 ms instead of 3.40.
-constexpr int kDWalk = 128;
+// own, and the last of them walks all of it. Stage D1 of a path whose gaps fall,
+// all walks whole / cut at 256 / 128 / 64 steps: 400,000 edges 166 / 0.88 / 0.61 /
+// 0.47 ms, 3M 4.4 s / 3.1 / 2.2 / 1.5 ms; of 200M hub edges 71.0 / 70.6 / 70.6 / 70.6
+// (their cut walks settle in 0.08 to 0.11 ms, 14 launches included; 8.3 with rounds
+// over all pointers instead of a list of the cut ones).
+constexpr int kDWalk = 64;
 // OWN: the limit is kDWalk, known when the loop is compiled.
 template <bool OWN>
 __device__ __forceinline__ void d_jump(const DArgs &a, const DRound &w) {
     const int limit = OWN ? kDWalk : a.walk;
     D_LIST;
     D_STRIDE;
-    bool cut = false;
     for (int64_t j = g0; j < na; j += gsize) {
         const int st = a.st[j];
         if (!st) continue;
@@ -299,23 +297,13 @@ __device__ __forceinline__ void d_jump(const DArgs &a, const DRound &w) {
                 r = rr;
                 atomicExch(a.gp + c, r);  // (not a store: see d_alloc)
             }
-            cut |= it == limit;
+            if (it == limit) list_cut(a.slot, a.tot + 4, c);
         }
     }
-    if (__syncthreads_or(cut) && threadIdx.x == 0) atomicOr(a.tot + 4, 1ull);
 }
-// The pointers of the live edges' ends, as jump_rounds takes them.
-struct DItem {
-    const unsigned char *st;
-    const int32_t *ecu, *ecv;
-    __device__ __forceinline__ int64_t operator()(int64_t i) const {
-        const int64_t j = i >> 1;
-        if (!((st[j] >> (i & 1)) & 1)) return -1;
-        return (i & 1) ? ecv[j] : ecu[j];
-    }
-};
-__device__ __forceinline__ JumpEnd d_settle(const DArgs &a, const DRound &w, GridBar &bar) {
-    return jump_rounds(bar, 2 * w.na, DItem{a.st, w.odd ? a.ecu2 : a.ecu, w.odd ? a.ecv2 : a.ecv}, a.gp, a.tot + 5);
+// Their number is in tot[4], they lie in `slot`, which d_accept fills later.
+__device__ __forceinline__ JumpEnd d_settle(const DArgs &a, GridBar &bar, int64_t n) {
+    return jump_rounds(bar, n, ListItem{a.slot}, a.gp, a.tot + 5);
 }
 __device__ __forceinline__ void d_tau(const DArgs &a, const DRound &w) {
     D_LIST;
@@ -738,12 +726,13 @@ __global__ void __launch_bounds__(kSThreads, 2) k_d_rows(const __grid_constant__
     d_rows(a, w, key, val);
 }
 
-// What d_jump left of a large round's walks: nothing unless one was cut.
-__global__ void __launch_bounds__(kSThreads, 2) k_d_settle(const __grid_constant__ DArgs a, const __grid_constant__ DRound w) {
-    if (a.tot[4] == 0) return;  // the same for every CTA: written before this launch
+// What d_jump left of a large round's walks: nothing unless some were cut.
+__global__ void __launch_bounds__(kSThreads, 2) k_d_settle(const __grid_constant__ DArgs a) {
+    const int64_t n = (int64_t)a.tot[4];
+    if (n == 0) return;  // the same for every CTA: written before this launch
     GridBar bar(a.bar);
     if (bar.stopped()) return;
-    const JumpEnd e = d_settle(a, w, bar);
+    const JumpEnd e = d_settle(a, bar, n);
     if (e == kJumpBarrier) return;
     if (e == kJumpBound && threadIdx.x == 0) bar.stop(kStopJump);
     bar.finish();
@@ -755,7 +744,7 @@ __device__ __noinline__ void dc_bid(const DArgs &a, const DRound &w) { d_bid(a, 
 __device__ __noinline__ void dc_ptr(const DArgs &a, const DRound &w) { d_ptr(a, w); }
 template <bool OWN>
 __device__ __noinline__ void dc_jump(const DArgs &a, const DRound &w) { d_jump<OWN>(a, w); }
-__device__ __noinline__ JumpEnd dc_settle(const DArgs &a, const DRound &w, GridBar &bar) { return d_settle(a, w, bar); }
+__device__ __noinline__ JumpEnd dc_settle(const DArgs &a, GridBar &bar, int64_t n) { return d_settle(a, bar, n); }
 __device__ __noinline__ void dc_tau(const DArgs &a, const DRound &w) { d_tau(a, w); }
 __device__ __noinline__ void dc_accept(const DArgs &a, const DRound &w) { d_accept(a, w); }
 __device__ __noinline__ void dc_alloc(const DArgs &a, const DRound &w) { d_alloc(a, w); }
@@ -795,8 +784,9 @@ __global__ void __launch_bounds__(kSThreads, 2) k_d_rounds(const __grid_constant
         if (a.walk == kDWalk) dc_jump<true>(a, w);
         else dc_jump<false>(a, w);
         if (!bar.sync()) return;
-        if (*(volatile unsigned long long *)(a.tot + 4)) {
-            const JumpEnd e = dc_settle(a, w, bar);
+        const int64_t cut = (int64_t) * (volatile unsigned long long *)(a.tot + 4);
+        if (cut > 0) {
+            const JumpEnd e = dc_settle(a, bar, cut);
             if (e == kJumpBarrier) return;
             if (e == kJumpBound) {
                 if (threadIdx.x == 0) bar.stop(kStopJump);
@@ -1226,7 +1216,7 @@ dgec_status stage_dendro(Ctx *c, const Problem &p, const Csr &g, const Msf &m, D
             w.G = std::min(w.G, c->num_sms);  // hardly ever with work to do: no more than it takes
             {
                 d.bar = c->next_bar();
-                void *args[] = {&d, &w};
+                void *args[] = {&d};
                 cudaError_t e;
                 TK(c, "k_d_settle", e = cudaLaunchCooperativeKernel((const void *)k_d_settle, dim3((unsigned)w.G),
                                                                     dim3(kSThreads), args, 0, st));

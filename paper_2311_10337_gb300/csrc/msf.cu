@@ -347,16 +347,13 @@ __global__ void k_m_hook(const int32_t *__restrict__ roots, int64_t nr, const un
 // Roots walk to their new root (own pointer compressed on the way). Walks are
 // cut after kMWalk steps and left to k_m_settle: on a long chain the threads
 // running meet only pointers as short as their own, and the last of them walks
-// all of it. A path of 3M edges whose gaps fall took 1.3 s in k_m_forest; with
-// walks cut at 256 / 128 / 64 steps it and k_m_labels take 1.2 / 0.93 / 0.77 ms.
-// At 256 steps hardly a walk of 100M hub edges is cut (k_m_settle 0.04 to 0.15 ms
-// in 7 rounds, 0.25 at 64).
-constexpr int kMWalk = 256;
+// all of it (3M roots: 2.3 s). The few cut walks of 200M hub edges settle in
+// 0.06 ms, 9 launches included.
+constexpr int kMWalk = 64;
 // OWN: the limit is kMWalk, known when the loop is compiled.
 template <bool OWN>
-__global__ void k_m_jump(const int32_t *roots, int64_t nr, int32_t *par, int steps, unsigned long long *cut) {
+__global__ void k_m_jump(const int32_t *roots, int64_t nr, int32_t *par, int steps, int32_t *list, unsigned long long *cut) {
     const int limit = OWN ? kMWalk : steps;
-    bool any = false;
     for (int64_t ix = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; ix < nr;
          ix += (int64_t)gridDim.x * blockDim.x) {
         int x = roots[ix];
@@ -368,22 +365,17 @@ __global__ void k_m_jump(const int32_t *roots, int64_t nr, int32_t *par, int ste
             r = rr;
             atomicExch(par + x, r);  // not a store: other CTAs read these lines meanwhile
         }
-        any |= it == limit;
+        if (it == limit) list_cut(list, cut, x);
     }
-    if (__syncthreads_or(any) && threadIdx.x == 0) atomicOr(cut, 1ull);
 }
-struct RootItem {
-    const int32_t *roots;
-    __device__ __forceinline__ int64_t operator()(int64_t i) const { return roots[i]; }
-};
 // Jumping rounds for the walks that were cut (cut[1 .. 3]: their flags): nothing
-// to do unless one was.
-__global__ void __launch_bounds__(kBlock) k_m_settle(const int32_t *roots, int64_t nr, int32_t *par, unsigned long long *cut,
-                                                     BarRef ref) {
-    if (cut[0] == 0) return;  // the same for every CTA: written before this launch
+// to do unless some were.
+__global__ void __launch_bounds__(kBlock) k_m_settle(const int32_t *list, int32_t *par, unsigned long long *cut, BarRef ref) {
+    const int64_t n = (int64_t)cut[0];
+    if (n == 0) return;  // the same for every CTA: written before this launch
     GridBar bar(ref);
     if (bar.stopped()) return;
-    const JumpEnd e = jump_rounds(bar, nr, RootItem{roots}, par, cut + 1);
+    const JumpEnd e = jump_rounds(bar, n, ListItem{list}, par, cut + 1);
     if (e == kJumpBarrier) return;
     if (e == kJumpBound && threadIdx.x == 0) bar.stop(kStopJump);
     bar.finish();
@@ -510,6 +502,10 @@ __device__ __forceinline__ void bid_u128(ulonglong2 *sa, u128 ka, ulonglong2 *sb
             if ((ob = cas_u128(sb, cb, kb)) == cb) break;
 }
 
+// Limit of a walk in k_m_forest. A path of 3M edges whose gaps fall took 1.3 s
+// there; it and k_m_labels take 1.2 ms cut at 256 steps (0.77 at 64, but then
+// relays of 30,000 edges stop and start again too, for 0.03 ms more).
+constexpr int kMCut = 256;
 // The root above label x after the hooks; x's own pointer is moved there when
 // the way was longer than one step (by an exchange, not a store: other CTAs
 // read these lines meanwhile). A walk is cut after `limit` steps, which *cut
@@ -956,14 +952,14 @@ dgec_status stage_msf(Ctx *c, const Problem &p, const Csr &g, const Skel &sk, Ms
             TK(c, "k_m_hook", k_m_hook<<<grk, kBlock, 0, st>>>(roots, nr, bw, buv, s.bp, s.win, cu, cv, cw, g.rank_of,
                                                             round == 0 ? g.orig_of : nullptr, s.par, s.fe, s.cnt + 4));
             CU_TRY(c, cudaMemsetAsync(s.cnt, 0, 4 * sizeof(unsigned long long), st));
-            if (c->own_walk(kMWalk)) TK(c, "k_m_jump", k_m_jump<true><<<gr, kBlock, 0, st>>>(roots, nr, s.par, kMWalk, s.cnt));
-            else TK(c, "k_m_jump", k_m_jump<false><<<gr, kBlock, 0, st>>>(roots, nr, s.par, c->walk_steps, s.cnt));
+            if (c->own_walk(kMWalk)) TK(c, "k_m_jump", k_m_jump<true><<<gr, kBlock, 0, st>>>(roots, nr, s.par, kMWalk, s.win, s.cnt));
+            else TK(c, "k_m_jump", k_m_jump<false><<<gr, kBlock, 0, st>>>(roots, nr, s.par, c->walk_steps, s.win, s.cnt));
             {
                 int grid = 1;
                 DG_TRY(coop_grid(c, kCoopMJump, (const void *)k_m_settle, kBlock, 0, &grid));
                 unsigned long long *cut = s.cnt;
                 BarRef ref = c->next_bar();
-                void *args[] = {&roots, &nr, &s.par, &cut, &ref};
+                void *args[] = {&s.win, &s.par, &cut, &ref};  // (win: read by the hooks, next written by the claims)
                 cudaError_t e;
                 TK(c, "k_m_settle", e = cudaLaunchCooperativeKernel((const void *)k_m_settle,
                                                                     dim3((unsigned)std::min({gr, grid, c->num_sms})), dim3(kBlock), args,
@@ -998,7 +994,7 @@ dgec_status stage_msf(Ctx *c, const Problem &p, const Csr &g, const Skel &sk, Ms
         // the kernel's first filter writes lb/kb: not the side its edges come from
         const LiveSide &in = s.side[which ^ 1], &out = s.side[which];
         MsfArgs f{nr, n, roots0, ccu, ccv, cu, cv, cw, g.rank_of, s.par, roots0 ? roots2 : roots, roots0 ? roots : roots2,
-                  s.bp, s.slot, s.slot2, in.lab, out.lab, in.key, out.key, s.fe, s.cnt, p.idbits, lbits, c->walk(kMWalk), c->next_bar()};
+                  s.bp, s.slot, s.slot2, in.lab, out.lab, in.key, out.key, s.fe, s.cnt, p.idbits, lbits, c->walk(kMCut), c->next_bar()};
         int grid = 1;
         DG_TRY(coop_grid(c, kCoopMsf, (const void *)k_m_forest, kBlock, 0, &grid));
         const int64_t want = cdiv(n > nr ? n : nr, kBlock * kRes);
