@@ -56,12 +56,6 @@ struct GridBar {
     }
 };
 
-// In-place pointer jumping, ptr[x] = ptr[ptr[x]], over the n pointers x =
-// item(i) (negative: none), in rounds until none moves. Pointers only move to
-// ancestors and fixed points are never written, so reading a neighbour's new
-// or old value is equally valid, and every distance to the fixed point at
-// least halves per round. flag[0 .. 2] are the rounds' flags in turn; flag[0]
-// is zero at the start and at the end.
 // The cut walks of a pass: their pointers' owners, in any order.
 __device__ __forceinline__ void list_cut(int32_t *list, unsigned long long *n, int x) {
     const unsigned m = __activemask();  // whichever lanes are here
@@ -71,11 +65,20 @@ __device__ __forceinline__ void list_cut(int32_t *list, unsigned long long *n, i
     at = __shfl_sync(m, at, leader);
     list[at + __popc(m & ((1u << lane_id()) - 1u))] = x;
 }
-// They alone are unsettled: the other walks ended at a fixed point.
+
+// The items of such a list. They alone are unsettled: the other walks ended at
+// a fixed point.
 struct ListItem {
     const int32_t *list;
     __device__ __forceinline__ int64_t operator()(int64_t i) const { return list[i]; }
 };
+
+// In-place pointer jumping, ptr[x] = ptr[ptr[x]], over the n pointers x =
+// item(i) (negative: none), in rounds until none moves. Pointers only move to
+// ancestors and fixed points are never written, so reading a neighbour's new
+// or old value is equally valid, and every distance to the fixed point at
+// least halves per round. flag[0 .. 2] are the rounds' flags in turn; flag[0]
+// is zero at the start and at the end.
 constexpr int kJumpRounds = 64;  // halvings of any distance below 2^31, twice over
 enum JumpEnd { kJumpDone, kJumpBarrier, kJumpBound };
 template <class Item>

@@ -1,6 +1,6 @@
 """Excess of mass on cluster trees of every shape the pass treats apart: deep
-spines (far above the height its first walk covers and above the 4,096 steps
-of a shortcut walk), several spines under one another, and bushy trees."""
+spines (far above the height its first walk covers and above the 64 steps of a
+shortcut walk), several spines under one another, and bushy trees."""
 import numpy as np
 import pytest
 
